@@ -131,7 +131,8 @@ typedef struct gbsbin_plan gbsbin_plan;
 typedef struct {
   double sum_P;              /* sum of the returned table (1 up to rounding on the folded grid) */
   double max_imag;           /* max |Im P~| before the real part is taken (round-off probe)    */
-  double min_pivot_re;       /* min over evaluated points of min_i Re u_ii (> 0 in theory)     */
+  double min_pivot_re;       /* min over evaluated points of min_i Re u_ii (one group: of the factors
+                                1 - w lambda_i); > 0 in theory                                 */
   long long n_bad_points;    /* evaluated points with a pivot Re <= 0 or a non-finite value    */
   long long n_points;        /* grid points prod(oversample (N_l + 1))                         */
   long long n_evaluated;     /* points evaluated: conjugate symmetry halves the last axis      */
@@ -162,11 +163,12 @@ typedef enum {
   GBSBIN_KERNEL_BLK_TC_FP32R = 7,  /* as 6, the trace-correction updates on the tensor
                                       cores (tcgen05, 3 x TF32, TMEM accumulator)         */
   GBSBIN_KERNEL_HESS_FP64 = 8,     /* one detector group (L = 1, the total photon number of
-                                      Sec. VIII): D(w) = w I, so one Hessenberg reduction
-                                      XA = Q H Q^H per state (host) serves every point,
-                                      O(n^2) per point (warp per point, FP64), displacement
-                                      through Q^T gamma and Q^H X gamma; chosen
-                                      automatically for GBSBIN_FP64 plans with L = 1       */
+                                      Sec. VIII): D(w) = w I and XA is Hermitian, so one
+                                      spectral decomposition XA = Q Lambda Q^H per state (host)
+                                      serves every point, O(n) per point: log det K(w) =
+                                      sum Log(1 - w lambda_i), displacement through Q^T gamma
+                                      and Q^H X gamma; FP64; chosen automatically for
+                                      GBSBIN_FP64 plans with L = 1                          */
   GBSBIN_KERNEL_FOCK_FP64 = 9,     /* Fock inputs (gbsbin_fock_*): FP64 throughout           */
   GBSBIN_KERNEL_FOCK_DF32 = 10,    /* Fock inputs: pairs of FP32 (hi + lo, ~46 bits) on the
                                       FMA pipe, running sums flushed to FP64               */
@@ -200,8 +202,7 @@ typedef enum {
                                       the same conditions                                   */
   GBSBIN_KERNEL_HERALD_FP64 = 15,  /* heralded states (gbsbin_herald_*): CTA per point, FP64;
                                       not a choice for gbsbin_plan_create                   */
-  GBSBIN_KERNEL_HESS_DF32 = 16     /* as 8 in pairs of FP32 on the FMA pipe (H, a, c stored as
-                                      pairs; FP64 results); chosen automatically for
+  GBSBIN_KERNEL_HESS_DF32 = 16     /* as 8 (FP64 throughout), the automatic choice of
                                       GBSBIN_FP32_REFINE plans with L = 1, also in batches   */
 } gbsbin_kernel;
 

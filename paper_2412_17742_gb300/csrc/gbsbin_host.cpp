@@ -42,12 +42,18 @@ struct gbsbin_plan {
   longlong2* d_NXA_fix = nullptr;
   double* d_ldfin = nullptr;          // warp kernel: unfinished log det per evaluated point
   unsigned* d_bar = nullptr;          // grid-barrier state of the fused DFT launch
-  double2* d_H = nullptr;             // Hessenberg form of XA (one-group, undisplaced plans)
+  // one-group plans: the spectral form of XA (device arrays in d_state) and what G = q / q(1) needs
+  const double* d_lam = nullptr;
+  const double2* d_gq = nullptr;
+  double lam_min = 0.0, lam_max = 0.0, sp_rt0 = 1.0;
+  int sp_e0 = 0;
+  double2 sp_ex0 = make_double2(0.0, 0.0);
   // tree plans: rows ordered by group (tree_perm[new] = old), depth-0 arrays in d_state,
   // depths 1 .. L-1 in d_tree
   std::vector<int> tree_perm;
   TreeArgs tree{};
-  bool tree_g = false;                // undisplaced tree plan: leaves write G, the DFT skips a stage
+  bool tree_g = false;                // undisplaced tree plan, or a one-group plan that is no shard: the
+                                      // point kernel writes G, the DFT skips a stage
   double tree_logq0 = 0.0;            // Re log q(1) from the host LU (diagnostics)
   unsigned char* d_tree = nullptr;
   // large-matrix tree plans (kernels 13, 14): the same row order, depth-0 augmented matrix in
@@ -418,7 +424,7 @@ int build_state(const gbsbin_problem* p, int n, std::vector<cd>& XA, std::vector
 void free_device(gbsbin_plan* P) {
   if (P->d_twdf) cudaFree(P->d_twdf);
   void* ptrs[] = {P->d_state, P->d_label, P->d_logq,  P->d_minpiv, P->d_bufA, P->d_bufB, P->d_tw,
-                  P->d_diag,  P->d_gws,   P->d_table, P->d_ldfin,  P->d_bar,  P->d_H,    P->d_tree};
+                  P->d_diag,  P->d_gws,   P->d_table, P->d_ldfin,  P->d_bar,  P->d_tree};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   for (int b = 0; b < 2; ++b) {
@@ -453,6 +459,7 @@ inline bool is_btree(int kernel) { return kernel == GBSBIN_KERNEL_BTREE_DF32 || 
 size_t tree_region_slots(int n, int kernel) {
   if (is_tree(kernel)) return (size_t)n * n + 2 * (size_t)n + 3;   // permuted XA, X gamma, gamma, path record
   if (is_btree(kernel)) return (size_t)(n + 1) * (n + 1) + 2;    // augmented matrix, path record
+  if (is_hess(kernel)) return (size_t)n + ((size_t)n + 1) / 2;    // g products, eigenvalues
   return 0;
 }
 
@@ -493,12 +500,12 @@ void split(cd v, float2* hi, float2* lo) {
   *lo = make_float2((float)(v.real() - (double)hr), (float)(v.imag() - (double)hi_));
 }
 
-int upload_hessenberg(gbsbin_plan* P, cudaStream_t stream);
+int spectral_state(gbsbin_plan* P, double2* gq, double* lam);
 
 // Stage the state and enqueue its upload on `stream`.
 int upload_state(gbsbin_plan* P, cudaStream_t stream) {
   const int n = P->n;
-  const bool tree = is_tree(P->kernel) || is_btree(P->kernel);
+  const bool tree = is_tree(P->kernel) || is_btree(P->kernel) || is_hess(P->kernel);
   const bool per_point = !tree || P->opt.want_backward;   // the reverse pass reads -XA, gamma, X gamma
   Stage s = stage_layout(n, tree_region_slots(n, P->kernel));
   // the copy that last read this staging buffer (two uploads back) must have finished
@@ -554,6 +561,10 @@ int upload_state(gbsbin_plan* P, cudaStream_t stream) {
     A0[n * D + n] = slot(cd(0.0, 0.0));                   // the exponent collected so far
     A0[D * D] = slot(cd(1.0, 0.0));                       // path record: pivot product
     A0[D * D + 1] = make_float4(0.f, 0.f, 3.0e38f, 0.f);  // argument sum, power of two, min Re pivot
+  } else if (is_hess(P->kernel)) {                 // the spectral form
+    double2* gq = (double2*)(h + s.off_tree);
+    const int st = spectral_state(P, gq, (double*)(gq + n));
+    if (st) return st;
   } else if (tree) {                               // depth 0 of the tree: the permuted state
     float4* A0 = (float4*)(h + s.off_tree);
     float4* c0 = A0 + (size_t)n * n;
@@ -630,83 +641,38 @@ int upload_state(gbsbin_plan* P, cudaStream_t stream) {
   P->upload_bytes = (long long)(s.total - off);
   e = cudaMemcpyAsync(P->d_state + off, h + off, s.total - off, cudaMemcpyHostToDevice, stream);
   if (e != cudaSuccess || cudaEventRecord(P->ev_stage[sb], stream) != cudaSuccess) return GBSBIN_ERR_CUDA;
-  if (is_hess(P->kernel)) return upload_hessenberg(P, stream);
   return GBSBIN_OK;
 }
 
-// In place: A (n x n, row-major) <- Q^H A Q upper Hessenberg, Q a product of Householder
-// reflectors (FP64); each reflector is also applied to the vectors in `vecs` (which become
-// Q^H vec).  Similar matrices share det(I - w A) for every w.
-void hessenberg(std::vector<cd>& A, int n, std::vector<std::vector<cd>*> vecs = {}) {
-  std::vector<cd> v(n), sv(n);
-  for (int k = 0; k + 2 < n; ++k) {
-    double nrm2 = 0.0;
-    for (int i = k + 1; i < n; ++i) nrm2 += std::norm(A[(size_t)i * n + k]);
-    if (nrm2 == 0.0) continue;
-    const double nrm = std::sqrt(nrm2);
-    const cd x0 = A[(size_t)(k + 1) * n + k];
-    const double ax0 = std::abs(x0);
-    const cd alpha = (ax0 > 0.0 ? -x0 / ax0 : cd(-1.0, 0.0)) * nrm;   // -e^{i arg x0} ||x||
-    for (int i = k + 1; i < n; ++i) v[i] = A[(size_t)i * n + k];
-    v[k + 1] -= alpha;
-    double vn2 = 0.0;
-    for (int i = k + 1; i < n; ++i) vn2 += std::norm(v[i]);
-    if (vn2 == 0.0) continue;
-    const double beta = 2.0 / vn2;
-    // rows k+1.. : A <- (I - beta v v^H) A
-    for (int j = 0; j < n; ++j) sv[j] = 0.0;
-    for (int i = k + 1; i < n; ++i) {
-      const cd vc = std::conj(v[i]);
-      const cd* row = &A[(size_t)i * n];
-      for (int j = 0; j < n; ++j) sv[j] += vc * row[j];
-    }
-    for (int i = k + 1; i < n; ++i) {
-      const cd vi = beta * v[i];
-      cd* row = &A[(size_t)i * n];
-      for (int j = 0; j < n; ++j) row[j] -= vi * sv[j];
-    }
-    // columns k+1.. : A <- A (I - beta v v^H)
-    for (int i = 0; i < n; ++i) {
-      cd* row = &A[(size_t)i * n];
-      cd t = 0.0;
-      for (int j = k + 1; j < n; ++j) t += row[j] * v[j];
-      t *= beta;
-      for (int j = k + 1; j < n; ++j) row[j] -= t * std::conj(v[j]);
-    }
-    for (std::vector<cd>* x : vecs) {           // x <- (I - beta v v^H) x
-      cd t = 0.0;
-      for (int i = k + 1; i < n; ++i) t += std::conj(v[i]) * (*x)[i];
-      t *= beta;
-      for (int i = k + 1; i < n; ++i) (*x)[i] -= t * v[i];
-    }
-    A[(size_t)(k + 1) * n + k] = alpha;
-    for (int i = k + 2; i < n; ++i) A[(size_t)i * n + k] = 0.0;
-  }
-}
-
-// The one-group plans' Hessenberg form of the current XA, followed by a = Q^T gamma and
-// c = Q^H X gamma (the exponent gamma^T (conj(w) - XA)^{-1} X gamma = a^T (conj(w) - H)^{-1} c),
-// uploaded on `stream`.
-int upload_hessenberg(gbsbin_plan* P, cudaStream_t stream) {
+// The one-group plans' spectral form of the current state: the eigenvalues of XA = Q Lambda Q^H, the
+// products g_i = (Q^T gamma)_i (Q^H X gamma)_i of the displacement term, and q at w = 1 from them.
+int spectral_state(gbsbin_plan* P, double2* gq, double* lam) {
   const int n = P->n;
-  std::vector<cd> H(P->XA), ga(n), c(P->Xgamma);
+  std::vector<cd> ga(n), c(P->Xgamma);
   for (int i = 0; i < n; ++i) ga[i] = std::conj(P->gamma[i]);     // Q^T g = conj(Q^H conj(g))
-  hessenberg(H, n, {&ga, &c});
-  std::vector<double2> h((size_t)n * n + 2 * (size_t)n);
-  for (size_t q = 0; q < (size_t)n * n; ++q) h[q] = make_double2(H[q].real(), H[q].imag());
+  std::vector<std::vector<cd>*> vecs;
+  if (P->has_gamma) vecs = {&ga, &c};
+  std::vector<double> ev;
+  if (!hermitian_spectrum(P->XA, n, ev, vecs)) return GBSBIN_ERR_NUMERIC;
+  P->lam_min = *std::min_element(ev.begin(), ev.end());
+  P->lam_max = *std::max_element(ev.begin(), ev.end());
+  double p0 = 1.0;
+  int e0 = 0;
+  cd ex0 = 0.0;
   for (int i = 0; i < n; ++i) {
-    h[(size_t)n * n + i] = make_double2(ga[i].real(), -ga[i].imag());
-    h[(size_t)n * n + n + i] = make_double2(c[i].real(), c[i].imag());
+    const cd g = P->has_gamma ? std::conj(ga[i]) * c[i] : cd(0.0);
+    gq[i] = make_double2(g.real(), g.imag());
+    lam[i] = ev[i];
+    int ex;
+    p0 = std::frexp(p0 * (1.0 - ev[i]), &ex);
+    e0 += ex;
+    ex0 += g / (1.0 - ev[i]);
   }
-  if (P->kernel == GBSBIN_KERNEL_HESS_DF32)        // pairs of FP32 in the same 16-byte slots
-    for (size_t q = 0; q < h.size(); ++q) {
-      const float4 f = split4(cd(h[q].x, h[q].y));
-      std::memcpy(&h[q], &f, sizeof(f));
-    }
-  // a pageable source: the call returns once the data are staged, so h may go out of scope
-  if (cudaMemcpyAsync(P->d_H, h.data(), h.size() * sizeof(double2), cudaMemcpyHostToDevice, stream) != cudaSuccess)
-    return GBSBIN_ERR_CUDA;
-  P->upload_bytes += (long long)(h.size() * sizeof(double2));
+  P->sp_rt0 = std::sqrt(p0);
+  P->sp_e0 = e0;
+  P->sp_ex0 = make_double2(ex0.real(), ex0.imag());
+  P->tree_g = P->grid.e_lo == 0 && P->grid.e_hi == P->grid.n_full;
+  P->tree_logq0 = 0.5 * ex0.real() - 0.5 * (std::log(p0) + e0 * 0.693147180559945309417232121458);
   return GBSBIN_OK;
 }
 
@@ -1317,10 +1283,9 @@ static int plan_create_impl(const gbsbin_problem* p, const gbsbin_options* o, gb
     }
     btree_pointers(P, sl);
   }
-  if (is_hess(P->kernel) && (st = dalloc(&P->d_H, nn + 2 * (size_t)n))) {
-    free_device(P);
-    delete P;
-    return st;
+  if (is_hess(P->kernel)) {
+    P->d_gq = (const double2*)(P->d_state + sl.off_tree);
+    P->d_lam = (const double*)(P->d_gq + n);
   }
   if (alloc_gws && (P->kernel == GBSBIN_KERNEL_GMEM_FP64 || P->kernel == GBSBIN_KERNEL_GMEM_FP32R ||
                     is_blk(P->kernel))) {
@@ -1479,7 +1444,14 @@ static PointArgs make_point_args(gbsbin_plan* P) {
   a.gws = P->d_gws;
   a.gws_slot_bytes = P->gws_slot_bytes;
   a.ldfin = P->d_ldfin;
-  a.H = P->d_H;
+  a.lam = P->d_lam;
+  a.gq = P->d_gq;
+  a.lam_min = P->lam_min;
+  a.lam_max = P->lam_max;
+  a.gout = is_hess(P->kernel) && P->tree_g ? P->d_bufA : nullptr;
+  a.sp_e0 = P->sp_e0;
+  a.sp_rt0 = P->sp_rt0;
+  a.sp_ex0 = P->sp_ex0;
   return a;
 }
 
@@ -1497,6 +1469,7 @@ static DftArgs make_dft_args(gbsbin_plan* P, double* P_out) {
   d.minpiv = P->d_minpiv;
   d.table_size = P->table_size;
   d.df = P->kernel == GBSBIN_KERNEL_TREE_DF32 ? 1 : 0;
+  d.g_ready = is_hess(P->kernel) && P->tree_g ? 1 : 0;
   return d;
 }
 
@@ -1556,7 +1529,7 @@ int gbsbin_execute(gbsbin_plan* P, double* P_out, void* stream) {
                                                                                              : GBSBIN_ERR_CUDA;
   }
   cudaError_t e = P->kernel == GBSBIN_KERNEL_WARP_FP32R  ? launch_points_warp(a, P->num_sms, s)
-                  : is_hess(P->kernel) ? launch_points_hess(a, PointBatch{}, 0, P->num_sms, s, P->kernel == GBSBIN_KERNEL_HESS_DF32)
+                  : is_hess(P->kernel) ? launch_points_spectral(a, P->num_sms, s)
                   : is_blk(P->kernel) ? launch_points_blk(a, PointBatch{}, 0, P->num_sms, s, P->kernel == GBSBIN_KERNEL_BLK_TC_FP32R)
                                                          : launch_points(a, P->kernel, P->num_sms, s);
   if (e != cudaSuccess) return GBSBIN_ERR_CUDA;
@@ -1604,7 +1577,7 @@ int gbsbin_diagnostics(gbsbin_plan* P, gbsbin_diag* out, void* stream) {
   out->max_imag = h[1];
   out->min_pivot_re = h[2];
   out->n_bad_points = (long long)h[3];
-  out->log_q1_re = (is_tree(P->kernel) && P->tree_g) ? P->tree_logq0 : h[4];
+  out->log_q1_re = P->tree_g ? P->tree_logq0 : h[4];
   out->n_points = P->grid.npts;
   out->n_evaluated = P->grid.n_eval;
   out->table_size = P->table_size;
@@ -1642,7 +1615,7 @@ int gbsbin_read_points(gbsbin_plan* P, double* logq_host, double* minpiv_host, v
   cudaStream_t s = (cudaStream_t)stream;
   const size_t ne = (size_t)P->grid.n_eval;
   // plans whose DFT took G directly left log q unfinished
-  if (is_tree(P->kernel) && P->tree_g &&
+  if (P->tree_g &&
       launch_finish_logq(P->d_ldfin, P->d_logq, (long long)ne, s) != cudaSuccess)
     return GBSBIN_ERR_CUDA;
   if (cudaMemcpyAsync(logq_host, P->d_logq, ne * sizeof(double2), cudaMemcpyDeviceToHost, s) != cudaSuccess)
@@ -1658,7 +1631,7 @@ int gbsbin_read_points(gbsbin_plan* P, double* logq_host, double* minpiv_host, v
 static int backward_enqueue(gbsbin_plan* P, const double* dLdP, cudaStream_t s) {
   int st = GBSBIN_OK;
   if (!P->logq_valid && (st = gbsbin_execute(P, P->d_table, s))) return st;   // log q of the current state
-  if (is_tree(P->kernel) && P->tree_g &&        // the tree's DFT took G directly: finish log q
+  if (P->tree_g &&                              // the DFT took G directly: finish log q
       launch_finish_logq(P->d_ldfin, P->d_logq, P->grid.n_eval, s) != cudaSuccess)
     return GBSBIN_ERR_CUDA;
   BackwardArgs b{};
@@ -2765,7 +2738,7 @@ int batch_launch(gbsbin_batch* B, double* const* P_out, cudaStream_t s) {
     if (cudaMemsetAsync(B->d_queue + c, 0, sizeof(unsigned long long), s) != cudaSuccess) return GBSBIN_ERR_CUDA;
     PointBatch pb{B->d_probs, C.d_jobs, (long long)C.jobs.size(), B->d_queue + c};
     cudaError_t e = C.kernel == GBSBIN_KERNEL_WARP_FP32R  ? launch_points_warp_batch(pb, C.np, B->num_sms, s)
-                    : is_hess(C.kernel) ? launch_points_hess(PointArgs{}, pb, C.np, B->num_sms, s, C.kernel == GBSBIN_KERNEL_HESS_DF32)
+                    : is_hess(C.kernel) ? launch_points_spectral_batch(pb, s)
                     : is_blk(C.kernel) ? launch_points_blk(PointArgs{}, pb, C.smem, B->num_sms, s, C.kernel == GBSBIN_KERNEL_BLK_TC_FP32R)
                                                           : launch_points_batch(pb, C.kernel, C.threads, C.smem, B->num_sms, s);
     if (e != cudaSuccess) return GBSBIN_ERR_CUDA;
@@ -2846,7 +2819,7 @@ int gbsbin_batch_create(const gbsbin_problem* probs, int nprob, const gbsbin_opt
         if (T) gbsbin_plan_destroy(T);
       }
     }
-    // one-group problems keep the Hessenberg path whatever the size's tuning
+    // one-group problems keep the spectral path whatever the size's tuning
     const bool one_group = probs[i].L == 1;
     if (autotune && !opt.tile_override && n <= GBSBIN_MAX_N && !one_group) {
       TuneVal v{};
@@ -2871,11 +2844,9 @@ int gbsbin_batch_create(const gbsbin_problem* probs, int nprob, const gbsbin_opt
                         : is_blk(P->kernel) ? 256
                                                                : points_threads(P->kernel, P->n);
     // warp kernel: padded size class; blocked kernel: problems whose shared memory allows
-    // two CTAs per SM run apart from the larger ones (a class launches with its largest need);
-    // Hessenberg kernels: the row slots per lane of the instantiation
+    // two CTAs per SM run apart from the larger ones (a class launches with its largest need)
     const int np = P->kernel == GBSBIN_KERNEL_WARP_FP32R ? (P->n <= 8 ? 8 : P->n <= 16 ? 16 : 32)
                    : is_blk(P->kernel) ? points_blk_ctas_per_sm(P->n)
-                   : is_hess(P->kernel) ? hess_slots(P->n)
                                                           : 0;
     auto key = std::make_tuple(P->kernel, threads, np);
     if (!class_of.count(key)) {
@@ -2886,7 +2857,7 @@ int gbsbin_batch_create(const gbsbin_problem* probs, int nprob, const gbsbin_opt
       B->classes.back().np = np;
     }
     auto& C = B->classes[class_of[key]];
-    const int group = (P->kernel == GBSBIN_KERNEL_WARP_FP32R || is_hess(P->kernel)) ? 4 : P->P;
+    const int group = P->kernel == GBSBIN_KERNEL_WARP_FP32R ? 4 : is_hess(P->kernel) ? GBSBIN_SPECTRAL_BATCH_POINTS : P->P;
     for (long long e0 = 0; e0 < P->grid.n_eval; e0 += group) C.jobs.push_back(PointJob{i, 0, e0});
     if (P->kernel == GBSBIN_KERNEL_SMEM_FP64 || P->kernel == GBSBIN_KERNEL_SMEM_FP32R ||
         P->kernel == GBSBIN_KERNEL_GMEM_FP64 || P->kernel == GBSBIN_KERNEL_GMEM_FP32R)

@@ -54,7 +54,13 @@ struct PointArgs {
   const float2* g_lo;       // n
   const int* label;         // n: detector group of each row
   const double2* tw;        // twiddles exp(-2 pi i m / radix[l]), m < radix[l], axis after axis
-  const double2* H;         // one-group plans: Hessenberg form of XA, n*n FP64 (else nullptr)
+  const double* lam;        // one-group plans: the eigenvalues of XA (n) and, per eigenvector, the
+  const double2* gq;        // product (Q^T gamma)_i (Q^H X gamma)_i (else nullptr)
+  double lam_min, lam_max;  // the smallest and the largest eigenvalue
+  double2* gout;            // one-group plans: G = q / q(1) per point (nullptr: not wanted), from
+  int sp_e0;                // prod (1 - lambda_i) = sp_rt0^2 2^sp_e0 and the displacement term at w = 1
+  double sp_rt0;
+  double2 sp_ex0;
   GridDesc grid;
   double2* logq;            // n_eval outputs: log q at each evaluated point
   double* minpiv;           // n_eval outputs: min_i Re u_ii
@@ -272,13 +278,11 @@ size_t points_blk_slot_bytes(int n);
 int points_blk_ctas_per_sm(int n);   // resident CTAs per SM that the shared memory allows (1 or 2)
 cudaError_t launch_points_blk(const PointArgs& a, const PointBatch& batch, size_t smem_batch, int num_sms,
                               cudaStream_t s, bool tensor_cores);
-// One-group (L = 1) undisplaced kernel (gbsbin_points_hess.cu): warp per point, four
-// points per CTA; batch jobs are groups of four consecutive points of one problem.
-// slots: row slots per lane of the instantiation (hess_slots(n) for the largest n it serves;
-// 0: from a.n)
-cudaError_t launch_points_hess(const PointArgs& a, const PointBatch& batch, int slots, int num_sms, cudaStream_t s,
-                               bool df);
-int hess_slots(int n);
+// One-group (L = 1) kernel (gbsbin_points_spectral.cu), FP64; batch jobs are groups of
+// GBSBIN_SPECTRAL_BATCH_POINTS consecutive points of one problem.
+#define GBSBIN_SPECTRAL_BATCH_POINTS 16
+cudaError_t launch_points_spectral(const PointArgs& a, int num_sms, cudaStream_t s);
+cudaError_t launch_points_spectral_batch(const PointBatch& batch, cudaStream_t s);
 size_t points_smem_bytes(int kernel, int n, int P, int L);
 size_t points_matrix_bytes(int kernel, int n, int P);
 int points_per_cta(int kernel, int n, int L);
