@@ -535,7 +535,11 @@ int gbsbin_prob_distinguishable_device(const gbsbin_problem* p, const int* patte
  * gbsbin_execute: the folded table P~(b), 0 <= b_l <= N_l, which is P(b) itself when every
  * N_l >= N (no group sees more than N photons).
  * Work: prod over the other occupied inputs of (p_k + 1) nodes x (half the output grid)
- * points, each factor O(L).  Options: precision GBSBIN_FP64 (kernel 9) or
+ * points, each factor O(L).  Where it costs less (no shard, automatic kernel choice), the plan takes
+ * the table's coefficients directly instead: the product of half the factors (B(z) x)_j as a polynomial in z
+ * per sub-multiset of the photons, for both halves, then the sum over complementary sub-multisets, in
+ * integer arithmetic of 50 bits or more for either precision (kernel 9 or 10 is reported as asked for).
+ * Options: precision GBSBIN_FP64 (kernel 9) or
  * GBSBIN_FP32_REFINE, which here selects pairs of FP32 (kernel 10); oversample,
  * want_diagnostics, want_timing and tile_override (9 or 10) as for gbsbin_plan_create;
  * want_backward is not supported (ERR_UNSUPPORTED).  shard_begin/shard_end select a range

@@ -1,0 +1,59 @@
+// Fock inputs by a convolution over sub-multisets of the photons: the interface between the host plan
+// (gbsbin_fock_host.cpp) and the kernels (gbsbin_fock_conv.cu).  Not part of the public ABI.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "gbsbin_internal.h"
+
+namespace gbsbin {
+
+#define GBSBIN_FC_NONE (-(1 << 28))       // exponent of an all-zero state or column
+
+// Coefficients in fixed point, round(b 2^kConvRowBits / 2^rowexp): components below 2^56, and a row's sum of
+// component magnitudes below 2^60, which keeps a layer's 64-bit sums (digits of 26 bits) below 2^62 and its
+// results four bits finer than a state's 52.
+constexpr int kConvRowBits = 56;
+struct FockConvArgs {
+  int nin, L, N, h[2];                    // occupied inputs, groups, photons, factors of each half
+  int stride[GBSBIN_FOCK_MAX_IN];         // code of a state m: sum m_k stride[k]
+  int radix[GBSBIN_FOCK_MAX_IN];          // p_k + 1
+  int full;                               // code of p
+  const int* rank;                        // code -> index within its layer
+  const int* order;                       // layer after layer: index -> code
+  const int* down;                        // [t][e]: monomial e without z_{t-1} (t = 0: e itself), -1: none
+  int ndown;                              // monomials of degree <= h[1] (the stride of `down`)
+  const longlong2* B;                     // [row][k][t], fixed point
+  const int4* F0;                         // the empty product: digits of 2^51, and its exponent 1
+  const int* E0;
+  int4* F[2][2];                          // [half][parity]: state x monomial, digits (re hi, lo, im hi, lo)
+  int* E[2][2];                           // [half][parity]: the state's exponent
+  int nd;                                 // digits of the sum over states: 2 (25 bits) or 3 (20 bits)
+  int2* F3[2];                            // with three: the last layers' third digits (re, im)
+  int* colexp[2];                         // per monomial of the last layer: exponent of its largest entry
+  int states, first, n1, n2;              // last layer of the first half: states, its codes in order; monomials
+                                          // of each half
+  int chunk, nchunks;                     // states per contraction CTA
+  int exponent;                           // sum of the rows' exponents
+  double2* parts;                         // nchunks x n1 x n2
+  const int* pair_first;                  // table entry -> its pairs (a n2 + b) in pair_list
+  const int* pair_list;
+  long long table_size;
+  double* P;
+  double* diag;
+};
+// One layer r >= 1 of both halves (those that reach it): states of r photons, nc monomials of degree
+// <= r, nc0 of degree <= r - 1; order[first ..] are its codes.  `last[half]` asks for the column maxima.
+struct FockConvLayer {
+  int r, states, first, nc, nc0, row[2];  // row[half]: row of B of this layer's factor
+  int halves, half0;                      // number of halves that reach this layer, and the first of them
+  int last[2];
+};
+constexpr int kConvRows = 24, kConvCols = 16;   // monomials of either half per contraction CTA
+constexpr int kConvMaxChunk = 1024;       // states per CTA: the 64-bit sums stay below 2^62
+int fock_conv_slots_per_sm(int nd);           // resident contraction CTAs of an SM
+size_t fock_conv_layer_smem(int nin, int L, int nc);
+cudaError_t launch_fock_conv(const FockConvArgs& a, const FockConvLayer* layers, int nlayers, int num_sms,
+                             cudaStream_t s, int* launches);
+
+}  // namespace gbsbin

@@ -1,13 +1,16 @@
 // Host side of the Fock-input path (arXiv:2412.17742, App. C): validation, the FP64
 // coefficient matrices I - T^dag T and T_l^dag T_l restricted to the occupied inputs, the
-// node and output-group roots, device workspaces and the two launches (nodes x points,
-// then the inverse DFT of the output groups).
+// node and output-group roots, device workspaces and the launches: the convolution over
+// sub-multisets of the photons (gbsbin_fock_conv.cu) where it costs less, else nodes x points
+// and the inverse DFT of the output groups.
 #include <algorithm>
 #include <cmath>
 #include <complex>
+#include <cstring>
 #include <new>
 #include <vector>
 
+#include "gbsbin_fock_conv.h"
 #include "gbsbin_internal.h"
 
 using cd = std::complex<double>;
@@ -42,6 +45,12 @@ struct gbsbin_fock_plan {
   unsigned char* h_stage = nullptr;      // pinned copy of the state block
   size_t state_bytes = 0;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+  // the convolution (whole plans where it costs less than the node walk)
+  bool conv = false;
+  FockConvArgs cv{};
+  std::vector<FockConvLayer> layers;
+  unsigned char* d_conv = nullptr;       // its tables, states and partial sums
+  int last_launches = 0;
 };
 
 namespace {
@@ -65,7 +74,7 @@ int dalloc(T** p, size_t count) {
 
 void free_all(gbsbin_fock_plan* P) {
   void* ptrs[] = {P->d_state, P->d_xtw, P->d_xtw_df, P->d_zr, P->d_zr_df, P->d_tw, P->d_parts,
-                  P->d_bufA, P->d_bufB, P->d_diag, P->d_bar, P->d_table};
+                  P->d_bufA, P->d_bufB, P->d_diag, P->d_bar, P->d_table, P->d_conv};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   if (P->h_stage) cudaFreeHost(P->h_stage);
@@ -122,6 +131,257 @@ int stage_transfer(gbsbin_fock_plan* P, const gbsbin_complex* Tin) {
         coef[q] = make_double2(s.real(), s.imag());
         coef_df[q] = split_df(s);
       }
+  if (P->conv) {   // the same by rows in fixed point, each row scaled by a power of two
+    longlong2* B = reinterpret_cast<longlong2*>(P->h_stage + P->coef_count * (sizeof(double2) + sizeof(float4)));
+    P->cv.exponent = 0;
+    for (int j = 0; j < nin; ++j) {
+      auto at = [&](int k, int m) { return coef[((size_t)m * nin + k) * nin + j]; };
+      double big = 0.0, all = 0.0;
+      for (int k = 0; k < nin; ++k)
+        for (int m = 0; m <= L; ++m) {
+          big = std::fmax(big, std::fmax(std::fabs(at(k, m).x), std::fabs(at(k, m).y)));
+          all += std::fabs(at(k, m).x) + std::fabs(at(k, m).y);
+        }
+      int e = 0, ea = 0;
+      std::frexp(big, &e);                      // big < 2^e, all < 16 x 2^e
+      std::frexp(all * 1.0001, &ea);
+      e = std::max(e, ea - 4);
+      for (int k = 0; k < nin; ++k)
+        for (int m = 0; m <= L; ++m)
+          B[((size_t)j * nin + k) * (L + 1) + m] =
+              make_longlong2(std::llrint(std::ldexp(at(k, m).x, kConvRowBits - e)),
+                             std::llrint(std::ldexp(at(k, m).y, kConvRowBits - e)));
+      P->cv.exponent += e * P->args.pw[j];
+    }
+  }
+  return GBSBIN_OK;
+}
+
+// Whether the convolution serves the plan, with its layers and sizes: its estimated time (60 clocks
+// of a scheduler per warp's multiply-add, as measured, and ~3 us per launch) against the node walk's at its measured rates (1.25e13 FP32 operations a second, 63 per
+// factor, in pairs of FP32; 4.5e11 FP64 operations, 10 per factor).  Bounded: 2^22 states in all, 2^20 monomial
+// pairs and 2^22 table entries, 1 GB of states, 48 KB of shared memory per layer CTA.
+bool conv_layout(gbsbin_fock_plan* P) {
+  const FockArgs& a = P->args;
+  FockConvArgs& c = P->cv;
+  int N = 0;
+  double codes = 1.0;
+  for (int j = 0; j < a.nin; ++j) {
+    codes *= a.pw[j] + 1.0;
+    if (codes > (double)(1 << 22)) return false;
+    N += a.pw[j];
+  }
+  if (N < 4 || P->table_size > (1 << 22)) return false;
+  c.nin = a.nin;
+  c.L = a.L;
+  c.N = N;
+  c.nd = P->df ? 2 : 3;
+  c.h[0] = N / 2;
+  c.h[1] = N - N / 2;
+  std::vector<double> mono(c.h[1] + 1, 1.0);            // monomials of degree <= r in L variables
+  for (int r = 1; r <= c.h[1]; ++r) {
+    mono[r] = mono[r - 1] * (r + a.L) / r;
+    if (mono[r] > 4096.0) return false;
+  }
+  c.n1 = (int)std::lround(mono[c.h[0]]);
+  c.n2 = (int)std::lround(mono[c.h[1]]);
+  if ((double)c.n1 * c.n2 > (double)(1 << 20) || fock_conv_layer_smem(a.nin, a.L, c.n2) > 48 * 1024) return false;
+  // states per layer: coefficients of prod (1 + x + .. + x^p_j)
+  std::vector<double> cnt(1, 1.0);
+  for (int j = 0; j < a.nin; ++j) {
+    std::vector<double> nx(cnt.size() + a.pw[j], 0.0);
+    for (size_t u = 0; u < cnt.size(); ++u)
+      for (int v = 0; v <= a.pw[j]; ++v) nx[u + v] += cnt[u];
+    cnt.swap(nx);
+  }
+  std::vector<int> row;
+  for (int j = 0; j < a.nin; ++j)
+    for (int v = 0; v < a.pw[j]; ++v) row.push_back(j);
+  P->layers.clear();
+  double clocks = 0.0, bytes = 0.0;
+  int first = 1;
+  for (int r = 1; r <= c.h[1]; ++r) {
+    FockConvLayer y{};
+    y.r = r;
+    y.states = (int)cnt[r];
+    y.first = first;
+    first += y.states;
+    y.nc = (int)std::lround(mono[r]);
+    y.nc0 = (int)std::lround(mono[r - 1]);
+    y.halves = r <= c.h[0] ? 2 : 1;
+    y.half0 = y.halves == 2 ? 0 : 1;
+    for (int h = 0; h < 2; ++h) {
+      if (h == 0 && r > c.h[0]) continue;
+      y.row[h] = row[(h ? c.h[0] : 0) + r - 1];
+      y.last[h] = r == c.h[h];
+    }
+    clocks += y.halves * (double)y.states * std::min(r, a.nin) * ((y.nc + 31) / 32) * (a.L + 1);
+    bytes = std::fmax(bytes, 16.0 * y.states * (y.nc + 1.0));
+    P->layers.push_back(y);
+  }
+  c.states = (int)cnt[c.h[0]];
+  c.first = P->layers[c.h[0] - 1].first;
+  clocks += (c.nd - 1) * (double)c.states * ((c.n1 + 23) / 24 * 24.0) * ((c.n2 + 15) / 16 * 16.0) / 32.0;
+  if (4.0 * bytes > (double)(1 << 30)) return false;
+  const double t_conv = 60.0 * clocks / (4.0 * P->num_sms * 1.9e9) + 3e-6 * (P->layers.size() + 3);
+  const double pairs = (double)(a.x_hi - a.x_lo) * a.grid.n_full * N;
+  const double t_walk = (P->df ? pairs * 63.0 / 1.25e13 : pairs * 10.0 / 4.5e11) + 25e-6;
+  return t_conv < t_walk;
+}
+
+// Tables and workspaces of the convolution in one device block.
+int conv_setup(gbsbin_fock_plan* P) {
+  FockConvArgs& c = P->cv;
+  const FockArgs& a = P->args;
+  const int L = c.L, nin = c.nin, hi = c.h[1];
+  int codes = 1;
+  for (int j = 0; j < nin; ++j) {
+    c.stride[j] = codes;
+    c.radix[j] = a.pw[j] + 1;
+    codes *= c.radix[j];
+  }
+  c.full = codes - 1;
+  // codes by layer: sum of digits by an odometer, then a counting sort
+  std::vector<int> sum(codes), rank(codes, 0), order(P->layers.back().first + P->layers.back().states);
+  {
+    std::vector<int> next(hi + 1, 0), dig(nin, 0);
+    for (int r = 1; r <= hi; ++r) next[r] = P->layers[r - 1].first;
+    const std::vector<int> begin(next);
+    int s = 0;
+    for (int q = 0; q < codes; ++q) {
+      if (s <= hi) {
+        rank[q] = next[s] - begin[s];
+        order[next[s]++] = q;
+      }
+      for (int j = 0; j < nin; ++j) {
+        if (++dig[j] < c.radix[j]) {
+          ++s;
+          break;
+        }
+        s -= dig[j] - 1;
+        dig[j] = 0;
+      }
+    }
+  }
+  // monomials by degree (a layer's are a prefix), and each without one of its variables
+  std::vector<std::vector<int>> mono;
+  for (int d = 0; d <= hi; ++d) {
+    std::vector<int> e(L, 0);
+    e[L - 1] = d;
+    for (;;) {                                  // compositions of d, the last variable running down
+      mono.push_back(e);
+      int l = L - 1;
+      while (l > 0 && e[l] == 0) --l;
+      if (l == 0) break;
+      const int v = e[l];
+      e[l] = 0;
+      e[l - 1] += 1;
+      e[L - 1] = v - 1;
+    }
+  }
+  if ((int)mono.size() != c.n2) return GBSBIN_ERR_UNSUPPORTED;
+  c.ndown = c.n2;
+  std::vector<int> down((size_t)(L + 1) * c.n2, -1);
+  {
+    std::vector<std::pair<std::vector<int>, int>> idx;
+    for (int e = 0; e < c.n2; ++e) idx.emplace_back(mono[e], e);
+    std::sort(idx.begin(), idx.end());
+    for (int e = 0; e < c.n2; ++e) {
+      down[e] = e;
+      for (int l = 0; l < L; ++l)
+        if (mono[e][l] > 0) {
+          std::vector<int> f(mono[e]);
+          --f[l];
+          down[(size_t)(l + 1) * c.n2 + e] = std::lower_bound(idx.begin(), idx.end(), std::make_pair(f, -1))->second;
+        }
+    }
+  }
+  // the pairs (a, b) of each table entry: exponents add, folded modulo the radices
+  const GridDesc& g = a.grid;
+  c.table_size = P->table_size;
+  std::vector<int> to((size_t)c.n1 * c.n2), first(P->table_size + 1, 0), list;
+  for (int x = 0; x < c.n1; ++x)
+    for (int y = 0; y < c.n2; ++y) {
+      long long t = 0;
+      for (int l = 0; l < L && t >= 0; ++l) {
+        const int b = (mono[x][l] + mono[y][l]) % g.radix[l];
+        t = b < g.nout[l] ? t * g.nout[l] + b : -1;
+      }
+      to[(size_t)x * c.n2 + y] = (int)t;
+      if (t >= 0) ++first[t + 1];
+    }
+  for (long long t = 0; t < P->table_size; ++t) first[t + 1] += first[t];
+  list.resize(std::max(1, first[P->table_size]));
+  {
+    std::vector<int> next(first);
+    for (size_t q = 0; q < to.size(); ++q)
+      if (to[q] >= 0) list[next[to[q]]++] = (int)q;
+  }
+  // chunks of states: one wave of resident CTAs, at most kConvMaxChunk states each
+  const long long tiles = (long long)((c.n1 + kConvRows - 1) / kConvRows) * ((c.n2 + kConvCols - 1) / kConvCols);
+  const long long slots = (long long)std::max(1, fock_conv_slots_per_sm(c.nd)) * P->num_sms;
+  long long nch = std::max<long long>(1, slots / tiles);
+  nch = std::min<long long>(nch, (c.states + 31) / 32);
+  c.chunk = (int)std::min<long long>((c.states + nch - 1) / nch, kConvMaxChunk);
+  c.nchunks = (c.states + c.chunk - 1) / c.chunk;
+  // one block: offsets in 16-byte units
+  size_t at = 0;
+  auto take = [&at](size_t bytes) {
+    const size_t o = at;
+    at += (bytes + 15) / 16 * 16;
+    return o;
+  };
+  size_t fmax[2] = {0, 0}, emax = 0;
+  for (const FockConvLayer& y : P->layers) {
+    for (int h = y.half0; h < 2; ++h) fmax[h] = std::max(fmax[h], (size_t)y.states * (y.nc + 1));
+    emax = std::max(emax, (size_t)y.states);
+  }
+  const size_t o_rank = take(rank.size() * 4), o_order = take(order.size() * 4), o_down = take(down.size() * 4),
+               o_first = take(first.size() * 4), o_list = take(list.size() * 4), o_f0 = take(32), o_e0 = take(4),
+               o_c0 = take(((size_t)c.n1 + c.n2) * 4);
+  size_t o_F[2][2], o_E[2][2];
+  for (int h = 0; h < 2; ++h)
+    for (int p = 0; p < 2; ++p) {
+      o_F[h][p] = take(fmax[h] * 16);
+      o_E[h][p] = take(emax * 4);
+    }
+  size_t o_F3[2] = {0, 0};
+  for (int h = 0; h < 2 && c.nd == 3; ++h) o_F3[h] = take((size_t)c.states * ((h ? c.n2 : c.n1) + 1) * 8);
+  const size_t o_parts = take((size_t)c.nchunks * c.n1 * c.n2 * 16);
+  const int st = dalloc(&P->d_conv, at);
+  if (st) return st;
+  unsigned char* d = P->d_conv;
+  const int f0[8] = {1 << 25, 0, 0, 0, 0, 0, 0, 0}, e0 = 1;   // 1 = 2^51 2^-52 2^1, then the row's zero entry
+  std::vector<unsigned char> tables(o_c0);               // the tables come first: one copy
+  auto put = [&tables](size_t o, const void* src, size_t bytes) { std::memcpy(tables.data() + o, src, bytes); };
+  put(o_rank, rank.data(), rank.size() * 4);
+  put(o_order, order.data(), order.size() * 4);
+  put(o_down, down.data(), down.size() * 4);
+  put(o_first, first.data(), first.size() * 4);
+  put(o_list, list.data(), list.size() * 4);
+  put(o_f0, f0, 32);
+  put(o_e0, &e0, 4);
+  if (cudaMemcpy(d, tables.data(), tables.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
+    cudaGetLastError();
+    return GBSBIN_ERR_CUDA;
+  }
+  c.rank = (const int*)(d + o_rank);
+  c.order = (const int*)(d + o_order);
+  c.down = (const int*)(d + o_down);
+  c.pair_first = (const int*)(d + o_first);
+  c.pair_list = (const int*)(d + o_list);
+  c.F0 = (const int4*)(d + o_f0);
+  c.E0 = (const int*)(d + o_e0);
+  c.colexp[0] = (int*)(d + o_c0);
+  c.colexp[1] = c.colexp[0] + c.n1;
+  for (int h = 0; h < 2; ++h)
+    for (int p = 0; p < 2; ++p) {
+      c.F[h][p] = (int4*)(d + o_F[h][p]);
+      c.E[h][p] = (int*)(d + o_E[h][p]);
+    }
+  for (int h = 0; h < 2; ++h) c.F3[h] = c.nd == 3 ? (int2*)(d + o_F3[h]) : nullptr;
+  c.parts = (double2*)(d + o_parts);
+  c.B = (const longlong2*)(P->d_state + P->coef_count * (sizeof(double2) + sizeof(float4)));
   return GBSBIN_OK;
 }
 
@@ -277,12 +537,13 @@ int gbsbin_fock_plan_create(const gbsbin_fock_problem* p, const gbsbin_options* 
   if (xr > a.nchunks) xr = a.nchunks;
   a.xr = (int)xr;
   P->coef_count = (size_t)(L + 1) * a.nin * a.nin;
-  P->state_bytes = P->coef_count * (sizeof(double2) + sizeof(float4));
+  P->conv = opt.shard_end == 0 && opt.shard_begin == 0 && opt.tile_override == 0 && conv_layout(P);
+  P->state_bytes = P->coef_count * (sizeof(double2) + sizeof(float4) + (P->conv ? sizeof(longlong2) : 0));
   int st = GBSBIN_OK;
   if ((st = dalloc(&P->d_state, P->state_bytes)) || (st = dalloc(&P->d_xtw, (size_t)xoff)) ||
       (st = dalloc(&P->d_xtw_df, (size_t)xoff)) || (st = dalloc(&P->d_zr, (size_t)a.rsum)) ||
       (st = dalloc(&P->d_zr_df, (size_t)a.rsum)) || (st = dalloc(&P->d_tw, (size_t)a.rsum)) ||
-      (st = dalloc(&P->d_parts, (size_t)xr * g.n_full)) || (st = dalloc(&P->d_bufA, (size_t)g.n_full)) ||
+      (st = dalloc(&P->d_parts, P->conv ? 0 : (size_t)xr * g.n_full)) || (st = dalloc(&P->d_bufA, (size_t)g.n_full)) ||
       (st = dalloc(&P->d_bufB, (size_t)g.n_full)) || (st = dalloc(&P->d_diag, GBSBIN_DIAG_DOUBLES)) ||
       (st = dalloc(&P->d_bar, 4)) || (st = dalloc(&P->d_table, (size_t)P->table_size))) {
     free_all(P);
@@ -310,6 +571,11 @@ int gbsbin_fock_plan_create(const gbsbin_fock_problem* p, const gbsbin_options* 
   a.zr = P->d_zr;
   a.zr_df = P->d_zr_df;
   a.parts = P->d_parts;
+  if (P->conv && (st = conv_setup(P))) {
+    free_all(P);
+    delete P;
+    return st;
+  }
   // roots from exact integer indices
   const double TWO_PI = 6.283185307179586476925286766559;
   std::vector<double2> xtw((size_t)std::max(xoff, 1)), zr((size_t)a.rsum), tw((size_t)a.rsum);
@@ -371,8 +637,18 @@ int gbsbin_fock_execute(gbsbin_fock_plan* P, double* P_out, void* stream) {
   if (!P || !P_out) return GBSBIN_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   if (P->ev0 && cudaEventRecord(P->ev0, s) != cudaSuccess) return GBSBIN_ERR_CUDA;
+  if (P->conv) {
+    FockConvArgs c = P->cv;
+    c.P = P_out;
+    c.diag = P->opt.want_diagnostics ? P->d_diag : nullptr;
+    if (launch_fock_conv(c, P->layers.data(), (int)P->layers.size(), P->num_sms, s, &P->last_launches) != cudaSuccess)
+      return GBSBIN_ERR_CUDA;
+    P->executed = true;
+    return P->ev1 && cudaEventRecord(P->ev1, s) != cudaSuccess ? GBSBIN_ERR_CUDA : GBSBIN_OK;
+  }
   if (launch_fock(P->args, P->df, P->zt, s) != cudaSuccess) return GBSBIN_ERR_CUDA;
   P->executed = true;
+  P->last_launches = 2;                           // the Fock kernel and the fused DFT
   if (P->ev1 && cudaEventRecord(P->ev1, s) != cudaSuccess) return GBSBIN_ERR_CUDA;
   DftArgs d{};
   d.grid = P->args.grid;
@@ -428,7 +704,7 @@ int gbsbin_fock_diagnostics(gbsbin_fock_plan* P, gbsbin_diag* out, void* stream)
   out->backward_kernel_ms = 0.0;
   out->backward_path = 0;
   out->state_upload_bytes = (long long)P->state_bytes;
-  out->launches = P->executed ? 2 : 0;            // the Fock kernel and the fused DFT
+  out->launches = P->last_launches;
   if (P->ev1 && P->executed) {
     float ms = 0.f;
     if (cudaEventSynchronize(P->ev1) != cudaSuccess || cudaEventElapsedTime(&ms, P->ev0, P->ev1) != cudaSuccess) {
