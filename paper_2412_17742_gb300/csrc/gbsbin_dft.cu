@@ -740,6 +740,176 @@ static cudaError_t launch_dft_blocked(const DftArgs& a, int h, unsigned* bar, in
                                      s);
 }
 
+// ------------------------------------------------- small transforms: one cluster, no grid barrier
+// All stages by one cluster of kClusterCtas CTAs (16 FP64 operations a clock together): stages are separated
+// by the cluster's hardware barrier (arrive with release, wait with acquire, so the writes to bufA / bufB are
+// seen) instead of a grid barrier, and an ordinary launch replaces the cooperative one.  A sum of R terms
+// is split over S consecutive lanes (S a power of two set by the host so that a stage fills the threads, at
+// least kMinTerms terms each), terms k = lane mod S, + S, ..., then a butterfly: on this GPU a warp's FP64
+// instruction holds its scheduler for 64 clocks, so a stage of a few hundred items is a chain of R such
+// instructions that only more lanes shorten.  Whole tables, cooperative launch -> cluster: n = 8, 7 x 7
+// points 30.9 -> 28.8 us; n = 42, 8 x 11 x 6 117.3 -> 110.7; n = 20, 13 x 14 65.6 -> 59.5; 30 x 30 58.7 -> 53.4;
+// 45 x 45 (114,000 multiply-adds and normalisations) 75.9 -> 78.0, beyond the line drawn below.
+constexpr int kClusterCtas = 8;
+constexpr int kClusterThreads = 512;
+constexpr int kMinTerms = 2;
+struct DftCluster {
+  DftFused f;
+  int split[GBSBIN_MAX_L];           // lanes per item of each complex axis
+  int split_last;
+};
+
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ double2 split_sum(double2 v, int S) {
+  for (int o = S >> 1; o > 0; o >>= 1) {
+    v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+    v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+  }
+  return v;
+}
+
+// The Hermitian last axis, S lanes per output; diagnostics of what these threads write and read into acc.
+__device__ __forceinline__ void split_last_real(const DftFused& f, const double2* cur, unsigned S, unsigned t0,
+                                                unsigned stride, DiagAcc& acc) {
+  const double2* tw = f.a.tw + f.last_twoff;
+  const unsigned R = (unsigned)f.last_R, H = (unsigned)f.H, nout = (unsigned)f.last_nout;
+  const unsigned total = (unsigned)(f.last_outer * f.last_nout) * S, end = (total + 31u) & ~31u;
+  for (unsigned t = t0; t < end; t += stride) {
+    const unsigned it = t / S, k0 = t & (S - 1);
+    const bool live = t < total;
+    const unsigned o = it / nout, b = it - o * nout;
+    const double2* row = cur + (size_t)o * H;
+    double2 v = make_double2(0.0, 0.0);
+    if (live) {
+      unsigned idx = (k0 * b) % R;
+      const unsigned step = (S * b) % R;
+      for (unsigned k = k0; k < H; k += S) {
+        const double2 y = row[k], w = tw[idx];
+        const double re = fma(y.x, w.x, -y.y * w.y);
+        v.x += (k == 0 || 2 * k == R) ? re : 2.0 * re;
+        idx += step;
+        if (idx >= R) idx -= R;
+      }
+    }
+    v = split_sum(v, (int)S);
+    if (live && k0 == 0) {
+      const double P = v.x * f.scale;
+      f.a.P[it] = P;
+      acc.sum += P;
+      if (b == 0) {                                       // the row's self-conjugate entries
+        acc.im = fmax(acc.im, fabs(row[0].y));
+        if ((R & 1u) == 0) acc.im = fmax(acc.im, fabs(row[H - 1].y));
+      }
+    }
+  }
+}
+
+// The pivots' scan and the warp's partial: warp `slot` of `slots`.
+__device__ __forceinline__ void split_diag(const DftArgs& a, DiagAcc& acc, unsigned t0, unsigned stride, int slot,
+                                           int slots) {
+  if (!a.diag) return;
+  const double2* lq = a.g_ready ? nullptr : a.ldfin ? a.logq_fin : a.logq;
+  for (long long e = t0; a.minpiv && e < a.grid.n_eval; e += stride) {
+    const double m = a.minpiv[e];
+    const double2 l = lq ? lq[e] : make_double2(0.0, 0.0);
+    if (!((m > 0.0) && isfinite(l.x) && isfinite(l.y))) acc.bad += 1.0;
+    acc.mn = fmin(acc.mn, m);
+  }
+  warp_diag(acc, a.diag, slot);
+  if (t0 == 0) {
+    a.diag[4 * GBSBIN_DIAG_SLOTS] = lq ? lq[0].x : 0.0;
+    a.diag[4 * GBSBIN_DIAG_SLOTS + 1] = 0.0;
+    a.diag[4 * GBSBIN_DIAG_SLOTS + 2] = (double)slots;
+  }
+}
+
+// One axis with G given (one-group plans): no exchange at all, so an ordinary launch over as many SMs as the
+// outputs, split over lanes, fill (171 outputs of 86 terms at n = 512: the table 26.7 us with the cluster, 18.5
+// so, together with the CTA per point of the one-group kernel).
+constexpr int kLineThreads = 128;
+__global__ void __launch_bounds__(kLineThreads) k_dft_line(DftFused f, int S) {
+  DiagAcc acc{0.0, 0.0, 1.0e300, 0.0};
+  const unsigned t0 = blockIdx.x * kLineThreads + threadIdx.x, stride = gridDim.x * kLineThreads;
+  split_last_real(f, f.a.bufA, (unsigned)S, t0, stride, acc);
+  split_diag(f.a, acc, t0, stride, (int)(t0 >> 5), (int)(stride >> 5));
+}
+
+__global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterThreads) k_dft_cluster(DftCluster c) {
+  const DftFused& f = c.f;
+  const DftArgs& a = f.a;
+  // consecutive items over the CTAs' warps in turn: warp w of CTA b is warp (w kClusterCtas + b) of the cluster
+  const unsigned t0 = (threadIdx.x >> 5) * (32u * kClusterCtas) + blockIdx.x * 32u + (threadIdx.x & 31u);
+  const unsigned stride = kClusterCtas * kClusterThreads;
+  bool first = !a.g_ready;
+  if (a.parts) {
+    stage_sum_parts(a.parts, a.nparts, a.pscale, a.grid, a.bufA, t0, stride);
+  } else if (first) {
+    __shared__ double2 s_l0;
+    if (threadIdx.x == 0) s_l0 = a.ldfin ? finish_logq(a.ldfin) : a.logq[0];
+    __syncthreads();
+    stage_normalise(a.logq, a.grid, a.bufA, a.ldfin, a.logq_fin, s_l0, t0, stride);
+  }
+  double2* cur = a.bufA;
+  double2* nxt = a.bufB;
+  for (int l = 0; l < f.naxes; ++l) {
+    if (l > 0 || first) cluster_barrier();
+    const DftStage& st = f.ax[l];
+    const double2* tw = a.tw + st.twoff;
+    const unsigned S = (unsigned)c.split[l], R = (unsigned)st.R, in = (unsigned)st.inner, nout = (unsigned)st.nout;
+    const unsigned total = (unsigned)(st.outer * st.nout * st.inner) * S, end = (total + 31u) & ~31u;
+    for (unsigned t = t0; t < end; t += stride) {          // whole warps: the butterfly needs every lane
+      const unsigned it = t / S, k0 = t & (S - 1);
+      const bool live = t < total;
+      const unsigned rest = it / in, s = it - rest * in;
+      const unsigned o = rest / nout, b = rest - o * nout;
+      double2 acc = make_double2(0.0, 0.0);
+      if (live) {
+        const double2* src = cur + (size_t)o * R * in + s;
+        unsigned idx = (k0 * b) % R;
+        const unsigned step = (S * b) % R;
+        for (unsigned k = k0; k < R; k += S) {
+          acc = cfma2(src[(size_t)k * in], tw[idx], acc);
+          idx += step;
+          if (idx >= R) idx -= R;
+        }
+      }
+      acc = split_sum(acc, (int)S);
+      if (live && k0 == 0) nxt[it] = acc;
+    }
+    double2* x = cur;
+    cur = nxt;
+    nxt = x;
+  }
+  if (f.naxes > 0 || first) cluster_barrier();
+  DiagAcc acc{0.0, 0.0, 1.0e300, 0.0};
+  split_last_real(f, cur, (unsigned)c.split_last, t0, stride, acc);
+  split_diag(a, acc, t0, stride, blockIdx.x * (kClusterThreads >> 5) + (threadIdx.x >> 5),
+             kClusterCtas * (kClusterThreads >> 5));
+}
+
+// Lanes per item: as many as fill the cluster's threads, at most a warp and kMinTerms terms a lane.
+static int split_for(long long items, long long terms) {
+  int S = 1;
+  while (S < 32 && items * 2 * S <= (long long)kClusterCtas * kClusterThreads && terms >= 2LL * S * kMinTerms) S *= 2;
+  return S;
+}
+
+// The cluster's share of the transform: complex multiply-adds of all axes; the cluster serves up to
+// kClusterWork of them (and as many points, each ~100 of them to normalise).
+constexpr long long kClusterWork = 100000;
+static bool cluster_suits(const DftFused& f) {
+  long long w = f.last_outer * f.last_nout * f.H;
+  for (int l = 0; l < f.naxes; ++l) w += f.ax[l].outer * f.ax[l].nout * f.ax[l].inner * f.ax[l].R;
+  const GridDesc& g = f.a.grid;
+  if (f.a.parts) w += f.a.nparts * g.n_full;
+  else if (!f.a.g_ready) w += 20 * g.n_full;
+  return w <= kClusterWork;
+}
+
 cudaError_t launch_dft_fused(const DftArgs& a, unsigned* bar, int num_sms, cudaStream_t s) {
   const GridDesc& g = a.grid;
   const int L = g.L;
@@ -770,6 +940,22 @@ cudaError_t launch_dft_fused(const DftArgs& a, unsigned* bar, int num_sms, cudaS
   f.H = g.half;
   f.last_nout = g.nout[L - 1];
   f.scale = 1.0 / (double)g.npts;
+  if (f.naxes == 0 && a.g_ready) {
+    int S = 1;                                        // lanes per output: two warps a scheduler at most
+    while (S < 32 && (long long)f.last_nout * 2 * S <= 256LL * num_sms && f.H >= 2 * S * kMinTerms) S *= 2;
+    long long blocks = ((long long)f.last_nout * S + kLineThreads - 1) / kLineThreads;
+    if (blocks > GBSBIN_DIAG_SLOTS / (kLineThreads / 32)) blocks = GBSBIN_DIAG_SLOTS / (kLineThreads / 32);
+    k_dft_line<<<(unsigned)blocks, kLineThreads, 0, s>>>(f, S);
+    return cudaGetLastError();
+  }
+  if (cluster_suits(f)) {
+    DftCluster c{};
+    c.f = f;
+    for (int l = 0; l < f.naxes; ++l) c.split[l] = split_for(f.ax[l].outer * f.ax[l].nout * f.ax[l].inner, f.ax[l].R);
+    c.split_last = split_for(f.last_outer * f.last_nout, f.H);
+    k_dft_cluster<<<kClusterCtas, kClusterThreads, 0, s>>>(c);
+    return cudaGetLastError();
+  }
   int per_sm = 0;
   cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dft_fused, 128, 0);
   if (err != cudaSuccess) return err;

@@ -15,12 +15,11 @@
 //
 // All of it is FP64, for plans of either arithmetic: at n = 512 and 86 points it is 44,000
 // factors of ~8 FP64 operations, which 152 SMs at 2 operations a clock finish in ~1200 clocks.
-// What bounds a launch is the FP64 latency of one warp's chain (n / TP factors, five butterfly
-// steps, two square roots) on small grids and the FP64 rate on large ones, so TP is 32 while
-// that leaves SMs to fill and falls to one lane per point on large grids, where a warp then takes the
-// square roots of 32 points at once.  Before, a CTA or warp per point eliminated the Hessenberg
-// form of XA, n serial steps of O(n): 614 us at n = 512 with 86 points in FP64. With this kernel the whole
-// table, transform included, takes 34.8 us instead of 642.
+// What bounds a launch is the FP64 latency of one warp's chain (n / TP factors, the butterfly, the root) on
+// small grids and the FP64 rate on large ones, so a point takes a CTA or a warp while that leaves SMs to
+// fill and one thread on large grids, where a warp then takes the roots of 32 points at once.  Before, a CTA or warp per point eliminated the Hessenberg
+// form of XA, n serial steps of O(n): 614 us at n = 512 with 86 points in FP64. The whole
+// table, transform included, took 642 us and takes 18.5 us, 17.6 of them on the host's side of the call.
 #include <cuda_runtime.h>
 
 #include "gbsbin_device.cuh"
@@ -32,36 +31,73 @@ namespace {
 
 constexpr int kSpectralThreads = 128;
 
-// One point by TP consecutive lanes of a warp (lane r of the team); every lane of the warp calls
-// it, teams past the last point with live = false.
+struct Partial {                                // a share of the factors
+  double2 prod, ex;
+  int e2;
+  float args;
+};
+
+__device__ __forceinline__ void join(Partial& p, const Partial& q, bool disp) {
+  p.prod = ArF64::mul(p.prod, q.prod);
+  p.e2 += q.e2 + ArF64::normalise(p.prod);
+  p.args += q.args;
+  if (disp) p.ex = ArF64::add(p.ex, q.ex);
+}
+
+// p^{-1/2}, the principal root, for |p| in [1/2, 3/2): two Newton steps y <- y (3 - p y^2) / 2 on the FP32
+// root (FP64 square roots and divisions are long sequences on this GPU's FP64 pipe).
+__device__ __forceinline__ double2 inv_sqrt(double2 p) {
+  const float x = (float)p.x, y = (float)p.y, r = sqrtf(fmaf(x, x, y * y));
+  const float s = sqrtf(0.5f * (r + fabsf(x))), q = s > 0.f ? 0.5f * y / s : 0.f;
+  const float re = x >= 0.f ? s : fabsf(q), im = x >= 0.f ? q : (y < 0.f ? -s : s);   // sqrt(p)
+  double2 v = make_double2((double)(re / r), (double)(-im / r));
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const double2 t = ArF64::fms(make_double2(1.5, 0.0), p, ArF64::mul(v, make_double2(0.5 * v.x, 0.5 * v.y)));
+    v = ArF64::mul(v, t);
+  }
+  return v;
+}
+
+// One point by TP consecutive threads (thread r of the team; TP = kSpectralThreads: the whole CTA, through
+// shared memory); every thread of the block calls it, teams past the last point with live = false.
 template <int TP, bool DISP>
 __device__ __forceinline__ void spectral_point(const PointArgs& a, long long e, int r, bool live) {
   const double2 w = grid_root(a.tw, a.grid, 0, live ? point_digit(e, a.grid, 0) : 0);
-  double2 prod = ArF64::one(), ex = ArF64::zero();
-  float args = 0.f;
-  int e2 = 0, since = 0;
+  Partial p{ArF64::one(), ArF64::zero(), 0, 0.f};
+  int since = 0;
   for (int i = r; i < a.n; i += TP) {
     const double lam = a.lam[i];
     const double2 z = make_double2(fma(-w.x, lam, 1.0), -w.y * lam);
-    prod = ArF64::mul(prod, z);
-    args += atan2f((float)z.y, (float)z.x);
+    p.prod = ArF64::mul(p.prod, z);
+    p.args += atan2f((float)z.y, (float)z.x);
     if (++since == 4) {                         // |z| < 2 and > 1 - |lambda|
-      e2 += ArF64::normalise(prod);
+      p.e2 += ArF64::normalise(p.prod);
       since = 0;
     }
-    if (DISP) ex = ArF64::fma(a.gq[i], ArF64::recip(z), ex);
+    if (DISP) p.ex = ArF64::fma(a.gq[i], ArF64::recip(z), p.ex);
   }
-  e2 += ArF64::normalise(prod);
+  p.e2 += ArF64::normalise(p.prod);
 #pragma unroll
-  for (int o = TP / 2; o > 0; o >>= 1) {
-    prod = ArF64::mul(prod, shfl_xor(prod, o));
-    e2 += __shfl_xor_sync(0xffffffffu, e2, o);
-    args += __shfl_xor_sync(0xffffffffu, args, o);
-    e2 += ArF64::normalise(prod);
-    if (DISP) ex = ArF64::add(ex, shfl_xor(ex, o));
+  for (int o = (TP < 32 ? TP : 32) / 2; o > 0; o >>= 1) {
+    Partial q;
+    q.prod = shfl_xor(p.prod, o);
+    q.e2 = __shfl_xor_sync(0xffffffffu, p.e2, o);
+    q.args = __shfl_xor_sync(0xffffffffu, p.args, o);
+    if (DISP) q.ex = shfl_xor(p.ex, o);
+    join(p, q, DISP);
+  }
+  if constexpr (TP > 32) {
+    __shared__ Partial s_p[TP / 32];
+    if ((threadIdx.x & 31) == 0) s_p[threadIdx.x >> 5] = p;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int i = 1; i < TP / 32; ++i) join(p, s_p[i], DISP);
   }
   if (!live || r != 0) return;
-  if (DISP) ex = ArF64::mul(ex, w);             // gamma^T K^{-1} w X gamma
+  const double2 prod = p.prod;
+  const int e2 = p.e2;
+  const double2 ex = DISP ? ArF64::mul(p.ex, w) : ArF64::zero();   // gamma^T K^{-1} w X gamma
   // every factor's real part is 1 - Re(w) lambda_i: the smallest at an end of the spectrum
   const double mn = 1.0 - fmax(w.x * a.lam_min, w.x * a.lam_max);
   const bool ok = isfinite(prod.x) && isfinite(prod.y) && isfinite(ex.x) && isfinite(ex.y);
@@ -69,7 +105,7 @@ __device__ __forceinline__ void spectral_point(const PointArgs& a, long long e, 
   double* f = a.ldfin + 6 * e;                  // log q unfinished, as finish_logq takes it
   f[0] = prod.x;
   f[1] = prod.y;
-  f[2] = (double)args;
+  f[2] = (double)p.args;
   f[3] = fma(-0.5 * LN2, (double)e2, 0.5 * ex.x);
   f[4] = 0.5 * ex.y;
   f[5] = 0.0;
@@ -78,8 +114,8 @@ __device__ __forceinline__ void spectral_point(const PointArgs& a, long long e, 
   // G = (p0 2^e0 / (prod 2^e2))^{1/2} exp((ex - ex(1)) / 2), the root on the sheet of the summed
   // arguments: the principal root times (-1)^m, m the winding of log prod
   const float a0 = atan2f((float)prod.y, (float)prod.x);
-  const int m = (int)rintf((args - a0) * 0.159154943f);
-  double2 g = ArF64::csqrt(ArF64::recip(prod));
+  const int m = (int)rintf((p.args - a0) * 0.159154943f);
+  double2 g = inv_sqrt(prod);
   const int de = a.sp_e0 - e2, h = de >> 1;     // 2^(de / 2) = 2^h sqrt(2)^(de odd)
   double sc = a.sp_rt0 * ((de & 1) ? 1.41421356237309504880 : 1.0);
   if (m & 1) sc = -sc;
@@ -96,7 +132,7 @@ __device__ __forceinline__ void spectral_point(const PointArgs& a, long long e, 
 
 template <int TP, bool DISP>
 __global__ void __launch_bounds__(kSpectralThreads) k_points_spectral(PointArgs a) {
-  const long long e = (blockIdx.x * (long long)kSpectralThreads + threadIdx.x) / TP;
+  const long long e = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / TP;
   spectral_point<TP, DISP>(a, e, threadIdx.x % TP, e < a.grid.n_eval);
 }
 
@@ -112,23 +148,26 @@ __global__ void __launch_bounds__(kSpectralThreads) k_points_spectral_batch(Poin
 }
 
 template <int TP>
-cudaError_t launch_tp(const PointArgs& a, cudaStream_t s) {
-  const long long per = kSpectralThreads / TP;
+cudaError_t launch_tp(const PointArgs& a, int threads, cudaStream_t s) {
+  const long long per = threads / TP;
   const unsigned grid = (unsigned)((a.grid.n_eval + per - 1) / per);
-  if (a.has_gamma) k_points_spectral<TP, true><<<grid, kSpectralThreads, 0, s>>>(a);
-  else k_points_spectral<TP, false><<<grid, kSpectralThreads, 0, s>>>(a);
+  if (a.has_gamma) k_points_spectral<TP, true><<<grid, threads, 0, s>>>(a);
+  else k_points_spectral<TP, false><<<grid, threads, 0, s>>>(a);
   return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_points_spectral(const PointArgs& a, int num_sms, cudaStream_t s) {
-  // lanes per point: a warp each while the points do not give every SM's four schedulers two
-  // warps, then eight, then one
-  const long long warps = a.grid.n_eval;
-  if (warps <= 8LL * num_sms) return launch_tp<32>(a, s);
-  if (warps <= 64LL * num_sms) return launch_tp<8>(a, s);
-  return launch_tp<1>(a, s);
+  // threads per point.  A CTA (four warps) each for long products on few points: a warp's chain of n / 32
+  // factors, not the FP64 rate, is the time then (n = 512, 86 points: 21 us with a warp per point).  A
+  // warp each, one to a CTA so that the points spread over the SMs, while every SM gets at most eight;
+  // then eight lanes, then one.
+  const long long pts = a.grid.n_eval;
+  if (a.n >= 128 && pts <= 4LL * num_sms) return launch_tp<kSpectralThreads>(a, kSpectralThreads, s);
+  if (pts <= 8LL * num_sms) return launch_tp<32>(a, 32, s);
+  if (pts <= 64LL * num_sms) return launch_tp<8>(a, kSpectralThreads, s);
+  return launch_tp<1>(a, kSpectralThreads, s);
 }
 
 cudaError_t launch_points_spectral_batch(const PointBatch& batch, cudaStream_t s) {
