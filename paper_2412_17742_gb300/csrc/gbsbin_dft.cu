@@ -38,35 +38,77 @@ __device__ __forceinline__ double2 finish_logq(const double* f) {
   return make_double2(f[3] - 0.5 * re, f[4] - 0.5 * im);
 }
 
-// G = exp(log q - log q_0) on the whole evaluated half grid (finishing log q first when the
-// point kernel left it unfinished).  A shard's plan evaluated point 0 and its slice
-// [e_lo, e_hi) only: G is zero off the slice, so the transform gives the slice's partial
-// table.  Items t0, t0 + stride, ... of the half grid; l0 = log q_0.
-// G at half-grid point t (see stage_normalise); with ldfin, also stores the finished log q.
+// What G at every point is taken relative to: log q_0, or the record of point 0 as (P^{1/2}, rest, winding).
+struct Point0 {
+  double2 l0;                        // log q_0, or the rest of it
+  double2 root;
+  int wind;
+};
+
+// P^{-1/2} of a record, principal root, and the winding of log P: |P| brought to [1/4, 1) by an even power of two.
+__device__ __forceinline__ double2 record_root(const double* f, int* wind) {
+  double2 p = make_double2(f[0], f[1]);
+  const int e = ArF64::normalise(p), odd = e & 1;         // f = p 2^e
+  if (odd) p = make_double2(0.5 * p.x, 0.5 * p.y);
+  const int h = (e + odd) / 2;
+  double2 v = inv_sqrt(p);
+  if (h != 0) v = make_double2(ldexp(v.x, -h), ldexp(v.y, -h));
+  *wind = (int)rintf(((float)f[2] - atan2f((float)p.y, (float)p.x)) * 0.159154943f);
+  return v;
+}
+
+__device__ __forceinline__ Point0 point0(const double2* logq, const double* ldfin) {
+  Point0 z;
+  z.wind = 0;
+  if (!ldfin) {
+    z.l0 = logq[0];
+    z.root = make_double2(1.0, 0.0);
+    return z;
+  }
+  const double2 v = record_root(ldfin, &z.wind);
+  z.root = ArF64::mul(make_double2(ldfin[0], ldfin[1]), v);   // P^{1/2}
+  z.l0 = make_double2(ldfin[3], ldfin[4]);
+  return z;
+}
+
+// G = exp(log q - log q_0) at half-grid point t of the evaluated half grid.  A shard's plan evaluated point 0 and
+// its slice [e_lo, e_hi) only: G is zero off the slice, so the transform gives the slice's partial table.
+// Where the point kernel left log q unfinished, G comes from the records: (P_0 / P)^{1/2} (-1)^(windings) times the
+// exponential of the rest, no logarithm or arctangent in FP64 (and log q itself is finished only when asked for).
 __device__ __forceinline__ double2 normalise_one(const double2* logq, const GridDesc& g, const double* __restrict__ ldfin,
-                                                 double2* logq_fin, double2 l0, long long t) {
-  const bool in_slice = t >= g.e_lo && t < g.e_hi;
-  // this plan's index of half-grid point t (-1: not evaluated here)
-  const long long loc = in_slice ? (g.e_lo > 0 ? t - g.e_lo + 1 : t) : (t == 0 ? 0 : -1);
-  if (loc < 0) return make_double2(0.0, 0.0);
-  double2 v;
+                                                 const Point0& z, long long t) {
+  if (t < g.e_lo || t >= g.e_hi) return make_double2(0.0, 0.0);
+  const long long loc = g.e_lo > 0 ? t - g.e_lo + 1 : t;   // this plan's index of half-grid point t
+  double2 v, r = make_double2(1.0, 0.0);
   if (ldfin) {
-    v = finish_logq(ldfin + 6 * loc);
-    logq_fin[loc] = v;
+    const double* f = ldfin + 6 * loc;
+    int wind;
+    r = ArF64::mul(z.root, record_root(f, &wind));
+    if ((wind - z.wind) & 1) r = make_double2(-r.x, -r.y);
+    v = make_double2(f[3], f[4]);
   } else {
     v = logq[loc];
   }
-  if (!in_slice) return make_double2(0.0, 0.0);     // point 0 of a later shard: normalisation only
-  double m = exp(v.x - l0.x);
+  const double m = exp(v.x - z.l0.x), ph = v.y - z.l0.y;
+  if (ph == 0.0) return make_double2(m * r.x, m * r.y);    // undisplaced records
   double s, c;
-  sincos(v.y - l0.y, &s, &c);
-  return make_double2(m * c, m * s);
+  sincos(ph, &s, &c);
+  return ArF64::mul(r, make_double2(m * c, m * s));
 }
 
 __device__ __forceinline__ void stage_normalise(const double2* logq, const GridDesc& g, double2* __restrict__ G,
-                                                const double* __restrict__ ldfin, double2* logq_fin, double2 l0,
-                                                long long t0, long long stride) {
-  for (long long t = t0; t < g.n_full; t += stride) G[t] = normalise_one(logq, g, ldfin, logq_fin, l0, t);
+                                                const double* __restrict__ ldfin, const Point0& z, long long t0,
+                                                long long stride) {
+  for (long long t = t0; t < g.n_full; t += stride) G[t] = normalise_one(logq, g, ldfin, z, t);
+}
+
+// Whether evaluated point e's log q is finite, from whichever form the point kernel left.
+__device__ __forceinline__ bool finite_point(const double2* logq, const double* ldfin, long long e) {
+  if (ldfin) {
+    const double* f = ldfin + 6 * e;
+    return isfinite(f[0]) && isfinite(f[1]) && isfinite(f[3]) && isfinite(f[4]);
+  }
+  return !logq || (isfinite(logq[e].x) && isfinite(logq[e].y));
 }
 
 // G given as partial sums over nparts ranges of some inner sum (Fock inputs: node ranges
@@ -89,11 +131,11 @@ __device__ __forceinline__ void stage_sum_parts(const double2* __restrict__ part
 }
 
 __global__ void k_normalise(const double2* logq, GridDesc g, double2* __restrict__ G,
-                            const double* __restrict__ ldfin, double2* logq_fin) {
-  __shared__ double2 s_l0;
-  if (threadIdx.x == 0) s_l0 = ldfin ? finish_logq(ldfin) : logq[0];
+                            const double* __restrict__ ldfin) {
+  __shared__ Point0 s_0;
+  if (threadIdx.x == 0) s_0 = point0(logq, ldfin);
   __syncthreads();
-  stage_normalise(logq, g, G, ldfin, logq_fin, s_l0, blockIdx.x * (long long)blockDim.x + threadIdx.x,
+  stage_normalise(logq, g, G, ldfin, s_0, blockIdx.x * (long long)blockDim.x + threadIdx.x,
                   (long long)gridDim.x * blockDim.x);
 }
 
@@ -235,8 +277,8 @@ __global__ void k_dft_last_real(const double2* __restrict__ Y, double* __restric
 // blocks of blockDim.x threads; the whole CTA calls it.
 __device__ __forceinline__ void stage_diag(const double* __restrict__ P, long long table, const double2* __restrict__ Y,
                                            long long outer, int H, int R, const double* __restrict__ minpiv,
-                                           const double2* logq, long long n_eval, double* __restrict__ part,
-                                           int vb, int nvb) {
+                                           const double2* logq, const double* __restrict__ ldfin, long long n_eval,
+                                           double* __restrict__ part, int vb, int nvb) {
   __shared__ double s_sum[32], s_im[32], s_min[32], s_bad[32];
   double sum = 0.0, im = 0.0, mn = 1.0e300, bad = 0.0;
   const long long stride = (long long)nvb * blockDim.x;
@@ -248,9 +290,7 @@ __device__ __forceinline__ void stage_diag(const double* __restrict__ P, long lo
   }
   for (long long e = t0; minpiv && e < n_eval; e += stride) {
     double m = minpiv[e];
-    double2 l = logq ? logq[e] : make_double2(0.0, 0.0);
-    bool ok = (m > 0.0) && isfinite(l.x) && isfinite(l.y);
-    if (!ok) bad += 1.0;
+    if (!((m > 0.0) && finite_point(logq, ldfin, e))) bad += 1.0;
     mn = fmin(mn, m);
   }
   for (int o = 16; o > 0; o >>= 1) {
@@ -281,7 +321,7 @@ __device__ __forceinline__ void stage_diag(const double* __restrict__ P, long lo
     out[2] = mn;
     out[3] = bad;
     if (vb == 0) {
-      part[4 * GBSBIN_DIAG_SLOTS] = logq ? logq[0].x : 0.0;
+      part[4 * GBSBIN_DIAG_SLOTS] = ldfin ? finish_logq(ldfin).x : logq ? logq[0].x : 0.0;
       part[4 * GBSBIN_DIAG_SLOTS + 2] = (double)nvb;
     }
   }
@@ -289,8 +329,9 @@ __device__ __forceinline__ void stage_diag(const double* __restrict__ P, long lo
 
 __global__ void k_diag(const double* __restrict__ P, long long table, const double2* __restrict__ Y,
                        long long outer, int H, int R, const double* __restrict__ minpiv,
-                       const double2* __restrict__ logq, long long n_eval, double* __restrict__ part) {
-  stage_diag(P, table, Y, outer, H, R, minpiv, logq, n_eval, part, blockIdx.x, gridDim.x);
+                       const double2* __restrict__ logq, const double* __restrict__ ldfin, long long n_eval,
+                       double* __restrict__ part) {
+  stage_diag(P, table, Y, outer, H, R, minpiv, logq, ldfin, n_eval, part, blockIdx.x, gridDim.x);
 }
 
 // ------------------------------------------------------- one cooperative launch, all stages
@@ -338,6 +379,18 @@ __device__ __forceinline__ void grid_barrier(unsigned* bar) {
   __syncthreads();
 }
 
+// The pivots' scan into acc, and Re log q(1) as the diagnostics report it (0 where G was given).
+__device__ __forceinline__ void scan_points(const DftArgs& a, long long e0, long long stride, DiagAcc& acc) {
+  for (long long e = e0; a.minpiv && e < a.grid.n_eval; e += stride) {
+    const double m = a.minpiv[e];
+    if (!((m > 0.0) && (a.g_ready || finite_point(a.logq, a.ldfin, e)))) acc.bad += 1.0;
+    acc.mn = fmin(acc.mn, m);
+  }
+}
+__device__ __forceinline__ double log_q1(const DftArgs& a) {
+  return a.g_ready ? 0.0 : a.ldfin ? finish_logq(a.ldfin).x : a.logq ? a.logq[0].x : 0.0;
+}
+
 __global__ void __launch_bounds__(128, 4) k_dft_fused(DftFused f) {
   const DftArgs& a = f.a;
   // the CTA's k-th item goes to lane k / 4 of warp k mod 4: a CTA's few items use all
@@ -351,10 +404,10 @@ __global__ void __launch_bounds__(128, 4) k_dft_fused(DftFused f) {
   } else if (a.parts) {
     stage_sum_parts(a.parts, a.nparts, a.pscale, a.grid, a.bufA, t0, stride);
   } else {
-    __shared__ double2 s_l0;
-    if (threadIdx.x == 0) s_l0 = a.ldfin ? finish_logq(a.ldfin) : a.logq[0];
+    __shared__ Point0 s_0;
+    if (threadIdx.x == 0) s_0 = point0(a.logq, a.ldfin);
     __syncthreads();
-    stage_normalise(a.logq, a.grid, a.bufA, a.ldfin, a.logq_fin, s_l0, t0, stride);
+    stage_normalise(a.logq, a.grid, a.bufA, a.ldfin, s_0, t0, stride);
   }
   double2* cur = a.bufA;
   double2* nxt = a.bufB;
@@ -373,16 +426,10 @@ __global__ void __launch_bounds__(128, 4) k_dft_fused(DftFused f) {
   stage_last_real(cur, a.P, f.last_outer, f.last_R, f.H, f.last_nout, f.scale, a.tw + f.last_twoff, t0, stride,
                   a.diag ? &acc : nullptr);
   if (a.diag) {
-    const double2* lq = a.g_ready ? nullptr : a.ldfin ? a.logq_fin : a.logq;
-    for (long long e = t0; a.minpiv && e < a.grid.n_eval; e += stride) {
-      const double m = a.minpiv[e];
-      const double2 l = lq ? lq[e] : make_double2(0.0, 0.0);
-      if (!((m > 0.0) && isfinite(l.x) && isfinite(l.y))) acc.bad += 1.0;
-      acc.mn = fmin(acc.mn, m);
-    }
+    scan_points(a, t0, stride, acc);
     block_diag(acc, a.diag, blockIdx.x);
     if (t0 == 0) {
-      a.diag[4 * GBSBIN_DIAG_SLOTS] = lq ? lq[0].x : 0.0;
+      a.diag[4 * GBSBIN_DIAG_SLOTS] = log_q1(a);
       a.diag[4 * GBSBIN_DIAG_SLOTS + 1] = (double)*(volatile unsigned*)(f.bar + 2);
       a.diag[4 * GBSBIN_DIAG_SLOTS + 2] = (double)gridDim.x;
     }
@@ -410,7 +457,7 @@ cudaError_t launch_dft(const DftArgs& a, cudaStream_t s) {
   if (a.parts)
     k_sum_parts<<<blocks_for(g.n_full), kDftThreads, 0, s>>>(a.parts, a.nparts, a.pscale, g, a.bufA);
   else
-    k_normalise<<<blocks_for(g.n_full), kDftThreads, 0, s>>>(a.logq, g, a.bufA, a.ldfin, a.logq_fin);
+    k_normalise<<<blocks_for(g.n_full), kDftThreads, 0, s>>>(a.logq, g, a.bufA, a.ldfin);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;
   long long dims[GBSBIN_MAX_L];
@@ -442,7 +489,7 @@ cudaError_t launch_dft(const DftArgs& a, cudaStream_t s) {
   if (err != cudaSuccess) return err;
   if (a.diag) {
     k_diag<<<GBSBIN_DIAG_BLOCKS, 256, 0, s>>>(a.P, a.table_size, cur, outer, g.half, g.radix[L - 1],
-                                              a.minpiv, a.logq, g.n_eval, a.diag);
+                                              a.minpiv, a.logq, a.ldfin, g.n_eval, a.diag);
     err = cudaGetLastError();
   }
   return err;
@@ -539,15 +586,14 @@ __global__ void __launch_bounds__(128) k_dft_blocked(DftBlocked f) {
   E* tws = S1 + f.buf;                               // all axes' twiddles
   E* Y = reinterpret_cast<E*>(a.bufB);               // 16-byte entries either way
   for (int j = threadIdx.x; j < f.ntw; j += blockDim.x) tws[j] = Ar::from(a.tw[j]);
-  __shared__ double2 s_l0;
+  __shared__ Point0 s_0;
   if (!a.g_ready && !a.parts) {
-    if (threadIdx.x == 0) s_l0 = a.ldfin ? finish_logq(a.ldfin) : a.logq[0];
+    if (threadIdx.x == 0) s_0 = point0(a.logq, a.ldfin);
     __syncthreads();
   }
   // the pivots' scan after phase 1 (log q may be finished there); its first pivot per
   // thread is loaded now, so that load's latency passes under phase 1
   DiagAcc acc{0.0, 0.0, 1.0e300, 0.0};
-  const double2* lq = a.g_ready ? nullptr : a.ldfin ? a.logq_fin : a.logq;
   const long long e_first = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const bool has_first = a.diag && a.minpiv && e_first < a.grid.n_eval;
   const double m_first = has_first ? a.minpiv[e_first] : 0.0;
@@ -555,8 +601,7 @@ __global__ void __launch_bounds__(128) k_dft_blocked(DftBlocked f) {
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long e = e_first; a.minpiv && e < a.grid.n_eval; e += stride) {
       const double m = e == e_first ? m_first : a.minpiv[e];
-      const double2 l = lq ? lq[e] : make_double2(0.0, 0.0);
-      if (!((m > 0.0) && isfinite(l.x) && isfinite(l.y))) acc.bad += 1.0;
+      if (!((m > 0.0) && (a.g_ready || finite_point(a.logq, a.ldfin, e)))) acc.bad += 1.0;
       acc.mn = fmin(acc.mn, m);
     }
   };
@@ -569,7 +614,7 @@ __global__ void __launch_bounds__(128) k_dft_blocked(DftBlocked f) {
       else
         S0[e] = Ar::from(a.g_ready ? a.bufA[t]
                          : a.parts ? sum_parts_one(a.parts, a.nparts, a.pscale, a.grid.n_full, t)
-                                   : normalise_one(a.logq, a.grid, a.ldfin, a.logq_fin, s_l0, t));
+                                   : normalise_one(a.logq, a.grid, a.ldfin, s_0, t));
     }
     __syncthreads();
     E* cur = S0;
@@ -639,7 +684,7 @@ __global__ void __launch_bounds__(128) k_dft_blocked(DftBlocked f) {
     const int nw = blockDim.x >> 5;
     warp_diag(acc, a.diag, blockIdx.x * nw + (threadIdx.x >> 5));
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-      a.diag[4 * GBSBIN_DIAG_SLOTS] = lq ? lq[0].x : 0.0;
+      a.diag[4 * GBSBIN_DIAG_SLOTS] = log_q1(a);
       a.diag[4 * GBSBIN_DIAG_SLOTS + 1] = (double)*(volatile unsigned*)(f.bar + 2);
       a.diag[4 * GBSBIN_DIAG_SLOTS + 2] = (double)(gridDim.x * nw);
     }
@@ -812,16 +857,10 @@ __device__ __forceinline__ void split_last_real(const DftFused& f, const double2
 __device__ __forceinline__ void split_diag(const DftArgs& a, DiagAcc& acc, unsigned t0, unsigned stride, int slot,
                                            int slots) {
   if (!a.diag) return;
-  const double2* lq = a.g_ready ? nullptr : a.ldfin ? a.logq_fin : a.logq;
-  for (long long e = t0; a.minpiv && e < a.grid.n_eval; e += stride) {
-    const double m = a.minpiv[e];
-    const double2 l = lq ? lq[e] : make_double2(0.0, 0.0);
-    if (!((m > 0.0) && isfinite(l.x) && isfinite(l.y))) acc.bad += 1.0;
-    acc.mn = fmin(acc.mn, m);
-  }
+  scan_points(a, t0, stride, acc);
   warp_diag(acc, a.diag, slot);
   if (t0 == 0) {
-    a.diag[4 * GBSBIN_DIAG_SLOTS] = lq ? lq[0].x : 0.0;
+    a.diag[4 * GBSBIN_DIAG_SLOTS] = log_q1(a);
     a.diag[4 * GBSBIN_DIAG_SLOTS + 1] = 0.0;
     a.diag[4 * GBSBIN_DIAG_SLOTS + 2] = (double)slots;
   }
@@ -848,10 +887,10 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterT
   if (a.parts) {
     stage_sum_parts(a.parts, a.nparts, a.pscale, a.grid, a.bufA, t0, stride);
   } else if (first) {
-    __shared__ double2 s_l0;
-    if (threadIdx.x == 0) s_l0 = a.ldfin ? finish_logq(a.ldfin) : a.logq[0];
+    __shared__ Point0 s_0;
+    if (threadIdx.x == 0) s_0 = point0(a.logq, a.ldfin);
     __syncthreads();
-    stage_normalise(a.logq, a.grid, a.bufA, a.ldfin, a.logq_fin, s_l0, t0, stride);
+    stage_normalise(a.logq, a.grid, a.bufA, a.ldfin, s_0, t0, stride);
   }
   double2* cur = a.bufA;
   double2* nxt = a.bufB;

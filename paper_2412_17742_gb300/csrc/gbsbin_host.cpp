@@ -457,7 +457,8 @@ inline bool is_hess(int kernel) { return kernel == GBSBIN_KERNEL_HESS_FP64 || ke
 inline bool is_btree(int kernel) { return kernel == GBSBIN_KERNEL_BTREE_DF32 || kernel == GBSBIN_KERNEL_BTREE_FP64; }
 // 16-byte slots of a tree plan's depth-0 region in the state block
 size_t tree_region_slots(int n, int kernel) {
-  if (is_tree(kernel)) return (size_t)n * n + 2 * (size_t)n + 3;   // permuted XA, X gamma, gamma, path record
+  // permuted XA, X gamma, gamma, path record; the first group's spectral form (at most n rows of n + 2 + 1)
+  if (is_tree(kernel)) return (size_t)n * n + 2 * (size_t)n + 3 + (size_t)n * (n + 3);
   if (is_btree(kernel)) return (size_t)(n + 1) * (n + 1) + 2;    // augmented matrix, path record
   if (is_hess(kernel)) return (size_t)n + ((size_t)n + 1) / 2;    // g products, eigenvalues
   return 0;
@@ -588,6 +589,28 @@ int upload_state(gbsbin_plan* P, cudaStream_t stream) {
     path[0] = slot(cd(1.0, 0.0));                       // pivot product
     path[1] = make_float4(0.f, 0.f, 3.0e38f, 0.f);    // argument sum, power of two, min Re pivot
     path[2] = slot(cd(0.0, 0.0));                       // exponent sum
+    {                                                   // the first group's spectral form
+      const int nb = P->tree.nb[0], rest = n - nb;
+      float4 *lam = path + 3, *B = lam + nb, *ru = B + (size_t)nb * (rest + 1);
+      std::vector<cd> A00((size_t)nb * nb);
+      for (int i = 0; i < nb; ++i)
+        for (int j = 0; j < nb; ++j) A00[(size_t)i * nb + j] = P->XA[(size_t)pm[i] * n + pm[j]];
+      std::vector<std::vector<cd>> col(rest + 2, std::vector<cd>(nb));
+      std::vector<std::vector<cd>*> vecs;
+      for (int i = 0; i < nb; ++i) {
+        for (int j = 0; j < rest; ++j) col[j][i] = P->XA[(size_t)pm[i] * n + pm[nb + j]];
+        col[rest][i] = P->Xgamma[pm[i]];
+        col[rest + 1][i] = std::conj(P->gamma[pm[i]]);
+      }
+      for (auto& v : col) vecs.push_back(&v);
+      std::vector<double> ev;
+      if (!hermitian_spectrum(A00, nb, ev, vecs)) return GBSBIN_ERR_NUMERIC;
+      for (int k = 0; k < nb; ++k) {
+        lam[k] = slot(cd(ev[k], 0.0));
+        for (int j = 0; j <= rest; ++j) B[(size_t)k * (rest + 1) + j] = slot(col[j][k]);
+        ru[k] = slot(std::conj(col[rest + 1][k]));
+      }
+    }
     // the w = 1 point on the host: unpivoted LU of I - XA in the tree's row order, its pivot
     // product p0 2^e0, argument and winding (each pivot has Re > 0)
     P->tree_g = !P->has_gamma;
@@ -946,6 +969,9 @@ void tree_pointers(gbsbin_plan* P, const Stage& sl) {
   t.c[0] = A0 + (size_t)n * n;
   t.u[0] = t.c[0] + n;
   t.path[0] = t.u[0] + n;
+  t.rlam = t.path[0] + 3;
+  t.rB = t.rlam + t.nb[0];
+  t.ru = t.rB + (size_t)t.nb[0] * (n - t.nb[0] + 1);
   float4* q = (float4*)P->d_tree;
   long long nodes = 1;
   for (int l = 0; l + 1 < P->L; ++l) {
@@ -1460,7 +1486,6 @@ static DftArgs make_dft_args(gbsbin_plan* P, double* P_out) {
   d.grid = P->grid;
   d.logq = P->d_logq;
   d.ldfin = P->d_ldfin;
-  d.logq_fin = P->d_logq;
   d.tw = P->d_tw;
   d.bufA = P->d_bufA;
   d.bufB = P->d_bufB;
@@ -1614,8 +1639,8 @@ int gbsbin_read_points(gbsbin_plan* P, double* logq_host, double* minpiv_host, v
   if (!P || !logq_host) return GBSBIN_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   const size_t ne = (size_t)P->grid.n_eval;
-  // plans whose DFT took G directly left log q unfinished
-  if (P->tree_g &&
+  // kernels that leave records: log q is finished here
+  if (P->d_ldfin &&
       launch_finish_logq(P->d_ldfin, P->d_logq, (long long)ne, s) != cudaSuccess)
     return GBSBIN_ERR_CUDA;
   if (cudaMemcpyAsync(logq_host, P->d_logq, ne * sizeof(double2), cudaMemcpyDeviceToHost, s) != cudaSuccess)
@@ -1631,7 +1656,7 @@ int gbsbin_read_points(gbsbin_plan* P, double* logq_host, double* minpiv_host, v
 static int backward_enqueue(gbsbin_plan* P, const double* dLdP, cudaStream_t s) {
   int st = GBSBIN_OK;
   if (!P->logq_valid && (st = gbsbin_execute(P, P->d_table, s))) return st;   // log q of the current state
-  if (P->tree_g &&                              // the DFT took G directly: finish log q
+  if (P->d_ldfin &&                             // kernels that leave records: finish log q
       launch_finish_logq(P->d_ldfin, P->d_logq, P->grid.n_eval, s) != cudaSuccess)
     return GBSBIN_ERR_CUDA;
   BackwardArgs b{};

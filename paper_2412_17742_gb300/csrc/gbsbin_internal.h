@@ -68,7 +68,7 @@ struct PointArgs {
   long long gws_slot_bytes; // bytes of one CTA's slot
   double* ldfin;            // warp kernel only: n_eval x 6 doubles (the product of the
                             // pivots d_i u'_ii re/im, the FP32 sum of their arguments, the
-                            // rest of log q re/im, unused); log q is finished by the DFT
+                            // rest of log q re/im, unused); log q is finished on demand
 };
 
 // A batch of problems for one point-kernel launch: jobs are (problem, first point) groups
@@ -123,8 +123,7 @@ struct DftArgs {
   long long nparts;
   double pscale;
   const double2* logq;      // n_eval
-  const double* ldfin;      // nullptr, or the warp kernel's unfinished log det (see PointArgs)
-  double2* logq_fin;        // with ldfin: where the finished log q go (n_eval)
+  const double* ldfin;      // nullptr, or the unfinished log q (see PointArgs), from which G is taken
   const double2* tw;        // concatenated exp(-2 pi i m / radix[l]), m < radix[l]
   double2* bufA;            // n_eval complex scratch
   double2* bufB;            // n_eval complex scratch
@@ -164,6 +163,9 @@ struct TreeArgs {
   double2* gout;
   int gout_df;              // nonzero (pairs plans whose DFT runs in pairs): G stored as a pair
                             // of FP32 (float4) in the 16-byte slots of gout
+  // the first group's block of XA is Hermitian, A_00 = Q Lambda Q^H (host, once per state): the eigenvalues
+  // (real parts of nb[0] slots), Q^H [A_0r, c_0] (nb[0] x (m[1] + 1)) and u_0^T Q (nb[0])
+  const float4 *rlam, *rB, *ru;
   double p0re, p0im;
   float4 p0df;              // p0 as a pair of FP32
   float p0arg, e0, m0;
@@ -288,8 +290,7 @@ size_t points_matrix_bytes(int kernel, int n, int P);
 int points_per_cta(int kernel, int n, int L);
 int points_threads(int kernel, int n);
 cudaError_t launch_dft(const DftArgs& a, cudaStream_t s);
-// log q of n evaluated points from the unfinished form (ldfin) - for plans whose DFT took G
-// directly and did not finish them.
+// log q of n evaluated points from the unfinished form (ldfin), which the transform leaves as it is.
 cudaError_t launch_finish_logq(const double* ldfin, double2* logq, long long n, cudaStream_t s);
 // All DFT stages and the diagnostics in one cooperative launch; bar: 4 zeroed unsigned ints
 // of grid-barrier state owned by the caller; diag (if any) holds GBSBIN_DIAG_DOUBLES.

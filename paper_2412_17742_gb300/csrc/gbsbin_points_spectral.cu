@@ -44,21 +44,6 @@ __device__ __forceinline__ void join(Partial& p, const Partial& q, bool disp) {
   if (disp) p.ex = ArF64::add(p.ex, q.ex);
 }
 
-// p^{-1/2}, the principal root, for |p| in [1/2, 3/2): two Newton steps y <- y (3 - p y^2) / 2 on the FP32
-// root (FP64 square roots and divisions are long sequences on this GPU's FP64 pipe).
-__device__ __forceinline__ double2 inv_sqrt(double2 p) {
-  const float x = (float)p.x, y = (float)p.y, r = sqrtf(fmaf(x, x, y * y));
-  const float s = sqrtf(0.5f * (r + fabsf(x))), q = s > 0.f ? 0.5f * y / s : 0.f;
-  const float re = x >= 0.f ? s : fabsf(q), im = x >= 0.f ? q : (y < 0.f ? -s : s);   // sqrt(p)
-  double2 v = make_double2((double)(re / r), (double)(-im / r));
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const double2 t = ArF64::fms(make_double2(1.5, 0.0), p, ArF64::mul(v, make_double2(0.5 * v.x, 0.5 * v.y)));
-    v = ArF64::mul(v, t);
-  }
-  return v;
-}
-
 // One point by TP consecutive threads (thread r of the team; TP = kSpectralThreads: the whole CTA, through
 // shared memory); every thread of the block calls it, teams past the last point with live = false.
 template <int TP, bool DISP>

@@ -34,6 +34,8 @@
 // its launch shapes are the same.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include <type_traits>
 
 #include "gbsbin_device.cuh"
@@ -107,6 +109,119 @@ __device__ __forceinline__ void path_warp(PathRec<typename Ar::E>& pr, typename 
   pr.meta = make_float4(__fadd_rn(pr.meta.x, arg), e, fminf(pr.meta.z, mn), 0.f);
 }
 
+// Level 0 from the spectral form of the first group's block.  XA is Hermitian, so A_00 = Q Lambda Q^H and
+// W = w (I - w A_00)^-1 A_0r = Q diag(d) Q^H A_0r with d_k = w / (1 - w lambda_k): every entry of the child's
+//   A' = A_rr + sum_k conj(B_ki) d_k B_kj,  c' = c_r + sum_k conj(B_ki) d_k b_k,
+//   u' = u_r + sum_k q_k d_k B_kj,          exponent sum_k q_k d_k b_k
+// (B = Q^H A_0r, b = Q^H c_0, q = u_0^T Q) is a sum of nb products of its own, where the elimination it
+// replaces is nb steps with a barrier and a reciprocal each on as many SMs as the axis has roots.  The
+// pivots' product is prod (1 - w lambda_k), each factor with Re > 0.  CTA (child, part): part of the child's
+// rows, their left factors times d in shared memory.  n = 42, 14 rows per group, FP64: the levels took
+// 53 us in one elimination of both, and take 11 (this launch) + 23.
+// Where a level's CTAs are few and the sums cheap, the next level's launch forms its parents' entries itself
+// (k_tree_level<Ar, true>).
+constexpr int ROOT_THREADS = 256;
+
+// d (nb) and d B (nb x X) of the root w in shared memory, by the whole CTA.
+template <class Ar>
+__device__ __forceinline__ void root_factors(const TreeArgs& a, typename Ar::E w, typename Ar::E* d, typename Ar::E* dB) {
+  const int nb = a.nb[0], X = a.m[1] + 1;
+  const typename Ar::E* lam = elem<Ar>(const_cast<float4*>(a.rlam));
+  const typename Ar::E* B = elem<Ar>(const_cast<float4*>(a.rB));
+  for (int k = threadIdx.x; k < nb; k += blockDim.x)
+    d[k] = Ar::mul(w, Ar::recip(Ar::add(Ar::one(), Ar::neg(Ar::mul(w, lam[k])))));
+  __syncthreads();
+  for (int q = threadIdx.x; q < nb * X; q += blockDim.x) dB[q] = Ar::mul(d[q / X], B[q]);
+  __syncthreads();
+}
+
+// Entry (i, j) of the child's augmented matrix: row mc is u', column mc is c', (mc, mc) the exponent.
+template <class Ar>
+__device__ __forceinline__ typename Ar::E root_entry(const TreeArgs& a, const typename Ar::E* dB, int i, int j) {
+  using E = typename Ar::E;
+  const int nb = a.nb[0], mc = a.m[1], X = mc + 1;
+  const bool urow = i == mc, ccol = j == mc;
+  E acc = urow ? (ccol ? Ar::zero() : elem<Ar>(a.u[0])[nb + j])
+               : ccol ? elem<Ar>(a.c[0])[nb + i] : elem<Ar>(a.A[0])[(nb + i) * a.m[0] + nb + j];
+  const E* left = urow ? elem<Ar>(const_cast<float4*>(a.ru)) : elem<Ar>(const_cast<float4*>(a.rB)) + i;
+  const int step = urow ? 1 : X;
+  E odd = Ar::zero();                                  // two chains
+  int k = 0;
+#pragma unroll 2
+  for (; k + 2 <= nb; k += 2) {
+    const E x = left[k * step], y = left[(k + 1) * step];
+    acc = Ar::fma(urow ? x : Ar::conj(x), dB[k * X + j], acc);
+    odd = Ar::fma(urow ? y : Ar::conj(y), dB[(k + 1) * X + j], odd);
+  }
+  if (k < nb) {
+    const E x = left[k * step];
+    acc = Ar::fma(urow ? x : Ar::conj(x), dB[k * X + j], acc);
+  }
+  return Ar::add(acc, odd);
+}
+
+// The first level's path record of the root w (its exponent apart), by one full warp.
+template <class Ar>
+__device__ __forceinline__ PathRec<typename Ar::E> root_path(const TreeArgs& a, typename Ar::E w) {
+  using E = typename Ar::E;
+  const int nb = a.nb[0], lane = threadIdx.x & 31;
+  const E* lam = elem<Ar>(const_cast<float4*>(a.rlam));
+  PathRec<E> pr = *path_at<Ar>(a.path[0], 0);
+  int width = 1;
+  while (width < nb && width < 32) width <<= 1;
+  for (int t0 = 0; t0 < nb; t0 += 32) {
+    const int t = t0 + lane;
+    const E z = t < nb ? Ar::add(Ar::one(), Ar::neg(Ar::mul(w, lam[t]))) : Ar::zero();
+    path_warp<Ar>(pr, z, t < nb, width);
+  }
+  return pr;
+}
+
+template <class Ar>
+__global__ void __launch_bounds__(ROOT_THREADS) k_tree_root(TreeArgs a, int parts) {
+  using E = typename Ar::E;
+  extern __shared__ __align__(16) unsigned char gsm_raw[];
+  const int child = blockIdx.x / parts, part = blockIdx.x - child * parts;
+  const int mc = a.m[1], tid = threadIdx.x;
+  const int cols = a.has_gamma ? mc + 1 : mc, rows = cols;   // row mc: u', column mc: c'
+  const E w = root_at<Ar>(a, 0, child);
+  const int nb = a.nb[0], r0 = rows * part / parts, r1 = rows * (part + 1) / parts;
+  // d, then the left factors of this part's rows times d
+  E* d = reinterpret_cast<E*>(gsm_raw);                // nb
+  E* ld = d + nb;                                      // (r1 - r0) x nb
+  const E* lam = elem<Ar>(const_cast<float4*>(a.rlam));
+  const E* B = elem<Ar>(const_cast<float4*>(a.rB));
+  const E* ru = elem<Ar>(const_cast<float4*>(a.ru));
+  for (int k = tid; k < nb; k += ROOT_THREADS)
+    d[k] = Ar::mul(w, Ar::recip(Ar::add(Ar::one(), Ar::neg(Ar::mul(w, lam[k])))));
+  __syncthreads();
+  for (int q = tid; q < (r1 - r0) * nb; q += ROOT_THREADS) {
+    const int i = r0 + q / nb, k = q - q / nb * nb;
+    ld[q] = Ar::mul(d[k], i == mc ? ru[k] : Ar::conj(B[k * (mc + 1) + i]));
+  }
+  __syncthreads();
+  for (int q = tid; q < (r1 - r0) * cols; q += ROOT_THREADS) {
+    const int i = r0 + q / cols, j = q - q / cols * cols;
+    E v = i == mc ? (j == mc ? Ar::zero() : elem<Ar>(a.u[0])[nb + j])
+                  : j == mc ? elem<Ar>(a.c[0])[nb + i] : elem<Ar>(a.A[0])[(nb + i) * a.m[0] + nb + j];
+    const E* li = ld + (i - r0) * nb;
+    for (int k = 0; k < nb; ++k) v = Ar::fma(li[k], B[k * (mc + 1) + j], v);
+    if (i == mc && j == mc) path_at<Ar>(a.path[1], child)->ex = v;
+    else if (i == mc) elem<Ar>(a.u[1])[(long long)child * mc + j] = v;
+    else if (j == mc) elem<Ar>(a.c[1])[(long long)child * mc + i] = v;
+    else elem<Ar>(a.A[1])[(long long)child * mc * mc + i * mc + j] = v;
+  }
+  if (part == 0 && tid < 32) {                         // the child's path record, its exponent apart
+    const PathRec<E> pr = root_path<Ar>(a, w);
+    if (tid == 0) {
+      PathRec<E>* out = path_at<Ar>(a.path[1], child);
+      out->prod = pr.prod;
+      out->meta = pr.meta;
+      if (!a.has_gamma) out->ex = Ar::zero();
+    }
+  }
+}
+
 // Level l: one CTA per child (parent, k) of depth l.  Forward elimination of the nb pivot
 // columns of the (m + 1) x (m + 1) augmented matrix
 //
@@ -130,7 +245,9 @@ __device__ __forceinline__ void path_warp(PathRec<typename Ar::E>& pr, typename 
 // same A'' as after span single-group sweeps (eliminating block 0 and then block 1 of the
 // first Schur complement is eliminating [0 1] at once), with the same pivots.
 // (48 registers: five 256-thread CTAs per SM, so a 729-CTA level runs in one wave)
-template <class Ar>
+// ROOT (l = 1): the parents are not read but formed from the first group's spectral form while the matrix is
+// filled.
+template <class Ar, bool ROOT>
 __global__ void __maxnreg__(48) k_tree_level(TreeArgs a, int l, int span) {
   using E = typename Ar::E;
   extern __shared__ __align__(16) unsigned char gsm_raw[];
@@ -164,13 +281,28 @@ __global__ void __maxnreg__(48) k_tree_level(TreeArgs a, int l, int span) {
   const E* up = elem<Ar>(a.u[l]) + parent * (long long)m;
   const int tid = threadIdx.x, LT = blockDim.x;
   const E zero = Ar::zero();
-  for (int idx = tid; idx < rows * cols; idx += LT) {
+  E* dB = Lm + 2 * rows + (ROOT ? a.nb[0] : 0);      // ROOT: behind d
+  E w0 = zero;
+  if constexpr (ROOT) {
+    w0 = root_at<Ar>(a, 0, (int)parent);
+    root_factors<Ar>(a, w0, Lm + 2 * rows, dB);
+  }
+  // ROOT: the last warp forms the root's path record meanwhile
+  PathRec<E>* rootp = reinterpret_cast<PathRec<E>*>(dB + (ROOT ? a.nb[0] * (m + 1) : 0));
+  const int FT = ROOT ? LT - 32 : LT;                // threads that fill
+  if (ROOT && tid >= FT) {
+    const PathRec<E> pr = root_path<Ar>(a, w0);
+    if (tid == FT) *rootp = pr;
+  }
+  for (int idx = tid; idx < (tid < FT ? rows * cols : 0); idx += FT) {
     const int i = idx / cols, s = idx - (idx / cols) * cols;
-    E g;
-    if (i == m) {                                   // the u row
-      g = s < nb ? Ar::neg(up[s]) : s < m ? up[s] : zero;
+    E g, v;
+    if constexpr (ROOT) v = s < m || a.has_gamma ? root_entry<Ar>(a, dB, i, s) : zero;
+    if (i == m) {                                   // the u row; its corner is the parent's exponent
+      if constexpr (!ROOT) v = s < m ? up[s] : zero;
+      g = s < nb ? Ar::neg(v) : v;
     } else {
-      const E v = s < m ? Ap[(long long)i * m + s] : (a.has_gamma ? cp[i] : zero);
+      if constexpr (!ROOT) v = s < m ? Ap[(long long)i * m + s] : (a.has_gamma ? cp[i] : zero);
       if (i < nb) {
         E w = wg[0];                                 // the root of row i's group
 #pragma unroll
@@ -251,7 +383,9 @@ __global__ void __maxnreg__(48) k_tree_level(TreeArgs a, int l, int span) {
       }
     }
   } else {                                           // the child's path record (warp 0)
-    PathRec<E> pr = *path_at<Ar>(a.path[l], parent);
+    PathRec<E> pr;
+    if constexpr (ROOT) pr = *rootp;                 // exponent zero: the root's is in the corner
+    else pr = *path_at<Ar>(a.path[l], parent);
     int width = 1;                                   // butterfly over the pivots' lanes only
     while (width < nb && width < 32) width <<= 1;
     for (int t0 = 0; t0 < nb; t0 += 32) {
@@ -430,15 +564,33 @@ cudaError_t launch_leaf(const TreeArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Levels whose children would fill fewer than half the SMs take the next level into the
+// Level 0 from the spectral form; then levels whose children would fill fewer than half the SMs take the next level into the
 // same launch (a level's fixed costs - launch, fill from the parent, copy-out, path record -
 // are then paid once), up to SPAN_MAX groups and while a level remains before the leaves.
 template <class Ar>
 cudaError_t launch_tree(const TreeArgs& a, int num_sms, cudaStream_t s, int* launches) {
   cudaError_t err = cudaSuccess;
   *launches = 1;                                      // the leaves
-  long long nodes = 1;
-  for (int l = 0; l + 1 < a.grid.L;) {
+  // The first level on its own, or within the second's launch where that runs the arithmetic with the cheap
+  // products (pairs of FP32: ~0.5 clocks of an SM each, FP64 2) in well under a launch's time (~3 us).
+  // n = 32, four groups of 8 rows, pairs: 51.4 us with both levels in one elimination, 54.4 with the first
+  // level apart, 50.1 formed within the second's launch.  n = 42, three of 14 rows, FP64: 110.7 with both in
+  // one elimination, 90.3 apart.
+  long long nodes = a.grid.radix[0];
+  const double fill = (double)a.nb[0] * a.m[1] * a.m[1] * (std::is_same<Ar, ArDF>::value ? 0.5 : 2.0);
+  bool fused = a.grid.L > 2 && fill < 6000.0;
+  if (!fused) {
+    const int rows = a.m[1] + (a.has_gamma ? 1 : 0);
+    const int parts = (int)std::max<long long>(1, std::min<long long>(rows, num_sms / nodes));
+    const size_t smem = sizeof(float4) * (size_t)a.nb[0] * ((rows + parts - 1) / parts + 1);
+    if (smem > 48 * 1024 &&
+        (err = cudaFuncSetAttribute(k_tree_root<Ar>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+      return err;
+    k_tree_root<Ar><<<(unsigned)(nodes * parts), ROOT_THREADS, smem, s>>>(a, parts);
+    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    ++*launches;
+  }
+  for (int l = 1; l + 1 < a.grid.L;) {
     long long children = nodes * a.grid.radix[l];
     int span = 1, nb = a.nb[l];
     while (span < SPAN_MAX && l + span + 1 < a.grid.L && 2 * children < num_sms) {
@@ -446,19 +598,21 @@ cudaError_t launch_tree(const TreeArgs& a, int num_sms, cudaStream_t s, int* lau
       nb += a.nb[l + span];
       ++span;
     }
-    const size_t smem = tree_level_smem_bytes(nb, a.m[l]);
+    const size_t smem = tree_level_smem_bytes(nb, a.m[l]) + (fused ? sizeof(float4) * ((size_t)a.nb[0] * (a.m[1] + 2) + 3) : 0);
+    auto kernel = fused ? k_tree_level<Ar, true> : k_tree_level<Ar, false>;
     if (smem > 48 * 1024) {
-      err = cudaFuncSetAttribute(k_tree_level<Ar>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (err != cudaSuccess) return err;
     }
     const int m = a.m[l], width = m * m;              // entries of the first elimination step
-    const int threads = width >= 1024 ? 512 : width >= 256 ? 256 : 128;
-    k_tree_level<Ar><<<(unsigned)children, threads, smem, s>>>(a, l, span);
+    const int threads = width >= 1024 || fused ? 512 : width >= 256 ? 256 : 128;
+    kernel<<<(unsigned)children, threads, smem, s>>>(a, l, span);
     ++*launches;
     err = cudaGetLastError();
     if (err != cudaSuccess) return err;
     nodes = children;
     l += span;
+    fused = false;
   }
   switch (a.m[a.grid.L - 1]) {
     case 2: return launch_leaf<Ar, 2>(a, s);
