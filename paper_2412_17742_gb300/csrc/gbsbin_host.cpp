@@ -1540,6 +1540,7 @@ int gbsbin_execute(gbsbin_plan* P, double* P_out, void* stream) {
     t.q1re = P->logq1.real();
     t.q1im = P->logq1.imag();
     t.q1minpiv = P->logq1_minpiv;
+    t.shared_gpu = P->dft_plain ? 1 : 0;
     int nl = 0;
     if (launch_points_btree(t, P->btree_steps.data(), (int)P->btree_steps.size(),
                             P->kernel == GBSBIN_KERNEL_BTREE_FP64, P->num_sms, s, &nl) != cudaSuccess)

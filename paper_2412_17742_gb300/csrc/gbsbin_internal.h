@@ -176,7 +176,7 @@ struct TreeArgs {
 // the first d axes' roots, and a path record (pivot product; FP32 argument sum, power of
 // two, smallest pivot real part).  Level l runs as sub-steps of nbs pivots of its group,
 // each a top launch (CTA per child) and a bottom launch (CTAs per row chunk); the last
-// group's blocks are reduced to Hessenberg form (a CTA per leaf parent) and every evaluated
+// group's blocks are reduced to Hessenberg form (a CTA, or a cluster of them, per leaf parent) and every evaluated
 // point is an O(m^2) Hessenberg elimination (a warp per point) writing the unfinished log q.
 #define GBSBIN_BT_MAX_HESS 116          // largest last group reduced in shared memory (225 KB at 116)
 #define GBSBIN_BT_MAX_LAST 192          // largest last group (above 116 rows the reduction works
@@ -205,6 +205,7 @@ struct BTreeArgs {
                             // k_{L-1} = 0 or 2 k_{L-1} >= radix[L-1], so every evaluated point of
                             // the half grid is written exactly once
   int halve_first;
+  int shared_gpu;           // other launches run beside this plan's (batches)
   long long n_leaves;       // leaves: prod cnt[l]
   // a shard (last axis halved): level 0 takes the roots k0_lo .. k0_lo + cnt[0] - 1, and the
   // leaves write only the evaluated points of the grid's slice [e_lo, e_hi) (grid), at their

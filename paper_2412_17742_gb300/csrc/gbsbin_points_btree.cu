@@ -61,6 +61,7 @@ namespace {
 constexpr int TOP_THREADS = 512;
 constexpr int BOT_WARPS = 16;
 constexpr int HESS_THREADS = 256;
+constexpr int HC_THREADS = 512;
 constexpr int LEAF_WARPS = 4;
 constexpr int LEAF_SMAX = (GBSBIN_BT_MAX_HESS + 31) / 32;       // leaves of last groups <= 128 rows
 constexpr int LEAF_SMAX_BIG = (GBSBIN_BT_MAX_LAST + 31) / 32;   // and above
@@ -315,6 +316,43 @@ __global__ void __launch_bounds__(BOT_WARPS * 32) k_bt_bottom(BTreeArgs a, BTree
   }
 }
 
+// The reflector of x (squared norm nrm2, first entry x0): alpha = -e^{i arg x0} ||x|| and
+// beta = 2 / ||x - alpha e_1||^2 = 1 / (||x||^2 + ||x|| |x0|).
+template <class Ar>
+__device__ __forceinline__ void reflector(typename Ar::E nrm2, typename Ar::E x0, typename Ar::E& alpha,
+                                          typename Ar::E& beta) {
+  using E = typename Ar::E;
+  const E nrm = Ar::rsqrt_real(nrm2);
+  const E ax0 = Ar::rsqrt_real(Ar::norm2(x0));
+  alpha = Ar::re(ax0) > 0.f ? Ar::neg(Ar::mul(x0, Ar::mul(nrm, Ar::rrecip(ax0)))) : Ar::neg(nrm);
+  beta = Ar::rrecip(Ar::add(nrm2, Ar::mul(nrm, ax0)));
+}
+// In FP64 by Newton steps on FP32 seeds, ~30 FP64 instructions instead of ~120 of square roots and divisions: one
+// warp runs this once per column, and each of its FP64 instructions takes 64 clocks.
+template <>
+__device__ __forceinline__ void reflector<ArF64>(double2 nrm2, double2 x0, double2& alpha, double2& beta) {
+  const double a = ::fma(x0.x, x0.x, x0.y * x0.y), b = nrm2.x;
+  if (!(a > 1e-30 && b < 1e30)) {                    // beyond the seeds' range
+    const double nrm = ::sqrt(b), ax = ::sqrt(a);
+    alpha = ax > 0.0 ? make_double2(-x0.x / ax * nrm, -x0.y / ax * nrm) : make_double2(-nrm, 0.0);
+    beta = make_double2(1.0 / ::fma(nrm, ax, b), 0.0);
+    return;
+  }
+  double ra = (double)rsqrtf((float)a), rb = (double)rsqrtf((float)b);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    ra *= ::fma(-0.5 * a * ra, ra, 1.5);
+    rb *= ::fma(-0.5 * b * rb, rb, 1.5);
+  }
+  const double nrm = b * rb, ax = a * ra, f = -nrm * ra;
+  alpha = make_double2(f * x0.x, f * x0.y);
+  const double d = ::fma(nrm, ax, b);
+  double y = (double)__frcp_rn((float)d);
+  y = ::fma(y, ::fma(-d, y, 1.0), y);
+  y = ::fma(y, ::fma(-d, y, 1.0), y);
+  beta = make_double2(y, 0.0);
+}
+
 // ------------------------------------------------------------------------- Hessenberg
 // One CTA per leaf parent: the m x m block A_L with c and conj(u) as two extra columns in
 // shared memory (row stride m + 3, odd in 16-byte units), or, for GM (m above
@@ -366,12 +404,7 @@ __global__ void __launch_bounds__(HESS_THREADS) k_bt_hess(BTreeArgs a) {
       const E x0 = at(k + 1, k);
       E alpha = Ar::zero(), beta = Ar::zero();
       if (Ar::re(nrm2) > 0.f) {
-        const E nrm = Ar::rsqrt_real(nrm2);
-        const E ax0 = Ar::rsqrt_real(Ar::norm2(x0));
-        alpha = Ar::re(ax0) > 0.f ? Ar::neg(Ar::mul(x0, Ar::mul(nrm, Ar::rrecip(ax0)))) : Ar::neg(nrm);
-        // ||v||^2 = ||x||^2 - 2 Re(conj(alpha) x0) + |alpha|^2 = 2 (||x||^2 + ||x|| |x0|)
-        const E vn2 = Ar::add(Ar::add(nrm2, nrm2), Ar::add(Ar::mul(nrm, ax0), Ar::mul(nrm, ax0)));
-        beta = Ar::add(Ar::rrecip(vn2), Ar::rrecip(vn2));
+        reflector<Ar>(nrm2, x0, alpha, beta);
       }
       for (int i = k + 1 + lane; i < m; i += 32) {
         E vi = at(i, k);
@@ -447,6 +480,166 @@ __global__ void __launch_bounds__(HESS_THREADS) k_bt_hess(BTreeArgs a) {
     hv[m + i] = at(i, m);               // b = Q^H c
   }
   if (tid == 0) hv[2 * m] = src[(long long)m * D + m];   // the exponent so far
+}
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// 16 bytes into the same shared-memory place of the cluster's CTA `rank`
+template <class E>
+__device__ __forceinline__ void put_cluster(E* p, int rank, const E& v) {
+  static_assert(sizeof(E) == 16, "16-byte elements");
+  const unsigned local = (unsigned)__cvta_generic_to_shared(p);
+  unsigned remote;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
+  const float4 f = *reinterpret_cast<const float4*>(&v);
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(remote), "f"(f.x), "f"(f.y), "f"(f.z), "f"(f.w)
+               : "memory");
+}
+
+// The same reduction by a cluster of C CTAs per node, for levels with too few nodes to fill the SMs (41 nodes of 100
+// rows at n = 200).  Column j of [A_L, c, conj(u)] lives in CTA j mod C (local column j / C), in shared memory,
+// m x ld with ld odd.  Step k: the owner of column k forms the reflector (one warp) and writes v and beta to every
+// CTA; each CTA then applies it from the left to its own columns (eight lanes per column: product and update by
+// the same lanes, no barrier between), forms its share of A v (eight lanes per row) and writes it to every
+// CTA; all sum the C shares in order and update their own columns from the right.  Two cluster barriers and two
+// block barriers per column.  v is double-buffered: the next reflector is written while others still read this
+// one.
+template <class Ar>
+__global__ void __launch_bounds__(HC_THREADS) k_bt_hess_cluster(BTreeArgs a, int C) {
+  using E = typename Ar::E;
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  const int m = a.mL, D = m + 1, cw = (m + 2 + C - 1) / C, ld = cw | 1;
+  const int rank = (int)(blockIdx.x % C);
+  const long long node = blockIdx.x / C;
+  E* A = reinterpret_cast<E*>(sm_raw);               // m x ld
+  E* vbuf = A + (size_t)m * ld;                      // 2 x (m + 1): v, then beta
+  E* tp = vbuf + 2 * (m + 1);                        // C x m shares of A v
+  E* Hn = elem<Ar>(a.H) + node * (long long)m * m;
+  E* hv = elem<Ar>(a.hv) + node * (long long)(2 * m + 1);
+  const E* src = elem<Ar>(a.mat[a.L - 1]) + node * (long long)D * D;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = tid & 7, q = tid & 3;
+  constexpr int GROUPS = HC_THREADS / 8, RGROUPS = HC_THREADS / 4;   // columns, rows at a time
+  auto scale = [](E b, E x) {                        // by a real factor
+    if constexpr (std::is_same<Ar, ArF64>::value) return make_double2(b.x * x.x, b.x * x.y);
+    else return Ar::mul(b, x);
+  };
+  const int mine = (m + 2 - rank + C - 1) / C;       // own columns (with c and conj(u))
+  const int mineA = (m - rank + C - 1) / C;          // of A_L alone
+  for (int idx = tid; idx < m * mine; idx += HC_THREADS) {
+    const int i = idx / mine, jl = idx - i * mine, j = jl * C + rank;
+    A[(size_t)i * ld + jl] = j < m    ? src[(long long)i * D + j]
+                             : j == m ? src[(long long)i * D + m]
+                                      : Ar::conj(src[(long long)m * D + i]);
+  }
+  __syncthreads();
+  for (int k = 0; k + 2 < m; ++k) {
+    E* v = vbuf + (k & 1) * (m + 1);
+    if (rank == k % C && warp == 0) {                // the reflector of column k, to every CTA
+      E* col = A + k / C;
+      E nrm2 = Ar::zero();
+      for (int i = k + 1 + lane; i < m; i += 32) nrm2 = Ar::add(nrm2, Ar::norm2(col[(size_t)i * ld]));
+      for (int o = 16; o > 0; o >>= 1) nrm2 = Ar::add(nrm2, shfl_xor(nrm2, o));
+      const E x0 = col[(size_t)(k + 1) * ld];
+      E alpha = Ar::zero(), beta = Ar::zero();
+      if (Ar::re(nrm2) > 0.f) reflector<Ar>(nrm2, x0, alpha, beta);
+      for (int i = k + 1 + lane; i < m; i += 32) {
+        E vi = col[(size_t)i * ld];
+        if (i == k + 1) vi = Ar::add(vi, Ar::neg(alpha));
+        for (int r = 0; r < C; ++r) put_cluster(v + i, r, vi);
+      }
+      if (lane < C) put_cluster(v + m, lane, beta);
+      if (lane == 0 && Ar::re(beta) > 0.f) col[(size_t)(k + 1) * ld] = alpha;
+    }
+    cluster_sync();
+    const E beta = v[m];
+    if (!(Ar::re(beta) > 0.f)) continue;             // the same for every CTA
+    // left: own columns j > k
+    const int j0 = (k + 1 - rank + C - 1) / C;       // first own column right of k
+    for (int w0 = j0 + 4 * warp; w0 < mine; w0 += GROUPS) {   // four columns a warp
+      const int jl = w0 + (lane >> 3);
+      const bool on = jl < mine;
+      E* col = A + (on ? jl : 0);
+      E s = Ar::zero();
+      for (int i = k + 1 + g; i < m; i += 8) s = Ar::fma(Ar::conj(v[i]), col[(size_t)i * ld], s);
+      for (int o = 4; o > 0; o >>= 1) s = Ar::add(s, shfl_xor(s, o));
+      s = scale(beta, s);
+      if (on)
+        for (int i = k + 1 + g; i < m; i += 8) col[(size_t)i * ld] = Ar::fms(col[(size_t)i * ld], v[i], s);
+    }
+    __syncthreads();
+    // right: this CTA's share of beta A v, to every CTA (four lanes per row: 8 or more columns each)
+    for (int w0 = 8 * warp; w0 < m; w0 += RGROUPS) {
+      const int i = w0 + (lane >> 2);
+      const bool on = i < m;
+      const E* row = A + (size_t)(on ? i : 0) * ld;
+      E t = Ar::zero();
+      for (int jl = j0 + q; jl < mineA; jl += 4) t = Ar::fma(row[jl], v[jl * C + rank], t);
+      for (int o = 2; o > 0; o >>= 1) t = Ar::add(t, shfl_xor(t, o));
+      t = scale(beta, t);
+      if (on)
+        for (int r = q; r < C; r += 4) put_cluster(tp + rank * m + i, r, t);
+    }
+    cluster_sync();
+    for (int i = tid >> 2; i < m; i += RGROUPS) {
+      E t = tp[i];
+      for (int r = 1; r < C; ++r) t = Ar::add(t, tp[r * m + i]);
+      E* row = A + (size_t)i * ld;
+      for (int jl = j0 + q; jl < mineA; jl += 4) row[jl] = Ar::fms(row[jl], t, Ar::conj(v[jl * C + rank]));
+    }
+    __syncthreads();
+  }
+  for (int idx = tid; idx < m * mineA; idx += HC_THREADS) {
+    const int i = idx / mineA, jl = idx - i * mineA;
+    Hn[(long long)i * m + jl * C + rank] = A[(size_t)i * ld + jl];
+  }
+  if (rank == m % C)
+    for (int i = tid; i < m; i += HC_THREADS) hv[m + i] = A[(size_t)i * ld + m / C];               // b = Q^H c
+  if (rank == (m + 1) % C)
+    for (int i = tid; i < m; i += HC_THREADS) hv[i] = Ar::conj(A[(size_t)i * ld + (m + 1) / C]);   // a = Q^T u
+  if (rank == 0 && tid == 0) hv[2 * m] = src[(long long)m * D + m];
+  cluster_sync();                                    // no CTA leaves while others may still write to it
+}
+
+size_t hess_cluster_smem(int m, int C) {
+  const int ld = ((m + 2 + C - 1) / C) | 1;
+  return sizeof(float4) * ((size_t)m * ld + 2 * (size_t)(m + 1) + (size_t)C * m);
+}
+
+// CTAs per node of the Householder launch: as many, up to HC_MAX, as leave every CTA an SM of its own (41 nodes of
+// 100 rows, whole tables: FP64 5249 us with one CTA, 4612 with two, 4370 with three, and a fourth, on 164 > 152
+// SMs, puts a second one on some and doubles their nodes' time; pairs 1961, 1483, 1391.  14 nodes of 60 rows: 552,
+// 472, 455).  Below 32 rows the two cluster barriers per column cost what the split saves (27 rows: 240, 231, 240).
+// With one CTA this kernel and k_bt_hess take the same time (231 nodes of 64 rows: 1613 and 1613).  Tables that
+// share the GPU with others (batches) keep one CTA per node: their other streams fill the SMs (48 problems: 15.1 ms,
+// with clusters 16.1).
+constexpr int HC_MAX = 4;
+int hess_cluster_size(int m, long long nodes, int num_sms) {
+  if (m < 32) return 1;
+  const int C = (int)std::min<long long>(HC_MAX, num_sms / nodes);
+  return C < 2 ? 1 : C;
+}
+
+template <class Ar>
+cudaError_t launch_hess_cluster(const BTreeArgs& a, long long nodes, int C, cudaStream_t s) {
+  const size_t smem = hess_cluster_smem(a.mL, C);
+  cudaError_t err = cudaSuccess;
+  if (smem > 48 * 1024 && (err = cudaFuncSetAttribute(k_bt_hess_cluster<Ar>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                      (int)smem)) != cudaSuccess)
+    return err;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(nodes * C));
+  cfg.blockDim = dim3(HC_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)C;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_bt_hess_cluster<Ar>, a, C);
 }
 
 // ----------------------------------------------------------------------------- leaves
@@ -687,7 +880,10 @@ cudaError_t launch_btree_ar(const BTreeArgs& a, const BTreeStep* steps, int nste
   long long parents = 1;
   for (int l = 0; l + 1 < a.grid.L; ++l) parents *= a.cnt[l];
   const size_t hsmem = btree_hess_smem_bytes(a.mL);
-  if (a.mL <= GBSBIN_BT_MAX_HESS) {
+  const int C = a.shared_gpu ? 1 : hess_cluster_size(a.mL, parents, num_sms);
+  if (C > 1 && hess_cluster_smem(a.mL, C) <= 225 * 1024) {
+    if ((err = launch_hess_cluster<Ar>(a, parents, C, s)) != cudaSuccess) return err;
+  } else if (a.mL <= GBSBIN_BT_MAX_HESS) {
     if (hsmem > 48 * 1024) {
       err = cudaFuncSetAttribute(k_bt_hess<Ar, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hsmem);
       if (err != cudaSuccess) return err;
