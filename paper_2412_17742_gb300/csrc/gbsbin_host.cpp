@@ -310,9 +310,23 @@ bool cholesky(std::vector<double>& re, std::vector<double>& im, int n) {
   return true;
 }
 
-// XA = I - Sigma^{-1}, Xgamma = Sigma^{-1} z-bar, gamma = X Xgamma, Sigma = I + Sigma^(1).
-int adjacency(const std::vector<cd>& S1, const std::vector<cd>& zbar, int n, std::vector<cd>& XA,
-              std::vector<cd>& gamma, std::vector<cd>& Xgamma) {
+// ERR_ARG for a non-finite entry, ERR_NONPHYSICAL where S1 is not Hermitian: an entry further than kHermTol times
+// the largest magnitude so far (at least 1) from its mirror image.  Almost every matrix passes at scale 1 already,
+// which is checked in tiles on the host threads; only the others take the row-by-row scan.
+int hermitian_check(const std::vector<cd>& S1, int n) {
+  constexpr int B = 32;
+  const int tiles = (n + B - 1) / B;
+  std::vector<char> fails(host_threads(), 0);
+  parallel_run(n >= 96 ? host_threads() : 1, [&](int t, int nth) {
+    for (int ti = t; ti < tiles; ti += nth)
+      for (int tj = 0; tj <= ti; ++tj)
+        for (int i = ti * B; i < std::min(n, (ti + 1) * B); ++i)
+          for (int j = tj * B; j < std::min(n, (tj + 1) * B); ++j) {
+            const cd a = S1[(size_t)i * n + j], b = S1[(size_t)j * n + i];
+            if (!(std::norm(a - std::conj(b)) <= kHermTol * kHermTol) || !(std::norm(a) < 1e300)) fails[t] = 1;
+          }
+  });
+  if (std::none_of(fails.begin(), fails.end(), [](char f) { return f != 0; })) return GBSBIN_OK;
   double scale2 = 1.0;                               // running max of |a|^2 (squares compared)
   for (int i = 0; i < n; ++i)
     for (int j = 0; j < n; ++j) {
@@ -321,6 +335,14 @@ int adjacency(const std::vector<cd>& S1, const std::vector<cd>& zbar, int n, std
       scale2 = std::fmax(scale2, std::norm(a));
       if (std::norm(a - std::conj(b)) > kHermTol * kHermTol * scale2) return GBSBIN_ERR_NONPHYSICAL;
     }
+  return GBSBIN_OK;
+}
+
+// XA = I - Sigma^{-1}, Xgamma = Sigma^{-1} z-bar, gamma = X Xgamma, Sigma = I + Sigma^(1).
+int adjacency(const std::vector<cd>& S1, const std::vector<cd>& zbar, int n, std::vector<cd>& XA,
+              std::vector<cd>& gamma, std::vector<cd>& Xgamma) {
+  const int hst = hermitian_check(S1, n);
+  if (hst) return hst;
   // physicality: Sigma - I/2 = Sigma^(1) + I/2 positive definite <=> ||I - Sigma^{-1}|| < 1
   const size_t nn = (size_t)n * n;
   std::vector<double> cr(nn), ci(nn);
@@ -397,24 +419,61 @@ int adjacency(const std::vector<cd>& S1, const std::vector<cd>& zbar, int n, std
   return GBSBIN_OK;
 }
 
-int build_state(const gbsbin_problem* p, int n, std::vector<cd>& XA, std::vector<cd>& gamma,
-                std::vector<cd>& Xgamma, int* has_gamma, std::vector<cd>* zbar_out = nullptr,
-                std::vector<cd>* s1_out = nullptr) {
-  std::vector<cd> S1, zbar;
-  if (p->sigma1) {
-    S1.resize((size_t)n * n);
-    for (size_t q = 0; q < S1.size(); ++q) S1[q] = cd(p->sigma1[q].re, p->sigma1[q].im);
-    zbar.assign(n, 0.0);
-    if (p->zbar)
-      for (int q = 0; q < n; ++q) zbar[q] = cd(p->zbar[q].re, p->zbar[q].im);
-  } else {
-    int st = physical_state(p, S1, zbar);
-    if (st) return st;
+// Sigma^(1) and z-bar of a problem's state, physical description or direct.
+int covariance(const gbsbin_problem* p, int n, std::vector<cd>& S1, std::vector<cd>& zbar) {
+  if (!p->sigma1) return physical_state(p, S1, zbar);
+  S1.resize((size_t)n * n);
+  for (size_t q = 0; q < S1.size(); ++q) S1[q] = cd(p->sigma1[q].re, p->sigma1[q].im);
+  zbar.assign(n, 0.0);
+  if (p->zbar)
+    for (int q = 0; q < n; ++q) zbar[q] = cd(p->zbar[q].re, p->zbar[q].im);
+  return GBSBIN_OK;
+}
+
+// What the cumulants need of the state: Sigma^(1), checked as for the adjacency, and for displaced states
+// Xgamma = Sigma^{-1} z-bar by two triangular solves with Sigma's Cholesky factor, gamma = X Xgamma; neither
+// Sigma^{-1} nor XA is formed (at n = 512 those were 2.8 ms of a 10.1 ms call, now 6.1).
+int moment_state(const gbsbin_problem* p, int n, std::vector<cd>& S1, std::vector<cd>& gamma, std::vector<cd>& Xgamma) {
+  std::vector<cd> zbar;
+  int st = covariance(p, n, S1, zbar);
+  if (st || (st = hermitian_check(S1, n))) return st;
+  std::vector<double> cr, ci;
+  auto factor = [&](double shift) {
+    cr.resize((size_t)n * n);
+    ci.resize((size_t)n * n);
+    for (size_t q = 0; q < cr.size(); ++q) {
+      cr[q] = S1[q].real();
+      ci[q] = S1[q].imag();
+    }
+    for (int i = 0; i < n; ++i) cr[(size_t)i * n + i] += shift;
+    return cholesky(cr, ci, n);
+  };
+  if (!factor(0.5)) return GBSBIN_ERR_NONPHYSICAL;
+  gamma.assign(n, 0.0);
+  Xgamma.assign(n, 0.0);
+  if (std::all_of(zbar.begin(), zbar.end(), [](const cd& z) { return z == cd(0.0); })) return GBSBIN_OK;
+  if (!factor(1.0)) return GBSBIN_ERR_NONPHYSICAL;
+  std::vector<cd>& x = Xgamma;
+  for (int i = 0; i < n; ++i) {                      // C y = z-bar
+    cd s = zbar[i];
+    for (int j = 0; j < i; ++j) s -= cd(cr[(size_t)i * n + j], ci[(size_t)i * n + j]) * x[j];
+    x[i] = s / cr[(size_t)i * n + i];
   }
-  int st = adjacency(S1, zbar, n, XA, gamma, Xgamma);
+  for (int i = n - 1; i >= 0; --i) {                 // C^H x = y, by rows of C
+    x[i] /= cr[(size_t)i * n + i];
+    for (int j = 0; j < i; ++j) x[j] -= cd(cr[(size_t)i * n + j], -ci[(size_t)i * n + j]) * x[i];
+  }
+  for (int i = 0; i < n; ++i) gamma[i] = x[i < n / 2 ? i + n / 2 : i - n / 2];
+  return GBSBIN_OK;
+}
+
+int build_state(const gbsbin_problem* p, int n, std::vector<cd>& XA, std::vector<cd>& gamma,
+                std::vector<cd>& Xgamma, int* has_gamma, std::vector<cd>* zbar_out = nullptr) {
+  std::vector<cd> S1, zbar;
+  int st = covariance(p, n, S1, zbar);
+  if (!st) st = adjacency(S1, zbar, n, XA, gamma, Xgamma);
   if (st) return st;
   if (zbar_out) *zbar_out = zbar;
-  if (s1_out) s1_out->swap(S1);
   *has_gamma = 0;
   for (int i = 0; i < n; ++i)
     if (gamma[i] != cd(0.0)) *has_gamma = 1;
@@ -2175,9 +2234,8 @@ int gbsbin_cumulants_device(const gbsbin_problem* p, int precision, double* mean
   if (st) return st;
   if (p->L > GBSBIN_MOM_MAX_L) return GBSBIN_ERR_UNSUPPORTED;
   const int MK = p->M * p->K, n = 2 * MK, L = p->L;
-  std::vector<cd> XA, gamma, Xgamma, S1;
-  int has_gamma = 0;
-  if ((st = build_state(p, n, XA, gamma, Xgamma, &has_gamma, nullptr, &S1))) return st;
+  std::vector<cd> gamma, Xgamma, S1;
+  if ((st = moment_state(p, n, S1, gamma, Xgamma))) return st;
   std::vector<int> perm, goff(L + 1, 0);
   for (int l = 0; l < L; ++l) {
     goff[l] = (int)perm.size();
@@ -2186,12 +2244,14 @@ int gbsbin_cumulants_device(const gbsbin_problem* p, int precision, double* mean
   }
   goff[L] = n;
   std::vector<cd> Wp((size_t)n * n), gp(n), Xgp(n);
-  for (int a = 0; a < n; ++a) {
-    for (int b = 0; b < n; ++b)
-      Wp[(size_t)a * n + b] = 0.5 * (S1[(size_t)perm[a] * n + perm[b]] + std::conj(S1[(size_t)perm[b] * n + perm[a]]));
-    gp[a] = gamma[perm[a]];
-    Xgp[a] = Xgamma[perm[a]];
-  }
+  parallel_run(n >= 96 ? host_threads() : 1, [&](int t, int nth) {
+    for (int a = t; a < n; a += nth) {
+      for (int b = 0; b < n; ++b)
+        Wp[(size_t)a * n + b] = 0.5 * (S1[(size_t)perm[a] * n + perm[b]] + std::conj(S1[(size_t)perm[b] * n + perm[a]]));
+      gp[a] = gamma[perm[a]];
+      Xgp[a] = Xgamma[perm[a]];
+    }
+  });
   double* out[4] = {mean, cov, k3, k4};
   float ms = 0.f;
   st = cumulants_device(n, L, goff.data(), reinterpret_cast<const double*>(Wp.data()),
