@@ -9,302 +9,351 @@
 //
 //   sum_{n, t} lhaf(A_{(n,t,u)+(n,t,v)}, ...) w^n / (n! t!) = u! v! [x^u y^v] F(w; x, y),
 //   F = exp(xi_F^T M xi_F / 2 + l^T xi_F + e) / sqrt(det(I - X D(w) A_DD)),
-//   N = (I - X D(w) A_DD)^-1 X D(w),  M = A_FF + A_DF^T N A_DF,  l = gamma_F + A_DF^T N gamma_D,
-//   e = gamma_D^T N gamma_D / 2,
 //
-// D the heralding and traced indices (both halves; w = 1 on traced modes), F the kept ones.
-// Hence <v|rho(b)|u> = Pr(0) sqrt(u! v!) [w^b][x^u y^v] F.  Per point of the roots-of-unity grid
-// over the heralding groups a CTA eliminates I - X D(w) A_DD without pivoting (a principal
-// block of I - D(w) XA with ||XA|| < 1: every pivot has Re > 0 and Sum Log is the branch of
-// the square root continuous from w = 0), solves for the kept modes' columns and gamma_D,
-// forms M, l, e, and the Taylor coefficients of exp(xi^T M xi / 2 + l^T xi) by
-// (p_i + 1) c_{p + e_i} = l_i c_p + sum_j M_ij c_{p - e_j} (shells of equal total degree in
-// parallel, from a table of each coefficient's neighbours).  The heralding probability's
-// generating function (every non-heralding mode traced, w = 1 on the kept ones) continues the
-// same elimination into the kept block: its Schur complement is I - X_F M, so it is
-// exp(e + l^T (I - X_F M)^{-1} X_F l / 2) / sqrt(det(I - X D A_DD) det(I - X_F M)), the
-// branch Sum Log of the pivots of the whole unpivoted elimination.  An inverse DFT over the
-// grid, one axis per launch, then extracts [w^b] for every coefficient.  FP64 throughout.
+// D the heralding and traced indices (both halves; w = 1 on traced modes), F the kept ones, and
+// <v|rho(b)|u> = Pr(0) sqrt(u! v!) [w^b][x^u y^v] F.  M, l and e are what block elimination of the D rows
+// of I - D(w) XA leaves in the kept rows: with the augmented form of the tree (gbsbin_tree.cuh) the Schur
+// complement is A'_F = X_F M, its row u' = l and its corner 2 e, and the pivots' product the determinant.  So the
+// points share eliminations like those of the binned tables: the traced rows go on the host once per
+// state (w = 1), the first group by its spectral form for all roots of its axis in one launch (k_tree_root), and a
+// CTA per point sweeps the other groups, from the first group's result of its root.  Then the Taylor
+// coefficients of exp(xi^T M xi / 2 + l^T xi) by (p_i + 1) c_{p + e_i} = l_i c_p + sum_j M_ij c_{p - e_j}
+// (shells of equal total degree in parallel, in shared memory, seven warps), while the eighth warp continues
+// the elimination into the kept block - its Schur complement is I - A'_F - for the heralding probability's
+// generating function (every non-heralding mode traced, w = 1 on the kept ones), and forms both factors
+// exp(e) / sqrt(det) from the pivots' products by inverse roots (no logarithms).  FP64 throughout.
+//
+// What bounds it is the FP64 pipe of the points' SMs (a warp's FP64 instruction takes its scheduler 64
+// clocks): every entry of a sweep is one multiply-add with its row's multiplier, where the elimination it
+// replaces recomputed the multiplier per entry, solved back and added e on one thread.  16 ports x 2 internal modes,
+// two groups of twelve modes, 81 points, 2401 coefficients each: 460 us before (425 of them the point stage, one
+// elimination of 60 rows per point), 117 with the three launches here.
+//
+// The inverse DFT over the heralding grid: rho(b) is Hermitian, so only the channels u <= v are transformed and
+// each is written with its conjugate; the first two axes in one launch through shared memory, sums over k and
+// R - k folded (x_k + x_{R-k} times the cosine, x_k - x_{R-k} times the sine: half the multiplications).
 #include <cuda_runtime.h>
 
-#include "gbsbin_device.cuh"
 #include "gbsbin_herald.h"
+#include "gbsbin_tree.cuh"
 
 namespace gbsbin {
 namespace {
 
 constexpr int HT = 256;
+constexpr int TAYLOR_THREADS = HT - 32;
+constexpr long long SMEM_COEF = 6144;                // coefficients kept in shared memory (96 KB)
 
-__device__ __forceinline__ double2 cadd2(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ double2 cneg2(double2 a) { return make_double2(-a.x, -a.y); }
-
-// Unpivoted elimination of the nr x nr block of G (row stride ld) with ncol right-hand-side
-// columns after it, then back substitution (column by column: each solved entry updates the
-// rows above it in parallel): the columns become the block's inverse times themselves.
-// Returns sum Log(pivots) (each Re > 0) and the smallest pivot real part in thread 0's
-// registers; all threads call it.
-// Sum Log of a sequence of pivots (each Re > 0) without a log or an atan2 per pivot (FP64
-// transcendentals are slow on this GPU): the running product, renormalised by powers of two,
-// and the FP32 sum of the pivots' arguments, which fixes the winding of the product's argument
-// (each argument lies in (-pi/2, pi/2); the FP32 sum errs by far less than pi).
-struct LogDet {
-  double2 prod = make_double2(1.0, 0.0);
-  int e2 = 0, count = 0;
-  float args = 0.f;
-  double mn = 1e300;
-  __device__ void add(double2 p) {
-    prod = cmul(prod, p);
-    args += atan2f((float)p.y, (float)p.x);
-    mn = fmin(mn, p.x);
-    if (!(p.x == p.x) || !(p.y == p.y)) mn = -1e300;
-    if ((++count & 7) == 0) renorm();
-  }
-  __device__ void renorm() {
-    const double m = fmax(fabs(prod.x), fabs(prod.y));
-    if (!(m > 0.0) || !(m < 1e300)) return;
-    const int ex = (int)((__double_as_longlong(m) >> 52) & 0x7ff) - 1022;
-    const double sc = __longlong_as_double((long long)(1023 - ex) << 52);
-    prod = make_double2(prod.x * sc, prod.y * sc);
-    e2 += ex;
-  }
-  __device__ double2 value() {
-    renorm();
-    const double TWO_PI = 6.283185307179586476925286766559, LN2 = 0.693147180559945309417232121458;
-    const double a0 = atan2(prod.y, prod.x);
-    const double wind = rint(((double)args - a0) / TWO_PI);
-    return make_double2(0.5 * log(fma(prod.x, prod.x, prod.y * prod.y)) + e2 * LN2, a0 + TWO_PI * wind);
-  }
-};
-
-__device__ void solve_block(double2* G, int nr, int ncol, int ld, double2* ldet, double* minre) {
-  const int tid = threadIdx.x, T = blockDim.x;
-  const int cols = nr + ncol;
-  LogDet acc;
-  for (int k = 0; k < nr; ++k) {
-    const double2 piv = G[k * ld + k];
-    const double2 r = crecip(piv);
-    if (tid == 0) acc.add(piv);
-    const int w = cols - k - 1;
-    for (int idx = tid; idx < (nr - k - 1) * w; idx += T) {
-      const int i = k + 1 + idx / w, j = k + 1 + idx % w;
-      const double2 li = cmul(G[i * ld + k], r);
-      G[i * ld + j] = cfnma(G[i * ld + j], li, G[k * ld + j]);
-    }
-    __syncthreads();
-  }
-  for (int k = nr - 1; k >= 0; --k) {                // x_k = rhs_k / u_kk; rhs_i -= u_ik x_k, i < k
-    if (tid < ncol) G[k * ld + nr + tid] = cmul(G[k * ld + nr + tid], crecip(G[k * ld + k]));
-    __syncthreads();
-    for (int idx = tid; idx < k * ncol; idx += T) {
-      const int i = idx / ncol, c = idx - (idx / ncol) * ncol;
-      G[i * ld + nr + c] = cfnma(G[i * ld + nr + c], G[i * ld + k], G[k * ld + nr + c]);
-    }
-    __syncthreads();
-  }
-  if (tid == 0) {
-    *ldet = acc.value();
-    *minre = acc.mn;
-  }
+// exp(x) P^{-1/2} for a pivots' record (product p 2^e2 with the sum of its factors' arguments), the root on the
+// sheet of that sum.
+__device__ double2 record_value(double2 p, float e2, float args, double2 x) {
+  e2 += (float)ArF64::normalise(p);
+  const int e = (int)e2, h = e >> 1;                  // e = 2 h + (e & 1)
+  const int wind = (int)rintf((args - atan2f((float)p.y, (float)p.x)) * 0.159154943f);
+  double2 v = inv_sqrt(p);
+  double s = ldexp(exp(x.x), -h) * ((e & 1) ? 0.70710678118654752440 : 1.0);
+  if (wind & 1) s = -s;
+  if (x.y == 0.0) return make_double2(v.x * s, v.y * s);
+  double sn, cs;
+  sincos(x.y, &sn, &cs);
+  return ArF64::mul(v, make_double2(s * cs, s * sn));
 }
 
-__global__ void __launch_bounds__(HT) k_herald_points(HeraldArgs a) {
+__device__ __forceinline__ void taylor_sync() { asm volatile("bar.sync 1, %0;" ::"n"(TAYLOR_THREADS) : "memory"); }
+
+__global__ void __launch_bounds__(HT) k_herald_points(HeraldArgs a, TreeArgs t) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
+  __shared__ double2 blk[(GBSBIN_HERALD_MAX_F + 1) * (GBSBIN_HERALD_MAX_F + 1)];   // [[A'_F, c'], [u', .]]
+  __shared__ double2 fin[(GBSBIN_HERALD_MAX_F + 1) * (GBSBIN_HERALD_MAX_F + 1)];
+  __shared__ double2 Mq[GBSBIN_HERALD_MAX_F * GBSBIN_HERALD_MAX_F], lq[GBSBIN_HERALD_MAX_F];
+  __shared__ double2 s_pref;
+  __shared__ PathRec<double2> s_rec;
   const long long k = blockIdx.x;
-  const int nd = a.nd, nf = a.nf, tid = threadIdx.x, T = blockDim.x;
-  const int cols = nd + nf + 1;
-  double2* G = reinterpret_cast<double2*>(sm_raw);   // nd x cols
-  double2* Mq = G + (size_t)nd * cols;                // nf x nf
-  double2* lq = Mq + nf * nf;                         // nf
-  double2* sc = lq + nf;                              // e, log det
-  double2* wg = sc + 2;                               // the heralding groups' roots at this point
-  double2* wd = wg + GBSBIN_MAX_L;                    // the root of each D row's mode
-  if (tid < a.L) {                                    // digit of group tid, w = exp(2 pi i d / R)
-    long long rest = k;
-    for (int q = a.L - 1; q > tid; --q) rest /= a.radix[q];
-    const int d = (int)(rest % a.radix[tid]);
-    int off = 0;
-    for (int q = 0; q < tid; ++q) off += a.radix[q];
-    const double2 t = a.tw[off + d];
-    wg[tid] = make_double2(t.x, -t.y);
-  }
-  __syncthreads();
-  for (int i = tid; i < nd; i += T) wd[i] = a.dgroup[i] >= 0 ? wg[a.dgroup[i]] : make_double2(1.0, 0.0);
-  __syncthreads();
-  // I - X D(w) A_DD with the right-hand sides X D(w) [A_DF | gamma_D]; row i of X D A is
-  // w_{partner(i)} A_{partner(i), .}
-  for (int idx = tid; idx < nd * cols; idx += T) {
-    const int i = idx / cols, j = idx - (idx / cols) * cols;
-    const int pi = a.dpart[i];                        // X partner of row i within D
-    const double2 w = wd[pi];
-    double2 v;
-    if (j < nd) v = cneg2(cmul(w, a.ADD[(size_t)pi * nd + j]));
-    else if (j < nd + nf) v = cmul(w, a.ADF[(size_t)pi * nf + (j - nd)]);
-    else v = cmul(w, a.gD[pi]);
-    if (j == i) v.x += 1.0;
-    G[idx] = v;
-  }
-  __syncthreads();
-  double2 ld;
-  double mn;
-  solve_block(G, nd, nf + 1, cols, &ld, &mn);
-  // M = A_FF + A_DF^T Y_F, l = gamma_F + A_DF^T y, e = gamma_D^T y / 2
-  for (int idx = tid; idx < nf * (nf + 1); idx += T) {
-    const int i = idx / (nf + 1), c = idx - (idx / (nf + 1)) * (nf + 1);
-    double2 s = c < nf ? a.AFF[i * nf + c] : a.gF[i];
-    for (int d = 0; d < nd; ++d) s = cadd2(s, cmul(a.ADF[(size_t)d * nf + i], G[d * cols + nd + c]));
-    if (c < nf) Mq[i * nf + c] = s;
-    else lq[i] = s;
-  }
-  if (tid == 0) {
-    double2 e = make_double2(0.0, 0.0);
-    for (int d = 0; d < nd; ++d) e = cadd2(e, cmul(a.gD[d], G[d * cols + nd + nf]));
-    sc[0] = make_double2(0.5 * e.x, 0.5 * e.y);
-    sc[1] = ld;
-  }
-  __syncthreads();
-  // the heralding probability's value: the kept block's Schur complement I - X_F M (X_F swaps
-  // the kept modes' halves) with the right-hand side X_F l, eliminated by one thread
-  if (tid == 0) {
-    const int h = nf / 2;
-    double2 Tm[GBSBIN_HERALD_MAX_F][GBSBIN_HERALD_MAX_F + 1];
-    for (int i = 0; i < nf; ++i) {
-      const int pi = i < h ? i + h : i - h;
-      for (int j = 0; j < nf; ++j) Tm[i][j] = cneg2(Mq[pi * nf + j]);
-      Tm[i][i].x += 1.0;
-      Tm[i][nf] = lq[pi];
+  const int nf = a.nf, f1 = nf + 1, tid = threadIdx.x;
+  if (a.L == 1) {                                     // the only group: its spectral form gives the kept block
+    double2* d = reinterpret_cast<double2*>(sm_raw);
+    double2* dB = d + t.nb[0];
+    const double2 w = root_at<ArF64>(t, 0, (int)k);
+    root_factors<ArF64>(t, w, d, dB);
+    for (int q = tid; q < f1 * f1; q += HT) {
+      const int i = q / f1, j = q - q / f1 * f1;
+      blk[q] = (i < nf && j < nf) || t.has_gamma ? root_entry<ArF64>(t, dB, i, j) : ArF64::zero();
     }
-    LogDet accf;
+    if (tid < 32) {
+      const PathRec<double2> pr = root_path<ArF64>(t, w);
+      if (tid == 0) s_rec = pr;                       // with the traced rows' exponent
+    }
+    __syncthreads();
+    if (tid == 0) s_rec.ex = ArF64::add(s_rec.ex, blk[f1 * f1 - 1]);
+  } else {
+    const Sweep<double2> w = level_sweep<ArF64, false, GBSBIN_MAX_L - 1>(t, 1, a.L - 1, k, sm_raw);
+    for (int q = tid; q < f1 * f1; q += HT) {
+      const int i = q / f1, j = q - q / f1 * f1;
+      blk[q] = (i < nf && j < nf) || t.has_gamma ? w.G[(w.nb + i) * w.cols + w.nb + j] : ArF64::zero();
+    }
+    if (tid < 32) {
+      const PathRec<double2> pr = sweep_path<ArF64, false>(t, 1, w);
+      if (tid == 0) s_rec = pr;
+    }
+  }
+  __syncthreads();
+  const PathRec<double2> rec = s_rec;
+  const int h = nf / 2;
+  for (int q = tid; q < nf * nf; q += HT) {           // M = X_F A'_F, l = u'
+    const int i = q / nf, j = q - q / nf * nf;
+    Mq[q] = blk[(i < h ? i + h : i - h) * f1 + j];
+  }
+  if (tid < nf) lq[tid] = blk[nf * f1 + tid];
+  // the coefficients in the sweep's memory (done with), or in the point's slot
+  double2* slot = a.gcoef + (size_t)k * (a.ncoef + 1);
+  double2* C = a.ncoef <= SMEM_COEF ? reinterpret_cast<double2*>(sm_raw) : slot;
+  if (tid == 0) C[0] = ArF64::one();
+  __syncthreads();
+  if (tid >= TAYLOR_THREADS) {                        // the eighth warp: the scalar factors
+    const int lane = tid & 31;
+    for (int q = lane; q < f1 * f1; q += 32) {        // [[I - A'_F, c'], [-u', 2 e]]
+      const int i = q / f1, j = q - q / f1 * f1;
+      double2 v = blk[q];
+      if (i < nf && j < nf) {
+        v = ArF64::neg(v);
+        if (i == j) v.x += 1.0;
+      } else if (i == nf) {
+        v = j == nf ? rec.ex : ArF64::neg(v);
+      }
+      fin[q] = v;
+    }
+    __syncwarp();
+    double2 prod = rec.prod;
+    float e2 = rec.meta.y, args = rec.meta.x, mn = rec.meta.z;
     for (int c = 0; c < nf; ++c) {
-      const double2 piv = Tm[c][c];
-      accf.add(piv);
-      const double2 r = crecip(piv);
-      for (int i = c + 1; i < nf; ++i) {
-        const double2 li = cmul(Tm[i][c], r);
-        for (int j = c + 1; j <= nf; ++j) Tm[i][j] = cfnma(Tm[i][j], li, Tm[c][j]);
+      const double2 piv = fin[c * f1 + c], r = ArF64::recip(piv);
+      prod = ArF64::mul(prod, piv);
+      e2 += (float)ArF64::normalise(prod);
+      args += atan2f((float)piv.y, (float)piv.x);
+      mn = fminf(mn, (float)piv.x);
+      if (!(piv.x == piv.x) || !(piv.y == piv.y)) mn = -3.0e38f;
+      const int n1 = nf - c;
+      for (int q = lane; q < n1 * n1; q += 32) {
+        const int i = c + 1 + q / n1, j = c + 1 + q - q / n1 * n1;
+        fin[i * f1 + j] = ArF64::fms(fin[i * f1 + j], ArF64::mul(fin[i * f1 + c], r), fin[c * f1 + j]);
+      }
+      __syncwarp();
+    }
+    // lane 0: exp(e) / sqrt(det); lane 1: the heralding probability's value; one pass of the same code
+    if (lane < 2) {
+      const double2 x = lane ? fin[f1 * f1 - 1] : rec.ex;
+      const double2 v = record_value(lane ? prod : rec.prod, lane ? e2 : rec.meta.y, lane ? args : rec.meta.x,
+                                     make_double2(0.5 * x.x, 0.5 * x.y));
+      if (lane) {
+        slot[a.ncoef] = v;
+        a.minpiv[k] = isfinite(v.x) && isfinite(v.y) ? (double)mn : -1.0e300;
+      } else {
+        s_pref = v;
       }
     }
-    double2 y[GBSBIN_HERALD_MAX_F];
-    for (int i = nf - 1; i >= 0; --i) {
-      double2 s = Tm[i][nf];
-      for (int j = i + 1; j < nf; ++j) s = cfnma(s, Tm[i][j], y[j]);
-      y[i] = cmul(s, crecip(Tm[i][i]));
+  } else {                                            // Taylor coefficients by shells, relative to the first
+    for (int sh = 1; sh <= nf * a.cut; ++sh) {
+      const int t1 = a.shell[sh + 1];
+      for (int e = a.shell[sh] + tid; e < t1; e += TAYLOR_THREADS) {
+        const int i0 = a.ti0[e];
+        double2 val = ArF64::mul(lq[i0], C[a.tqm[e]]);
+        const int* nb = a.tnb + (size_t)e * nf;
+        for (int j = 0; j < nf; ++j)
+          if (nb[j] >= 0) val = ArF64::fma(Mq[i0 * nf + j], C[nb[j]], val);
+        const double p = (double)a.tp[e];
+        double inv = (double)__frcp_rn((float)p);     // 1 / p: an exact small integer, two Newton steps
+        inv = fma(inv, fma(-p, inv, 1.0), inv);
+        inv = fma(inv, fma(-p, inv, 1.0), inv);
+        C[a.tq[e]] = make_double2(val.x * inv, val.y * inv);
+      }
+      taylor_sync();
     }
-    double2 ly = make_double2(0.0, 0.0);
-    for (int i = 0; i < nf; ++i) ly = cadd2(ly, cmul(lq[i], y[i]));
-    const double2 lf = accf.value();
-    const double mnf = accf.mn;
-    const double re = sc[0].x + 0.5 * ly.x - 0.5 * (ld.x + lf.x), im = sc[0].y + 0.5 * ly.y - 0.5 * (ld.y + lf.y);
-    const double m = exp(re);
-    double s, c;
-    sincos(im, &s, &c);
-    a.gcoef[(size_t)k * (a.ncoef + 1) + a.ncoef] = make_double2(m * c, m * s);
-    a.minpiv[k] = fmin(mn, mnf);
   }
-  // Taylor coefficients by shells of total degree, in this point's slot of ncoef + 1 entries
-  // (index p = sum_i p_i (c + 1)^(nf - 1 - i)), from the plan's table of neighbours
-  double2* C = a.gcoef + (size_t)k * (a.ncoef + 1);
-  const double2 e = sc[0], l0 = sc[1];
-  const double m0 = exp(e.x - 0.5 * l0.x);
-  double s0, c0;
-  sincos(e.y - 0.5 * l0.y, &s0, &c0);
-  if (tid == 0) C[0] = make_double2(m0 * c0, m0 * s0);   // exp(e) / sqrt(det) times c_0 = 1
   __syncthreads();
-  for (int shell = 1; shell <= nf * a.cut; ++shell) {
-    for (int t = a.shell[shell] + tid; t < a.shell[shell + 1]; t += T) {
-      const int i0 = a.ti0[t];
-      double2 val = cmul(lq[i0], C[a.tqm[t]]);
-      const int* nb = a.tnb + (size_t)t * nf;
-      for (int j = 0; j < nf; ++j)
-        if (nb[j] >= 0) val = cadd2(val, cmul(Mq[i0 * nf + j], C[nb[j]]));
-      const double inv = 1.0 / (double)a.tp[t];
-      C[a.tq[t]] = make_double2(val.x * inv, val.y * inv);
-    }
-    __syncthreads();
+  const double2 pref = s_pref;
+  for (long long q = tid; q < a.ncoef; q += HT) slot[q] = ArF64::mul(pref, C[q]);
+}
+
+// ------------------------------------------------------------------------------ inverse DFT
+// Sum over k < R of x_k exp(-2 pi i k b / R) from folded values at stride st: entry k holds x_k + x_{R-k} and entry
+// R - k holds x_k - x_{R-k} (0 < k < R/2); entries 0 and R/2 as they are.
+__device__ __forceinline__ double2 folded_sum(const double2* x, int st, int R, int b, const double2* __restrict__ tw) {
+  double2 acc = x[0];
+  if ((R & 1) == 0) {
+    const double2 y = x[(R / 2) * st];
+    acc = (b & 1) ? make_double2(acc.x - y.x, acc.y - y.y) : make_double2(acc.x + y.x, acc.y + y.y);
+  }
+  int idx = b;
+  for (int k = 1; 2 * k < R; ++k) {
+    const double2 s = x[k * st], d = x[(R - k) * st], w = tw[idx];   // w = (cos, -sin)
+    acc.x = fma(w.x, s.x, fma(-w.y, d.y, acc.x));
+    acc.y = fma(w.x, s.y, fma(w.y, d.x, acc.y));
+    idx += b;
+    if (idx >= R) idx -= R;
+  }
+  return acc;
+}
+
+// A finished entry of channel c (position in the list) at heralding outcome `cell`: rho and its mirror image, or
+// Pr(b).
+__device__ __forceinline__ void write_channel(const HeraldArgs& a, long long cell, int c, double2 v,
+                                              double2* __restrict__ rho, double* __restrict__ prob) {
+  const double s = a.pr0 / (double)a.npts;
+  if (c == a.nchan - 1) {
+    prob[cell] = v.x * s;
+    a.prob_own[cell] = v.x * s;
+    return;
+  }
+  const int ch = a.chan[c], u = ch / a.side, w = ch - u * a.side;
+  const double f = s * a.chscale[ch];
+  double2* r = rho + cell * a.ncoef;
+  v = make_double2(v.x * f, u == w ? 0.0 : v.y * f);
+  r[ch] = v;
+  if (u != w) r[w * a.side + u] = make_double2(v.x, -v.y);
+}
+
+// Folds R entries at stride st in place, for each of n lines (base(line)), by the whole CTA.
+template <class Base>
+__device__ __forceinline__ void fold_lines(double2* X, int n, int R, int st, Base base) {
+  const int half = (R - 1) / 2;
+  for (int q = threadIdx.x; q < n * half; q += blockDim.x) {
+    const int line = q / half, k = 1 + q - q / half * half;
+    double2* x = X + base(line);
+    const double2 p = x[k * st], m = x[(R - k) * st];
+    x[k * st] = make_double2(p.x + m.x, p.y + m.y);
+    x[(R - k) * st] = make_double2(p.x - m.x, p.y - m.y);
   }
 }
 
-// One axis of the inverse DFT over the heralding grid: out[pre][b][post][ch] = sum over
-// k < R_l of in[pre][k][post][ch] exp(-2 pi i k b / R_l), b < nout_l (pre runs over the
-// axes already transformed, extent nout; post over the later ones, extent radix; ch over the
-// ncoef Taylor coefficients and the heralding probability's value).  One thread per output
-// element, consecutive threads on consecutive channels (coalesced reads of the input).  The
-// last axis scales by Pr(0) / N (and prod sqrt(p_i!) per coefficient) and writes rho and
-// Pr(b).
-__global__ void k_herald_dft_axis(HeraldArgs a, int l, const double2* __restrict__ in, double2* __restrict__ out,
-                                  double2* __restrict__ rho, double* __restrict__ prob) {
-  const long long nch = a.ncoef + 1;
+// The first two axes: CTA = (index of the later axes, block of CB channels); in: the points' slots, out (when axes
+// follow): [b_0][b_1][later][channel].
+__global__ void __launch_bounds__(HT) k_herald_dft2(HeraldArgs a, int CB, long long later, double2* __restrict__ out,
+                                                    double2* __restrict__ rho, double* __restrict__ prob) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  const int R0 = a.radix[0], R1 = a.radix[1], n0 = a.nout[0], n1 = a.nout[1];
+  double2* X = reinterpret_cast<double2*>(sm_raw);    // [k0][k1][cb]
+  double2* Y = X + (size_t)R0 * R1 * CB;              // [k0][b1][cb]
+  const int blocks = (a.nchan + CB - 1) / CB;
+  const long long p = blockIdx.x / blocks;
+  const int c0 = (int)(blockIdx.x - p * blocks) * CB;
+  for (int q = threadIdx.x; q < R0 * R1 * CB; q += HT) {
+    const int cb = q % CB, kk = q / CB, c = c0 + cb;
+    X[q] = c < a.nchan ? a.gcoef[((long long)kk * later + p) * (a.ncoef + 1) + (c == a.nchan - 1 ? a.ncoef : a.chan[c])]
+                       : make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  fold_lines(X, R0 * CB, R1, CB, [=](int line) { return line / CB * R1 * CB + line % CB; });
+  __syncthreads();
+  for (int q = threadIdx.x; q < R0 * n1 * CB; q += HT) {
+    const int cb = q % CB, r = q / CB, b1 = r % n1, k0 = r / n1;
+    Y[q] = folded_sum(X + (size_t)k0 * R1 * CB + cb, CB, R1, b1, a.tw + R0);
+  }
+  __syncthreads();
+  fold_lines(Y, n1 * CB, R0, n1 * CB, [](int line) { return line; });
+  __syncthreads();
+  for (int q = threadIdx.x; q < n0 * n1 * CB; q += HT) {
+    const int cb = q % CB, r = q / CB, b1 = r % n1, b0 = r / n1, c = c0 + cb;
+    if (c >= a.nchan) continue;
+    const double2 v = folded_sum(Y + (size_t)b1 * CB + cb, n1 * CB, R0, b0, a.tw);
+    if (a.L == 2) write_channel(a, (long long)b0 * n1 + b1, c, v, rho, prob);
+    else out[(((long long)b0 * n1 + b1) * later + p) * a.nchan + c] = v;
+  }
+}
+
+// One axis: out[pre][b][post][c] = sum over k < R_l of in[pre][k][post][c] exp(-2 pi i k b / R_l), b < nout_l (pre
+// runs over the axes already transformed, post over the later ones, c over the channels); slots: the input is the
+// points' slots, every channel.  One thread per output element, consecutive threads on consecutive channels.
+__global__ void k_herald_dft_axis(HeraldArgs a, int l, int slots, const double2* __restrict__ in,
+                                  double2* __restrict__ out, double2* __restrict__ rho, double* __restrict__ prob) {
   long long pre = 1, post = 1;
   for (int q = 0; q < l; ++q) pre *= a.nout[q];
   for (int q = l + 1; q < a.L; ++q) post *= a.radix[q];
   const int R = a.radix[l], nb = a.nout[l];
   int off = 0;
   for (int q = 0; q < l; ++q) off += a.radix[q];
-  const bool last = l == a.L - 1;
-  const long long total = pre * nb * post * nch;
+  const long long total = pre * nb * post * a.nchan, nch = slots ? a.ncoef + 1 : a.nchan;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
     long long rest = t;
-    const long long ch = rest % nch;
-    rest /= nch;
+    const int c = (int)(rest % a.nchan);
+    rest /= a.nchan;
     const long long pi = rest % post;
     rest /= post;
     const int b = (int)(rest % nb);
     const long long pr = rest / nb;
+    const long long ch = !slots ? c : c == a.nchan - 1 ? a.ncoef : a.chan[c];
     const double2* src = in + ((pr * R) * post + pi) * nch + ch;
     const long long step = post * nch;
     double2 acc = make_double2(0.0, 0.0);
-    int idx = 0;                                     // k b mod R, advanced by b per k
+    int idx = 0;                                      // k b mod R, advanced by b per k
     for (int k = 0; k < R; ++k) {
-      acc = cadd2(acc, cmul(src[(long long)k * step], a.tw[off + idx]));
+      acc = ArF64::fma(src[(long long)k * step], a.tw[off + idx], acc);
       idx += b;
       if (idx >= R) idx -= R;
     }
-    if (!last) {
-      out[((pr * nb + b) * post + pi) * nch + ch] = acc;
-      continue;
-    }
-    const long long cell = pr * nb + b;              // post = 1 on the last axis
-    const double s = a.pr0 / (double)a.npts;
-    if (ch < a.ncoef) {
-      const double f = s * a.chscale[ch];
-      rho[cell * a.ncoef + ch] = make_double2(acc.x * f, acc.y * f);
-    } else {
-      prob[cell] = acc.x * s;
-      a.prob_own[cell] = acc.x * s;
-    }
+    if (l + 1 < a.L) out[((pr * nb + b) * post + pi) * a.nchan + c] = acc;
+    else write_channel(a, pr * nb + b, c, acc, rho, prob);   // post = 1 on the last axis
   }
 }
 
 }  // namespace
 
-size_t herald_smem_bytes(int nd, int nf, int n2) {
-  (void)n2;
-  return sizeof(double2) * ((size_t)nd * (nd + nf + 1) + (size_t)nf * nf + nf + 2 + GBSBIN_MAX_L + nd);
+size_t herald_sweep_smem(int L, int nb0, int m1) {
+  if (L == 1) return sizeof(double2) * (size_t)nb0 * (m1 + 2);
+  return tree_level_smem_bytes(m1, m1);
 }
 
-cudaError_t launch_herald(const HeraldArgs& a, double2* out, double* prob, cudaStream_t s) {
-  const size_t smem = herald_smem_bytes(a.nd, a.nf, a.n2);
+cudaError_t launch_herald(const HeraldArgs& a, const TreeArgs& t, int num_sms, double2* out, double* prob,
+                          cudaStream_t s, int* launches) {
   cudaError_t err = cudaSuccess;
-  if (smem > 48 * 1024) {
-    err = cudaFuncSetAttribute(k_herald_points, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
+  *launches = 0;
+  if (a.L > 1) {
+    if ((err = launch_tree_root_fp64(t, num_sms, s)) != cudaSuccess) return err;
+    ++*launches;
   }
-  k_herald_points<<<(unsigned)a.npts, HT, smem, s>>>(a);
+  const size_t sweep = herald_sweep_smem(a.L, t.nb[0], t.m[1]);
+  const size_t coef = a.ncoef <= SMEM_COEF ? sizeof(double2) * (size_t)a.ncoef : 0, smem = sweep > coef ? sweep : coef;
+  if (smem > 32 * 1024 &&
+      (err = cudaFuncSetAttribute(k_herald_points, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    return err;
+  k_herald_points<<<(unsigned)a.npts, HT, smem, s>>>(a, t);
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
-  // axis by axis, ping-pong between the coefficient slots and the scratch buffer (each
-  // output is at most as large as its input)
-  const long long nch = a.ncoef + 1;
+  ++*launches;
+  int l = 0;
   long long pre = 1;
   const double2* in = a.gcoef;
-  for (int l = 0; l < a.L; ++l) {
+  if (a.L > 1) {                                      // two axes at once where a block of channels fits 96 KB
+    const long long cell = (long long)a.radix[0] * (a.radix[1] + a.nout[1]);
+    const int CB = (int)(cell < 6144 ? 6144 / cell : 0);
+    if (CB >= 1) {
+      const int cb = CB > 8 ? 8 : CB;
+      long long later = 1;
+      for (int q = 2; q < a.L; ++q) later *= a.radix[q];
+      const size_t sm = sizeof(double2) * (size_t)cell * cb;
+      if (sm > 48 * 1024 &&
+          (err = cudaFuncSetAttribute(k_herald_dft2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
+        return err;
+      const long long blocks = later * ((a.nchan + cb - 1) / cb);
+      k_herald_dft2<<<(unsigned)blocks, HT, sm, s>>>(a, cb, later, a.scratch, out, prob);
+      if ((err = cudaGetLastError()) != cudaSuccess) return err;
+      ++*launches;
+      in = a.scratch;
+      pre = (long long)a.nout[0] * a.nout[1];
+      l = 2;
+    }
+  }
+  // the other axes one by one, ping-pong between the slots and the scratch buffer (each output is at most as
+  // large as its input)
+  for (; l < a.L; ++l) {
     long long post = 1;
     for (int q = l + 1; q < a.L; ++q) post *= a.radix[q];
-    const long long work = pre * a.nout[l] * post * nch;
+    const long long work = pre * a.nout[l] * post * a.nchan;
     long long blocks = (work + 255) / 256;
     if (blocks > 65535) blocks = 65535;
     double2* o = (in == a.gcoef) ? a.scratch : a.gcoef;
-    k_herald_dft_axis<<<(unsigned)blocks, 256, 0, s>>>(a, l, in, o, out, prob);
+    k_herald_dft_axis<<<(unsigned)blocks, 256, 0, s>>>(a, l, l == 0 ? 1 : 0, in, o, out, prob);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    ++*launches;
     in = o;
     pre *= a.nout[l];
   }

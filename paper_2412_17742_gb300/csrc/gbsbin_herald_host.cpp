@@ -19,10 +19,13 @@ struct gbsbin_herald_plan {
   int n2 = 0;
   long long table_size = 0;              // complex elements of rho
   bool executed = false;
+  int last_launches = 0, num_sms = 0;
+  TreeArgs tree{};                       // the heralding groups' levels
+  double2* d_depth1 = nullptr;           // depth 1: matrices, vectors, path records
   double logq1_re = 0.0;
   size_t upload_bytes = 0;
   // device
-  unsigned char* d_const = nullptr;      // role, dpart, dmode, tw, blocks, chscale
+  unsigned char* d_const = nullptr;      // tree inputs, tw, chscale, channel and Taylor tables
   double2* d_gcoef = nullptr;
   double2* d_scratch = nullptr;
   double* d_minpiv = nullptr;
@@ -47,7 +50,7 @@ int dalloc(T** p, size_t count) {
 }
 
 void free_all(gbsbin_herald_plan* P) {
-  void* ptrs[] = {P->d_const, P->d_gcoef, P->d_scratch, P->d_minpiv, P->d_prob, P->d_rho_tmp, P->d_prob_tmp};
+  void* ptrs[] = {P->d_const, P->d_gcoef, P->d_scratch, P->d_minpiv, P->d_prob, P->d_rho_tmp, P->d_prob_tmp, P->d_depth1};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   if (P->ev0) cudaEventDestroy(P->ev0);
@@ -102,7 +105,7 @@ int gbsbin_herald_plan_create(const gbsbin_herald_problem* p, const gbsbin_optio
     if (cnt[l] == 0) return GBSBIN_ERR_PARTITION;
   const int nk = (int)kept.size();
   if (nk < 1 || nk > GBSBIN_HERALD_MAX_KEPT) return GBSBIN_ERR_UNSUPPORTED;
-  const int nf = 2 * nk, nd = 2 * (int)Dm.size(), cut = p->fock_cutoff;
+  const int nf = 2 * nk, cut = p->fock_cutoff;
   long long ncoef = 1;
   for (int i = 0; i < nf; ++i) {
     ncoef *= cut + 1;
@@ -110,9 +113,7 @@ int gbsbin_herald_plan_create(const gbsbin_herald_problem* p, const gbsbin_optio
   }
   HeraldArgs a{};
   a.L = L;
-  a.nd = nd;
   a.nf = nf;
-  a.n2 = n2;
   a.cut = cut;
   a.ncoef = ncoef;
   a.npts = 1;
@@ -134,33 +135,92 @@ int gbsbin_herald_plan_create(const gbsbin_herald_problem* p, const gbsbin_optio
   std::vector<cd> XA, gamma, Xgamma;
   int st = host_state(s, n2, XA, gamma, Xgamma);
   if (st) return st;
-  // A = X XA: row i of A is row partner(i) of XA
-  std::vector<cd> A((size_t)n2 * n2);
+  // row order: traced modes, the heralding groups, the kept modes; each set's annihilation rows, then its
+  // creation rows.  The traced rows are eliminated here (w = 1): the same augmented form as the tree's levels,
+  // [[I - A_TT, A_T., c_T], [-A_.T, A_.., c_.], [-u_T, u_., 0]], whose trailing block is the traced-out state's
+  std::vector<int> order;
+  TreeArgs t{};
+  auto add_role = [&](int role) {
+    const size_t before = order.size();
+    for (int half = 0; half < 2; ++half)
+      for (int m = 0; m < nm; ++m)
+        if (p->role[m] == role) order.push_back(m + half * nm);
+    return (int)(order.size() - before);
+  };
+  const int nt = add_role(GBSBIN_HERALD_TRACED), nr = n2 - nt, W = n2 + 1;
+  for (int l = 0; l < L; ++l) t.nb[l] = add_role(l);
+  add_role(GBSBIN_HERALD_KEPT);
+  int rem = nr;
+  for (int l = 0; l < L; ++l) {
+    t.m[l] = rem;
+    rem -= t.nb[l];
+  }
+  if (L == 1) t.m[1] = nf;
+  std::vector<cd> Z((size_t)W * W, cd(0.0));
   for (int i = 0; i < n2; ++i) {
-    const int pi = i < nm ? i + nm : i - nm;
-    for (int j = 0; j < n2; ++j) A[(size_t)i * n2 + j] = XA[(size_t)pi * n2 + j];
+    for (int j = 0; j < n2; ++j) {
+      const cd v = XA[(size_t)order[i] * n2 + order[j]];
+      Z[(size_t)i * W + j] = j < nt ? (i == j ? 1.0 : 0.0) - v : v;
+      if (i < nt && j >= nt) Z[(size_t)i * W + j] = v;
+      if (i >= nt && j < nt) Z[(size_t)i * W + j] = -v;
+    }
+    Z[(size_t)i * W + n2] = Xgamma[order[i]];
+    Z[(size_t)n2 * W + i] = i < nt ? -gamma[order[i]] : gamma[order[i]];
   }
-  std::vector<int> D, F;
-  for (int m : Dm) D.push_back(m);
-  for (int m : Dm) D.push_back(m + nm);
-  for (int m : kept) F.push_back(m);
-  for (int m : kept) F.push_back(m + nm);
-  std::vector<cd> ADD((size_t)nd * nd), ADF((size_t)nd * nf), AFF((size_t)nf * nf), gD(nd), gF(nf);
-  for (int i = 0; i < nd; ++i) {
-    for (int j = 0; j < nd; ++j) ADD[(size_t)i * nd + j] = A[(size_t)D[i] * n2 + D[j]];
-    for (int j = 0; j < nf; ++j) ADF[(size_t)i * nf + j] = A[(size_t)D[i] * n2 + F[j]];
-    gD[i] = gamma[D[i]];
+  cd tprod = 1.0;
+  double targ = 0.0, tmin = 3.0e38;
+  int te2 = 0;
+  for (int k = 0; k < nt; ++k) {
+    const cd piv = Z[(size_t)k * W + k];
+    tprod *= piv;
+    int ex;
+    std::frexp(std::max(std::fabs(tprod.real()), std::fabs(tprod.imag())), &ex);
+    tprod = cd(std::ldexp(tprod.real(), -ex), std::ldexp(tprod.imag(), -ex));
+    te2 += ex;
+    targ += std::atan2(piv.imag(), piv.real());
+    tmin = std::min(tmin, piv.real());
+    for (int i = k + 1; i < W; ++i) {
+      const cd f = Z[(size_t)i * W + k] / piv;
+      if (f == cd(0.0)) continue;
+      for (int j = k + 1; j < W; ++j) Z[(size_t)i * W + j] -= f * Z[(size_t)k * W + j];
+    }
   }
-  for (int i = 0; i < nf; ++i) {
-    for (int j = 0; j < nf; ++j) AFF[(size_t)i * nf + j] = A[(size_t)F[i] * n2 + F[j]];
-    gF[i] = gamma[F[i]];
+  std::vector<cd> A0((size_t)nr * nr), c0(nr), u0(nr);
+  for (int i = 0; i < nr; ++i) {                     // Hermitian up to rounding: made exactly so
+    for (int j = 0; j < nr; ++j)
+      A0[(size_t)i * nr + j] = 0.5 * (Z[(size_t)(nt + i) * W + nt + j] + std::conj(Z[(size_t)(nt + j) * W + nt + i]));
+    c0[i] = Z[(size_t)(nt + i) * W + n2];
+    u0[i] = Z[(size_t)n2 * W + nt + i];
   }
-  std::vector<int> dpart(nd), dgroup(nd);
-  const int hd = nd / 2;
-  for (int i = 0; i < nd; ++i) {
-    dpart[i] = i < hd ? i + hd : i - hd;
-    dgroup[i] = p->role[Dm[i % hd]] >= 0 ? p->role[Dm[i % hd]] : -1;
+  for (int i = 0; i < n2; ++i)
+    if (gamma[i] != cd(0.0)) t.has_gamma = 1;
+  // the first group's spectral form
+  const int nb0 = t.nb[0], rest = nr - nb0;
+  std::vector<cd> A00((size_t)nb0 * nb0), rlam(nb0), rB((size_t)nb0 * (rest + 1)), ru(nb0);
+  {
+    std::vector<std::vector<cd>> col(rest + 2, std::vector<cd>(nb0));
+    std::vector<std::vector<cd>*> vecs;
+    for (int i = 0; i < nb0; ++i) {
+      for (int j = 0; j < nb0; ++j) A00[(size_t)i * nb0 + j] = A0[(size_t)i * nr + j];
+      for (int j = 0; j < rest; ++j) col[j][i] = A0[(size_t)i * nr + nb0 + j];
+      col[rest][i] = c0[i];
+      col[rest + 1][i] = std::conj(u0[i]);
+    }
+    for (auto& v : col) vecs.push_back(&v);
+    std::vector<double> ev;
+    if (!hermitian_spectrum(A00, nb0, ev, vecs)) return GBSBIN_ERR_NUMERIC;
+    for (int k = 0; k < nb0; ++k) {
+      rlam[k] = ev[k];
+      for (int j = 0; j <= rest; ++j) rB[(size_t)k * (rest + 1) + j] = col[j][k];
+      ru[k] = std::conj(col[rest + 1][k]);
+    }
   }
+  struct {
+    double2 prod;
+    float4 meta;
+    double2 ex;
+  } path0 = {make_double2(tprod.real(), tprod.imag()), make_float4((float)targ, (float)te2, (float)tmin, 0.f),
+             make_double2(Z[(size_t)n2 * W + n2].real(), Z[(size_t)n2 * W + n2].imag())};
   // the Taylor coefficients in order of total degree, each with its predecessor p - e_i0 (i0
   // its first non-zero digit) and that predecessor's neighbours p - e_i0 - e_j
   const int cp1 = cut + 1, nsh = nf * cut;
@@ -204,6 +264,13 @@ int gbsbin_herald_plan_create(const gbsbin_herald_problem* p, const gbsbin_optio
       const cd v = std::polar(1.0, -TWO_PI * (double)d / (double)a.radix[l]);
       tw[off + d] = make_double2(v.real(), v.imag());
     }
+  // the channels (u, v) with u <= v
+  a.side = 1;
+  for (int i = 0; i < nk; ++i) a.side *= cp1;
+  std::vector<int> chan;
+  for (int u = 0; u < a.side; ++u)
+    for (int v = u; v < a.side; ++v) chan.push_back(u * a.side + v);
+  a.nchan = (int)chan.size() + 1;
   std::vector<double> fs(cut + 1), chs((size_t)ncoef);
   fs[0] = 1.0;
   for (int i = 1; i <= cut; ++i) fs[i] = fs[i - 1] * std::sqrt((double)i);   // sqrt(i!)
@@ -222,16 +289,14 @@ int gbsbin_herald_plan_create(const gbsbin_herald_problem* p, const gbsbin_optio
   a.pr0 = std::exp(-lq1.real());
 
   Blob b;
-  const size_t o_dgroup = b.put(dgroup.data(), dgroup.size() * sizeof(int));
-  const size_t o_dpart = b.put(dpart.data(), dpart.size() * sizeof(int));
   const size_t o_tw = b.put(tw.data(), tw.size() * sizeof(double2));
-  const std::vector<double2> vADD = to_d2(ADD), vADF = to_d2(ADF), vAFF = to_d2(AFF), vgD = to_d2(gD),
-                             vgF = to_d2(gF);
-  const size_t o_ADD = b.put(vADD.data(), vADD.size() * sizeof(double2));
-  const size_t o_ADF = b.put(vADF.data(), vADF.size() * sizeof(double2));
-  const size_t o_AFF = b.put(vAFF.data(), vAFF.size() * sizeof(double2));
-  const size_t o_gD = b.put(vgD.data(), vgD.size() * sizeof(double2));
-  const size_t o_gF = b.put(vgF.data(), vgF.size() * sizeof(double2));
+  auto put_d2 = [&b](const std::vector<cd>& v) {
+    const std::vector<double2> d = to_d2(v);
+    return b.put(d.data(), d.size() * sizeof(double2));
+  };
+  const size_t o_A0 = put_d2(A0), o_c0 = put_d2(c0), o_u0 = put_d2(u0), o_rlam = put_d2(rlam), o_rB = put_d2(rB),
+               o_ru = put_d2(ru), o_path = b.put(&path0, sizeof(path0));
+  const size_t o_chan = b.put(chan.data(), chan.size() * sizeof(int));
   const size_t o_chs = b.put(chs.data(), chs.size() * sizeof(double));
   const size_t o_shell = b.put(shell.data(), shell.size() * sizeof(int));
   const size_t o_tq = b.put(tq.data(), tq.size() * sizeof(int));
@@ -249,12 +314,16 @@ int gbsbin_herald_plan_create(const gbsbin_herald_problem* p, const gbsbin_optio
   P->upload_bytes = b.bytes.size();
   if ((st = dalloc(&P->d_const, b.bytes.size())) || (st = dalloc(&P->d_gcoef, (size_t)(a.npts * (ncoef + 1)))) ||
       (st = dalloc(&P->d_scratch, (size_t)(a.npts * (ncoef + 1)))) || (st = dalloc(&P->d_minpiv, (size_t)a.npts)) ||
-      (st = dalloc(&P->d_prob, (size_t)a.table))) {
+      (st = dalloc(&P->d_prob, (size_t)a.table)) ||
+      (st = dalloc(&P->d_depth1, L > 1 ? (size_t)a.radix[0] * ((size_t)t.m[1] * (t.m[1] + 2) + 3) : 0))) {
     free_all(P);
     delete P;
     return st;
   }
-  if (cudaMemcpy(P->d_const, b.bytes.data(), b.bytes.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+  int device = 0;
+  if (cudaGetDevice(&device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&P->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+      cudaMemcpy(P->d_const, b.bytes.data(), b.bytes.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemset(P->d_prob, 0, (size_t)a.table * sizeof(double)) != cudaSuccess ||
       (opt.want_timing && (cudaEventCreate(&P->ev0) != cudaSuccess || cudaEventCreate(&P->ev1) != cudaSuccess))) {
     cudaGetLastError();
@@ -263,14 +332,27 @@ int gbsbin_herald_plan_create(const gbsbin_herald_problem* p, const gbsbin_optio
     return GBSBIN_ERR_CUDA;
   }
   unsigned char* c = P->d_const;
-  a.dgroup = reinterpret_cast<const int*>(c + o_dgroup);
-  a.dpart = reinterpret_cast<const int*>(c + o_dpart);
   a.tw = reinterpret_cast<const double2*>(c + o_tw);
-  a.ADD = reinterpret_cast<const double2*>(c + o_ADD);
-  a.ADF = reinterpret_cast<const double2*>(c + o_ADF);
-  a.AFF = reinterpret_cast<const double2*>(c + o_AFF);
-  a.gD = reinterpret_cast<const double2*>(c + o_gD);
-  a.gF = reinterpret_cast<const double2*>(c + o_gF);
+  a.chan = reinterpret_cast<const int*>(c + o_chan);
+  t.A[0] = reinterpret_cast<float4*>(c + o_A0);
+  t.c[0] = reinterpret_cast<float4*>(c + o_c0);
+  t.u[0] = reinterpret_cast<float4*>(c + o_u0);
+  t.path[0] = reinterpret_cast<float4*>(c + o_path);
+  t.rlam = reinterpret_cast<const float4*>(c + o_rlam);
+  t.rB = reinterpret_cast<const float4*>(c + o_rB);
+  t.ru = reinterpret_cast<const float4*>(c + o_ru);
+  t.tw = a.tw;
+  t.grid.L = L;
+  for (int l = 0; l < L; ++l) t.grid.radix[l] = a.radix[l];
+  if (L > 1) {
+    float4* q = reinterpret_cast<float4*>(P->d_depth1);
+    const size_t R0 = (size_t)a.radix[0], m1 = (size_t)t.m[1];
+    t.A[1] = q;
+    t.c[1] = t.A[1] + R0 * m1 * m1;
+    t.u[1] = t.c[1] + R0 * m1;
+    t.path[1] = t.u[1] + R0 * m1;
+  }
+  P->tree = t;
   a.chscale = reinterpret_cast<const double*>(c + o_chs);
   a.shell = reinterpret_cast<const int*>(c + o_shell);
   a.tq = reinterpret_cast<const int*>(c + o_tq);
@@ -295,7 +377,7 @@ int gbsbin_herald_execute(gbsbin_herald_plan* P, gbsbin_complex* rho_out, double
   if (!P || !rho_out || !prob_out) return GBSBIN_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   if (P->ev0 && cudaEventRecord(P->ev0, s) != cudaSuccess) return GBSBIN_ERR_CUDA;
-  if (launch_herald(P->args, reinterpret_cast<double2*>(rho_out), prob_out, s) != cudaSuccess) {
+  if (launch_herald(P->args, P->tree, P->num_sms, reinterpret_cast<double2*>(rho_out), prob_out, s, &P->last_launches) != cudaSuccess) {
     cudaGetLastError();
     return GBSBIN_ERR_CUDA;
   }
@@ -353,7 +435,7 @@ int gbsbin_herald_diagnostics(gbsbin_herald_plan* P, gbsbin_diag* out, void* str
   out->log_q1_re = P->logq1_re;
   out->point_kernel_ms = 0.0;
   out->state_upload_bytes = (long long)P->upload_bytes;
-  out->launches = P->executed ? 1 + a.L : 0;
+  out->launches = P->last_launches;
   if (P->ev1 && P->executed) {
     float ms = 0.f;
     if (cudaEventSynchronize(P->ev1) != cudaSuccess || cudaEventElapsedTime(&ms, P->ev0, P->ev1) != cudaSuccess) {

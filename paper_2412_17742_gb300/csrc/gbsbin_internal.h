@@ -231,6 +231,8 @@ cudaError_t launch_points_btree(const BTreeArgs& a, const BTreeStep* steps, int 
                                 cudaStream_t s, int* launches);
 size_t tree_level_smem_bytes(int nb, int m);
 int tree_leaf_threads(int n);   // lanes per leaf (0: no kernel for a last group of n rows)
+// The first level alone (FP64), from the spectral form: depth 1's matrices, vectors and path records.
+cudaError_t launch_tree_root_fp64(const TreeArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_points_tree(const TreeArgs& a, bool fp64, int num_sms, cudaStream_t s, int* launches);
 
 // Fock inputs through a lossy circuit (gbsbin_fock.cu).  nin occupied inputs in position
