@@ -60,7 +60,7 @@ struct gbsbin_plan {
   // d_state, the other depths, sub-step scratch and Hessenberg leaves in d_tree
   BTreeArgs btree{};
   std::vector<BTreeStep> btree_steps;
-  size_t bt_scratch[3] = {0, 0, 0};   // 16-byte slots: each trailing-block buffer, pivot rows, reciprocals
+  size_t bt_scratch[2] = {0, 0};      // 16-byte slots: each trailing-block buffer, pivot rows
   cd logq1 = 0.0;                     // sharded large-matrix tree plans: log q(1) of the state (host FP64)
   double logq1_minpiv = 1.0;          // and the smallest real part of its pivots
   int last_launches = 0;              // kernel launches of the last execute
@@ -900,7 +900,7 @@ size_t btree_configure(gbsbin_plan* P, int halve_first, const int* nb, const int
   t.n_leaves = 1;
   for (int l = 0; l < L; ++l) t.n_leaves *= t.cnt[l];
   P->btree_steps.clear();
-  size_t bytes = 0, tmp_max = 0, u_max = 0, inv_max = 0;
+  size_t bytes = 0, tmp_max = 0, u_max = 0;
   long long nodes = 1;
   for (int l = 0; l + 1 < L; ++l) {
     const long long children = nodes * t.cnt[l];
@@ -918,7 +918,6 @@ size_t btree_configure(gbsbin_plan* P, int halve_first, const int* nb, const int
       st.D = D;
       P->btree_steps.push_back(st);
       u_max = std::max(u_max, (size_t)children * st.nbs * D);
-      inv_max = std::max(inv_max, (size_t)children * st.nbs);
       D -= st.nbs;
       if (p0 + st.nbs < nb[l]) tmp_max = std::max(tmp_max, (size_t)children * D * D);
     }
@@ -928,8 +927,7 @@ size_t btree_configure(gbsbin_plan* P, int halve_first, const int* nb, const int
   const size_t hslots = (size_t)nodes * ((size_t)t.mL * t.mL + 2 * (size_t)t.mL + 1);
   P->bt_scratch[0] = tmp_max;
   P->bt_scratch[1] = u_max;
-  P->bt_scratch[2] = inv_max;
-  return bytes + 2 * tmp_max + u_max + inv_max + hslots;
+  return bytes + 2 * tmp_max + u_max + hslots;
 }
 
 // Large-matrix tree plans: rows ordered by group (as for kernels 11 and 12), each level's
@@ -998,13 +996,11 @@ void btree_pointers(gbsbin_plan* P, const Stage& sl) {
     t.path[l + 1] = q;
     q += 2 * (size_t)nodes;
   }
-  const size_t tmp_max = P->bt_scratch[0], u_max = P->bt_scratch[1], inv_max = P->bt_scratch[2];
+  const size_t tmp_max = P->bt_scratch[0], u_max = P->bt_scratch[1];
   float4* tmp[2] = {q, q + tmp_max};
   q += 2 * tmp_max;
   t.U = q;
   q += u_max;
-  t.inv = q;
-  q += inv_max;
   t.H = q;
   q += (size_t)nodes * t.mL * t.mL;
   t.hv = q;

@@ -218,8 +218,7 @@ struct BTreeArgs {
   const float4* twdf;
   float4* mat[GBSBIN_MAX_L];
   float4* path[GBSBIN_MAX_L];
-  float4* U;                // per child of the current sub-step: nbs x D pivot rows
-  float4* inv;              // per child: nbs reciprocal pivots
+  float4* U;                // per child of the current sub-step: nbs x D pivot rows, right of each pivot divided by it
   float4* H;                // per leaf parent: mL x mL Hessenberg form
   float4* hv;               // per leaf parent: a = Q^T u (mL), b = Q^H c (mL), the exponent so far
   double* ldfin;

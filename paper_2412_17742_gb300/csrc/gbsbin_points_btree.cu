@@ -25,7 +25,7 @@
 // A level runs in sub-steps of nbs pivots (as many as fit in shared memory), each in two
 // launches:
 //   top:    one CTA per child eliminates the nbs pivot rows among themselves in shared
-//           memory (one barrier per step) and writes them with their reciprocal pivots; one
+//           memory (one barrier per step) and writes them divided by their pivots; one
 //           warp folds the pivots into the child's path record;
 //   bottom: several CTAs per child stage those pivot rows in shared memory and stream the
 //           other rows through registers (a warp per row: lane t holds columns t + 32 s),
@@ -169,10 +169,13 @@ __device__ __forceinline__ const typename Ar::E* step_input(const BTreeArgs& a, 
 // CTA (child, part): the nbs pivot rows in shared memory - their first nbs columns (the pivot
 // block) and the part's share of the columns right of it (every column when parts = 1; the
 // parts split the right-hand columns when a level has few children, each redoing the pivot
-// block) - and their forward elimination among themselves.  Step kk: every warp forms
-// 1 / u_kk and the multipliers of its own rows (column kk and row kk are not written in step
-// kk), then updates its rows right of kk; one barrier per step.  Part 0 also writes the pivot
-// block, the reciprocal pivots and the child's path record.
+// block) - and their forward elimination among themselves.  The multipliers run one step ahead: in step
+// kk warp 0 updates column kk + 1 and forms pivot kk + 1's reciprocal and the next multipliers into the
+// other buffer, while the other warps update the columns right of it; one barrier per step.  (Every warp
+// forming the reciprocal and its rows' multipliers itself took a fifth of the launch's issue slots: 11
+// children of 64 pivots 104 us, 231 of them 284; now 88 and 252.)  The rows are written divided by their
+// pivots, so that the bottom rows' multipliers need no product of their own.  Part 0 also writes the pivot block and
+// the child's path record.
 template <class Ar>
 __global__ void __launch_bounds__(TOP_THREADS) k_bt_top(BTreeArgs a, BTreeStep st, int parts, int W) {
   using E = typename Ar::E;
@@ -197,26 +200,44 @@ __global__ void __launch_bounds__(TOP_THREADS) k_bt_top(BTreeArgs a, BTreeStep s
     U[idx] = v;
   }
   __syncthreads();
+  E* Lm = pinv + nbs;                                // 2 x nbs: multipliers, this step's and the next's
+  if (warp == 0) {                                   // pivot 0
+    const E r = Ar::recip(U[0]);
+    if (lane == 0) pinv[0] = r;
+    for (int i = 1 + lane; i < nbs; i += 32) Lm[i] = Ar::mul(U[(size_t)i * Dl], r);
+  }
+  __syncthreads();
   for (int kk = 0; kk < nbs; ++kk) {
     const E* Uk = U + (size_t)kk * Dl;
-    const E r = Ar::recip(Uk[kk]);
-    if (tid == 0) pinv[kk] = r;
-    for (int i = kk + 1 + warp; i < nbs; i += NW) {
-      E* Ui = U + (size_t)i * Dl;
-      const E li = Ar::mul(Ui[kk], r);
-      for (int j = kk + 1 + lane; j < Dl; j += 32) Ui[j] = Ar::fms(Ui[j], li, Uk[j]);
+    const E* Lc = Lm + (kk & 1) * nbs;
+    const int s1 = kk + 1;
+    if (warp == 0) {
+      if (s1 < Dl)
+        for (int i = s1 + lane; i < nbs; i += 32) U[(size_t)i * Dl + s1] = Ar::fms(U[(size_t)i * Dl + s1], Lc[i], Uk[s1]);
+      if (s1 < nbs) {
+        __syncwarp();
+        const E r = Ar::recip(U[(size_t)s1 * Dl + s1]);
+        if (lane == 0) pinv[s1] = r;
+        E* Ln = Lm + (s1 & 1) * nbs;
+        for (int i = s1 + 1 + lane; i < nbs; i += 32) Ln[i] = Ar::mul(U[(size_t)i * Dl + s1], r);
+      }
+    } else {
+      for (int i = s1 + warp - 1; i < nbs; i += NW - 1) {
+        E* Ui = U + (size_t)i * Dl;
+        const E li = Lc[i];
+        for (int j = s1 + 1 + lane; j < Dl; j += 32) Ui[j] = Ar::fms(Ui[j], li, Uk[j]);
+      }
     }
     __syncthreads();
   }
   E* Ug = elem<Ar>(a.U) + child * (long long)nbs * D;
   for (int idx = tid; idx < nbs * Dl; idx += T) {
     const int i = idx / Dl, c = idx - i * Dl;
-    if (c >= nbs) Ug[(long long)i * D + c0 + (c - nbs)] = U[idx];
-    else if (part == 0) Ug[(long long)i * D + c] = U[idx];
+    const E v = c > i ? Ar::mul(pinv[i], U[idx]) : U[idx];   // row i divided by its pivot
+    if (c >= nbs) Ug[(long long)i * D + c0 + (c - nbs)] = v;
+    else if (part == 0) Ug[(long long)i * D + c] = v;
   }
   if (part != 0) return;
-  E* pg = elem<Ar>(a.inv) + child * (long long)nbs;
-  for (int k = tid; k < nbs; k += T) pg[k] = pinv[k];
   if (warp == 0) {
     const BRec<E> in = st.first ? *rec_at<Ar>(a.path[st.l], parent) : *rec_at<Ar>(a.path[st.l + 1], child);
     const BRec<E> out = fold_pivots<Ar>(in, nbs, [&](int k) { return U[(size_t)k * Dl + k]; });
@@ -227,10 +248,10 @@ __global__ void __launch_bounds__(TOP_THREADS) k_bt_top(BTreeArgs a, BTreeStep s
 // ---------------------------------------------------------------------------- bottom
 // The other rows of every child, D - nbs per child, taken as one sequence (child-major) and
 // split evenly over the CTAs (one per resident slot): a CTA walks its share child by child,
-// staging each child's nbs pivot rows and reciprocals in shared memory.  A warp per row: the
+// staging each child's nbs pivot rows, divided by their pivots, in shared memory.  A warp per row: the
 // row's first Dm columns in registers (lane t: columns t + 32 s), eliminated against pivot
-// rows 0 .. nbs - 1 in order (the multiplier is the row's current entry kk, broadcast from
-// its lane; lane kk mod 32 keeps it), then the trailing part (columns nbs ..) written as row
+// rows 0 .. nbs - 1 in order (with the rows divided the multiplier is the row's current entry kk itself,
+// broadcast from its lane; lane kk mod 32 keeps it), then the trailing part (columns nbs ..) written as row
 // - nbs of the output.  Columns Dm .. D - 1 (a short tail, such as the augmented column when
 // D = 32 s + 1) need no register slot: each is its initial value minus the dot product of the
 // kept multipliers with the pivot rows' entries, summed over the lanes by a fixed butterfly.
@@ -241,7 +262,6 @@ __global__ void __launch_bounds__(BOT_WARPS * 32) k_bt_bottom(BTreeArgs a, BTree
   extern __shared__ __align__(16) unsigned char sm_raw[];
   const int D = st.D, nbs = st.nbs, Do = D - nbs, S = (Dm + 31) >> 5;
   E* U = reinterpret_cast<E*>(sm_raw);
-  E* pinv = U + (size_t)nbs * D;
   const int R = a.cnt[st.l];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long g0 = rows_total * blockIdx.x / gridDim.x, g1 = rows_total * (blockIdx.x + 1) / gridDim.x;
@@ -253,10 +273,8 @@ __global__ void __launch_bounds__(BOT_WARPS * 32) k_bt_bottom(BTreeArgs a, BTree
     const E* src = step_input<Ar>(a, st, child, parent);
     E* dst = elem<Ar>(st.out) + child * (long long)Do * Do;
     const E* Ug = elem<Ar>(a.U) + child * (long long)nbs * D;
-    const E* pg = elem<Ar>(a.inv) + child * (long long)nbs;
     __syncthreads();                                 // the previous child's rows are done
     for (int idx = tid; idx < nbs * D; idx += blockDim.x) U[idx] = Ug[idx];
-    for (int k = tid; k < nbs; k += blockDim.x) pinv[k] = pg[k];
     __syncthreads();
     for (long long gr = gs + warp; gr < ge; gr += BOT_WARPS) {
       const int i = nbs + (int)(gr - child * Do);
@@ -280,8 +298,7 @@ __global__ void __launch_bounds__(BOT_WARPS * 32) k_bt_bottom(BTreeArgs a, BTree
         const int kend = min(32, nbs - 32 * sb);
         for (int il = 0; il < kend; ++il) {
           const int kk = 32 * sb + il;
-          const E x = shfl(r[sb], il);
-          const E li = Ar::mul(x, pinv[kk]);
+          const E li = shfl(r[sb], il);
           if (sb < LMS && lane == il) lm[sb < LMS ? sb : 0] = li;
           const E* Uk = U + (size_t)kk * D;
 #pragma unroll
@@ -354,6 +371,11 @@ __device__ __forceinline__ void reflector<ArF64>(double2 nrm2, double2 x0, doubl
 }
 
 // ------------------------------------------------------------------------- Hessenberg
+// floor(idx / w) from the reciprocal of w: for idx < 2^16 and w < 256 the product errs by under 256 x 2^-22, and
+// (idx + 1/2) / w lies 1 / (2 w) from an integer.  (An integer division per updated entry was a quarter of the
+// reduction: 231 nodes of 64 rows 516 us, now 489.)
+__device__ __forceinline__ int row_of(int idx, float rw) { return (int)(((float)idx + 0.5f) * rw); }
+
 // One CTA per leaf parent: the m x m block A_L with c and conj(u) as two extra columns in
 // shared memory (row stride m + 3, odd in 16-byte units), or, for GM (m above
 // GBSBIN_BT_MAX_HESS), A_L in the node's slot of the Hessenberg buffer H (row stride m, read and
@@ -438,8 +460,9 @@ __global__ void __launch_bounds__(HESS_THREADS) k_bt_hess(BTreeArgs a) {
       }
       __syncthreads();
       const int wl = m + 2 - (k + 1);
+      const float rwl = 1.0f / (float)wl;
       for (int idx = tid; idx < (m - k - 1) * wl; idx += T) {
-        const int i = k + 1 + idx / wl, j = k + 1 + idx % wl;
+        const int q = row_of(idx, rwl), i = k + 1 + q, j = k + 1 + idx - q * wl;
         at(i, j) = Ar::fms(at(i, j), v[i], sv[j]);
       }
       __syncthreads();
@@ -461,8 +484,9 @@ __global__ void __launch_bounds__(HESS_THREADS) k_bt_hess(BTreeArgs a) {
       }
       __syncthreads();
       const int wr = m - (k + 1);
+      const float rwr = 1.0f / (float)wr;
       for (int idx = tid; idx < m * wr; idx += T) {
-        const int i = idx / wr, j = k + 1 + idx % wr;
+        const int i = row_of(idx, rwr), j = k + 1 + idx - i * wr;
         at(i, j) = Ar::fms(at(i, j), tv[i], Ar::conj(v[j]));
       }
       if (tid == 0) at(k + 1, k) = sc[0];
@@ -812,7 +836,7 @@ __global__ void __launch_bounds__(LEAF_WARPS * 32, SMX <= LEAF_SMAX ? (DISP ? 3 
 }
 
 // ---------------------------------------------------------------------------- launch
-size_t top_smem(const BTreeStep& st) { return sizeof(float4) * ((size_t)st.nbs * st.D + st.nbs); }
+size_t bottom_smem(const BTreeStep& st) { return sizeof(float4) * (size_t)st.nbs * st.D; }
 
 // Columns of the bottom rows kept in registers: all D, or D rounded down to a multiple of 32
 // when the rest (the tail) is cheaper as dot products of the kept multipliers (~280 pair
@@ -826,7 +850,7 @@ int bottom_main_columns(int D, int nbs) {
 template <class Ar, int SMAX>
 cudaError_t launch_bottom(const BTreeArgs& a, const BTreeStep& st, long long children, int Dm, int num_sms,
                           cudaStream_t s) {
-  const size_t smem = top_smem(st);
+  const size_t smem = bottom_smem(st);
   cudaError_t err = cudaSuccess;
   if (smem > 48 * 1024) {
     err = cudaFuncSetAttribute(k_bt_bottom<Ar, SMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -907,7 +931,7 @@ cudaError_t launch_btree_ar(const BTreeArgs& a, const BTreeStep* steps, int nste
 
 }  // namespace
 
-size_t btree_step_smem_bytes(int nbs, int D) { return sizeof(float4) * ((size_t)nbs * D + nbs); }
+size_t btree_step_smem_bytes(int nbs, int D) { return sizeof(float4) * ((size_t)nbs * D + 3 * nbs); }   // rows, reciprocals, multipliers
 size_t btree_hess_smem_bytes(int m) {
   const size_t vecs = (size_t)m + (m + 2) + m + 2 + HESS_THREADS;
   if (m > GBSBIN_BT_MAX_HESS) return sizeof(float4) * (vecs + 2 * (size_t)m);   // the block in H
