@@ -26,6 +26,7 @@
 #include "gbsbin_device.cuh"
 #include "gbsbin_df.cuh"
 #include "gbsbin_gj.cuh"
+#include "gbsbin_hess.cuh"
 
 namespace gbsbin {
 namespace {
@@ -203,6 +204,394 @@ __global__ void __launch_bounds__(kBwdLeafThreads, 2) k_bwdt_leaf(BackwardArgs b
   }
 }
 
+// ---------------------------------------------------------------- leaves in the Hessenberg basis
+// The leaves of a parent differ by conj(w) I only, so one unitary reduction C = Q H Q^H serves them all:
+// inv(S) = Q inv(N) Q^H with N = conj(w) I - H, and with c' = Q^H c_F, d' = Q^T d_F
+//   s = Q s',  t = conj(Q) t',  Q + R^T = conj(Q) (Q' + R'^T) Q^T,
+// the primed sums those of the leaves with N, c', d'.  N = L U by the forward's unpivoted Hessenberg elimination (L
+// unit lower bidiagonal with multipliers l), so the inverse takes the m^3 / 6 multiply-adds of the triangular one
+// and O(m^2) more, instead of m^3: inv(N) L = inv(U) gives row i of inv(N) from the right,
+// x_ij = inv(U)_ij - l_j x_i,j+1.  At n = 200 (81 parents, 3321 leaves of 100 rows, pairs of FP32) the Gauss-Jordan
+// leaves took 10.1 ms; the reduction takes 0.87, the leaves 2.91 and the way back 1.08.
+constexpr int kBwdHessMax = GBSBIN_BT_MAX_HESS;
+constexpr int kBwdHessThreads = 512;
+constexpr int kRotThreads = 256;
+constexpr int kRotSlots = (kBwdHessMax + 7) / 8;
+
+template <class E>
+struct Rotated {                                       // what the Hessenberg leaves add to a parent's slot
+  E *Z, *ss, *st, *v0, *beta;
+  static __device__ Rotated map(E* P, int n, int mF) {
+    Rotated r;
+    r.Z = P + (size_t)n * n + 2 * n;
+    r.ss = r.Z + mF * mF;
+    r.st = r.ss + mF;
+    r.v0 = r.st + mF;
+    r.beta = r.v0 + mF;
+    return r;
+  }
+};
+
+// Sum over the g = 2^k lanes of a group.
+template <class Ar>
+__device__ __forceinline__ typename Ar::E group_sum(typename Ar::E v, int g) {
+  for (int o = g >> 1; o > 0; o >>= 1) v = Ar::add(v, shfl_xor(v, o));
+  return v;
+}
+
+// C -> H in place, a CTA per parent, [C, c_F, conj(d_F)] in shared memory (row stride odd).  The lanes of a column
+// form its product with the reflector and update it, then the lanes of a row: three barriers per step.  Below the
+// subdiagonal the reflectors' entries stay; their first entries and factors go to v0 and beta.
+template <class Ar>
+__global__ void __launch_bounds__(kBwdHessThreads) k_bwdt_hess(BackwardArgs b, BwdTree t) {
+  using E = typename Ar::E;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int m = t.mF, ld = (m + 2) | 1, tid = threadIdx.x, T = kBwdHessThreads, lane = tid & 31;
+  E* M = reinterpret_cast<E*>(smem);
+  E* v = M + (size_t)m * ld;
+  E* sc = v + m;
+  E* const P = reinterpret_cast<E*>(t.pbuf) + (size_t)blockIdx.x * t.pstride;
+  E *A, *U, *V, *C, *aE, *eE, *cF, *dF;
+  Parent::map(P, t.mE, m, &A, &U, &V, &C, &aE, &eE, &cF, &dF);
+  const Rotated<E> rot = Rotated<E>::map(P, b.n, m);
+  for (int q = tid; q < m * m; q += T) M[(size_t)(q / m) * ld + q % m] = C[q];
+  for (int i = tid; i < m; i += T) {
+    M[(size_t)i * ld + m] = cF[i];
+    M[(size_t)i * ld + m + 1] = Ar::conj(dF[i]);
+  }
+  __syncthreads();
+  const int extra = t.has_gamma ? 2 : 0;
+  for (int k = 0; k + 2 < m; ++k) {
+    if (tid < 32) {
+      E nrm2 = Ar::zero();
+      for (int i = k + 1 + lane; i < m; i += 32) nrm2 = Ar::add(nrm2, Ar::norm2(M[(size_t)i * ld + k]));
+      nrm2 = group_sum<Ar>(nrm2, 32);
+      const E x0 = M[(size_t)(k + 1) * ld + k];
+      E alpha = x0, beta = Ar::zero();
+      if (Ar::re(nrm2) > 0.f) reflector<Ar>(nrm2, x0, alpha, beta);
+      for (int i = k + 1 + lane; i < m; i += 32) {
+        E vi = M[(size_t)i * ld + k];
+        if (i == k + 1) vi = Ar::add(vi, Ar::neg(alpha));
+        v[i] = vi;
+      }
+      if (lane == 0) {
+        sc[0] = beta;
+        rot.v0[k] = v[k + 1];
+        rot.beta[k] = beta;
+      }
+      __syncwarp();
+      if (lane == 0) M[(size_t)(k + 1) * ld + k] = alpha;
+    }
+    __syncthreads();
+    const E beta = sc[0];
+    if (Ar::re(beta) > 0.f) {
+      {                                                // columns k + 1 .. m + 1 from the left
+        const int nc = m - 1 - k + extra, g = nc * 8 <= T ? 8 : 4, q = tid & (g - 1);
+        const int groups = T / g, rounds = (nc + groups - 1) / groups;
+        for (int r = 0; r < rounds; ++r) {
+          const int c = r * groups + tid / g, j = k + 1 + c;
+          E sum = Ar::zero();
+          if (c < nc)
+            for (int i = k + 1 + q; i < m; i += g) sum = Ar::fma(Ar::conj(v[i]), M[(size_t)i * ld + j], sum);
+          sum = Ar::mul(beta, group_sum<Ar>(sum, g));
+          if (c < nc)
+            for (int i = k + 1 + q; i < m; i += g) M[(size_t)i * ld + j] = Ar::fms(M[(size_t)i * ld + j], v[i], sum);
+        }
+      }
+      __syncthreads();
+      {                                                // rows from the right
+        const int g = m * 8 <= T ? 8 : 4, q = tid & (g - 1), i = tid / g;
+        E sum = Ar::zero();
+        if (i < m)
+          for (int j = k + 1 + q; j < m; j += g) sum = Ar::fma(M[(size_t)i * ld + j], v[j], sum);
+        sum = Ar::mul(beta, group_sum<Ar>(sum, g));
+        if (i < m)
+          for (int j = k + 1 + q; j < m; j += g) M[(size_t)i * ld + j] = Ar::fms(M[(size_t)i * ld + j], sum, Ar::conj(v[j]));
+      }
+    }
+    __syncthreads();
+  }
+  for (int q = tid; q < m * m; q += T) C[q] = M[(size_t)(q / m) * ld + q % m];
+  for (int i = tid; i < m; i += T) {
+    cF[i] = M[(size_t)i * ld + m];
+    dF[i] = Ar::conj(M[(size_t)i * ld + m + 1]);
+  }
+}
+
+// Leaves: CTA c takes leaves [c per, (c + 1) per) of the wave.  Four phases: one warp eliminates the Hessenberg
+// matrix (its row in registers, four columns a lane) and leaves U in shared memory (packed by rows, the diagonal
+// inverted); U is inverted in place, the 8 x 8 diagonal blocks first, then block columns left to right,
+// X_J = -X (U_J X_JJ) in 1 x 4 tiles; a thread per row then runs the recurrence of inv(N) and adds to the sums.
+template <class Ar, bool DISP>
+__global__ void __launch_bounds__(kBwdLeafThreads, 2) k_bwdt_hleaf(BackwardArgs b, BwdTree t) {
+  using E = typename Ar::E;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int m = t.mF, tid = threadIdx.x, NT = kBwdLeafThreads, lane = tid & 31, warp = tid >> 5;
+  E* Up = reinterpret_cast<E*>(smem);                  // U, then its inverse: row i at row(i) + j, j >= i
+  E* Tb = Up + (size_t)m * (m + 1) / 2;                // m x 8
+  E* lv = Tb + (size_t)8 * m;
+  E* yv = lv + m;
+  E* zv = yv + m;
+  auto row = [&](int i) { return i * m - i * (i + 1) / 2; };
+  const long long nleaves = (t.p1 - t.p0) * t.half;
+  const long long l0 = (long long)blockIdx.x * t.per, l1 = min(l0 + t.per, nleaves);
+  const long long pfirst = l0 / t.half;
+  long long cur = -1;
+  const E *H = nullptr, *cs = nullptr, *ds = nullptr;
+  for (long long l = l0; l < l1; ++l) {
+    const long long pr = l / t.half, kl = l - pr * t.half;
+    E* Z = reinterpret_cast<E*>(t.part) + ((size_t)blockIdx.x * t.maxspan + (size_t)(pr - pfirst)) * t.lstride;
+    E* ss = Z + m * m;
+    E* st = ss + m;
+    E* bb = st + m;
+    if (pr != cur) {
+      E *A, *U, *V, *C, *aE, *eE, *cF, *dF;
+      Parent::map(reinterpret_cast<E*>(t.pbuf) + (size_t)pr * t.pstride, t.mE, m, &A, &U, &V, &C, &aE, &eE, &cF, &dF);
+      H = C;
+      cs = cF;
+      ds = dF;
+      for (long long q = tid; q < t.lstride; q += NT) Z[q] = Ar::zero();
+      cur = pr;
+      __syncthreads();
+    }
+    const long long e = (t.p0 + pr) * t.half + kl;
+    const double2 beta = b.beta[e];
+    if (beta.x == 0.0 && beta.y == 0.0) continue;
+    const double2 w = grid_root(b.tw, b.grid, t.L - 1, (int)kl);
+    const E wc = Ar::from(make_double2(w.x, -w.y)), be = Ar::from(beta);
+    if (warp == 0) {
+      E r[4], hn[4];
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        const int j = lane + 32 * s;
+        r[s] = j < m ? Ar::neg(H[j]) : Ar::zero();
+        hn[s] = j < m ? H[m + j] : Ar::zero();
+      }
+      if (lane == 0) r[0] = Ar::add(r[0], wc);
+      E y = DISP ? cs[0] : Ar::zero();
+#pragma unroll
+      for (int sb = 0; sb < 4; ++sb) {
+        const int iend = min(m, 32 * sb + 32);
+        for (int i = 32 * sb; i < iend; ++i) {
+          const int il = i & 31;
+          const E rp = Ar::recip(shfl(r[sb], il));
+#pragma unroll
+          for (int s = 0; s < 4; ++s) {
+            const int j = lane + 32 * s;
+            if (s >= sb && j >= i && j < m) Up[row(i) + j] = j == i ? rp : r[s];
+          }
+          if (DISP && lane == 0) yv[i] = y;
+          if (i + 1 < m) {
+            const E lm = Ar::neg(Ar::mul(shfl(hn[sb], il), rp));
+            if (lane == 0) lv[i] = lm;
+            if (DISP) y = Ar::fms(cs[i + 1], lm, y);
+            const E* hrow = H + (size_t)min(i + 2, m - 1) * m;
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+              const int j = lane + 32 * s;
+              if (s < sb) continue;
+              E x = Ar::neg(hn[s]);
+              if (j == i + 1) x = Ar::add(x, wc);
+              hn[s] = j < m ? hrow[j] : Ar::zero();
+              r[s] = Ar::fms(x, lm, r[s]);
+            }
+          } else if (lane == 0) {
+            lv[i] = Ar::zero();
+          }
+        }
+      }
+    }
+    __syncthreads();
+    {                                                  // the diagonal blocks, a thread per column
+      const int j = tid, K = j & ~7, jj = j & 7;
+      E x[8];
+#pragma unroll
+      for (int ii = 7; ii >= 0; --ii) {
+        x[ii] = Ar::zero();
+        if (j < m && ii <= jj) {
+          const E rp = Up[row(K + ii) + K + ii];
+          if (ii == jj) {
+            x[ii] = rp;
+          } else {
+            E acc = Ar::zero();
+#pragma unroll
+            for (int kk = ii + 1; kk < 8; ++kk)
+              if (kk <= jj) acc = Ar::fms(acc, Up[row(K + ii) + K + kk], x[kk]);
+            x[ii] = Ar::mul(acc, rp);
+          }
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int ii = 0; ii < 7; ++ii)
+        if (j < m && ii < jj) Up[row(K + ii) + j] = x[ii];
+    }
+    __syncthreads();
+    for (int K = 8; K < m; K += 8) {
+      const int bs = min(8, m - K);
+      for (int q = tid; q < 8 * K; q += NT) {          // T = U_J X_JJ
+        const int k = q >> 3, c = q & 7;
+        E acc = Ar::zero();
+        if (c < bs)
+          for (int cc = 0; cc <= c; ++cc) acc = Ar::fma(Up[row(k) + K + cc], Up[row(K + cc) + K + c], acc);
+        Tb[q] = acc;
+      }
+      __syncthreads();
+      const int nw = (2 * K + 31) / 32;                // warps' items of 16 rows, the longest with the shortest
+      for (int rd = 0; rd * 4 < nw; ++rd) {
+        const int wi = rd * 4 + ((rd & 1) ? 3 - warp : warp);
+        if (wi >= nw) continue;
+        const int i = wi * 16 + (lane >> 1), h = 4 * (lane & 1);
+        E acc[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[c] = Ar::zero();
+        const int base = i < K ? row(i) : 0;
+        for (int k = wi * 16; k < K; ++k) {
+          const E u = (i < K && k >= i) ? Up[base + k] : Ar::zero();
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[c] = Ar::fms(acc[c], u, Tb[8 * k + h + c]);
+        }
+        if (i < K)
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (h + c < bs) Up[base + K + h + c] = acc[c];
+      }
+      __syncthreads();
+    }
+    E bs_i = Ar::zero();                               // beta s_i
+    if (DISP) {                                        // s = inv(U) y, z = inv(U)^T d: m + 1 terms a thread
+      if (tid < m) {
+        E sa = Ar::zero(), za = Ar::zero();
+        for (int j = tid; j < m; ++j) sa = Ar::fma(Up[row(tid) + j], yv[j], sa);
+        for (int i = 0; i <= tid; ++i) za = Ar::fma(Up[row(i) + tid], ds[i], za);
+        zv[tid] = za;
+        bs_i = Ar::mul(be, sa);
+        ss[tid] = Ar::add(ss[tid], bs_i);
+      }
+      __syncthreads();
+    }
+    if (tid < m) {                                     // row tid of inv(N); Z[j][i] += beta (t_j s_i + x_ij)
+      E x = Ar::zero(), tj = Ar::zero();
+      const int base = row(tid);
+      for (int jb = m - 1; jb >= 0; jb -= 4) {
+        E zo[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (jb - c >= 0) zo[c] = Z[(size_t)(jb - c) * m + tid];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int j = jb - c;
+          if (j < 0) continue;
+          const E lj = lv[j];
+          x = Ar::fms(j >= tid ? Up[base + j] : Ar::zero(), lj, x);
+          E z = Ar::fma(be, x, zo[c]);
+          if (DISP) {
+            tj = Ar::fms(zv[j], lj, tj);
+            z = Ar::fma(tj, bs_i, z);
+            if (j == tid) st[j] = Ar::fma(be, tj, st[j]);
+          }
+          Z[(size_t)j * m + tid] = z;
+        }
+      }
+    }
+    if (tid == 0) bb[0] = Ar::add(bb[0], be);
+    __syncthreads();
+  }
+}
+
+// Back from the Hessenberg basis: RIGHT 0: Z <- conj(Q) Z', sigma_t <- conj(Q) sigma_t' from the leaf CTAs' sums;
+// RIGHT 1: Z <- Z Q^T, sigma_s <- Q sigma_s'.  The columns (then the rows) are independent: eight lanes each hold
+// one in registers and apply the reflectors last to first, all of them in shared memory, without a barrier.
+template <class Ar, bool RIGHT>
+__global__ void __launch_bounds__(kRotThreads, 2) k_bwdt_unrot(BackwardArgs b, BwdTree t) {
+  using E = typename Ar::E;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int m = t.mF, tid = threadIdx.x, NT = kRotThreads, g = tid & 7;
+  const long long pr = blockIdx.x;
+  E* Vs = reinterpret_cast<E*>(smem);                  // reflector k at off(k) + i, i = k + 1 .. m - 1
+  E* bet = Vs + (size_t)m * (m - 1) / 2;
+  auto off = [&](int k) { return k * (m - 1) - k * (k - 1) / 2 - (k + 1); };
+  E *A, *U, *V, *C, *aE, *eE, *cF, *dF;
+  E* const P = reinterpret_cast<E*>(t.pbuf) + (size_t)pr * t.pstride;
+  Parent::map(P, t.mE, m, &A, &U, &V, &C, &aE, &eE, &cF, &dF);
+  const Rotated<E> rot = Rotated<E>::map(P, b.n, m);
+  for (int q = tid; q < m * m; q += NT) {
+    const int i = q / m, k = q - (q / m) * m;
+    if (k + 2 < m && i > k) Vs[off(k) + i] = i == k + 1 ? rot.v0[k] : C[q];
+  }
+  for (int k = tid; k + 2 < m; k += NT) bet[k] = rot.beta[k];
+  __syncthreads();
+  const int j = blockIdx.y * (NT / 8) + tid / 8;       // the column (or row); m: the vector
+  const long long c0 = (pr * t.half) / t.per, c1 = (pr * t.half + t.half - 1) / t.per;
+  E z[kRotSlots];
+#pragma unroll
+  for (int q = 0; q < kRotSlots; ++q) {
+    const int i = g + 8 * q;
+    z[q] = Ar::zero();
+    if (i >= m || j > m) continue;
+    if (RIGHT && j < m) {
+      z[q] = rot.Z[(size_t)j * m + i];
+      continue;
+    }
+    for (long long c = c0; c <= c1; ++c) {
+      const E* part = reinterpret_cast<const E*>(t.part) +
+                      ((size_t)c * t.maxspan + (size_t)(pr - (c * t.per) / t.half)) * t.lstride;
+      z[q] = Ar::add(z[q], j < m ? part[(size_t)i * m + j] : part[m * m + (RIGHT ? 0 : m) + i]);
+    }
+  }
+  for (int k = m - 3; k >= 0; --k) {
+    const E* v = Vs + off(k);
+    const int q0 = (k + 1) >> 3;
+    E s0 = Ar::zero();
+#pragma unroll
+    for (int q = 0; q < kRotSlots; ++q) {
+      const int i = g + 8 * q;
+      if (q >= q0 && i > k && i < m) s0 = Ar::fma(RIGHT ? Ar::conj(v[i]) : v[i], z[q], s0);
+    }
+    s0 = Ar::mul(bet[k], group_sum<Ar>(s0, 8));
+#pragma unroll
+    for (int q = 0; q < kRotSlots; ++q) {
+      const int i = g + 8 * q;
+      if (q >= q0 && i > k && i < m) z[q] = Ar::fms(z[q], RIGHT ? v[i] : Ar::conj(v[i]), s0);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < kRotSlots; ++q) {
+    const int i = g + 8 * q;
+    if (i >= m || j > m) continue;
+    if (j < m) rot.Z[RIGHT ? (size_t)j * m + i : (size_t)i * m + j] = z[q];
+    else (RIGHT ? rot.ss : rot.st)[i] = z[q];
+  }
+}
+
+template <class Ar>
+cudaError_t launch_hess_leaves(const BackwardArgs& b, const BwdTree& t, long long parents, long long leaf_ctas,
+                               cudaStream_t s) {
+  const int m = t.mF;
+  const size_t hsm = (size_t)16 * ((size_t)m * ((m + 2) | 1) + m + 1);
+  const size_t lsm = (size_t)16 * ((size_t)m * (m + 1) / 2 + 11 * (size_t)m);
+  const size_t rsm = (size_t)16 * ((size_t)m * (m - 1) / 2 + m);
+  auto leaf = t.has_gamma ? k_bwdt_hleaf<Ar, true> : k_bwdt_hleaf<Ar, false>;
+  cudaError_t err;
+  if ((err = cudaFuncSetAttribute(k_bwdt_hess<Ar>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hsm)) !=
+          cudaSuccess ||
+      (err = cudaFuncSetAttribute(leaf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm)) != cudaSuccess ||
+      (err = cudaFuncSetAttribute(k_bwdt_unrot<Ar, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm)) !=
+          cudaSuccess ||
+      (err = cudaFuncSetAttribute(k_bwdt_unrot<Ar, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm)) !=
+          cudaSuccess)
+    return err;
+  k_bwdt_hess<Ar><<<(unsigned)parents, kBwdHessThreads, hsm, s>>>(b, t);
+  if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  leaf<<<(unsigned)leaf_ctas, kBwdLeafThreads, lsm, s>>>(b, t);
+  if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  const dim3 rg((unsigned)parents, (unsigned)((m + 1 + kRotThreads / 8 - 1) / (kRotThreads / 8)));
+  k_bwdt_unrot<Ar, false><<<rg, kRotThreads, rsm, s>>>(b, t);
+  if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  k_bwdt_unrot<Ar, true><<<rg, kRotThreads, rsm, s>>>(b, t);
+  return cudaGetLastError();
+}
+
 // Per parent: the leaves' sums, Z = Q + R^T, the three products, and 1/2 (Phi + Psi^T) into this
 // CTA's partials in the original row order (ST[j][i] = S[i][j]).
 template <class Ar>
@@ -232,9 +621,12 @@ __global__ void __launch_bounds__(kBtThreads) k_bwdt_assemble(BackwardArgs b, Bw
   for (long long p = t.p0 + blockIdx.x; p < t.p1; p += gridDim.x) {
     const long long pr = p - t.p0;
     E *A, *U, *V, *C, *aE, *eE, *cF, *dF;
-    Parent::map(reinterpret_cast<E*>(t.pbuf) + (size_t)pr * t.pstride, mE, mF, &A, &U, &V, &C, &aE, &eE, &cF, &dF);
+    E* const P = reinterpret_cast<E*>(t.pbuf);
+    Parent::map(P + (size_t)pr * t.pstride, mE, mF, &A, &U, &V, &C, &aE, &eE, &cF, &dF);
     const long long c0 = (pr * t.half) / t.per, c1 = (pr * t.half + t.half - 1) / t.per;
-    for (int q = tid; q < mF * mF; q += NT) {
+    const Rotated<E> rot = Rotated<E>::map(P + (size_t)pr * t.pstride, b.n, mF);
+    const E* Zp = t.hess ? rot.Z : Z;
+    for (int q = tid; !t.hess && q < mF * mF; q += NT) {
       const int i = q / mF, j = q - (q / mF) * mF;
       E z = Ar::zero();
       for (long long c = c0; c <= c1; ++c) {
@@ -249,16 +641,17 @@ __global__ void __launch_bounds__(kBtThreads) k_bwdt_assemble(BackwardArgs b, Bw
       for (long long c = c0; c <= c1; ++c) {
         const E* part = reinterpret_cast<const E*>(t.part) +
                         ((size_t)c * t.maxspan + (size_t)(pr - (c * t.per) / t.half)) * t.lstride;
-        v = Ar::add(v, part[2 * mF * mF + f]);
+        v = Ar::add(v, part[(t.hess ? 1 : 2) * mF * mF + f]);
       }
+      if (t.hess && f < 2 * mF) v = f < mF ? rot.ss[f] : rot.st[f - mF];
       if (f < mF) ss[f] = v;
       else if (f < 2 * mF) st[f - mF] = v;
       else bbs[0] = v;
     }
     __syncthreads();
-    gemm_staged<Ar>(X1, mE, Z, mF, 1, U, 1, mF, mF, mE, mF, false, false, nb, Pc, Rx);
+    gemm_staged<Ar>(X1, mE, Zp, mF, 1, U, 1, mF, mF, mE, mF, false, false, nb, Pc, Rx);
     gemm_staged<Ar>(X2, mE, V, 1, mE, X1, mE, 1, mE, mE, mF, false, false, nb, Pc, Rx);
-    gemm_staged<Ar>(X3, mF, V, 1, mE, Z, mF, 1, mE, mF, mF, false, false, nb, Pc, Rx);
+    gemm_staged<Ar>(X3, mF, V, 1, mE, Zp, mF, 1, mE, mF, mF, false, false, nb, Pc, Rx);
     for (int i = tid; i < mE; i += NT) {             // U sigma_s, V^T sigma_t
       E su = Ar::zero(), sv = Ar::zero();
       for (int k = 0; k < mF; ++k) {
@@ -284,7 +677,7 @@ __global__ void __launch_bounds__(kBtThreads) k_bwdt_assemble(BackwardArgs b, Bw
       else if (c < mE)
         v = Ar::fms(Ar::mul(st[a - mE], aE[c]), Ar::one(), X1[(size_t)(a - mE) * mE + c]);
       else
-        v = Z[(size_t)(a - mE) * mF + (c - mE)];
+        v = Zp[(size_t)(a - mE) * mF + (c - mE)];
       ST[q] = Ar::fma(half, v, ST[q]);
     }
     for (int io = tid; io < n; io += NT) {           // 1/2 (sum beta x + X sum beta y)
@@ -316,12 +709,16 @@ cudaError_t tree_wave(const BackwardArgs& b, const BwdTree& t0, cudaStream_t s) 
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
   const long long nleaves = parents * t.half;
   const long long gl = (nleaves + t.per - 1) / t.per;
-  const size_t lsmem = backward_leaf_smem_bytes(t.mF);
-  if ((err = cudaFuncSetAttribute(k_bwdt_leaf<Ar>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsmem)) !=
-      cudaSuccess)
-    return err;
-  k_bwdt_leaf<Ar><<<(unsigned)gl, kBwdLeafThreads, lsmem, s>>>(b, t);
-  if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  if (t.hess) {
+    if ((err = launch_hess_leaves<Ar>(b, t, parents, gl, s)) != cudaSuccess) return err;
+  } else {
+    const size_t lsmem = backward_leaf_smem_bytes(t.mF);
+    if ((err = cudaFuncSetAttribute(k_bwdt_leaf<Ar>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsmem)) !=
+        cudaSuccess)
+      return err;
+    k_bwdt_leaf<Ar><<<(unsigned)gl, kBwdLeafThreads, lsmem, s>>>(b, t);
+    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  }
   k_bwdt_assemble<Ar><<<(unsigned)t.nparts, kBtThreads, smem, s>>>(b, t);
   return cudaGetLastError();
 }
@@ -330,6 +727,18 @@ cudaError_t tree_wave(const BackwardArgs& b, const BwdTree& t0, cudaStream_t s) 
 
 size_t backward_leaf_smem_bytes(int mF) {
   return (size_t)16 * ((size_t)3 * mF * kBwdLeafNb + (size_t)kBwdLeafNb * kBwdLeafNb + 4 * (size_t)mF);
+}
+
+// The reduction and the way back are launches of one or a few CTAs per parent, O(mF^3) each, as long for one parent
+// as for an SM each; the saving grows with the leaves per SM.  Measured (reverse-pass kernels, us, Gauss-Jordan
+// leaves / Hessenberg leaves, 61 parents; pairs, FP64): mF = 40, 6.8 leaves per SM 823 / 896, 1950 / 2438; mF = 60,
+// 5.2 per SM 1636 / 1689, 4235 / 4763, 6.8 per SM 1901 / 1819, 4945 / 5055; mF = 80, 5.2 per SM 3564 / 3393,
+// 8886 / 10008, 6.8 per SM 4116 / 3575, 10361 / 10449.  Eight leaves per SM, per parent an SM takes, is past the
+// crossing of all but the smallest blocks.
+bool backward_hess_suits(int mF, long long parents, long long half, int num_sms) {
+  if (mF < 32 || mF > kBwdHessMax) return false;
+  const long long rounds = (parents + num_sms - 1) / num_sms;
+  return parents * half >= 8 * rounds * num_sms;
 }
 
 size_t backward_tree_smem_bytes(int n, int nb) {

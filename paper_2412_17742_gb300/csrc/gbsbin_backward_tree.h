@@ -21,14 +21,18 @@ struct BwdTree {
   long long half;           // leaves per parent
   long long p0, p1;         // the parents of this wave
   void* pbuf;               // (p1 - p0) x pstride: inv(M_EE), U, V, C, a_E, e_E, c_F, d_F
-  long long pstride;        // n^2 + 2 n
+  long long pstride;        // n^2 + 2 n, and for the Hessenberg leaves mF^2 + 4 mF: Z, sigma_s, sigma_t, and the
+                            // reflectors' first entries and factors
   void* part;               // leaf partials: leaf CTAs x maxspan x lstride
-  long long lstride;        // 2 mF^2 + 2 mF + 1: R, Q, sigma_s, sigma_t, beta sum
+  long long lstride;        // 2 mF^2 + 2 mF + 1: R, Q, sigma_s, sigma_t, beta sum; for the Hessenberg leaves
+                            // mF^2 + 2 mF + 1: Q + R^T, the rest
   int per;                  // leaves per CTA of the leaf launch
   int maxspan;              // parents one leaf CTA can touch
   int nparts;               // CTAs of the assembly launch (its partials)
   int zero_partials;        // first wave: the assembly zeroes its partials
   int rn;                   // the kernels' shared memory holds the block-row buffer (nb x n)
+  int hess;                 // the leaves invert in the Hessenberg basis of their parent's C
+  int has_gamma;
   int leaf_ctas;            // CTAs of the leaf launch: two per SM (128 threads each) where two
                             // mF x mF slots fit in an SM's n x n workspace slot, else one
 };
@@ -46,5 +50,7 @@ cudaError_t launch_backward_tree_wave(const BackwardArgs& b, const BwdTree& t, c
 cudaError_t launch_backward_reduce(const BackwardArgs& b, int nparts, cudaStream_t s);
 size_t backward_tree_smem_bytes(int n, int nb);
 size_t backward_leaf_smem_bytes(int mF);
+// Whether the leaves' inverses go through the Hessenberg form of each parent's C.
+bool backward_hess_suits(int mF, long long parents, long long half, int num_sms);
 
 }  // namespace gbsbin

@@ -1067,8 +1067,9 @@ int backward_tree_setup(gbsbin_plan* P) {
   t.D = n + 1;
   t.A0 = P->btree.mat[0];
   t.half = half;
-  t.pstride = (long long)n * n + 2LL * n;
-  t.lstride = 2LL * mF * mF + 2LL * mF + 1;
+  t.hess = backward_hess_suits(mF, parents, half, P->num_sms);
+  t.pstride = (long long)n * n + 2LL * n + (t.hess ? (long long)mF * mF + 4LL * mF : 0);
+  t.lstride = (t.hess ? 1LL : 2LL) * mF * mF + 2LL * mF + 1;
   int off = 0;
   for (int l = 0; l < L; ++l) {
     t.goff[l] = off;
@@ -1078,7 +1079,8 @@ int backward_tree_setup(gbsbin_plan* P) {
   const long long budget = 512LL << 20;
   const long long wave = std::max(1LL, std::min(parents, budget / (t.pstride * 16)));
   // leaves: two CTAs per SM where two mF x mF matrices fit in an SM's n x n slot
-  t.leaf_ctas = 2LL * mF * mF <= (long long)n * n ? 2 * P->num_sms : P->num_sms;
+  // (the Hessenberg leaves keep theirs in shared memory)
+  t.leaf_ctas = t.hess || 2LL * mF * mF <= (long long)n * n ? 2 * P->num_sms : P->num_sms;
   t.per = (int)((wave * half + t.leaf_ctas - 1) / t.leaf_ctas);
   t.maxspan = (int)((t.per - 1) / half + 2);
   t.nparts = (int)std::min<long long>(parents, P->num_sms);
@@ -1749,6 +1751,7 @@ static int backward_enqueue(gbsbin_plan* P, const double* dLdP, cudaStream_t s) 
       t.p0 = p0;
       t.p1 = std::min(P->bt_parents, p0 + P->bt_wave);
       t.zero_partials = p0 == 0;
+      t.has_gamma = P->has_gamma;
       e = launch_backward_tree_wave(b, t, s);
     }
     if (e == cudaSuccess && b.ev1) e = cudaEventRecord(b.ev1, s);
