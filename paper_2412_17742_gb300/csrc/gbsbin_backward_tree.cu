@@ -16,9 +16,9 @@
 //   EF = e_E sigma_s^T - V^T Z,   FE = sigma_t a_E^T - Z U^T,   FF = Z,
 // and 1/2 sum beta (x + X y) from sum beta x = (b a_E - U sigma_s, sigma_s), sum beta y =
 // (b e_E - V^T sigma_t, sigma_t).  So a leaf inverts an mF x mF matrix instead of n x n, and the
-// parent's O(n^3) products are shared by its leaves.  Three launches per wave of parents: the
-// parents' inverse and products, the leaves (each CTA a contiguous run of leaves, its sums per
-// parent in its own slots), the parents' assembly into per-CTA partials (in the original row
+// parent's O(n^3) products are shared by its leaves.  Launches per wave of parents: the parents'
+// inverses, their products, the leaves (each CTA a contiguous run of leaves, its sums per parent in
+// its own slots), the leaves' sums, the parents' assembly into partials (in the original row
 // order, transposed as the per-point kernel keeps them), reduced once at the end in FP64.
 #include <cuda_runtime.h>
 
@@ -32,6 +32,8 @@ namespace gbsbin {
 namespace {
 
 constexpr int kBtThreads = 256;
+// The products of few parents are split by columns over several CTAs each, two to an SM: panels of eight.
+constexpr int kBwdSplitNb = 8;
 
 // The block-row buffer (nb x n) after the kernels' other shared arrays.
 __host__ __device__ __forceinline__ size_t backward_tree_rn_offset(int n, int nb) {
@@ -58,7 +60,7 @@ __device__ __forceinline__ int group_of(const BwdTree& t, int a) {
   return l;
 }
 
-// Per parent: A = inv(M_EE), U = -A XA_EF, V = -XA_FE A, C = XA_FF - XA_FE U and the vectors.
+// Per parent: A = inv(M_EE) and the vectors.
 template <class Ar>
 __global__ void __launch_bounds__(kBtThreads) k_bwdt_parent(BackwardArgs b, BwdTree t) {
   using E = typename Ar::E;
@@ -86,12 +88,6 @@ __global__ void __launch_bounds__(kBtThreads) k_bwdt_parent(BackwardArgs b, BwdT
     }
     __syncthreads();
     gj_invert<Ar>(A, mE, mE, nb, Pc, Rx, Dg, t.rn ? reinterpret_cast<E*>(smem + backward_tree_rn_offset(n, nb)) : nullptr);
-    // U = -A XA_EF, V = -XA_FE A, C = XA_FF - XA_FE U
-    gemm_staged<Ar>(U, mF, A, mE, 1, A0 + mE, D, 1, mE, mF, mE, false, true, nb, Pc, Rx);
-    gemm_staged<Ar>(V, mE, A0 + (size_t)mE * D, D, 1, A, mE, 1, mF, mE, mE, false, true, nb, Pc, Rx);
-    for (int q = tid; q < mF * mF; q += NT) C[q] = A0[(size_t)(mE + q / mF) * D + mE + q % mF];
-    __syncthreads();
-    gemm_staged<Ar>(C, mF, A0 + (size_t)mE * D, D, 1, U, mF, 1, mF, mF, mE, true, true, nb, Pc, Rx);
     // a_E = A b_E, e_E = A^T g_E (b = X gamma: column n; g = gamma: row n)
     for (int i = tid; i < mE; i += NT) {
       E sa = Ar::zero(), se = Ar::zero();
@@ -102,17 +98,54 @@ __global__ void __launch_bounds__(kBtThreads) k_bwdt_parent(BackwardArgs b, BwdT
       aE[i] = sa;
       eE[i] = se;
     }
-    // c_F = b_F - V b_E, d_F = g_F - U^T g_E
+    __syncthreads();
+    // c_F = b_F - V b_E = b_F + XA_FE a_E, d_F = g_F - U^T g_E = g_F + XA_EF^T e_E
     for (int f = tid; f < mF; f += NT) {
       E sc = A0[(size_t)(mE + f) * D + n], sd = A0[(size_t)n * D + mE + f];
       for (int k = 0; k < mE; ++k) {
-        sc = Ar::fms(sc, V[(size_t)f * mE + k], A0[(size_t)k * D + n]);
-        sd = Ar::fms(sd, U[(size_t)k * mF + f], A0[(size_t)n * D + k]);
+        sc = Ar::fma(A0[(size_t)(mE + f) * D + k], aE[k], sc);
+        sd = Ar::fma(A0[(size_t)k * D + mE + f], eE[k], sd);
       }
       cF[f] = sc;
       dF[f] = sd;
     }
     __syncthreads();
+  }
+}
+
+// The columns [lo, hi) of m that split y of `splits` takes.
+__device__ __forceinline__ void split_range(int m, int y, int splits, int& lo, int& hi) {
+  lo = (int)((long long)m * y / splits);
+  hi = (int)((long long)m * (y + 1) / splits);
+}
+
+// Per parent and split: U = -A XA_EF, C = XA_FF - XA_FE U and V = -XA_FE A on its columns.
+template <class Ar>
+__global__ void __launch_bounds__(kBtThreads, 2) k_bwdt_products(BackwardArgs b, BwdTree t) {
+  using E = typename Ar::E;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int nb = kBwdSplitNb, mE = t.mE, mF = t.mF, D = t.D, tid = threadIdx.x, NT = kBtThreads;
+  E* Pc = reinterpret_cast<E*>(smem);
+  E* Rx = Pc + (size_t)b.n * nb;
+  const E* A0 = reinterpret_cast<const E*>(t.A0);
+  int f0, f1, e0, e1;
+  split_range(mF, blockIdx.y, gridDim.y, f0, f1);
+  split_range(mE, blockIdx.y, gridDim.y, e0, e1);
+  const int nf = f1 - f0;
+  for (long long pr = blockIdx.x; pr < t.p1 - t.p0; pr += gridDim.x) {
+    E *A, *U, *V, *C, *aE, *eE, *cF, *dF;
+    Parent::map(reinterpret_cast<E*>(t.pbuf) + (size_t)pr * t.pstride, mE, mF, &A, &U, &V, &C, &aE, &eE, &cF, &dF);
+    for (int q = tid; q < mF * nf; q += NT) {
+      const int i = q / nf, j = f0 + q - (q / nf) * nf;
+      C[(size_t)i * mF + j] = A0[(size_t)(mE + i) * D + mE + j];
+    }
+    __syncthreads();
+    const E* AF = A0 + (size_t)mE * D;
+#pragma unroll 1
+    for (int g = 0; g < 3; ++g)                        // U, V, C (one call: the compiler inlines each)
+      gemm_staged<Ar>(g == 0 ? U + f0 : (g == 1 ? V + e0 : C + f0), g == 1 ? mE : mF, g == 0 ? A : AF, g == 0 ? mE : D, 1,
+                      g == 0 ? A0 + mE + f0 : (g == 1 ? A + e0 : U + f0), g == 0 ? D : (g == 1 ? mE : mF), 1,
+                      g == 0 ? mE : mF, g == 1 ? e1 - e0 : nf, mE, g == 2, true, nb, Pc, Rx);
   }
 }
 
@@ -219,7 +252,7 @@ constexpr int kRotThreads = 256;
 constexpr int kRotSlots = (kBwdHessMax + 7) / 8;
 
 template <class E>
-struct Rotated {                                       // what the Hessenberg leaves add to a parent's slot
+struct Rotated {                                       // the rest of a parent's slot: its leaves' sums
   E *Z, *ss, *st, *v0, *beta;
   static __device__ Rotated map(E* P, int n, int mF) {
     Rotated r;
@@ -592,66 +625,81 @@ cudaError_t launch_hess_leaves(const BackwardArgs& b, const BwdTree& t, long lon
   return cudaGetLastError();
 }
 
-// Per parent: the leaves' sums, Z = Q + R^T, the three products, and 1/2 (Phi + Psi^T) into this
-// CTA's partials in the original row order (ST[j][i] = S[i][j]).
+// The sums of Gauss-Jordan leaves over their CTAs: Z = Q + R^T, sigma_s, sigma_t per parent.
 template <class Ar>
-__global__ void __launch_bounds__(kBtThreads) k_bwdt_assemble(BackwardArgs b, BwdTree t) {
+__global__ void __launch_bounds__(kBtThreads) k_bwdt_sum(BackwardArgs b, BwdTree t) {
+  using E = typename Ar::E;
+  const int mF = t.mF, q = blockIdx.y * kBtThreads + threadIdx.x;
+  const long long pr = blockIdx.x;
+  const Rotated<E> rot = Rotated<E>::map(reinterpret_cast<E*>(t.pbuf) + (size_t)pr * t.pstride, b.n, mF);
+  const long long c0 = (pr * t.half) / t.per, c1 = (pr * t.half + t.half - 1) / t.per;
+  if (q >= mF * mF + 2 * mF) return;
+  E z = Ar::zero();
+  for (long long c = c0; c <= c1; ++c) {
+    const E* part = reinterpret_cast<const E*>(t.part) +
+                    ((size_t)c * t.maxspan + (size_t)(pr - (c * t.per) / t.half)) * t.lstride;
+    z = Ar::add(z, part[mF * mF + q]);
+    if (q < mF * mF) z = Ar::add(z, part[(size_t)(q % mF) * mF + q / mF]);
+  }
+  rot.Z[q] = z;                                        // (sigma_s and sigma_t follow Z in both)
+}
+
+// Per parent and split: the three products on its columns of E and of F, and 1/2 (Phi + Psi^T) of them into the
+// parent's partial in the original row order (ST[j][i] = S[i][j]); the splits of a partial write different rows
+// of ST.  Bound by the issue of the products' multiply-adds (one warp's latency where the blocks are small).  81
+// parents of 100 + 100 rows in pairs on 152 SMs: one CTA each 1.72 ms, three 1.05; with the parents' products, 1.60
+// -> 0.56 + 0.84 ms.  13 parents of 24 + 24 rows in FP64: parents, leaves and assembly 617 us -> 250 (entry by entry
+// instead of 36 tiles of 4 x 4, three splits).
+template <class Ar>
+__global__ void __launch_bounds__(kBtThreads, 2) k_bwdt_assemble(BackwardArgs b, BwdTree t) {
   using E = typename Ar::E;
   extern __shared__ __align__(16) unsigned char smem[];
-  const int n = b.n, nb = b.nb, mE = t.mE, mF = t.mF, tid = threadIdx.x, NT = kBtThreads;
+  const int n = b.n, nb = kBwdSplitNb, mE = t.mE, mF = t.mF, tid = threadIdx.x, NT = kBtThreads;
+  const int lane = tid & 31, warp = tid >> 5;
   E* Pc = reinterpret_cast<E*>(smem);
   E* Rx = Pc + (size_t)n * nb;
-  E* Dg = Rx + (size_t)nb * n;
-  E* ss = Dg + nb * nb;
-  E* st = ss + mF;
-  E* uS = st + mF;
+  E* uS = Rx + (size_t)nb * n;
   E* vT = uS + mE;
   E* bbs = vT + mE;
   E* ST = reinterpret_cast<E*>(b.partS) + (size_t)blockIdx.x * n * n;
   E* sg = reinterpret_cast<E*>(b.partg) + (size_t)blockIdx.x * n;
   E* W = reinterpret_cast<E*>(reinterpret_cast<char*>(b.ws) + (size_t)blockIdx.x * (size_t)b.ws_slot_bytes);
-  E* Z = W;
-  E* X1 = Z + mF * mF;                                 // Z U^T (mF x mE)
+  E* X1 = W;                                           // Z U^T (mF x mE)
   E* X2 = X1 + mF * mE;                                // V^T Z U^T (mE x mE)
   E* X3 = X2 + mE * mE;                                // V^T Z (mE x mF)
+  int f0, f1, e0, e1;
+  split_range(mF, blockIdx.y, gridDim.y, f0, f1);
+  split_range(mE, blockIdx.y, gridDim.y, e0, e1);
+  auto mine = [&](int c) { return c < mE ? c >= e0 && c < e1 : c - mE >= f0 && c - mE < f1; };
   if (t.zero_partials) {
-    for (long long q = tid; q < (long long)n * n; q += NT) ST[q] = Ar::zero();
-    for (int q = tid; q < n; q += NT) sg[q] = Ar::zero();
+    for (int jo = warp; jo < n; jo += NT / 32)
+      if (mine(t.pinv[jo]))
+        for (int io = lane; io < n; io += 32) ST[(size_t)jo * n + io] = Ar::zero();
+    if (blockIdx.y == 0)
+      for (int q = tid; q < n; q += NT) sg[q] = Ar::zero();
+    __syncthreads();
   }
   for (long long p = t.p0 + blockIdx.x; p < t.p1; p += gridDim.x) {
     const long long pr = p - t.p0;
     E *A, *U, *V, *C, *aE, *eE, *cF, *dF;
-    E* const P = reinterpret_cast<E*>(t.pbuf);
-    Parent::map(P + (size_t)pr * t.pstride, mE, mF, &A, &U, &V, &C, &aE, &eE, &cF, &dF);
-    const long long c0 = (pr * t.half) / t.per, c1 = (pr * t.half + t.half - 1) / t.per;
-    const Rotated<E> rot = Rotated<E>::map(P + (size_t)pr * t.pstride, b.n, mF);
-    const E* Zp = t.hess ? rot.Z : Z;
-    for (int q = tid; !t.hess && q < mF * mF; q += NT) {
-      const int i = q / mF, j = q - (q / mF) * mF;
-      E z = Ar::zero();
-      for (long long c = c0; c <= c1; ++c) {
-        const E* part = reinterpret_cast<const E*>(t.part) +
-                        ((size_t)c * t.maxspan + (size_t)(pr - (c * t.per) / t.half)) * t.lstride;
-        z = Ar::add(z, Ar::add(part[mF * mF + q], part[(size_t)j * mF + i]));   // Q + R^T
-      }
-      Z[q] = z;
-    }
-    for (int f = tid; f < 2 * mF + 1; f += NT) {
+    E* const P = reinterpret_cast<E*>(t.pbuf) + (size_t)pr * t.pstride;
+    Parent::map(P, mE, mF, &A, &U, &V, &C, &aE, &eE, &cF, &dF);
+    const Rotated<E> rot = Rotated<E>::map(P, n, mF);
+    const E *Z = rot.Z, *ss = rot.ss, *st = rot.st;
+    if (tid == 0) {
+      const long long c0 = (pr * t.half) / t.per, c1 = (pr * t.half + t.half - 1) / t.per;
       E v = Ar::zero();
-      for (long long c = c0; c <= c1; ++c) {
-        const E* part = reinterpret_cast<const E*>(t.part) +
-                        ((size_t)c * t.maxspan + (size_t)(pr - (c * t.per) / t.half)) * t.lstride;
-        v = Ar::add(v, part[(t.hess ? 1 : 2) * mF * mF + f]);
-      }
-      if (t.hess && f < 2 * mF) v = f < mF ? rot.ss[f] : rot.st[f - mF];
-      if (f < mF) ss[f] = v;
-      else if (f < 2 * mF) st[f - mF] = v;
-      else bbs[0] = v;
+      for (long long c = c0; c <= c1; ++c)
+        v = Ar::add(v, reinterpret_cast<const E*>(t.part)[((size_t)c * t.maxspan +
+                                                           (size_t)(pr - (c * t.per) / t.half) + 1) * t.lstride - 1]);
+      bbs[0] = v;
     }
-    __syncthreads();
-    gemm_staged<Ar>(X1, mE, Zp, mF, 1, U, 1, mF, mF, mE, mF, false, false, nb, Pc, Rx);
-    gemm_staged<Ar>(X2, mE, V, 1, mE, X1, mE, 1, mE, mE, mF, false, false, nb, Pc, Rx);
-    gemm_staged<Ar>(X3, mF, V, 1, mE, Zp, mF, 1, mE, mF, mF, false, false, nb, Pc, Rx);
+#pragma unroll 1
+    for (int g = 0; g < 3; ++g)                        // X1, X2, X3
+      gemm_staged<Ar>(g == 0 ? X1 + e0 : (g == 1 ? X2 + e0 : X3 + f0), g == 2 ? mF : mE, g == 0 ? Z : V,
+                      g == 0 ? mF : 1, g == 0 ? 1 : mE,
+                      g == 0 ? U + (size_t)e0 * mF : (g == 1 ? X1 + e0 : Z + f0), g == 0 ? 1 : (g == 1 ? mE : mF),
+                      g == 0 ? mF : 1, g == 0 ? mF : mE, g == 2 ? f1 - f0 : e1 - e0, mF, false, false, nb, Pc, Rx);
     for (int i = tid; i < mE; i += NT) {             // U sigma_s, V^T sigma_t
       E su = Ar::zero(), sv = Ar::zero();
       for (int k = 0; k < mF; ++k) {
@@ -664,23 +712,27 @@ __global__ void __launch_bounds__(kBtThreads) k_bwdt_assemble(BackwardArgs b, Bw
     __syncthreads();
     const E bsum = bbs[0];
     const E half = Ar::from(make_double2(0.5, 0.0));
-    for (long long q = tid; q < (long long)n * n; q += NT) {
-      const int jo = (int)(q / n), io = (int)(q - (q / n) * n);   // ST[jo][io] = S[io][jo]
-      const int a = t.pinv[io], c = t.pinv[jo];
-      E v;
-      if (a < mE && c < mE)
-        v = Ar::add(Ar::fma(bsum, Ar::add(Ar::mul(eE[a], aE[c]), A[(size_t)c * mE + a]),
-                            Ar::neg(Ar::add(Ar::mul(eE[a], uS[c]), Ar::mul(vT[a], aE[c])))),
-                    X2[(size_t)a * mE + c]);
-      else if (a < mE)
-        v = Ar::fms(Ar::mul(eE[a], ss[c - mE]), Ar::one(), X3[(size_t)a * mF + (c - mE)]);
-      else if (c < mE)
-        v = Ar::fms(Ar::mul(st[a - mE], aE[c]), Ar::one(), X1[(size_t)(a - mE) * mE + c]);
-      else
-        v = Zp[(size_t)(a - mE) * mF + (c - mE)];
-      ST[q] = Ar::fma(half, v, ST[q]);
+    for (int jo = warp; jo < n; jo += NT / 32) {
+      const int c = t.pinv[jo];
+      if (!mine(c)) continue;
+      for (int io = lane; io < n; io += 32) {        // ST[jo][io] = S[io][jo]
+        const int a = t.pinv[io];
+        E v;
+        if (a < mE && c < mE)
+          v = Ar::add(Ar::fma(bsum, Ar::add(Ar::mul(eE[a], aE[c]), A[(size_t)c * mE + a]),
+                              Ar::neg(Ar::add(Ar::mul(eE[a], uS[c]), Ar::mul(vT[a], aE[c])))),
+                      X2[(size_t)a * mE + c]);
+        else if (a < mE)
+          v = Ar::fms(Ar::mul(eE[a], ss[c - mE]), Ar::one(), X3[(size_t)a * mF + (c - mE)]);
+        else if (c < mE)
+          v = Ar::fms(Ar::mul(st[a - mE], aE[c]), Ar::one(), X1[(size_t)(a - mE) * mE + c]);
+        else
+          v = Z[(size_t)(a - mE) * mF + (c - mE)];
+        const size_t q = (size_t)jo * n + io;
+        ST[q] = Ar::fma(half, v, ST[q]);
+      }
     }
-    for (int io = tid; io < n; io += NT) {           // 1/2 (sum beta x + X sum beta y)
+    for (int io = tid; blockIdx.y == 0 && io < n; io += NT) {   // 1/2 (sum beta x + X sum beta y)
       const int h = n / 2, po = io < h ? io + h : io - h;
       const int a = t.pinv[io], ap = t.pinv[po];
       const E xs = a < mE ? Ar::fms(Ar::mul(bsum, aE[a]), Ar::one(), uS[a]) : ss[a - mE];
@@ -696,16 +748,24 @@ cudaError_t tree_wave(const BackwardArgs& b, const BwdTree& t0, cudaStream_t s) 
   BwdTree t = t0;
   const size_t base = backward_tree_smem_bytes(b.n, b.nb), with = base + (size_t)16 * b.nb * b.n;
   t.rn = with <= 226 * 1024 ? 1 : 0;
-  const size_t smem = t.rn ? with : base;
+  const size_t smem = t.rn ? with : base, ssmem = backward_tree_smem_bytes(b.n, kBwdSplitNb);
   cudaError_t err;
   if ((err = cudaFuncSetAttribute(k_bwdt_parent<Ar>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
           cudaSuccess ||
-      (err = cudaFuncSetAttribute(k_bwdt_assemble<Ar>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
+      (err = cudaFuncSetAttribute(k_bwdt_products<Ar>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem)) !=
+          cudaSuccess ||
+      (err = cudaFuncSetAttribute(k_bwdt_assemble<Ar>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem)) !=
           cudaSuccess)
     return err;
   const long long parents = t.p1 - t.p0;
   const long long gp = parents < b.nparts ? parents : b.nparts;
+  // splits: two CTAs an SM in one wave, at least eight columns each (one CTA a parent: 81 parents 0.7 ms more, 13
+  // parents of 24 + 24 rows 0.3 ms more of 2.0)
+  const int cols = (t.mE < t.mF ? t.mE : t.mF) / 8, fill = (int)(2 * b.nparts / t.nparts);
+  const int splits = cols < 1 || fill < 1 ? 1 : (cols < fill ? cols : fill);
   k_bwdt_parent<Ar><<<(unsigned)gp, kBtThreads, smem, s>>>(b, t);
+  if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  k_bwdt_products<Ar><<<dim3((unsigned)gp, (unsigned)splits), kBtThreads, ssmem, s>>>(b, t);
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
   const long long nleaves = parents * t.half;
   const long long gl = (nleaves + t.per - 1) / t.per;
@@ -718,8 +778,11 @@ cudaError_t tree_wave(const BackwardArgs& b, const BwdTree& t0, cudaStream_t s) 
       return err;
     k_bwdt_leaf<Ar><<<(unsigned)gl, kBwdLeafThreads, lsmem, s>>>(b, t);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    const int words = t.mF * t.mF + 2 * t.mF;
+    k_bwdt_sum<Ar><<<dim3((unsigned)parents, (unsigned)((words + kBtThreads - 1) / kBtThreads)), kBtThreads, 0, s>>>(b, t);
+    if ((err = cudaGetLastError()) != cudaSuccess) return err;
   }
-  k_bwdt_assemble<Ar><<<(unsigned)t.nparts, kBtThreads, smem, s>>>(b, t);
+  k_bwdt_assemble<Ar><<<dim3((unsigned)t.nparts, (unsigned)splits), kBtThreads, ssmem, s>>>(b, t);
   return cudaGetLastError();
 }
 

@@ -20,8 +20,8 @@ struct BwdTree {
   int goff[GBSBIN_MAX_L + 1];   // first permuted row of each group
   long long half;           // leaves per parent
   long long p0, p1;         // the parents of this wave
-  void* pbuf;               // (p1 - p0) x pstride: inv(M_EE), U, V, C, a_E, e_E, c_F, d_F
-  long long pstride;        // n^2 + 2 n, and for the Hessenberg leaves mF^2 + 4 mF: Z, sigma_s, sigma_t, and the
+  void* pbuf;               // (p1 - p0) x pstride: inv(M_EE), U, V, C, a_E, e_E, c_F, d_F, Z, ...
+  long long pstride;        // n^2 + 2 n, and mF^2 + 4 mF: Z, sigma_s, sigma_t, and for the Hessenberg leaves the
                             // reflectors' first entries and factors
   void* part;               // leaf partials: leaf CTAs x maxspan x lstride
   long long lstride;        // 2 mF^2 + 2 mF + 1: R, Q, sigma_s, sigma_t, beta sum; for the Hessenberg leaves
@@ -43,8 +43,8 @@ constexpr int kBwdLeafNb = 8;             // pivots per Gauss-Jordan step in the
 cudaError_t launch_backward_weights(const BackwardArgs& b, const double* dLdP, cudaStream_t s, const double2** beta);
 // The per-point kernel and the reduce over its CTAs (b.beta set).
 cudaError_t launch_backward_points(const BackwardArgs& b, cudaStream_t s);
-// One wave of the tree's reverse pass: the parents' products, the leaves' inverses and sums,
-// the parents' assembly into the partials (b.beta set).
+// One wave of the tree's reverse pass: the parents' inverses and products, the leaves' inverses and
+// sums, the parents' assembly into the partials (b.beta set).
 cudaError_t launch_backward_tree_wave(const BackwardArgs& b, const BwdTree& t, cudaStream_t s);
 // outS, outg from the first nparts partials.
 cudaError_t launch_backward_reduce(const BackwardArgs& b, int nparts, cudaStream_t s);

@@ -2,9 +2,9 @@
 // ArDF, gbsbin_df.cuh): the in-place inverse of a matrix in global (L2-resident) memory by
 // blocked Gauss-Jordan elimination without pivoting, and a staged product C (+)= +-A B with
 // strided operands.  Both stage nb-wide panels in shared memory (Pc: m x nb, Rx: nb x m,
-// Dg: nb x nb) and update the matrix in 4 x 4 register tiles.  Every thread of the CTA calls
-// them; they end with a barrier.  A thread's 4 x 4 tile takes four consecutive rows and four
-// columns tcols apart (tcols = ceil(columns / 4)), so that the threads of a warp read
+// Dg: nb x nb) and update the matrix in register tiles of 4 x 4, or entry by entry where those
+// would be few.  Every thread of the CTA calls them; they end with a barrier.  A thread's tile takes consecutive rows and
+// columns tcols apart (tcols = ceil(columns / side)), so that the threads of a warp read
 // consecutive 16-byte entries of the staged rows (no shared-memory bank conflicts) and of the
 // matrix (coalesced).
 #pragma once
@@ -15,8 +15,59 @@
 
 namespace gbsbin {
 
-constexpr int kGjTile = 4;
 constexpr int kGjMaxNb = 16;
+
+// The side of a thread's register tile for m x n outputs: 4 x 4 reuses its operands most, but a warp's instruction
+// costs the same for one lane as for 32, so the fewest turns of the busiest scheduler decide: 24 x 24 outputs are 36
+// tiles, two warps of 16 multiply-adds, or 18 warps of one (turns 16 and 5).
+__device__ __forceinline__ int tile_side(int m, int n, int threads) {
+  const int warps = threads / 32;
+  auto turns = [&](int t) {
+    const int w = (((m + t - 1) / t) * ((n + t - 1) / t) + 31) / 32;
+    const int rounds = (w + warps - 1) / warps, last = w - (rounds - 1) * warps;
+    return ((rounds - 1) * ((warps + 3) / 4) + (last + 3) / 4) * t * t;
+  };
+  return turns(1) * 4 <= turns(4) * 3 ? 1 : 4;
+}
+
+// The rest's rank-bs update of gj_invert, and its rows' and columns' new values.
+template <class Ar, int TS>
+__device__ void gj_update(typename Ar::E* W, int m, int ld, int nbm, int K, int bs, const typename Ar::E* Pc,
+                          const typename Ar::E* Rb) {
+  using E = typename Ar::E;
+  const int tid = threadIdx.x, NT = blockDim.x;
+  const int tcols = (m + TS - 1) / TS, ntiles = tcols * tcols;
+  for (int tt = tid; tt < ntiles; tt += NT) {
+    const int i0 = (tt / tcols) * TS, jt = tt - (tt / tcols) * tcols;
+    E acc[TS][TS];
+#pragma unroll
+    for (int r = 0; r < TS; ++r)
+#pragma unroll
+      for (int q = 0; q < TS; ++q) {
+        const int i = i0 + r, j = jt + q * tcols;
+        acc[r][q] = (i < m && j < m && (j < K || j >= K + bs)) ? W[(size_t)i * ld + j] : Ar::zero();
+      }
+    for (int c = 0; c < bs; ++c) {
+      E pv[TS], rv[TS];
+#pragma unroll
+      for (int r = 0; r < TS; ++r) pv[r] = i0 + r < m ? Pc[(i0 + r) * nbm + c] : Ar::zero();
+#pragma unroll
+      for (int q = 0; q < TS; ++q) rv[q] = jt + q * tcols < m ? Rb[c * m + jt + q * tcols] : Ar::zero();
+#pragma unroll
+      for (int r = 0; r < TS; ++r)
+#pragma unroll
+        for (int q = 0; q < TS; ++q) acc[r][q] = Ar::fms(acc[r][q], pv[r], rv[q]);
+    }
+#pragma unroll
+    for (int r = 0; r < TS; ++r)
+#pragma unroll
+      for (int q = 0; q < TS; ++q) {
+        const int i = i0 + r, j = jt + q * tcols;
+        if (i >= m || j >= m) continue;
+        W[(size_t)i * ld + j] = (i >= K && i < K + bs) ? Rb[(i - K) * m + j] : acc[r][q];
+      }
+  }
+}
 
 // W (m x m, row stride ld) <- W^{-1}.  Per step of nb pivots B = [K, K + bs): the bs x bs
 // block W_BB is inverted in shared memory (one element per thread per pivot: the scalar rule
@@ -29,7 +80,7 @@ __device__ void gj_invert(typename Ar::E* W, int m, int ld, int nbm, typename Ar
                           typename Ar::E* Dg, typename Ar::E* Rn) {
   using E = typename Ar::E;
   const int tid = threadIdx.x, NT = blockDim.x;
-  const int tcols = (m + kGjTile - 1) / kGjTile, ntiles = tcols * tcols;
+  const int tile = tile_side(m, m, NT);
   for (int K = 0; K < m; K += nbm) {
     const int bs = min(nbm, m - K);
     for (int t = tid; t < m * bs; t += NT) {
@@ -90,37 +141,47 @@ __device__ void gj_invert(typename Ar::E* W, int m, int ld, int nbm, typename Ar
       }
     }
     __syncthreads();
-    for (int tt = tid; tt < ntiles; tt += NT) {
-      const int i0 = (tt / tcols) * kGjTile, jt = tt - (tt / tcols) * tcols;
-      E acc[kGjTile][kGjTile];
-#pragma unroll
-      for (int r = 0; r < kGjTile; ++r)
-#pragma unroll
-        for (int q = 0; q < kGjTile; ++q) {
-          const int i = i0 + r, j = jt + q * tcols;
-          acc[r][q] = (i < m && j < m && (j < K || j >= K + bs)) ? W[(size_t)i * ld + j] : Ar::zero();
-        }
-      for (int c = 0; c < bs; ++c) {
-        E pv[kGjTile], rv[kGjTile];
-#pragma unroll
-        for (int r = 0; r < kGjTile; ++r) pv[r] = i0 + r < m ? Pc[(i0 + r) * nbm + c] : Ar::zero();
-#pragma unroll
-        for (int q = 0; q < kGjTile; ++q) rv[q] = jt + q * tcols < m ? Rb[c * m + jt + q * tcols] : Ar::zero();
-#pragma unroll
-        for (int r = 0; r < kGjTile; ++r)
-#pragma unroll
-          for (int q = 0; q < kGjTile; ++q) acc[r][q] = Ar::fms(acc[r][q], pv[r], rv[q]);
-      }
-#pragma unroll
-      for (int r = 0; r < kGjTile; ++r)
-#pragma unroll
-        for (int q = 0; q < kGjTile; ++q) {
-          const int i = i0 + r, j = jt + q * tcols;
-          if (i >= m || j >= m) continue;
-          W[(size_t)i * ld + j] = (i >= K && i < K + bs) ? Rb[(i - K) * m + j] : acc[r][q];
-        }
-    }
+    if (tile == 4) gj_update<Ar, 4>(W, m, ld, nbm, K, bs, Pc, Rb);
+    else gj_update<Ar, 1>(W, m, ld, nbm, K, bs, Pc, Rb);
     __syncthreads();
+  }
+}
+
+// One k-block of gemm_staged.
+template <class Ar, int TS>
+__device__ void gemm_block(typename Ar::E* C, int ldc, int m, int n, int bs, int kb, bool first,
+                           const typename Ar::E* As, const typename Ar::E* Bs) {
+  using E = typename Ar::E;
+  const int tid = threadIdx.x, NT = blockDim.x;
+  const int tcols = (n + TS - 1) / TS, ntiles = (m + TS - 1) / TS * tcols;
+  for (int tt = tid; tt < ntiles; tt += NT) {
+    const int i0 = (tt / tcols) * TS, jt = tt - (tt / tcols) * tcols;
+    E cv[TS][TS];
+#pragma unroll
+    for (int r = 0; r < TS; ++r)
+#pragma unroll
+      for (int q = 0; q < TS; ++q) {
+        const int i = i0 + r, j = jt + q * tcols;
+        cv[r][q] = (!first && i < m && j < n) ? C[(size_t)i * ldc + j] : Ar::zero();
+      }
+    for (int c = 0; c < bs; ++c) {
+      E av[TS], bv[TS];
+#pragma unroll
+      for (int r = 0; r < TS; ++r) av[r] = i0 + r < m ? As[(i0 + r) * kb + c] : Ar::zero();
+#pragma unroll
+      for (int q = 0; q < TS; ++q) bv[q] = jt + q * tcols < n ? Bs[c * n + jt + q * tcols] : Ar::zero();
+#pragma unroll
+      for (int r = 0; r < TS; ++r)
+#pragma unroll
+        for (int q = 0; q < TS; ++q) cv[r][q] = Ar::fma(av[r], bv[q], cv[r][q]);
+    }
+#pragma unroll
+    for (int r = 0; r < TS; ++r)
+#pragma unroll
+      for (int q = 0; q < TS; ++q) {
+        const int i = i0 + r, j = jt + q * tcols;
+        if (i < m && j < n) C[(size_t)i * ldc + j] = cv[r][q];
+      }
   }
 }
 
@@ -134,7 +195,7 @@ __device__ void gemm_staged(typename Ar::E* C, int ldc, const typename Ar::E* A,
                             bool neg, int kb, typename Ar::E* As, typename Ar::E* Bs) {
   using E = typename Ar::E;
   const int tid = threadIdx.x, NT = blockDim.x;
-  const int trows = (m + kGjTile - 1) / kGjTile, tcols = (n + kGjTile - 1) / kGjTile, ntiles = trows * tcols;
+  const int tile = tile_side(m, n, NT);
   if (k == 0 && !acc) {
     for (int t = tid; t < m * n; t += NT) C[(size_t)(t / n) * ldc + t % n] = Ar::zero();
     __syncthreads();
@@ -153,35 +214,8 @@ __device__ void gemm_staged(typename Ar::E* C, int ldc, const typename Ar::E* A,
     }
     __syncthreads();
     const bool first = K == 0 && !acc;
-    for (int tt = tid; tt < ntiles; tt += NT) {
-      const int i0 = (tt / tcols) * kGjTile, jt = tt - (tt / tcols) * tcols;
-      E cv[kGjTile][kGjTile];
-#pragma unroll
-      for (int r = 0; r < kGjTile; ++r)
-#pragma unroll
-        for (int q = 0; q < kGjTile; ++q) {
-          const int i = i0 + r, j = jt + q * tcols;
-          cv[r][q] = (!first && i < m && j < n) ? C[(size_t)i * ldc + j] : Ar::zero();
-        }
-      for (int c = 0; c < bs; ++c) {
-        E av[kGjTile], bv[kGjTile];
-#pragma unroll
-        for (int r = 0; r < kGjTile; ++r) av[r] = i0 + r < m ? As[(i0 + r) * kb + c] : Ar::zero();
-#pragma unroll
-        for (int q = 0; q < kGjTile; ++q) bv[q] = jt + q * tcols < n ? Bs[c * n + jt + q * tcols] : Ar::zero();
-#pragma unroll
-        for (int r = 0; r < kGjTile; ++r)
-#pragma unroll
-          for (int q = 0; q < kGjTile; ++q) cv[r][q] = Ar::fma(av[r], bv[q], cv[r][q]);
-      }
-#pragma unroll
-      for (int r = 0; r < kGjTile; ++r)
-#pragma unroll
-        for (int q = 0; q < kGjTile; ++q) {
-          const int i = i0 + r, j = jt + q * tcols;
-          if (i < m && j < n) C[(size_t)i * ldc + j] = cv[r][q];
-        }
-    }
+    if (tile == 4) gemm_block<Ar, 4>(C, ldc, m, n, bs, kb, first, As, Bs);
+    else gemm_block<Ar, 1>(C, ldc, m, n, bs, kb, first, As, Bs);
     __syncthreads();
   }
 }
