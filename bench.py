@@ -25,6 +25,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import math
 import os
 import statistics
 import subprocess
@@ -661,26 +662,23 @@ def _extra_distinguishable(gb, torch, steps):
 
 def _extra_fock(gb, torch, stream, flush, steps, world):
     """Fock inputs through a lossy circuit (App. C): 16 single photons in 32 ports, output
-    loss eta_i ~ U(0.4, 0.9), three detector groups, the whole table (N_l = 16): 2^15 input
-    nodes x 2601 output-group points.  FP64 kernel against FP32 pairs; the pipe operations
-    per (node, point) pair are counted from the kernels' inner loop (FP64: 2L additions and
-    4 multiply-adds per photon plus 2; FP32 pairs: 4L additions, 12 for the renormalisation
-    and 38 per product per photon, plus 16)."""
+    loss eta_i ~ U(0.4, 0.9), three detector groups, the whole table (N_l = 16), by the
+    convolution over sub-multisets of the input photons.  Plans of either arithmetic; the work
+    is its complex multiply-adds for single photons (layers r = 1 .. of both halves: C(N, r)
+    states x C(r + L, L) monomials x r inputs x L + 1 terms; then C(N, N/2) states x both
+    halves' monomials), against the rate of one in 64-bit integer sums of two digits (47
+    scheduler clocks a warp, measured in a register-tiled loop); three digits in FP64 plans'
+    sum over states count as two multiply-adds."""
     fp = synth.fock_config()
     nin = int(np.count_nonzero(fp.photons))
     L = fp.L
-    nodes = 1
-    for c in sorted(fp.photons[fp.photons > 0])[1:]:
-        nodes *= int(c) + 1
-    radix = [int(c) + 1 for c in fp.cutoff]
-    half = radix[-1] // 2 + 1
-    points = int(np.prod(radix[:-1])) * half
-    pairs = nodes * points
     N = int(fp.photons.sum())
-    ops = {"fp64": nin * 2 * L + 4 * N + 2, "df32": nin * (4 * L + 12) + 38 * N + 16}
-    peaks = {"fp64": (0.5 * 1.05e12, "FP64 pipe: measured 1.05 TFLOP/s dependent-FMA rate / 2"),
-             "df32": (152 * 128 * 2.07e9, "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz")}
-    res = {"nodes": nodes, "points": points, "occupied_inputs": nin}
+    halves = (N // 2, N - N // 2)
+    layers = sum(math.comb(N, r) * math.comb(r + L, L) * r * (L + 1) for h in halves for r in range(1, h + 1))
+    pair_sum = math.comb(N, halves[0]) * math.comb(halves[0] + L, L) * math.comb(halves[1] + L, L)
+    work = {"fp64": layers + 2 * pair_sum, "df32": layers + pair_sum}
+    peak = 152 * 4 * 32 * 2.07e9 / 47.1
+    res = {"photons": N, "occupied_inputs": nin}
     tables = {}
     for name, prec in (("fp64", 0), ("df32", 1)):
         with gb.FockPlan(fp, precision=prec, want_timing=True) as p:
@@ -690,11 +688,11 @@ def _extra_fock(gb, torch, stream, flush, steps, world):
             d = p.diagnostics(stream)
             tables[name] = t.cpu().numpy()
         kms = d["point_kernel_ms"]
-        achieved = pairs * ops[name] / (kms * 1e-3)
+        achieved = work[name] / (kms * 1e-3)
         res[name] = {"ms_per_table": ms / steps, "tables_per_s": 1e3 * steps / ms, "kernel_ms": kms,
-                     "pairs_per_s": pairs / (kms * 1e-3), "pipe_ops_per_pair": ops[name],
-                     "pipe_ops_per_s": achieved, "pipe_peak": peaks[name][0], "pipe_peak_source": peaks[name][1],
-                     "pipe_frac": achieved / peaks[name][0], "sum_P": d["sum_P"], "status": d["status"]}
+                     "multiply_adds": work[name], "multiply_adds_per_s": achieved, "pipe_peak": peak,
+                     "pipe_peak_source": "152 SMs x 4 schedulers x 32 lanes x 2070 MHz / 47.1 clocks (measured loop)",
+                     "pipe_frac": achieved / peak, "sum_P": d["sum_P"], "status": d["status"]}
     res["max_abs_diff_fp64_df32"] = float(np.abs(tables["fp64"] - tables["df32"]).max())
     P = tables["df32"]
     means = [float(np.dot(np.arange(P.shape[l]), P.sum(axis=tuple(m for m in range(L) if m != l)))) for l in range(L)]
@@ -706,14 +704,14 @@ def _extra_fock(gb, torch, stream, flush, steps, world):
 
 def _extra_e3(gb, torch, stream, flush, steps, world):
     """Total photon number of the largest uniform-loss setup of Sec. VIII: M = 256 (n = 512),
-    xi = 0.89, eta = 0.36, Haar U, one detector group, N_max = 170: the one-group Hessenberg
-    path in pairs of FP32 and in FP64 against the general FP64 LU kernel on the same table."""
+    xi = 0.89, eta = 0.36, Haar U, one detector group, N_max = 170: the one-group path
+    (spectral, FP64 for plans of either arithmetic) against the general FP64 LU kernel on the same table."""
     M, Nmax, xi, eta = 256, 170, 0.89, 0.36
     prob = synth.Problem(M, 1, np.full((M, 1), xi), np.sqrt(eta) * synth.haar_unitary(M, np.random.default_rng(61)),
                          np.zeros(M, np.int32), np.array([Nmax], np.int32))
     res = {}
     tables = {}
-    for name, precision, tile in (("hessenberg_fp32_pairs", 1, 0), ("hessenberg_fp64", 0, 0),
+    for name, precision, tile in (("one_group_fp32_plan", 1, 0), ("one_group_fp64_plan", 0, 0),
                                   ("general_lu_fp64", 0, 3)):
         t0 = time.perf_counter()
         with gb.Plan(prob, precision=precision, want_timing=True, tile_override=tile) as p:
@@ -725,8 +723,8 @@ def _extra_e3(gb, torch, stream, flush, steps, world):
             tables[name] = t.cpu().numpy()
             res[name] = {"ms_per_table": ms / steps, "point_kernel_ms": d["point_kernel_ms"],
                          "kernel": d["kernel_name"], "plan_create_s": plan_s, "status": st}
-    res["max_abs_diff"] = float(np.abs(tables["hessenberg_fp64"] - tables["general_lu_fp64"]).max())
-    res["max_abs_diff_pairs"] = float(np.abs(tables["hessenberg_fp32_pairs"] - tables["general_lu_fp64"]).max())
+    res["max_abs_diff"] = float(np.abs(tables["one_group_fp64_plan"] - tables["general_lu_fp64"]).max())
+    res["max_abs_diff_pairs"] = float(np.abs(tables["one_group_fp32_plan"] - tables["general_lu_fp64"]).max())
     return {"E3_M256_n512_L1_N170": res}
 
 
@@ -783,7 +781,10 @@ def backward_work(prob, d):
     per evaluated point (n^3), or along the tree (backward_path 2): per parent (combination of
     the first L - 1 axes' roots) the inverse of the leading groups' block (mE^3), U, V, C
     (2 mE^2 mF + mE mF^2) and the assembly's three products (mF^2 mE + mE^2 mF + mE mF^2), per
-    evaluated point the last group's mF^3 inverse."""
+    evaluated point the last group's mF^3 inverse - or, where the leaves go through the Hessenberg
+    form of their parent's block (32 <= mF <= 116 and eight leaves per SM), per parent the
+    reduction (10/3 mF^3) and the rotation back (2 mF^3), per evaluated point a triangular inverse
+    (mF^3 / 6), the elimination and the recurrence (1.5 mF^2)."""
     n = prob.n
     if d.get("backward_path") != 2:
         return (float(n) ** 3 * d["n_evaluated"], "k_backward_gj (blocked Gauss-Jordan, per point)",
@@ -793,8 +794,14 @@ def backward_work(prob, d):
     mE = float(n) - mF
     parents = float(np.prod(prob.radix[:-1]))
     per_parent = mE ** 3 + 2 * mE * mE * mF + mE * mF * mF + (mF * mF * mE + mE * mE * mF + mE * mF * mF)
+    leaves = parents * (prob.radix[-1] // 2 + 1)
+    if 32 <= mF <= 116 and leaves >= 8 * SMS * -(-int(parents) // SMS):
+        macs = parents * (per_parent + 16 / 3 * mF ** 3) + d["n_evaluated"] * (mF ** 3 / 6 + 1.5 * mF ** 2)
+        return (macs, "k_bwdt_parent, products, hess, hleaf, unrot, assemble (along the tree)",
+                "tree complex multiply-adds (parents' inverses, products, Hessenberg forms and rotations, leaves' "
+                "triangular inverses) x 8 flops")
     macs = parents * per_parent + d["n_evaluated"] * mF ** 3
-    return (macs, "k_bwdt_parent + k_bwdt_leaf + k_bwdt_assemble (along the tree)",
+    return (macs, "k_bwdt_parent, products, leaf, sum, assemble (along the tree)",
             "tree complex multiply-adds (parents' inverses and products, leaves' mF^3 inverses) x 8 flops")
 
 

@@ -190,7 +190,8 @@ typedef enum {
                                       shared memory, the other rows streamed through
                                       registers by many CTAs per child - and the last
                                       group's block I - w A_L of every leaf parent reduced
-                                      once to Hessenberg form (A_L = Q H Q^H), so each grid
+                                      once to Hessenberg form (A_L = Q H Q^H; a CTA per leaf
+                                      parent, a cluster of them where few), so each grid
                                       point is an O(m^2) elimination of H - conj(w) I;
                                       pairs of FP32; chosen automatically for standalone
                                       GBSBIN_FP32_REFINE plans where kernel 11 does not
@@ -605,8 +606,9 @@ int gbsbin_fock_plan_destroy(gbsbin_fock_plan* plan);
  * expectation, so that
  *   <v| rho(b) |u> = Pr(0) sqrt(u! v!) [w^b][x^u y^v] exp(xi^T M(w) xi / 2 + l(w)^T xi + e(w))
  *                  / sqrt(det(I - X D(w) A_DD)),
- * xi = (x, y) on the kept modes' two halves, M(w), l(w), e(w) from one solve with the
- * heralding and traced block I - X D(w) A_DD (w = 1 on traced modes), and the coefficient of
+ * xi = (x, y) on the kept modes' two halves, M(w), l(w), e(w) from the elimination of the
+ * heralding and traced rows (w = 1 on traced modes; the traced rows once per state on the
+ * host, the first group's by its spectral form, the others' per point), and the coefficient of
  * w^b by an inverse DFT over the grid w_l = exp(2 pi i k_l / R_l), R_l = oversample
  * (cutoff[l] + 1) (folded: photon numbers beyond R_l - 1 alias onto b, as for the binned
  * tables; oversample to unfold).  Pr(b) is the binned table of the heralding groups with
@@ -649,8 +651,8 @@ int gbsbin_herald_plan_create(const gbsbin_herald_problem* p, const gbsbin_optio
  * + 1)^(2k) entries. */
 long long gbsbin_herald_table_size(const gbsbin_herald_plan* plan);
 long long gbsbin_herald_prob_size(const gbsbin_herald_plan* plan);
-/* rho_out, prob_out device memory; asynchronous on `stream` (1 + L launches: the points, then the
- * inverse DFT one heralding axis at a time). */
+/* rho_out, prob_out device memory; asynchronous on `stream` (the first group's roots, the points,
+ * then the inverse DFT, its first two axes in one launch). */
 int gbsbin_herald_execute(gbsbin_herald_plan* plan, gbsbin_complex* rho_out, double* prob_out, void* stream);
 /* The same into host memory; synchronises `stream`. */
 int gbsbin_herald_execute_host(gbsbin_herald_plan* plan, gbsbin_complex* rho_out_host, double* prob_out_host,
