@@ -55,11 +55,6 @@ __device__ __forceinline__ long long shift_round(long long v, int s) {
   if (s >= 63) return 0;
   return (v + (1ll << (s - 1))) >> s;
 }
-template <int BITS>
-__device__ __forceinline__ void digits(long long v, int& hi, int& lo) {   // v = hi 2^BITS + lo, |lo| <= 2^(BITS-1)
-  lo = ((int)((unsigned)v << (32 - BITS))) >> (32 - BITS);
-  hi = (int)((v - lo) >> BITS);
-}
 __device__ __forceinline__ int bit_length(long long v) {                  // of |v|
   return 64 - __clzll(v < 0 ? -v : v);
 }

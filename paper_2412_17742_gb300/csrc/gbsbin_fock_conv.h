@@ -4,16 +4,33 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cmath>
+
 #include "gbsbin_internal.h"
 
 namespace gbsbin {
 
 #define GBSBIN_FC_NONE (-(1 << 28))       // exponent of an all-zero state or column
 
-// Coefficients in fixed point, round(b 2^kConvRowBits / 2^rowexp): components below 2^56, and a row's sum of
-// component magnitudes below 2^60, which keeps a layer's 64-bit sums (digits of 26 bits) below 2^62 and its
-// results four bits finer than a state's 52.
-constexpr int kConvRowBits = 56;
+// Coefficients in fixed point, round(b 2^kConvRowBits / 2^e) with e the row's exponent: components up to 2^55, so that
+// a high digit of 26 bits is at most 2^29 and the sum of two (the third factor of a complex product by three
+// real ones) at most 2^30, and a row's sum of component magnitudes below 2^59, which keeps a layer's 64-bit sums below
+// 2^62 and its results three bits finer than a state's 52.
+constexpr int kConvRowBits = 55;
+// e of a row whose largest component is `big` and whose component magnitudes add to `all`: big < 2^e, all < 16 x 2^e
+inline int conv_row_exponent(double big, double all) {
+  int e = 0, ea = 0;
+  std::frexp(big, &e);
+  std::frexp(all * 1.0001, &ea);
+  return std::max(e, ea - 4);
+}
+inline long long conv_fixed(double v, int e) { return std::llrint(std::ldexp(v, kConvRowBits - e)); }
+template <int BITS>
+__host__ __device__ __forceinline__ void digits(long long v, int& hi, int& lo) {   // v = hi 2^BITS + lo, |lo| <= 2^(BITS-1)
+  lo = ((int)((unsigned)v << (32 - BITS))) >> (32 - BITS);
+  hi = (int)((v - lo) >> BITS);
+}
 struct FockConvArgs {
   int nin, L, N, h[2];                    // occupied inputs, groups, photons, factors of each half
   int stride[GBSBIN_FOCK_MAX_IN];         // code of a state m: sum m_k stride[k]

@@ -142,15 +142,10 @@ int stage_transfer(gbsbin_fock_plan* P, const gbsbin_complex* Tin) {
           big = std::fmax(big, std::fmax(std::fabs(at(k, m).x), std::fabs(at(k, m).y)));
           all += std::fabs(at(k, m).x) + std::fabs(at(k, m).y);
         }
-      int e = 0, ea = 0;
-      std::frexp(big, &e);                      // big < 2^e, all < 16 x 2^e
-      std::frexp(all * 1.0001, &ea);
-      e = std::max(e, ea - 4);
+      const int e = conv_row_exponent(big, all);
       for (int k = 0; k < nin; ++k)
         for (int m = 0; m <= L; ++m)
-          B[((size_t)j * nin + k) * (L + 1) + m] =
-              make_longlong2(std::llrint(std::ldexp(at(k, m).x, kConvRowBits - e)),
-                             std::llrint(std::ldexp(at(k, m).y, kConvRowBits - e)));
+          B[((size_t)j * nin + k) * (L + 1) + m] = make_longlong2(conv_fixed(at(k, m).x, e), conv_fixed(at(k, m).y, e));
       P->cv.exponent += e * P->args.pw[j];
     }
   }
