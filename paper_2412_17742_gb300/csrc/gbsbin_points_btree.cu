@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(HC_THREADS) k_bt_hess_cluster(BTreeArgs a, int
                              : j == m ? src[(long long)i * D + m]
                                       : Ar::conj(src[(long long)m * D + i]);
   }
-  __syncthreads();
+  cluster_sync();                                    // the fill, and every CTA has started: the first stores into them follow
   for (int k = 0; k + 2 < m; ++k) {
     E* v = vbuf + (k & 1) * (m + 1);
     if (rank == k % C && warp == 0) {                // the reflector of column k, to every CTA
