@@ -198,21 +198,22 @@ int gbsbin_herald_plan_create(const gbsbin_herald_problem* p, const gbsbin_optio
   const int nb0 = t.nb[0], rest = nr - nb0;
   std::vector<cd> A00((size_t)nb0 * nb0), rlam(nb0), rB((size_t)nb0 * (rest + 1)), ru(nb0);
   {
-    std::vector<std::vector<cd>> col(rest + 2, std::vector<cd>(nb0));
-    std::vector<std::vector<cd>*> vecs;
+    const int X = rest + 2;                          // columns: A_0r, c_0, conj(u_0)
+    std::vector<double> xr((size_t)nb0 * X), xi((size_t)nb0 * X), ev;
     for (int i = 0; i < nb0; ++i) {
       for (int j = 0; j < nb0; ++j) A00[(size_t)i * nb0 + j] = A0[(size_t)i * nr + j];
-      for (int j = 0; j < rest; ++j) col[j][i] = A0[(size_t)i * nr + nb0 + j];
-      col[rest][i] = c0[i];
-      col[rest + 1][i] = std::conj(u0[i]);
+      for (int j = 0; j < X; ++j) {
+        const cd v = j < rest ? A0[(size_t)i * nr + nb0 + j] : j == rest ? c0[i] : std::conj(u0[i]);
+        xr[(size_t)i * X + j] = v.real();
+        xi[(size_t)i * X + j] = v.imag();
+      }
     }
-    for (auto& v : col) vecs.push_back(&v);
-    std::vector<double> ev;
-    if (!hermitian_spectrum(A00, nb0, ev, vecs)) return GBSBIN_ERR_NUMERIC;
+    if (!hermitian_spectrum(A00, nb0, ev, xr.data(), xi.data(), X)) return GBSBIN_ERR_NUMERIC;
     for (int k = 0; k < nb0; ++k) {
+      const double *yr = &xr[(size_t)k * X], *yi = &xi[(size_t)k * X];
       rlam[k] = ev[k];
-      for (int j = 0; j <= rest; ++j) rB[(size_t)k * (rest + 1) + j] = col[j][k];
-      ru[k] = std::conj(col[rest + 1][k]);
+      for (int j = 0; j <= rest; ++j) rB[(size_t)k * (rest + 1) + j] = cd(yr[j], yi[j]);
+      ru[k] = cd(yr[rest + 1], -yi[rest + 1]);
     }
   }
   struct {

@@ -54,7 +54,7 @@ struct gbsbin_plan {
   TreeArgs tree{};
   bool tree_g = false;                // undisplaced tree plan, or a one-group plan that is no shard: the
                                       // point kernel writes G, the DFT skips a stage
-  double tree_logq0 = 0.0;            // Re log q(1) from the host LU (diagnostics)
+  double tree_logq0 = 0.0;            // Re log q(1) from the host's elimination or spectrum (diagnostics)
   unsigned char* d_tree = nullptr;
   // large-matrix tree plans (kernels 13, 14): the same row order, depth-0 augmented matrix in
   // d_state, the other depths, sub-step scratch and Hessenberg leaves in d_tree
@@ -515,9 +515,9 @@ inline bool is_tree(int kernel) { return kernel == GBSBIN_KERNEL_TREE_DF32 || ke
 inline bool is_hess(int kernel) { return kernel == GBSBIN_KERNEL_HESS_FP64 || kernel == GBSBIN_KERNEL_HESS_DF32; }
 inline bool is_btree(int kernel) { return kernel == GBSBIN_KERNEL_BTREE_DF32 || kernel == GBSBIN_KERNEL_BTREE_FP64; }
 // 16-byte slots of a tree plan's depth-0 region in the state block
-size_t tree_region_slots(int n, int kernel) {
-  // permuted XA, X gamma, gamma, path record; the first group's spectral form (at most n rows of n + 2 + 1)
-  if (is_tree(kernel)) return (size_t)n * n + 2 * (size_t)n + 3 + (size_t)n * (n + 3);
+size_t tree_region_slots(int n, int kernel, const TreeArgs& t) {
+  // permuted XA, X gamma, gamma, path record; the first group's spectral form, if taken (a row per eigenvalue)
+  if (is_tree(kernel)) return (size_t)n * n + 2 * (size_t)n + 3 + (t.spectral ? (size_t)t.nb[0] * (n - t.nb[0] + 3) : 0);
   if (is_btree(kernel)) return (size_t)(n + 1) * (n + 1) + 2;    // augmented matrix, path record
   if (is_hess(kernel)) return (size_t)n + ((size_t)n + 1) / 2;    // g products, eigenvalues
   return 0;
@@ -567,7 +567,7 @@ int upload_state(gbsbin_plan* P, cudaStream_t stream) {
   const int n = P->n;
   const bool tree = is_tree(P->kernel) || is_btree(P->kernel) || is_hess(P->kernel);
   const bool per_point = !tree || P->opt.want_backward;   // the reverse pass reads -XA, gamma, X gamma
-  Stage s = stage_layout(n, tree_region_slots(n, P->kernel));
+  Stage s = stage_layout(n, tree_region_slots(n, P->kernel, P->tree));
   // the copy that last read this staging buffer (two uploads back) must have finished
   const int sb = P->stage_next;
   P->stage_next ^= 1;
@@ -648,73 +648,72 @@ int upload_state(gbsbin_plan* P, cudaStream_t stream) {
     path[0] = slot(cd(1.0, 0.0));                       // pivot product
     path[1] = make_float4(0.f, 0.f, 3.0e38f, 0.f);    // argument sum, power of two, min Re pivot
     path[2] = slot(cd(0.0, 0.0));                       // exponent sum
-    {                                                   // the first group's spectral form
+    if (P->tree.spectral) {                             // the first group's spectral form
       const int nb = P->tree.nb[0], rest = n - nb;
       float4 *lam = path + 3, *B = lam + nb, *ru = B + (size_t)nb * (rest + 1);
       std::vector<cd> A00((size_t)nb * nb);
       for (int i = 0; i < nb; ++i)
         for (int j = 0; j < nb; ++j) A00[(size_t)i * nb + j] = P->XA[(size_t)pm[i] * n + pm[j]];
-      std::vector<std::vector<cd>> col(rest + 2, std::vector<cd>(nb));
-      std::vector<std::vector<cd>*> vecs;
-      for (int i = 0; i < nb; ++i) {
-        for (int j = 0; j < rest; ++j) col[j][i] = P->XA[(size_t)pm[i] * n + pm[nb + j]];
-        col[rest][i] = P->Xgamma[pm[i]];
-        col[rest + 1][i] = std::conj(P->gamma[pm[i]]);
-      }
-      for (auto& v : col) vecs.push_back(&v);
-      std::vector<double> ev;
-      if (!hermitian_spectrum(A00, nb, ev, vecs)) return GBSBIN_ERR_NUMERIC;
+      // columns: A_0r, c_0, conj(u_0)
+      const int X = rest + 2;
+      std::vector<double> xr((size_t)nb * X), xi((size_t)nb * X), ev;
+      for (int i = 0; i < nb; ++i)
+        for (int j = 0; j < X; ++j) {
+          const cd v = j < rest ? P->XA[(size_t)pm[i] * n + pm[nb + j]]
+                                : j == rest ? P->Xgamma[pm[i]] : std::conj(P->gamma[pm[i]]);
+          xr[(size_t)i * X + j] = v.real();
+          xi[(size_t)i * X + j] = v.imag();
+        }
+      if (!hermitian_spectrum(A00, nb, ev, xr.data(), xi.data(), X)) return GBSBIN_ERR_NUMERIC;
       for (int k = 0; k < nb; ++k) {
+        const double *yr = &xr[(size_t)k * X], *yi = &xi[(size_t)k * X];
         lam[k] = slot(cd(ev[k], 0.0));
-        for (int j = 0; j <= rest; ++j) B[(size_t)k * (rest + 1) + j] = slot(col[j][k]);
-        ru[k] = slot(std::conj(col[rest + 1][k]));
+        for (int j = 0; j <= rest; ++j) B[(size_t)k * (rest + 1) + j] = slot(cd(yr[j], yi[j]));
+        ru[k] = slot(cd(yr[rest + 1], -yi[rest + 1]));
       }
     }
-    // the w = 1 point on the host: unpivoted LU of I - XA in the tree's row order, its pivot
-    // product p0 2^e0, argument and winding (each pivot has Re > 0)
+    // the w = 1 point on the host: the pivots of I - XA in the tree's row order, their product p0 2^e0, its argument and
+    // winding.  I - XA is Hermitian positive definite: real pivots, and the upper triangle is enough, row i's
+    // multiplier being conj(row k's entry i) / pivot (both triangles took 14 us of set_state's 85 at n = 42)
     P->tree_g = !P->has_gamma;
     if (P->tree_g) {
-      // split real / imaginary rows; each pivot's reciprocal once, rows updated contiguously
+      // split real / imaginary rows, updated contiguously
       std::vector<double> kr((size_t)n * n), ki((size_t)n * n);
       for (int i = 0; i < n; ++i)
-        for (int j = 0; j < n; ++j) {
+        for (int j = i; j < n; ++j) {
           const cd v = (i == j ? 1.0 : 0.0) - P->XA[(size_t)pm[i] * n + pm[j]];
           kr[(size_t)i * n + j] = v.real();
           ki[(size_t)i * n + j] = v.imag();
         }
-      cd prod = 1.0;
+      double prod = 1.0, args = 0.0;
       int e0 = 0;
-      double args = 0.0;
       for (int k = 0; k < n; ++k) {
-        const cd piv(kr[(size_t)k * n + k], ki[(size_t)k * n + k]);
-        prod *= piv;
-        int ex;
-        std::frexp(std::max(std::fabs(prod.real()), std::fabs(prod.imag())), &ex);
-        prod = cd(std::ldexp(prod.real(), -ex), std::ldexp(prod.imag(), -ex));
-        e0 += ex;
-        args += std::atan2(piv.imag(), piv.real());
-        const double d = std::norm(piv), pr = piv.real() / d, pi = -piv.imag() / d;   // 1 / piv
         const double* rk = &kr[(size_t)k * n];
         const double* ik = &ki[(size_t)k * n];
+        int ex;
+        prod = std::frexp(prod * rk[k], &ex);
+        e0 += ex;
+        args += std::atan2(0.0, rk[k]);
+        const double rp = 1.0 / rk[k];
         for (int i = k + 1; i < n; ++i) {
           double* ri = &kr[(size_t)i * n];
           double* ii = &ki[(size_t)i * n];
-          const double lr = ri[k] * pr - ii[k] * pi, lim = ri[k] * pi + ii[k] * pr;
-          for (int j = k + 1; j < n; ++j) {
+          const double lr = rk[i] * rp, lim = -ik[i] * rp;
+          for (int j = i; j < n; ++j) {
             ri[j] -= lr * rk[j] - lim * ik[j];
             ii[j] -= lr * ik[j] + lim * rk[j];
           }
         }
       }
       const double TWO_PI = 6.283185307179586476925286766559;
-      const double arg0 = std::atan2(prod.imag(), prod.real());
-      P->tree.p0re = prod.real();
-      P->tree.p0im = prod.imag();
-      P->tree.p0df = split4(prod);
+      const double arg0 = std::atan2(0.0, prod);
+      P->tree.p0re = prod;
+      P->tree.p0im = 0.0;
+      P->tree.p0df = split4(cd(prod, 0.0));
       P->tree.p0arg = (float)arg0;
       P->tree.e0 = (float)e0;
       P->tree.m0 = (float)std::nearbyint((args - arg0) / TWO_PI);
-      P->tree_logq0 = -0.5 * (std::log(std::abs(prod)) + e0 * 0.693147180559945309417232121458);
+      P->tree_logq0 = -0.5 * (std::log(std::fabs(prod)) + e0 * 0.693147180559945309417232121458);
     }
   }
   // the device block has the staging layout: one copy (of the tree region alone for trees
@@ -730,19 +729,23 @@ int upload_state(gbsbin_plan* P, cudaStream_t stream) {
 // products g_i = (Q^T gamma)_i (Q^H X gamma)_i of the displacement term, and q at w = 1 from them.
 int spectral_state(gbsbin_plan* P, double2* gq, double* lam) {
   const int n = P->n;
-  std::vector<cd> ga(n), c(P->Xgamma);
-  for (int i = 0; i < n; ++i) ga[i] = std::conj(P->gamma[i]);     // Q^T g = conj(Q^H conj(g))
-  std::vector<std::vector<cd>*> vecs;
-  if (P->has_gamma) vecs = {&ga, &c};
-  std::vector<double> ev;
-  if (!hermitian_spectrum(P->XA, n, ev, vecs)) return GBSBIN_ERR_NUMERIC;
+  const int m = P->has_gamma ? 2 : 0;                              // columns: conj(gamma), X gamma
+  std::vector<double> xr((size_t)n * m), xi((size_t)n * m), ev;
+  for (int i = 0; i < n && m; ++i) {                               // Q^T g = conj(Q^H conj(g))
+    xr[2 * (size_t)i] = P->gamma[i].real();
+    xi[2 * (size_t)i] = -P->gamma[i].imag();
+    xr[2 * (size_t)i + 1] = P->Xgamma[i].real();
+    xi[2 * (size_t)i + 1] = P->Xgamma[i].imag();
+  }
+  if (!hermitian_spectrum(P->XA, n, ev, xr.data(), xi.data(), m)) return GBSBIN_ERR_NUMERIC;
   P->lam_min = *std::min_element(ev.begin(), ev.end());
   P->lam_max = *std::max_element(ev.begin(), ev.end());
   double p0 = 1.0;
   int e0 = 0;
   cd ex0 = 0.0;
   for (int i = 0; i < n; ++i) {
-    const cd g = P->has_gamma ? std::conj(ga[i]) * c[i] : cd(0.0);
+    const size_t q = 2 * (size_t)i;
+    const cd g = m ? cd(xr[q], -xi[q]) * cd(xr[q + 1], xi[q + 1]) : cd(0.0);
     gq[i] = make_double2(g.real(), g.imag());
     lam[i] = ev[i];
     int ex;
@@ -1024,9 +1027,11 @@ void tree_pointers(gbsbin_plan* P, const Stage& sl) {
   t.c[0] = A0 + (size_t)n * n;
   t.u[0] = t.c[0] + n;
   t.path[0] = t.u[0] + n;
-  t.rlam = t.path[0] + 3;
-  t.rB = t.rlam + t.nb[0];
-  t.ru = t.rB + (size_t)t.nb[0] * (n - t.nb[0] + 1);
+  if (t.spectral) {
+    t.rlam = t.path[0] + 3;
+    t.rB = t.rlam + t.nb[0];
+    t.ru = t.rB + (size_t)t.nb[0] * (n - t.nb[0] + 1);
+  }
   float4* q = (float4*)P->d_tree;
   long long nodes = 1;
   for (int l = 0; l + 1 < P->L; ++l) {
@@ -1309,7 +1314,9 @@ static int plan_create_impl(const gbsbin_problem* p, const gbsbin_options* o, gb
     return GBSBIN_ERR_CUDA;
   }
   const size_t nn = (size_t)n * n;
-  Stage sl = stage_layout(n, tree_region_slots(n, P->kernel));
+  if (is_tree(P->kernel))
+    P->tree.spectral = tree_spectral_suits(P->tree, g, P->num_sms, P->kernel == GBSBIN_KERNEL_TREE_FP64) ? 1 : 0;
+  Stage sl = stage_layout(n, tree_region_slots(n, P->kernel, P->tree));
   (void)nn;
   if ((st = dalloc(&P->d_state, sl.total)) || (st = dalloc(&P->d_label, n)) || (st = dalloc(&P->d_logq, g.n_eval)) ||
       (st = dalloc(&P->d_minpiv, g.n_eval)) || (st = dalloc(&P->d_bufA, g.n_full)) ||

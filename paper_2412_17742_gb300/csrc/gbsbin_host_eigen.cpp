@@ -1,7 +1,8 @@
-// Spectral form of a Hermitian matrix for the one-group plans, FP64 on the host: Householder
-// reduction to tridiagonal form, then the implicitly shifted QR iteration with Wilkinson's shift
-// (Golub and Van Loan, Matrix Computations, 8.3), the unitary applied to given vectors instead of
-// being formed: O(n^3) for the reduction, O(n^2) for the rest.
+// Spectral form of a Hermitian matrix for the one-group plans, the small trees' first group and heralded states,
+// FP64 on the host: Householder reduction to tridiagonal form, then the implicitly shifted QR iteration with
+// Wilkinson's shift (Golub and Van Loan, Matrix Computations, 8.3), the unitary applied to given vectors instead
+// of being formed: O(n^3) for the reduction, O(n^2) per vector for the rest.  The vectors are the columns of
+// an n x m array held by rows, so that a reflector's products and a plane rotation run along contiguous entries.
 #include <algorithm>
 #include <cmath>
 #include <limits>
@@ -31,11 +32,33 @@ inline void row_dot(const double* ar, const double* ai, const double* vr, const 
   *im = (m[0] + m[1]) + (m[2] + m[3]);
 }
 
+// y += a x of split rows (complex a)
+inline void axpy(double ar, double ai, const double* __restrict__ xr, const double* __restrict__ xi,
+                 double* __restrict__ yr, double* __restrict__ yi, int m) {
+  for (int j = 0; j < m; ++j) {
+    yr[j] += ar * xr[j] - ai * xi[j];
+    yi[j] += ar * xi[j] + ai * xr[j];
+  }
+}
+
+// |(x, z)|: the square root of the sum of squares where neither overflows nor loses digits
+inline double norm2d(double x, double z) {
+  const double q = x * x + z * z;
+  return q > 1e-280 && q < 1e280 ? std::sqrt(q) : std::hypot(x, z);
+}
+
 // Eigenvalues of the real symmetric tridiagonal (d, e) into d; every plane rotation is also applied
-// to the entries of the vectors (which become Z^T vec).  False if a block does not converge.
-bool tridiagonal_qr(std::vector<double>& d, std::vector<double>& e, const std::vector<std::vector<cd>*>& vecs) {
+// to the vectors' rows (which become Z^T X).  False if a block does not converge.
+bool tridiagonal_qr(std::vector<double>& d, std::vector<double>& e, double* xr, double* xi, int m) {
   const int n = (int)d.size();
   const double eps = std::numeric_limits<double>::epsilon();
+  auto rotate = [m](double c, double s, double* __restrict__ p, double* __restrict__ q) {
+    for (int j = 0; j < m; ++j) {
+      const double a = p[j], b = q[j];
+      p[j] = c * a + s * b;
+      q[j] = c * b - s * a;
+    }
+  };
   int hi = n - 1;
   long long budget = 60LL * n + 60;
   while (hi > 0) {
@@ -57,7 +80,7 @@ bool tridiagonal_qr(std::vector<double>& d, std::vector<double>& e, const std::v
     const double mu = d[hi] - b * (b / (g + std::copysign(std::hypot(g, b), g)));
     double x = d[lo] - mu, z = e[lo];
     for (int k = lo; k < hi; ++k) {             // chase the bulge down the block
-      const double h = std::hypot(x, z);
+      const double h = norm2d(x, z);
       const double c = h > 0.0 ? x / h : 1.0, s = h > 0.0 ? z / h : 0.0;
       if (k > lo) e[k - 1] = h;
       const double t = s * (d[k + 1] - d[k]) + 2.0 * c * e[k];   // d_k' + d_{k+1}' = d_k + d_{k+1}
@@ -69,11 +92,8 @@ bool tridiagonal_qr(std::vector<double>& d, std::vector<double>& e, const std::v
         z = s * e[k + 1];
         e[k + 1] *= c;
       }
-      for (std::vector<cd>* v : vecs) {
-        const cd p = (*v)[k], q = (*v)[k + 1];
-        (*v)[k] = c * p + s * q;
-        (*v)[k + 1] = c * q - s * p;
-      }
+      rotate(c, s, xr + (size_t)k * m, xr + (size_t)(k + 1) * m);
+      rotate(c, s, xi + (size_t)k * m, xi + (size_t)(k + 1) * m);
     }
   }
   return true;
@@ -85,8 +105,7 @@ bool tridiagonal_qr(std::vector<double>& d, std::vector<double>& e, const std::v
 // the next column known (its column updated first, O(n)), every remaining row takes the last
 // column's rank-2 update and its product with the next reflector together; rows dealt cyclically
 // to the host threads, each row's sums in a fixed order.
-bool hermitian_spectrum(const std::vector<cd>& A, int n, std::vector<double>& lam,
-                        const std::vector<std::vector<cd>*>& vecs) {
+bool hermitian_spectrum(const std::vector<cd>& A, int n, std::vector<double>& lam, double* xr, double* xi, int m) {
   std::vector<double> re((size_t)n * n), im((size_t)n * n);
   for (size_t q = 0; q < re.size(); ++q) {
     re[q] = A[q].real();
@@ -94,6 +113,7 @@ bool hermitian_spectrum(const std::vector<cd>& A, int n, std::vector<double>& la
   }
   const int nt = host_threads();
   std::vector<double> vr(n, 0.0), vi(n, 0.0), wr(n, 0.0), wi(n, 0.0), pr(n), pi(n), nvr(n, 0.0), nvi(n, 0.0);
+  std::vector<double> tr(m), ti(m);             // v^H X
   std::vector<cd> sub(n, cd(0.0));              // sub[k] = entry (k + 1, k) of the tridiagonal form
   bool pending = false;                         // (v, w): the rank-2 update not yet applied
   for (int k = 0; k + 1 < n; ++k) {
@@ -110,8 +130,8 @@ bool hermitian_spectrum(const std::vector<cd>& A, int n, std::vector<double>& la
     const cd x0(rk[k + 1], -ik[k + 1]);
     const double ax0 = std::abs(x0), nrm = std::sqrt(nrm2 + std::norm(x0));
     double beta = 0.0;
-    std::fill(nvr.begin(), nvr.end(), 0.0);
-    std::fill(nvi.begin(), nvi.end(), 0.0);
+    std::fill(nvr.begin() + k, nvr.end(), 0.0);
+    std::fill(nvi.begin() + k, nvi.end(), 0.0);
     if (nrm2 > 0.0) {                           // v = x - alpha e, alpha = -e^{i arg x0} |x|
       const cd alpha = (ax0 > 0.0 ? -x0 / ax0 : cd(-1.0, 0.0)) * nrm;
       for (int j = k + 2; j < n; ++j) {
@@ -125,20 +145,23 @@ bool hermitian_spectrum(const std::vector<cd>& A, int n, std::vector<double>& la
     } else {
       sub[k] = x0;
     }
-    parallel_run(n - k >= 160 ? nt : 1, [&](int t, int nth) {   // the rows below: update, then p = A v
+    auto rows = [&](int t, int nth) {           // the rows below: update, then p = A v
       for (int i = k + 1 + t; i < n; i += nth) {
         double* ri = &re[(size_t)i * n];
         double* ii = &im[(size_t)i * n];
         if (pending) {
           const double a = vr[i], b = vi[i], c = wr[i], d = wi[i];
+          const double *w0 = wr.data(), *w1 = wi.data(), *v0 = vr.data(), *v1 = vi.data();
           for (int j = k + 1; j < n; ++j) {
-            ri[j] -= a * wr[j] + b * wi[j] + c * vr[j] + d * vi[j];
-            ii[j] -= b * wr[j] - a * wi[j] + d * vr[j] - c * vi[j];
+            ri[j] -= a * w0[j] + b * w1[j] + c * v0[j] + d * v1[j];
+            ii[j] -= b * w0[j] - a * w1[j] + d * v0[j] - c * v1[j];
           }
         }
         if (beta != 0.0) row_dot(ri, ii, nvr.data(), nvi.data(), k + 1, n, &pr[i], &pi[i]);
       }
-    });
+    };
+    if (n - k >= 160) parallel_run(nt, rows);
+    else rows(0, 1);
     pending = beta != 0.0;
     if (!pending) continue;
     // w = beta p - (beta^2 (v^H p) / 2) v;  A <- A - v w^H - w v^H
@@ -149,14 +172,16 @@ bool hermitian_spectrum(const std::vector<cd>& A, int n, std::vector<double>& la
       wr[j] = beta * pr[j] - half * nvr[j];
       wi[j] = beta * pi[j] - half * nvi[j];
     }
-    for (int j = 0; j <= k; ++j) wr[j] = wi[j] = 0.0;
+    wr[k] = wi[k] = 0.0;
     vr.swap(nvr);
     vi.swap(nvi);
-    for (std::vector<cd>* x : vecs) {           // x <- (I - beta v v^H) x
-      cd t = 0.0;
-      for (int i = k + 1; i < n; ++i) t += cd(vr[i], -vi[i]) * (*x)[i];
-      t *= beta;
-      for (int i = k + 1; i < n; ++i) (*x)[i] -= t * cd(vr[i], vi[i]);
+    if (m > 0) {                                // X <- (I - beta v v^H) X
+      std::fill(tr.begin(), tr.end(), 0.0);
+      std::fill(ti.begin(), ti.end(), 0.0);
+      for (int i = k + 1; i < n; ++i)
+        axpy(vr[i], -vi[i], xr + (size_t)i * m, xi + (size_t)i * m, tr.data(), ti.data(), m);
+      for (int i = k + 1; i < n; ++i)
+        axpy(-beta * vr[i], -beta * vi[i], tr.data(), ti.data(), xr + (size_t)i * m, xi + (size_t)i * m, m);
     }
   }
   if (pending) {                                // the last diagonal entry
@@ -169,14 +194,20 @@ bool hermitian_spectrum(const std::vector<cd>& A, int n, std::vector<double>& la
   cd f = 1.0;
   for (int k = 0; k < n; ++k) {
     lam[k] = re[(size_t)k * n + k];
-    for (std::vector<cd>* x : vecs) (*x)[k] *= std::conj(f);
+    double* row_r = xr + (size_t)k * m;
+    double* row_i = xi + (size_t)k * m;
+    for (int j = 0; j < m; ++j) {               // times conj(f)
+      const double a = row_r[j], b = row_i[j];
+      row_r[j] = f.real() * a + f.imag() * b;
+      row_i[j] = f.real() * b - f.imag() * a;
+    }
     if (k + 1 < n) {
-      const double m = std::abs(sub[k]);
-      if (m > 0.0) f *= sub[k] / m;
-      e[k] = m;
+      const double g = std::abs(sub[k]);
+      if (g > 0.0) f *= sub[k] / g;
+      e[k] = g;
     }
   }
-  return tridiagonal_qr(lam, e, vecs);
+  return tridiagonal_qr(lam, e, xr, xi, m);
 }
 
 }  // namespace gbsbin

@@ -25,10 +25,10 @@ std::complex<double> host_logq1(const std::vector<std::complex<double>>& XA,
                                 const std::vector<std::complex<double>>& gamma,
                                 const std::vector<std::complex<double>>& Xgamma, int n, double* minpiv);
 
-// Eigenvalues (ascending order not implied) of the Hermitian n x n matrix A = Q Lambda Q^H, and each
-// vector in vecs replaced by Q^H vec; false if the iteration does not converge.
-bool hermitian_spectrum(const std::vector<std::complex<double>>& A, int n, std::vector<double>& lam,
-                        const std::vector<std::vector<std::complex<double>>*>& vecs);
+// Eigenvalues (ascending order not implied) of the Hermitian n x n matrix A = Q Lambda Q^H, and the n x m array X (split
+// real and imaginary parts, row-major: its columns are vectors) replaced by Q^H X; false if the iteration does not converge.
+bool hermitian_spectrum(const std::vector<std::complex<double>>& A, int n, std::vector<double>& lam, double* xr,
+                        double* xi, int m);
 
 // Host threads the state algebra uses: the hardware concurrency capped at 16, or the
 // environment variable GBSBIN_HOST_THREADS.

@@ -163,8 +163,9 @@ struct TreeArgs {
   double2* gout;
   int gout_df;              // nonzero (pairs plans whose DFT runs in pairs): G stored as a pair
                             // of FP32 (float4) in the 16-byte slots of gout
-  // the first group's block of XA is Hermitian, A_00 = Q Lambda Q^H (host, once per state): the eigenvalues
-  // (real parts of nb[0] slots), Q^H [A_0r, c_0] (nb[0] x (m[1] + 1)) and u_0^T Q (nb[0])
+  // spectral (tree_spectral_suits): the first group's block of XA is Hermitian, A_00 = Q Lambda Q^H (host, once per
+  // state): the eigenvalues (real parts of nb[0] slots), Q^H [A_0r, c_0] (nb[0] x (m[1] + 1)) and u_0^T Q (nb[0])
+  int spectral;
   const float4 *rlam, *rB, *ru;
   double p0re, p0im;
   float4 p0df;              // p0 as a pair of FP32
@@ -230,6 +231,8 @@ cudaError_t launch_points_btree(const BTreeArgs& a, const BTreeStep* steps, int 
                                 cudaStream_t s, int* launches);
 size_t tree_level_smem_bytes(int nb, int m);
 int tree_leaf_threads(int n);   // lanes per leaf (0: no kernel for a last group of n rows)
+// Whether a plan's first level starts from the spectral form (nb and m of its levels set).
+bool tree_spectral_suits(const TreeArgs& a, const GridDesc& g, int num_sms, bool fp64);
 // The first level alone (FP64), from the spectral form: depth 1's matrices, vectors and path records.
 cudaError_t launch_tree_root_fp64(const TreeArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_points_tree(const TreeArgs& a, bool fp64, int num_sms, cudaStream_t s, int* launches);

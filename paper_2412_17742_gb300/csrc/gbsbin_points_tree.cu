@@ -301,9 +301,16 @@ cudaError_t launch_root(const TreeArgs& a, int num_sms, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Level 0 from the spectral form; then levels whose children would fill fewer than half the SMs take the next level into the
-// same launch (a level's fixed costs - launch, fill from the parent, copy-out, path record -
-// are then paid once), up to SPAN_MAX groups and while a level remains before the leaves.
+// Children of the launch that starts at level l (nodes of them above it): levels whose children would fill fewer than
+// half the SMs take the next level into the same launch (a level's fixed costs - launch, fill from the parent, copy-out,
+// path record - are then paid once), up to SPAN_MAX groups and while a level remains before the leaves.
+long long level_children(const GridDesc& g, int l, long long nodes, int num_sms, int* span) {
+  long long children = nodes * g.radix[l];
+  for (*span = 1; *span < SPAN_MAX && l + *span + 1 < g.L && 2 * children < num_sms; ++*span) children *= g.radix[l + *span];
+  return children;
+}
+
+// Level 0 from the spectral form or, where the plan does without it, by elimination like the other levels.
 template <class Ar>
 cudaError_t launch_tree(const TreeArgs& a, int num_sms, cudaStream_t s, int* launches) {
   cudaError_t err = cudaSuccess;
@@ -313,21 +320,17 @@ cudaError_t launch_tree(const TreeArgs& a, int num_sms, cudaStream_t s, int* lau
   // n = 32, four groups of 8 rows, pairs: 51.4 us with both levels in one elimination, 54.4 with the first
   // level apart, 50.1 formed within the second's launch.  n = 42, three of 14 rows, FP64: 110.7 with both in
   // one elimination, 90.3 apart.
-  long long nodes = a.grid.radix[0];
+  long long nodes = a.spectral ? a.grid.radix[0] : 1;
   const double fill = (double)a.nb[0] * a.m[1] * a.m[1] * (std::is_same<Ar, ArDF>::value ? 0.5 : 2.0);
-  bool fused = a.grid.L > 2 && fill < 6000.0;
-  if (!fused) {
+  bool fused = a.spectral && a.grid.L > 2 && fill < 6000.0;
+  if (a.spectral && !fused) {
     if ((err = launch_root<Ar>(a, num_sms, s)) != cudaSuccess) return err;
     ++*launches;
   }
-  for (int l = 1; l + 1 < a.grid.L;) {
-    long long children = nodes * a.grid.radix[l];
+  for (int l = a.spectral ? 1 : 0; l + 1 < a.grid.L;) {
     int span = 1, nb = a.nb[l];
-    while (span < SPAN_MAX && l + span + 1 < a.grid.L && 2 * children < num_sms) {
-      children *= a.grid.radix[l + span];
-      nb += a.nb[l + span];
-      ++span;
-    }
+    const long long children = level_children(a.grid, l, nodes, num_sms, &span);
+    for (int g = 1; g < span; ++g) nb += a.nb[l + g];
     const size_t smem = tree_level_smem_bytes(nb, a.m[l]) + (fused ? sizeof(float4) * ((size_t)a.nb[0] * (a.m[1] + 2) + 3) : 0);
     auto kernel = fused ? k_tree_level<Ar, true> : k_tree_level<Ar, false>;
     if (smem > 48 * 1024) {
@@ -358,6 +361,22 @@ cudaError_t launch_tree(const TreeArgs& a, int num_sms, cudaStream_t s, int* lau
 }
 
 }  // namespace
+
+// The spectral form saves the first level's pivots in every child of the launch that would hold them, and costs the
+// host an eigendecomposition per state, so it is taken where a state with one table gains or loses no more than 3 us (then
+// further tables of the state decide).  Both in us, fitted to measured calls: the host 1.5 + 1e-3 nb^3 + 1.9e-3 nb^2 x
+// (columns) (8 rows and 26 columns 5, 14 and 30 16, 32 and 18 64, 48 and 18 187); a pivot saved, per turn of the
+// SMs, grows with the matrix, 0.04 m - 0.35 in FP64 and 0.0105 m in pairs (first groups of 14 of 42 rows 18 and 6 us, 32 of
+// 48 49 and 18, 48 of 64 107 and 41).  set_state and one table at 48 of 64 rows in pairs: 332 us by elimination, 442
+// from the spectral form; at 14 of 42 rows in FP64 194 and 184.
+bool tree_spectral_suits(const TreeArgs& a, const GridDesc& g, int num_sms, bool fp64) {
+  int span = 1;
+  const double turns = (double)((level_children(g, 0, 1, num_sms, &span) + num_sms - 1) / num_sms);
+  const double nb = a.nb[0], m = a.m[0], cols = m - nb + 2.0;
+  const double host = 1.5 + 1e-3 * nb * nb * nb + 1.9e-3 * nb * nb * cols;
+  const double gain = nb * turns * std::max(0.0, fp64 ? 0.04 * m - 0.35 : 0.0105 * m);
+  return host <= gain + 3.0;
+}
 
 size_t tree_level_smem_bytes(int nb, int m) { return sizeof(float4) * ((size_t)(m + 1) * (m + 1) + nb + 2 * (m + 1)); }
 
