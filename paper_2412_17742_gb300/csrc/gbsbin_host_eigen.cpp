@@ -64,7 +64,7 @@ bool tridiagonal_qr(std::vector<double>& d, std::vector<double>& e, double* xr, 
   while (hi > 0) {
     int lo = hi;                                // the unreduced block ending at hi
     while (lo > 0) {
-      if (std::fabs(e[lo - 1]) <= eps * (std::fabs(d[lo - 1]) + std::fabs(d[lo])) || std::fabs(e[lo - 1]) < 1e-300) {
+      if (std::fabs(e[lo - 1]) <= eps * (std::fabs(d[lo - 1]) + std::fabs(d[lo])) || std::fabs(e[lo - 1]) < std::numeric_limits<double>::min()) {
         e[lo - 1] = 0.0;
         break;
       }
@@ -125,25 +125,32 @@ bool hermitian_spectrum(const std::vector<cd>& A, int n, std::vector<double>& la
         rk[j] -= vr[k] * wr[j] + vi[k] * wi[j] + wr[k] * vr[j] + wi[k] * vi[j];
         ik[j] -= vi[k] * wr[j] - vr[k] * wi[j] + wi[k] * vr[j] - wr[k] * vi[j];
       }
+    // the column scaled by a power of two (exact) that brings its largest component to [1/2, 1): the squares of
+    // small entries and the square of beta leave FP64's range from magnitudes of 1e-77 on
+    double big = 0.0;
+    for (int j = k + 1; j < n; ++j) big = std::max(big, std::max(std::fabs(rk[j]), std::fabs(ik[j])));
+    int ex = 0;
+    std::frexp(big, &ex);
+    ex = std::max(ex, -1000);
+    const double up = std::ldexp(1.0, -ex);
     double nrm2 = 0.0;
-    for (int j = k + 2; j < n; ++j) nrm2 += rk[j] * rk[j] + ik[j] * ik[j];
-    const cd x0(rk[k + 1], -ik[k + 1]);
+    for (int j = k + 2; j < n; ++j) {
+      nvr[j] = rk[j] * up;
+      nvi[j] = -ik[j] * up;
+      nrm2 += nvr[j] * nvr[j] + nvi[j] * nvi[j];
+    }
+    nvr[k] = nvi[k] = 0.0;
+    const cd x0(rk[k + 1] * up, -ik[k + 1] * up);
     const double ax0 = std::abs(x0), nrm = std::sqrt(nrm2 + std::norm(x0));
     double beta = 0.0;
-    std::fill(nvr.begin() + k, nvr.end(), 0.0);
-    std::fill(nvi.begin() + k, nvi.end(), 0.0);
     if (nrm2 > 0.0) {                           // v = x - alpha e, alpha = -e^{i arg x0} |x|
       const cd alpha = (ax0 > 0.0 ? -x0 / ax0 : cd(-1.0, 0.0)) * nrm;
-      for (int j = k + 2; j < n; ++j) {
-        nvr[j] = rk[j];
-        nvi[j] = -ik[j];
-      }
       nvr[k + 1] = x0.real() - alpha.real();
       nvi[k + 1] = x0.imag() - alpha.imag();
       beta = 2.0 / (nrm2 + nvr[k + 1] * nvr[k + 1] + nvi[k + 1] * nvi[k + 1]);
-      sub[k] = alpha;
+      sub[k] = std::ldexp(1.0, ex) * alpha;
     } else {
-      sub[k] = x0;
+      sub[k] = cd(rk[k + 1], -ik[k + 1]);
     }
     auto rows = [&](int t, int nth) {           // the rows below: update, then p = A v
       for (int i = k + 1 + t; i < n; i += nth) {
