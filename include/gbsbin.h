@@ -225,6 +225,10 @@ int gbsbin_plan_create(const gbsbin_problem* p, const gbsbin_options* o, gbsbin_
  * pinned buffers used in turn, so the call waits only for the upload two calls back, not
  * for the stream: the host algebra of the next state overlaps the device work of the
  * current one.  Same errors as plan_create; ERR_ARG if a shape differs.
+ * The kernels read the state from device memory, so a caller's own CUDA graph of gbsbin_execute gives the
+ * new state's table when it is replayed after this call, provided both states are displaced or neither is.
+ * Two plans take log q(1) as a launch argument and have to be captured again: those of kernels 11 and 12
+ * without displacement, and shards of kernels 13 and 14.
  */
 int gbsbin_plan_set_state(gbsbin_plan* plan, const gbsbin_problem* p, void* stream);
 
@@ -577,7 +581,8 @@ typedef struct {
 typedef struct gbsbin_fock_plan gbsbin_fock_plan;
 int gbsbin_fock_plan_create(const gbsbin_fock_problem* p, const gbsbin_options* o, gbsbin_fock_plan** out);
 /* New transfer matrix T (same M, photons, grouping, cutoffs): host FP64 algebra, one
- * upload enqueued on `stream`.  ERR_ARG / ERR_NONPHYSICAL as for plan creation. */
+ * upload enqueued on `stream`.  ERR_ARG / ERR_NONPHYSICAL as for plan creation.  A caller's own CUDA graph of
+ * gbsbin_fock_execute replayed after it gives the new circuit's table. */
 int gbsbin_fock_plan_set_transfer(gbsbin_fock_plan* plan, const gbsbin_complex* T, void* stream);
 long long gbsbin_fock_plan_table_size(const gbsbin_fock_plan* plan);
 /* Input nodes of the whole problem, prod over the occupied inputs but the held one of

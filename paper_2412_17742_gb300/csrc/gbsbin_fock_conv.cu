@@ -320,6 +320,7 @@ __global__ void __launch_bounds__(kSumThreads, ND == 3 ? 4 : 5) k_conv_sum(FockC
     __syncthreads();                             // the buffer is refilled by the next iteration's stage
   }
   double2* out = a.parts + (size_t)blockIdx.z * a.n1 * a.n2;
+  const int exponent = *a.exponent;
   constexpr int B = ND == 3 ? 20 : 25;
   const double k = 1.0 / (double)(1 << B);
 #pragma unroll
@@ -337,7 +338,7 @@ __global__ void __launch_bounds__(kSumThreads, ND == 3 ? 4 : 5) k_conv_sum(FockC
           re = fma(re, k, (double)(m1s[i][j][w] - m2s[i][j][w]));
           im = fma(im, k, (double)(m3s[i][j][w] - m1s[i][j][w] - m2s[i][j][w]));
         }
-        const int s = ca + cb + a.exponent - 2 * B;
+        const int s = ca + cb + exponent - 2 * B;
         v = make_double2(ldexp(re, s), ldexp(im, s));
       }
       out[(size_t)ea * a.n2 + eb] = v;

@@ -51,7 +51,8 @@ struct FockConvArgs {
   int states, first, n1, n2;              // last layer of the first half: states, its codes in order; monomials
                                           // of each half
   int chunk, nchunks;                     // states per contraction CTA
-  int exponent;                           // sum of the rows' exponents
+  const int* exponent;                    // sum of the rows' exponents (of the circuit, so in device memory: a captured
+                                          // launch then serves later circuits)
   double2* parts;                         // nchunks x n1 x n2
   const int* pair_first;                  // table entry -> its pairs (a n2 + b) in pair_list
   const int* pair_list;

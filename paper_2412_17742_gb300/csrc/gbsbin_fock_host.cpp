@@ -133,7 +133,7 @@ int stage_transfer(gbsbin_fock_plan* P, const gbsbin_complex* Tin) {
       }
   if (P->conv) {   // the same by rows in fixed point, each row scaled by a power of two
     longlong2* B = reinterpret_cast<longlong2*>(P->h_stage + P->coef_count * (sizeof(double2) + sizeof(float4)));
-    P->cv.exponent = 0;
+    int exponent = 0;
     for (int j = 0; j < nin; ++j) {
       auto at = [&](int k, int m) { return coef[((size_t)m * nin + k) * nin + j]; };
       double big = 0.0, all = 0.0;
@@ -146,8 +146,9 @@ int stage_transfer(gbsbin_fock_plan* P, const gbsbin_complex* Tin) {
       for (int k = 0; k < nin; ++k)
         for (int m = 0; m <= L; ++m)
           B[((size_t)j * nin + k) * (L + 1) + m] = make_longlong2(conv_fixed(at(k, m).x, e), conv_fixed(at(k, m).y, e));
-      P->cv.exponent += e * P->args.pw[j];
+      exponent += e * P->args.pw[j];
     }
+    std::memcpy(B + P->coef_count, &exponent, sizeof(exponent));
   }
   return GBSBIN_OK;
 }
@@ -377,6 +378,7 @@ int conv_setup(gbsbin_fock_plan* P) {
   for (int h = 0; h < 2; ++h) c.F3[h] = c.nd == 3 ? (int2*)(d + o_F3[h]) : nullptr;
   c.parts = (double2*)(d + o_parts);
   c.B = (const longlong2*)(P->d_state + P->coef_count * (sizeof(double2) + sizeof(float4)));
+  c.exponent = (const int*)(c.B + P->coef_count);
   return GBSBIN_OK;
 }
 
@@ -533,7 +535,8 @@ int gbsbin_fock_plan_create(const gbsbin_fock_problem* p, const gbsbin_options* 
   a.xr = (int)xr;
   P->coef_count = (size_t)(L + 1) * a.nin * a.nin;
   P->conv = opt.shard_end == 0 && opt.shard_begin == 0 && opt.tile_override == 0 && conv_layout(P);
-  P->state_bytes = P->coef_count * (sizeof(double2) + sizeof(float4) + (P->conv ? sizeof(longlong2) : 0));
+  P->state_bytes = P->coef_count * (sizeof(double2) + sizeof(float4));
+  if (P->conv) P->state_bytes += (P->coef_count + 1) * sizeof(longlong2);   // and the exponent
   int st = GBSBIN_OK;
   if ((st = dalloc(&P->d_state, P->state_bytes)) || (st = dalloc(&P->d_xtw, (size_t)xoff)) ||
       (st = dalloc(&P->d_xtw_df, (size_t)xoff)) || (st = dalloc(&P->d_zr, (size_t)a.rsum)) ||

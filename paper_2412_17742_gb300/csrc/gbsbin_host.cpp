@@ -45,9 +45,7 @@ struct gbsbin_plan {
   // one-group plans: the spectral form of XA (device arrays in d_state) and what G = q / q(1) needs
   const double* d_lam = nullptr;
   const double2* d_gq = nullptr;
-  double lam_min = 0.0, lam_max = 0.0, sp_rt0 = 1.0;
-  int sp_e0 = 0;
-  double2 sp_ex0 = make_double2(0.0, 0.0);
+  const double* d_sp = nullptr;
   // tree plans: rows ordered by group (tree_perm[new] = old), depth-0 arrays in d_state,
   // depths 1 .. L-1 in d_tree
   std::vector<int> tree_perm;
@@ -519,7 +517,7 @@ size_t tree_region_slots(int n, int kernel, const TreeArgs& t) {
   // permuted XA, X gamma, gamma, path record; the first group's spectral form, if taken (a row per eigenvalue)
   if (is_tree(kernel)) return (size_t)n * n + 2 * (size_t)n + 3 + (t.spectral ? (size_t)t.nb[0] * (n - t.nb[0] + 3) : 0);
   if (is_btree(kernel)) return (size_t)(n + 1) * (n + 1) + 2;    // augmented matrix, path record
-  if (is_hess(kernel)) return (size_t)n + ((size_t)n + 1) / 2;    // g products, eigenvalues
+  if (is_hess(kernel)) return (size_t)n + ((size_t)n + 1) / 2 + 3;   // g products, eigenvalues, the values at w = 1
   return 0;
 }
 
@@ -738,8 +736,6 @@ int spectral_state(gbsbin_plan* P, double2* gq, double* lam) {
     xi[2 * (size_t)i + 1] = P->Xgamma[i].imag();
   }
   if (!hermitian_spectrum(P->XA, n, ev, xr.data(), xi.data(), m)) return GBSBIN_ERR_NUMERIC;
-  P->lam_min = *std::min_element(ev.begin(), ev.end());
-  P->lam_max = *std::max_element(ev.begin(), ev.end());
   double p0 = 1.0;
   int e0 = 0;
   cd ex0 = 0.0;
@@ -753,9 +749,13 @@ int spectral_state(gbsbin_plan* P, double2* gq, double* lam) {
     e0 += ex;
     ex0 += g / (1.0 - ev[i]);
   }
-  P->sp_rt0 = std::sqrt(p0);
-  P->sp_e0 = e0;
-  P->sp_ex0 = make_double2(ex0.real(), ex0.imag());
+  double* sp = lam + 2 * (((size_t)n + 1) / 2);
+  sp[0] = std::sqrt(p0);
+  sp[1] = e0;
+  sp[2] = ex0.real();
+  sp[3] = ex0.imag();
+  sp[4] = *std::min_element(ev.begin(), ev.end());
+  sp[5] = *std::max_element(ev.begin(), ev.end());
   P->tree_g = P->grid.e_lo == 0 && P->grid.e_hi == P->grid.n_full;
   P->tree_logq0 = 0.5 * ex0.real() - 0.5 * (std::log(p0) + e0 * 0.693147180559945309417232121458);
   return GBSBIN_OK;
@@ -1376,6 +1376,7 @@ static int plan_create_impl(const gbsbin_problem* p, const gbsbin_options* o, gb
   if (is_hess(P->kernel)) {
     P->d_gq = (const double2*)(P->d_state + sl.off_tree);
     P->d_lam = (const double*)(P->d_gq + n);
+    P->d_sp = P->d_lam + 2 * (((size_t)n + 1) / 2);
   }
   if (alloc_gws && (P->kernel == GBSBIN_KERNEL_GMEM_FP64 || P->kernel == GBSBIN_KERNEL_GMEM_FP32R ||
                     is_blk(P->kernel))) {
@@ -1536,12 +1537,8 @@ static PointArgs make_point_args(gbsbin_plan* P) {
   a.ldfin = P->d_ldfin;
   a.lam = P->d_lam;
   a.gq = P->d_gq;
-  a.lam_min = P->lam_min;
-  a.lam_max = P->lam_max;
+  a.sp = P->d_sp;
   a.gout = is_hess(P->kernel) && P->tree_g ? P->d_bufA : nullptr;
-  a.sp_e0 = P->sp_e0;
-  a.sp_rt0 = P->sp_rt0;
-  a.sp_ex0 = P->sp_ex0;
   return a;
 }
 

@@ -56,11 +56,11 @@ struct PointArgs {
   const double2* tw;        // twiddles exp(-2 pi i m / radix[l]), m < radix[l], axis after axis
   const double* lam;        // one-group plans: the eigenvalues of XA (n) and, per eigenvector, the
   const double2* gq;        // product (Q^T gamma)_i (Q^H X gamma)_i (else nullptr)
-  double lam_min, lam_max;  // the smallest and the largest eigenvalue
-  double2* gout;            // one-group plans: G = q / q(1) per point (nullptr: not wanted), from
-  int sp_e0;                // prod (1 - lambda_i) = sp_rt0^2 2^sp_e0 and the displacement term at w = 1
-  double sp_rt0;
-  double2 sp_ex0;
+  // of the state, read by the kernel like its matrices (a captured launch then serves later states): [0] sp_rt0, [1]
+  // sp_e0, [2] [3] the displacement term at w = 1, where prod (1 - lambda_i) = sp_rt0^2 2^sp_e0; [4] [5] the
+  // smallest and the largest eigenvalue
+  const double* sp;
+  double2* gout;            // one-group plans: G = q / q(1) per point (nullptr: not wanted)
   GridDesc grid;
   double2* logq;            // n_eval outputs: log q at each evaluated point
   double* minpiv;           // n_eval outputs: min_i Re u_ii

@@ -49,6 +49,8 @@ __device__ __forceinline__ void join(Partial& p, const Partial& q, bool disp) {
 template <int TP, bool DISP>
 __device__ __forceinline__ void spectral_point(const PointArgs& a, long long e, int r, bool live) {
   const double2 w = grid_root(a.tw, a.grid, 0, live ? point_digit(e, a.grid, 0) : 0);
+  const double rt0 = a.sp[0], e0 = a.sp[1], lam_min = a.sp[4], lam_max = a.sp[5];   // (the loads pass under the product)
+  const double2 ex0 = make_double2(a.sp[2], a.sp[3]);
   Partial p{ArF64::one(), ArF64::zero(), 0, 0.f};
   int since = 0;
   for (int i = r; i < a.n; i += TP) {
@@ -84,7 +86,7 @@ __device__ __forceinline__ void spectral_point(const PointArgs& a, long long e, 
   const int e2 = p.e2;
   const double2 ex = DISP ? ArF64::mul(p.ex, w) : ArF64::zero();   // gamma^T K^{-1} w X gamma
   // every factor's real part is 1 - Re(w) lambda_i: the smallest at an end of the spectrum
-  const double mn = 1.0 - fmax(w.x * a.lam_min, w.x * a.lam_max);
+  const double mn = 1.0 - fmax(w.x * lam_min, w.x * lam_max);
   const bool ok = isfinite(prod.x) && isfinite(prod.y) && isfinite(ex.x) && isfinite(ex.y);
   const double LN2 = 0.693147180559945309417232121458;
   double* f = a.ldfin + 6 * e;                  // log q unfinished, as finish_logq takes it
@@ -101,15 +103,15 @@ __device__ __forceinline__ void spectral_point(const PointArgs& a, long long e, 
   const float a0 = atan2f((float)prod.y, (float)prod.x);
   const int m = (int)rintf((p.args - a0) * 0.159154943f);
   double2 g = inv_sqrt(prod);
-  const int de = a.sp_e0 - e2, h = de >> 1;     // 2^(de / 2) = 2^h sqrt(2)^(de odd)
-  double sc = a.sp_rt0 * ((de & 1) ? 1.41421356237309504880 : 1.0);
+  const int de = (int)e0 - e2, h = de >> 1;     // 2^(de / 2) = 2^h sqrt(2)^(de odd)
+  double sc = rt0 * ((de & 1) ? 1.41421356237309504880 : 1.0);
   if (m & 1) sc = -sc;
   sc = ldexp(sc, h);
   g = make_double2(g.x * sc, g.y * sc);
   if (DISP) {
     double sn, cs;
-    sincos(0.5 * (ex.y - a.sp_ex0.y), &sn, &cs);
-    const double m2 = exp(0.5 * (ex.x - a.sp_ex0.x));
+    sincos(0.5 * (ex.y - ex0.y), &sn, &cs);
+    const double m2 = exp(0.5 * (ex.x - ex0.x));
     g = ArF64::mul(g, make_double2(m2 * cs, m2 * sn));
   }
   a.gout[e] = g;
