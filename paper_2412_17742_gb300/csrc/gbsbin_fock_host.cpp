@@ -377,8 +377,6 @@ int conv_setup(gbsbin_fock_plan* P) {
     }
   for (int h = 0; h < 2; ++h) c.F3[h] = c.nd == 3 ? (int2*)(d + o_F3[h]) : nullptr;
   c.parts = (double2*)(d + o_parts);
-  c.B = (const longlong2*)(P->d_state + P->coef_count * (sizeof(double2) + sizeof(float4)));
-  c.exponent = (const int*)(c.B + P->coef_count);
   return GBSBIN_OK;
 }
 
@@ -535,15 +533,22 @@ int gbsbin_fock_plan_create(const gbsbin_fock_problem* p, const gbsbin_options* 
   a.xr = (int)xr;
   P->coef_count = (size_t)(L + 1) * a.nin * a.nin;
   P->conv = opt.shard_end == 0 && opt.shard_begin == 0 && opt.tile_override == 0 && conv_layout(P);
+  int st = GBSBIN_OK;
+  // the convolution's tables and states; where the device has no room for them the walk serves the plan
+  if (P->conv && (st = conv_setup(P)) == GBSBIN_ERR_NOMEM) {
+    P->conv = false;
+    st = GBSBIN_OK;
+  }
   P->state_bytes = P->coef_count * (sizeof(double2) + sizeof(float4));
   if (P->conv) P->state_bytes += (P->coef_count + 1) * sizeof(longlong2);   // and the exponent
-  int st = GBSBIN_OK;
-  if ((st = dalloc(&P->d_state, P->state_bytes)) || (st = dalloc(&P->d_xtw, (size_t)xoff)) ||
-      (st = dalloc(&P->d_xtw_df, (size_t)xoff)) || (st = dalloc(&P->d_zr, (size_t)a.rsum)) ||
-      (st = dalloc(&P->d_zr_df, (size_t)a.rsum)) || (st = dalloc(&P->d_tw, (size_t)a.rsum)) ||
-      (st = dalloc(&P->d_parts, P->conv ? 0 : (size_t)xr * g.n_full)) || (st = dalloc(&P->d_bufA, (size_t)g.n_full)) ||
-      (st = dalloc(&P->d_bufB, (size_t)g.n_full)) || (st = dalloc(&P->d_diag, GBSBIN_DIAG_DOUBLES)) ||
-      (st = dalloc(&P->d_bar, 4)) || (st = dalloc(&P->d_table, (size_t)P->table_size))) {
+  if (!st)
+    (st = dalloc(&P->d_state, P->state_bytes)) || (st = dalloc(&P->d_xtw, (size_t)xoff)) ||
+        (st = dalloc(&P->d_xtw_df, (size_t)xoff)) || (st = dalloc(&P->d_zr, (size_t)a.rsum)) ||
+        (st = dalloc(&P->d_zr_df, (size_t)a.rsum)) || (st = dalloc(&P->d_tw, (size_t)a.rsum)) ||
+        (st = dalloc(&P->d_parts, P->conv ? 0 : (size_t)xr * g.n_full)) || (st = dalloc(&P->d_bufA, (size_t)g.n_full)) ||
+        (st = dalloc(&P->d_bufB, (size_t)g.n_full)) || (st = dalloc(&P->d_diag, GBSBIN_DIAG_DOUBLES)) ||
+        (st = dalloc(&P->d_bar, 4)) || (st = dalloc(&P->d_table, (size_t)P->table_size));
+  if (st) {
     free_all(P);
     delete P;
     return st;
@@ -569,10 +574,9 @@ int gbsbin_fock_plan_create(const gbsbin_fock_problem* p, const gbsbin_options* 
   a.zr = P->d_zr;
   a.zr_df = P->d_zr_df;
   a.parts = P->d_parts;
-  if (P->conv && (st = conv_setup(P))) {
-    free_all(P);
-    delete P;
-    return st;
+  if (P->conv) {
+    P->cv.B = (const longlong2*)(P->d_state + P->coef_count * (sizeof(double2) + sizeof(float4)));
+    P->cv.exponent = (const int*)(P->cv.B + P->coef_count);
   }
   // roots from exact integer indices
   const double TWO_PI = 6.283185307179586476925286766559;
