@@ -237,35 +237,31 @@ int conv_setup(gbsbin_fock_plan* P) {
     codes *= c.radix[j];
   }
   c.full = codes - 1;
-  // codes by layer: sum of digits by an odometer, then a counting sort
-  std::vector<int> sum(codes), rank(codes, 0), order(P->layers.back().first + P->layers.back().states);
+  // codes by layer: the sum of digits, digit after digit over all lower codes, then a counting sort
+  std::vector<int> rank(codes, 0), order(P->layers.back().first + P->layers.back().states);
   {
-    std::vector<int> next(hi + 1, 0), dig(nin, 0);
+    std::vector<int> sum(codes, 0), next(hi + 1, 0);
+    for (int j = 0; j < nin; ++j)
+      for (int v = 1; v < c.radix[j]; ++v)
+        for (int q = 0; q < c.stride[j]; ++q) sum[(size_t)v * c.stride[j] + q] = sum[q] + v;
     for (int r = 1; r <= hi; ++r) next[r] = P->layers[r - 1].first;
     const std::vector<int> begin(next);
-    int s = 0;
     for (int q = 0; q < codes; ++q) {
-      if (s <= hi) {
-        rank[q] = next[s] - begin[s];
-        order[next[s]++] = q;
-      }
-      for (int j = 0; j < nin; ++j) {
-        if (++dig[j] < c.radix[j]) {
-          ++s;
-          break;
-        }
-        s -= dig[j] - 1;
-        dig[j] = 0;
-      }
+      const int r = sum[q];
+      if (r > hi) continue;
+      rank[q] = next[r] - begin[r];
+      order[next[r]++] = q;
     }
   }
-  // monomials by degree (a layer's are a prefix), and each without one of its variables
-  std::vector<std::vector<int>> mono;
+  // monomials by degree (a layer's are a prefix), L exponents each, and each without one of its variables
+  std::vector<int> mono((size_t)c.n2 * L);
+  int nm = 0;
   for (int d = 0; d <= hi; ++d) {
     std::vector<int> e(L, 0);
     e[L - 1] = d;
-    for (;;) {                                  // compositions of d, the last variable running down
-      mono.push_back(e);
+    for (;; ++nm) {                             // compositions of d, the last variable running down
+      if (nm == c.n2) return GBSBIN_ERR_UNSUPPORTED;
+      std::copy(e.begin(), e.end(), mono.begin() + (size_t)nm * L);
       int l = L - 1;
       while (l > 0 && e[l] == 0) --l;
       if (l == 0) break;
@@ -274,38 +270,50 @@ int conv_setup(gbsbin_fock_plan* P) {
       e[l - 1] += 1;
       e[L - 1] = v - 1;
     }
+    ++nm;
   }
-  if ((int)mono.size() != c.n2) return GBSBIN_ERR_UNSUPPORTED;
+  if (nm != c.n2) return GBSBIN_ERR_UNSUPPORTED;
   c.ndown = c.n2;
   std::vector<int> down((size_t)(L + 1) * c.n2, -1);
   {
-    std::vector<std::pair<std::vector<int>, int>> idx;
-    for (int e = 0; e < c.n2; ++e) idx.emplace_back(mono[e], e);
-    std::sort(idx.begin(), idx.end());
+    std::vector<long long> unit(L, 1);          // a monomial's key: its exponents as digits of base hi + 1
+    for (int l = L - 2; l >= 0; --l) unit[l] = unit[l + 1] * (hi + 1);
+    std::vector<std::pair<long long, int>> idx(c.n2);
     for (int e = 0; e < c.n2; ++e) {
-      down[e] = e;
+      long long key = 0;
+      for (int l = 0; l < L; ++l) key += unit[l] * mono[(size_t)e * L + l];
+      idx[e] = std::make_pair(key, e);
+    }
+    std::sort(idx.begin(), idx.end());
+    for (const std::pair<long long, int>& k : idx) {
+      down[k.second] = k.second;
       for (int l = 0; l < L; ++l)
-        if (mono[e][l] > 0) {
-          std::vector<int> f(mono[e]);
-          --f[l];
-          down[(size_t)(l + 1) * c.n2 + e] = std::lower_bound(idx.begin(), idx.end(), std::make_pair(f, -1))->second;
-        }
+        if (mono[(size_t)k.second * L + l] > 0)
+          down[(size_t)(l + 1) * c.n2 + k.second] =
+              std::lower_bound(idx.begin(), idx.end(), std::make_pair(k.first - unit[l], -1))->second;
     }
   }
   // the pairs (a, b) of each table entry: exponents add, folded modulo the radices
   const GridDesc& g = a.grid;
   c.table_size = P->table_size;
   std::vector<int> to((size_t)c.n1 * c.n2), first(P->table_size + 1, 0), list;
-  for (int x = 0; x < c.n1; ++x)
-    for (int y = 0; y < c.n2; ++y) {
-      long long t = 0;
-      for (int l = 0; l < L && t >= 0; ++l) {
-        const int b = (mono[x][l] + mono[y][l]) % g.radix[l];
-        t = b < g.nout[l] ? t * g.nout[l] + b : -1;
-      }
-      to[(size_t)x * c.n2 + y] = (int)t;
-      if (t >= 0) ++first[t + 1];
+  {
+    std::vector<long long> part((size_t)L * (c.N + 1));   // an exponent's share of the entry, below any sum if cut off
+    long long stride = 1;
+    for (int l = L - 1; l >= 0; --l) {
+      for (int b = 0; b <= c.N; ++b)
+        part[(size_t)l * (c.N + 1) + b] = b % g.radix[l] < g.nout[l] ? stride * (b % g.radix[l]) : -(1LL << 40);
+      stride *= g.nout[l];
     }
+    for (int x = 0; x < c.n1; ++x)
+      for (int y = 0; y < c.n2; ++y) {
+        const int *ex = &mono[(size_t)x * L], *ey = &mono[(size_t)y * L];
+        long long t = 0;
+        for (int l = 0; l < L; ++l) t += part[(size_t)l * (c.N + 1) + ex[l] + ey[l]];
+        to[(size_t)x * c.n2 + y] = t >= 0 ? (int)t : -1;
+        if (t >= 0) ++first[t + 1];
+      }
+  }
   for (long long t = 0; t < P->table_size; ++t) first[t + 1] += first[t];
   list.resize(std::max(1, first[P->table_size]));
   {
@@ -542,12 +550,14 @@ int gbsbin_fock_plan_create(const gbsbin_fock_problem* p, const gbsbin_options* 
   P->state_bytes = P->coef_count * (sizeof(double2) + sizeof(float4));
   if (P->conv) P->state_bytes += (P->coef_count + 1) * sizeof(longlong2);   // and the exponent
   if (!st)
-    (st = dalloc(&P->d_state, P->state_bytes)) || (st = dalloc(&P->d_xtw, (size_t)xoff)) ||
-        (st = dalloc(&P->d_xtw_df, (size_t)xoff)) || (st = dalloc(&P->d_zr, (size_t)a.rsum)) ||
-        (st = dalloc(&P->d_zr_df, (size_t)a.rsum)) || (st = dalloc(&P->d_tw, (size_t)a.rsum)) ||
-        (st = dalloc(&P->d_parts, P->conv ? 0 : (size_t)xr * g.n_full)) || (st = dalloc(&P->d_bufA, (size_t)g.n_full)) ||
-        (st = dalloc(&P->d_bufB, (size_t)g.n_full)) || (st = dalloc(&P->d_diag, GBSBIN_DIAG_DOUBLES)) ||
-        (st = dalloc(&P->d_bar, 4)) || (st = dalloc(&P->d_table, (size_t)P->table_size));
+    (st = dalloc(&P->d_state, P->state_bytes)) || (st = dalloc(&P->d_diag, GBSBIN_DIAG_DOUBLES)) ||
+        (st = dalloc(&P->d_table, (size_t)P->table_size));
+  if (!st && !P->conv)                           // the walk's roots, partial sums and transform
+    (st = dalloc(&P->d_xtw, (size_t)xoff)) || (st = dalloc(&P->d_xtw_df, (size_t)xoff)) ||
+        (st = dalloc(&P->d_zr, (size_t)a.rsum)) || (st = dalloc(&P->d_zr_df, (size_t)a.rsum)) ||
+        (st = dalloc(&P->d_tw, (size_t)a.rsum)) || (st = dalloc(&P->d_parts, (size_t)xr * g.n_full)) ||
+        (st = dalloc(&P->d_bufA, (size_t)g.n_full)) || (st = dalloc(&P->d_bufB, (size_t)g.n_full)) ||
+        (st = dalloc(&P->d_bar, 4));
   if (st) {
     free_all(P);
     delete P;
@@ -578,33 +588,36 @@ int gbsbin_fock_plan_create(const gbsbin_fock_problem* p, const gbsbin_options* 
     P->cv.B = (const longlong2*)(P->d_state + P->coef_count * (sizeof(double2) + sizeof(float4)));
     P->cv.exponent = (const int*)(P->cv.B + P->coef_count);
   }
-  // roots from exact integer indices
-  const double TWO_PI = 6.283185307179586476925286766559;
-  std::vector<double2> xtw((size_t)std::max(xoff, 1)), zr((size_t)a.rsum), tw((size_t)a.rsum);
-  std::vector<float4> xtw_df((size_t)std::max(xoff, 1)), zr_df((size_t)a.rsum);
-  for (int d = 0; d < a.nd; ++d)
-    for (int q = 0; q < a.drad[d]; ++q) {
-      const cd v = std::polar(1.0, TWO_PI * (double)q / (double)a.drad[d]);
-      xtw[a.doff[d] + q] = make_double2(v.real(), v.imag());
-      xtw_df[a.doff[d] + q] = split_df(v);
-    }
-  for (int l = 0; l < L; ++l)
-    for (int q = 0; q < g.radix[l]; ++q) {
-      const cd v = std::polar(1.0, TWO_PI * (double)q / (double)g.radix[l]);
-      zr[a.roff[l] + q] = make_double2(v.real(), v.imag());
-      zr_df[a.roff[l] + q] = split_df(v);
-      tw[a.roff[l] + q] = make_double2(v.real(), -v.imag());
-    }
   st = stage_transfer(P, p->T);
-  if (!st) {
+  if (!st && (cudaMemcpy(P->d_state, P->h_stage, P->state_bytes, cudaMemcpyHostToDevice) != cudaSuccess ||
+              cudaMemset(P->d_diag, 0, GBSBIN_DIAG_DOUBLES * sizeof(double)) != cudaSuccess)) {
+    cudaGetLastError();
+    st = GBSBIN_ERR_CUDA;
+  }
+  if (!st && !P->conv) {
+    // roots from exact integer indices
+    const double TWO_PI = 6.283185307179586476925286766559;
+    std::vector<double2> xtw((size_t)std::max(xoff, 1)), zr((size_t)a.rsum), tw((size_t)a.rsum);
+    std::vector<float4> xtw_df((size_t)std::max(xoff, 1)), zr_df((size_t)a.rsum);
+    for (int d = 0; d < a.nd; ++d)
+      for (int q = 0; q < a.drad[d]; ++q) {
+        const cd v = std::polar(1.0, TWO_PI * (double)q / (double)a.drad[d]);
+        xtw[a.doff[d] + q] = make_double2(v.real(), v.imag());
+        xtw_df[a.doff[d] + q] = split_df(v);
+      }
+    for (int l = 0; l < L; ++l)
+      for (int q = 0; q < g.radix[l]; ++q) {
+        const cd v = std::polar(1.0, TWO_PI * (double)q / (double)g.radix[l]);
+        zr[a.roff[l] + q] = make_double2(v.real(), v.imag());
+        zr_df[a.roff[l] + q] = split_df(v);
+        tw[a.roff[l] + q] = make_double2(v.real(), -v.imag());
+      }
     if (cudaMemcpy(P->d_xtw, xtw.data(), (size_t)xoff * sizeof(double2), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(P->d_xtw_df, xtw_df.data(), (size_t)xoff * sizeof(float4), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(P->d_zr, zr.data(), zr.size() * sizeof(double2), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(P->d_zr_df, zr_df.data(), zr_df.size() * sizeof(float4), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(P->d_tw, tw.data(), tw.size() * sizeof(double2), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(P->d_state, P->h_stage, P->state_bytes, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemset(P->d_bar, 0, 4 * sizeof(unsigned)) != cudaSuccess ||
-        cudaMemset(P->d_diag, 0, GBSBIN_DIAG_DOUBLES * sizeof(double)) != cudaSuccess) {
+        cudaMemset(P->d_bar, 0, 4 * sizeof(unsigned)) != cudaSuccess) {
       cudaGetLastError();
       st = GBSBIN_ERR_CUDA;
     }

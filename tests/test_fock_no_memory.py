@@ -16,10 +16,11 @@ MAIN = '''
 #include "gbsbin_fock_conv.h"
 
 static size_t largest = 0, refuse_from = ~(size_t)0;
-static int refused = 0, walks = 0, convs = 0, live = 0;
+static int refused = 0, walks = 0, convs = 0, live = 0, calls = 0;
 
 extern "C" {
 cudaError_t cudaMalloc(void** p, size_t n) {
+  ++calls;
   largest = std::max(largest, n);
   if (n >= refuse_from) {
     ++refused;
@@ -34,7 +35,7 @@ cudaError_t cudaFree(void* p) { if (p) --live; std::free(p); return cudaSuccess;
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { *p = std::calloc(1, n); return cudaSuccess; }
 cudaError_t cudaMallocHost(void** p, size_t n) { return cudaHostAlloc(p, n, 0); }
 cudaError_t cudaFreeHost(void* p) { std::free(p); return cudaSuccess; }
-cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { std::memcpy(d, s, n); return cudaSuccess; }
+cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { ++calls; std::memcpy(d, s, n); return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) { std::memcpy(d, s, n); return cudaSuccess; }
 cudaError_t cudaMemset(void* d, int v, size_t n) { std::memset(d, v, n); return cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
@@ -89,12 +90,13 @@ int main() {
   std::vector<double> P(13 * 13 * 13);
   for (int pass = 0; pass < 2; ++pass) {       // with room for everything, then none for the largest block
     gbsbin_fock_plan* h = nullptr;
-    walks = convs = refused = 0;
+    walks = convs = refused = calls = 0;
     const int st = gbsbin_fock_plan_create(&p, nullptr, &h);
+    const int made = calls;
     const int ex = st ? -1 : gbsbin_fock_execute(h, P.data(), nullptr);
     const int tr = st ? -1 : gbsbin_fock_plan_set_transfer(h, T.data(), nullptr);
     if (h) gbsbin_fock_plan_destroy(h);
-    std::printf("%d %d %d %d %d %d %d\\n", st, ex, tr, convs, walks, refused, live);
+    std::printf("%d %d %d %d %d %d %d %d\\n", st, ex, tr, convs, walks, refused, live, made);
     refuse_from = largest;
   }
 }
@@ -114,9 +116,14 @@ def passes(tmp_path_factory):
 
 
 def test_convolution_with_room(passes):
-    assert passes[0] == [0, 0, 0, 1, 0, 0, 0]
+    assert passes[0][:7] == [0, 0, 0, 1, 0, 0, 0]
+
+
+def test_convolution_makes_its_own_arrays_only(passes):
+    # state, diagnostics, table and the convolution's block; one copy of its tables, one of the circuit
+    assert passes[0][7] == 6
 
 
 def test_walk_without_room(passes):
-    st, execute, transfer, convs, walks, refused, live = passes[1]
+    st, execute, transfer, convs, walks, refused, live, _ = passes[1]
     assert refused == 1 and (st, execute, transfer, convs, walks, live) == (0, 0, 0, 0, 1, 0)
