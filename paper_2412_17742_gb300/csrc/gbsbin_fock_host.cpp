@@ -73,6 +73,11 @@ int dalloc(T** p, size_t count) {
 }
 
 void free_all(gbsbin_fock_plan* P) {
+  if (P->d_conv) {                       // one block holds everything
+    P->d_state = nullptr;
+    P->d_diag = nullptr;
+    P->d_table = nullptr;
+  }
   void* ptrs[] = {P->d_state, P->d_xtw, P->d_xtw_df, P->d_zr, P->d_zr_df, P->d_tw, P->d_parts,
                   P->d_bufA, P->d_bufB, P->d_diag, P->d_bar, P->d_table, P->d_conv};
   for (void* q : ptrs)
@@ -225,7 +230,8 @@ bool conv_layout(gbsbin_fock_plan* P) {
   return t_conv < t_walk;
 }
 
-// Tables and workspaces of the convolution in one device block.
+// Tables and workspaces of the convolution and the plan's state, diagnostics and table in one device block (a block of
+// its own for each small array is one of 2 MB more to allocate and give back, ~65 us).
 int conv_setup(gbsbin_fock_plan* P) {
   FockConvArgs& c = P->cv;
   const FockArgs& a = P->args;
@@ -351,7 +357,8 @@ int conv_setup(gbsbin_fock_plan* P) {
     }
   size_t o_F3[2] = {0, 0};
   for (int h = 0; h < 2 && c.nd == 3; ++h) o_F3[h] = take((size_t)c.states * ((h ? c.n2 : c.n1) + 1) * 8);
-  const size_t o_parts = take((size_t)c.nchunks * c.n1 * c.n2 * 16);
+  const size_t o_parts = take((size_t)c.nchunks * c.n1 * c.n2 * 16), o_state = take(P->state_bytes),
+               o_diag = take(GBSBIN_DIAG_DOUBLES * sizeof(double)), o_table = take((size_t)P->table_size * sizeof(double));
   const int st = dalloc(&P->d_conv, at);
   if (st) return st;
   unsigned char* d = P->d_conv;
@@ -385,6 +392,11 @@ int conv_setup(gbsbin_fock_plan* P) {
     }
   for (int h = 0; h < 2; ++h) c.F3[h] = c.nd == 3 ? (int2*)(d + o_F3[h]) : nullptr;
   c.parts = (double2*)(d + o_parts);
+  P->d_state = d + o_state;
+  P->d_diag = (double*)(d + o_diag);
+  P->d_table = (double*)(d + o_table);
+  c.B = (const longlong2*)(P->d_state + P->coef_count * (sizeof(double2) + sizeof(float4)));
+  c.exponent = (const int*)(c.B + P->coef_count);
   return GBSBIN_OK;
 }
 
@@ -542,16 +554,20 @@ int gbsbin_fock_plan_create(const gbsbin_fock_problem* p, const gbsbin_options* 
   P->coef_count = (size_t)(L + 1) * a.nin * a.nin;
   P->conv = opt.shard_end == 0 && opt.shard_begin == 0 && opt.tile_override == 0 && conv_layout(P);
   int st = GBSBIN_OK;
+  const size_t walk_state = P->coef_count * (sizeof(double2) + sizeof(float4));
   // the convolution's tables and states; where the device has no room for them the walk serves the plan
-  if (P->conv && (st = conv_setup(P)) == GBSBIN_ERR_NOMEM) {
-    P->conv = false;
-    st = GBSBIN_OK;
+  if (P->conv) {
+    P->state_bytes = walk_state + (P->coef_count + 1) * sizeof(longlong2);   // and the exponent
+    if ((st = conv_setup(P)) == GBSBIN_ERR_NOMEM) {
+      P->conv = false;
+      st = GBSBIN_OK;
+    }
   }
-  P->state_bytes = P->coef_count * (sizeof(double2) + sizeof(float4));
-  if (P->conv) P->state_bytes += (P->coef_count + 1) * sizeof(longlong2);   // and the exponent
-  if (!st)
+  if (!P->conv) {
+    P->state_bytes = walk_state;
     (st = dalloc(&P->d_state, P->state_bytes)) || (st = dalloc(&P->d_diag, GBSBIN_DIAG_DOUBLES)) ||
         (st = dalloc(&P->d_table, (size_t)P->table_size));
+  }
   if (!st && !P->conv)                           // the walk's roots, partial sums and transform
     (st = dalloc(&P->d_xtw, (size_t)xoff)) || (st = dalloc(&P->d_xtw_df, (size_t)xoff)) ||
         (st = dalloc(&P->d_zr, (size_t)a.rsum)) || (st = dalloc(&P->d_zr_df, (size_t)a.rsum)) ||
@@ -584,10 +600,6 @@ int gbsbin_fock_plan_create(const gbsbin_fock_problem* p, const gbsbin_options* 
   a.zr = P->d_zr;
   a.zr_df = P->d_zr_df;
   a.parts = P->d_parts;
-  if (P->conv) {
-    P->cv.B = (const longlong2*)(P->d_state + P->coef_count * (sizeof(double2) + sizeof(float4)));
-    P->cv.exponent = (const int*)(P->cv.B + P->coef_count);
-  }
   st = stage_transfer(P, p->T);
   if (!st && (cudaMemcpy(P->d_state, P->h_stage, P->state_bytes, cudaMemcpyHostToDevice) != cudaSuccess ||
               cudaMemset(P->d_diag, 0, GBSBIN_DIAG_DOUBLES * sizeof(double)) != cudaSuccess)) {

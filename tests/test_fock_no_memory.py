@@ -120,8 +120,8 @@ def test_convolution_with_room(passes):
 
 
 def test_convolution_makes_its_own_arrays_only(passes):
-    # state, diagnostics, table and the convolution's block; one copy of its tables, one of the circuit
-    assert passes[0][7] == 6
+    # one block; one copy of its tables, one of the circuit
+    assert passes[0][7] == 3
 
 
 def test_walk_without_room(passes):
