@@ -173,6 +173,10 @@ bool conv_layout(gbsbin_fock_plan* P) {
     N += a.pw[j];
   }
   if (N < 4 || P->table_size > (1 << 22)) return false;
+  // The walk of few nodes is shorter than the convolution's launches (N / 2 layers and three more, ~6 us each): one or
+  // two occupied inputs (2 + 2 photons, one group, pairs 20 us against 29, 6 + 6 32 against 49, three groups FP64 10 + 10 123
+  // against 127), three of up to five photons in one group (27 to 36 us against 29 to 37).
+  if (a.nin <= 2 || (a.nin == 3 && N <= 5 && a.L == 1)) return false;
   c.nin = a.nin;
   c.L = a.L;
   c.N = N;
