@@ -944,6 +944,10 @@ static bool cluster_suits(const DftFused& f) {
   long long w = f.last_outer * f.last_nout * f.H;
   for (int l = 0; l < f.naxes; ++l) w += f.ax[l].outer * f.ax[l].nout * f.ax[l].inner * f.ax[l].R;
   const GridDesc& g = f.a.grid;
+  // sums of many parts are chains that end sooner over more SMs than a cluster's (Fock walks, whole tables,
+  // cooperative launch and cluster: 8 sums of 256 parts 194 and 199 us, 9 of 1024 486 and 520, 144 of 512 351 and 363;
+  // 7 of 128 160 and 160)
+  if (f.a.parts && f.a.nparts > 128) return false;
   if (f.a.parts) w += f.a.nparts * g.n_full;
   else if (!f.a.g_ready) w += 20 * g.n_full;
   return w <= kClusterWork;
