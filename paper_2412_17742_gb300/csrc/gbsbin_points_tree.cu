@@ -310,19 +310,28 @@ long long level_children(const GridDesc& g, int l, long long nodes, int num_sms,
   return children;
 }
 
+// The first level on its own, or formed by every child of the second's launch, which saves a launch and the way
+// through memory and repeats the sums per child.  In clocks, per turn of the SMs: m^2 entries of nb products and
+// ~10 more, 1 each in FP64 and 0.35 in pairs, at least a CTA's turn; against ~11000 saved in FP64, 7600 in pairs.  Whole
+// tables, apart / fused: three groups of 8 rows, FP64, 81 children 54.5 / 48.1 us, 256 59.4 / 59.4, 729 81.9 / 111,
+// 1600 145 / 204; of 12 rows 69.6 / 73.7, 80 / 94, 141 / 203, 291 / 422; in pairs 8 rows 38.0 / 34.8, 44.0 / 42.5, 53 / 64, 64 / 89;
+// 12 rows 49.2 / 47.0, 55.3 / 55.4, 74 / 93, 112 / 159; four of 8 rows, pairs 53.2 / 49.8, FP64 87.8 / 88.1.
+bool first_level_fused(const TreeArgs& a, const GridDesc& g, int num_sms, bool fp64) {
+  if (g.L <= 2) return false;
+  int span = 1;
+  const long long turns = (level_children(g, 1, g.radix[0], num_sms, &span) + num_sms - 1) / num_sms;
+  const double sums = (a.nb[0] + 10.0) * a.m[1] * a.m[1] * (fp64 ? 1.0 : 0.35);
+  return (double)turns * std::max(fp64 ? 5400.0 : 3000.0, sums) < (fp64 ? 11000.0 : 7600.0);
+}
+
 // Level 0 from the spectral form or, where the plan does without it, by elimination like the other levels.
 template <class Ar>
 cudaError_t launch_tree(const TreeArgs& a, int num_sms, cudaStream_t s, int* launches) {
   cudaError_t err = cudaSuccess;
   *launches = 1;                                      // the leaves
-  // The first level on its own, or within the second's launch where that runs the arithmetic with the cheap
-  // products (pairs of FP32: ~0.5 clocks of an SM each, FP64 2) in well under a launch's time (~3 us).
-  // n = 32, four groups of 8 rows, pairs: 51.4 us with both levels in one elimination, 54.4 with the first
-  // level apart, 50.1 formed within the second's launch.  n = 42, three of 14 rows, FP64: 110.7 with both in
-  // one elimination, 90.3 apart.
+  constexpr bool fp64 = !std::is_same<Ar, ArDF>::value;
   long long nodes = a.spectral ? a.grid.radix[0] : 1;
-  const double fill = (double)a.nb[0] * a.m[1] * a.m[1] * (std::is_same<Ar, ArDF>::value ? 0.5 : 2.0);
-  bool fused = a.spectral && a.grid.L > 2 && fill < 6000.0;
+  bool fused = a.spectral && first_level_fused(a, a.grid, num_sms, fp64);
   if (a.spectral && !fused) {
     if ((err = launch_root<Ar>(a, num_sms, s)) != cudaSuccess) return err;
     ++*launches;
@@ -375,7 +384,9 @@ bool tree_spectral_suits(const TreeArgs& a, const GridDesc& g, int num_sms, bool
   const double nb = a.nb[0], m = a.m[0], cols = m - nb + 2.0;
   const double host = 1.5 + 1e-3 * nb * nb * nb + 1.9e-3 * nb * nb * cols;
   const double gain = nb * turns * std::max(0.0, fp64 ? 0.04 * m - 0.35 : 0.0105 * m);
-  return host <= gain + 3.0;
+  // (apart from the second level's launch it is one launch more, ~4 us: groups of 4 rows, 729 children, pairs 43 us
+  // apart, 39 by elimination)
+  return host <= gain + 3.0 && (gain >= 4.0 || g.L == 2 || first_level_fused(a, g, num_sms, fp64));
 }
 
 size_t tree_level_smem_bytes(int nb, int m) { return sizeof(float4) * ((size_t)(m + 1) * (m + 1) + nb + 2 * (m + 1)); }
