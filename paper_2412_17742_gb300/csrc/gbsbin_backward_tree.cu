@@ -296,17 +296,13 @@ __global__ void __launch_bounds__(kBwdHessThreads) k_bwdt_hess(BackwardArgs b, B
   const int extra = t.has_gamma ? 2 : 0;
   for (int k = 0; k + 2 < m; ++k) {
     if (tid < 32) {
-      E nrm2 = Ar::zero();
-      for (int i = k + 1 + lane; i < m; i += 32) nrm2 = Ar::add(nrm2, Ar::norm2(M[(size_t)i * ld + k]));
-      nrm2 = group_sum<Ar>(nrm2, 32);
+      E rest = Ar::zero();
+      for (int i = k + 2 + lane; i < m; i += 32) rest = Ar::add(rest, Ar::norm2(M[(size_t)i * ld + k]));
+      rest = group_sum<Ar>(rest, 32);
       const E x0 = M[(size_t)(k + 1) * ld + k];
-      E alpha = x0, beta = Ar::zero();
-      if (Ar::re(nrm2) > 0.f) reflector<Ar>(nrm2, x0, alpha, beta);
-      for (int i = k + 1 + lane; i < m; i += 32) {
-        E vi = M[(size_t)i * ld + k];
-        if (i == k + 1) vi = Ar::add(vi, Ar::neg(alpha));
-        v[i] = vi;
-      }
+      E alpha = x0, v0 = Ar::zero(), beta = Ar::zero();
+      if (Ar::re(rest) > 0.f) reflector<Ar>(rest, x0, alpha, v0, beta);
+      for (int i = k + 1 + lane; i < m; i += 32) v[i] = i == k + 1 ? v0 : M[(size_t)i * ld + k];
       if (lane == 0) {
         sc[0] = beta;
         rot.v0[k] = v[k + 1];

@@ -384,19 +384,12 @@ __global__ void __launch_bounds__(HESS_THREADS) k_bt_hess(BTreeArgs a) {
   __syncthreads();
   for (int k = 0; k + 2 < m; ++k) {
     if (warp == 0) {                                 // the reflector of column k
-      E nrm2 = Ar::zero();
-      for (int i = k + 1 + lane; i < m; i += 32) nrm2 = Ar::add(nrm2, Ar::norm2(at(i, k)));
-      for (int o = 16; o > 0; o >>= 1) nrm2 = Ar::add(nrm2, shfl_xor(nrm2, o));
-      const E x0 = at(k + 1, k);
-      E alpha = Ar::zero(), beta = Ar::zero();
-      if (Ar::re(nrm2) > 0.f) {
-        reflector<Ar>(nrm2, x0, alpha, beta);
-      }
-      for (int i = k + 1 + lane; i < m; i += 32) {
-        E vi = at(i, k);
-        if (i == k + 1) vi = Ar::add(vi, Ar::neg(alpha));
-        v[i] = vi;
-      }
+      E rest = Ar::zero();
+      for (int i = k + 2 + lane; i < m; i += 32) rest = Ar::add(rest, Ar::norm2(at(i, k)));
+      for (int o = 16; o > 0; o >>= 1) rest = Ar::add(rest, shfl_xor(rest, o));
+      E alpha = Ar::zero(), v0 = Ar::zero(), beta = Ar::zero();
+      if (Ar::re(rest) > 0.f) reflector<Ar>(rest, at(k + 1, k), alpha, v0, beta);
+      for (int i = k + 1 + lane; i < m; i += 32) v[i] = i == k + 1 ? v0 : at(i, k);
       if (lane == 0) {
         sc[0] = alpha;
         sc[1] = beta;
@@ -526,15 +519,13 @@ __global__ void __launch_bounds__(HC_THREADS) k_bt_hess_cluster(BTreeArgs a, int
     E* v = vbuf + (k & 1) * (m + 1);
     if (rank == k % C && warp == 0) {                // the reflector of column k, to every CTA
       E* col = A + k / C;
-      E nrm2 = Ar::zero();
-      for (int i = k + 1 + lane; i < m; i += 32) nrm2 = Ar::add(nrm2, Ar::norm2(col[(size_t)i * ld]));
-      for (int o = 16; o > 0; o >>= 1) nrm2 = Ar::add(nrm2, shfl_xor(nrm2, o));
-      const E x0 = col[(size_t)(k + 1) * ld];
-      E alpha = Ar::zero(), beta = Ar::zero();
-      if (Ar::re(nrm2) > 0.f) reflector<Ar>(nrm2, x0, alpha, beta);
+      E rest = Ar::zero();
+      for (int i = k + 2 + lane; i < m; i += 32) rest = Ar::add(rest, Ar::norm2(col[(size_t)i * ld]));
+      for (int o = 16; o > 0; o >>= 1) rest = Ar::add(rest, shfl_xor(rest, o));
+      E alpha = Ar::zero(), v0 = Ar::zero(), beta = Ar::zero();
+      if (Ar::re(rest) > 0.f) reflector<Ar>(rest, col[(size_t)(k + 1) * ld], alpha, v0, beta);
       for (int i = k + 1 + lane; i < m; i += 32) {
-        E vi = col[(size_t)i * ld];
-        if (i == k + 1) vi = Ar::add(vi, Ar::neg(alpha));
+        const E vi = i == k + 1 ? v0 : col[(size_t)i * ld];
         for (int r = 0; r < C; ++r) put_cluster(v + i, r, vi);
       }
       if (lane < C) put_cluster(v + m, lane, beta);
