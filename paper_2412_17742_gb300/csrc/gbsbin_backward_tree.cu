@@ -789,15 +789,23 @@ size_t backward_leaf_smem_bytes(int mF) {
 }
 
 // The reduction and the way back are launches of one or a few CTAs per parent, O(mF^3) each, as long for one parent
-// as for an SM each; the saving grows with the leaves per SM.  Measured (reverse-pass kernels, us, Gauss-Jordan
-// leaves / Hessenberg leaves, 61 parents; pairs, FP64): mF = 40, 6.8 leaves per SM 823 / 896, 1950 / 2438; mF = 60,
-// 5.2 per SM 1636 / 1689, 4235 / 4763, 6.8 per SM 1901 / 1819, 4945 / 5055; mF = 80, 5.2 per SM 3564 / 3393,
-// 8886 / 10008, 6.8 per SM 4116 / 3575, 10361 / 10449.  Eight leaves per SM, per parent an SM takes, is past the
-// crossing of all but the smallest blocks.
-bool backward_hess_suits(int mF, long long parents, long long half, int num_sms) {
-  if (mF < 32 || mF > kBwdHessMax) return false;
+// as for an SM each, and the way back grows with the parents; the saving grows with the leaves per SM and faster with
+// mF, the less in FP64 whose leaves are bound by their products. Reverse-pass kernels, Hessenberg over Gauss-Jordan
+// leaves, at 8 / 16 / 24 leaves per SM (61 parents; 140 parents):
+//   rows  pairs                                  FP64
+//   32    1.14 / 0.97 / 0.88; 1.15 / 1.02 / 0.92   1.48 / 1.22 / 1.10; 1.85 / 1.57 / 1.36
+//   40    1.04 / 0.87 / 0.78; 1.08 / 0.93 / 0.82   1.20 / 0.95 / 0.83; 1.52 / 1.23 / 1.04
+//   48    0.91 / 0.74 / 0.67; 0.95 / 0.81 / 0.71   1.18 / 0.92 / 0.81; 1.48 / 1.20 / 1.00
+//   60    0.88 / 0.72 / 0.65; 0.94 / 0.80 / 0.71   0.94 / 0.73 / 0.64; 1.18 / 0.94 / 0.78
+//   80    0.74 / 0.56 / 0.49; 0.82 / 0.65 / 0.55   0.90 / 0.65 / 0.55; 1.06 / 0.81 / 0.66
+//   100   0.55 / 0.40 / 0.34; 0.65 / 0.45 / 0.37   0.71 / 0.49 / 0.41; 0.94 / 0.64 / 0.51
+// The line: leaves per SM by the rows and the arithmetic, times 1 + parents / SMs, and eight in any case.
+bool backward_hess_suits(int mF, long long parents, long long half, int num_sms, bool df) {
+  if (mF < (df ? 32 : 40) || mF > kBwdHessMax) return false;
+  const double least = df ? (mF < 40 ? 14.5 : mF < 48 ? 9.2 : 4.0) : (mF < 60 ? 14.0 : mF < 80 ? 7.5 : mF < 100 ? 5.3 : 4.0);
   const long long rounds = (parents + num_sms - 1) / num_sms;
-  return parents * half >= 8 * rounds * num_sms;
+  const double leaves = (double)(parents * half) / num_sms;
+  return leaves >= 8.0 * rounds && leaves >= least * (1.0 + (double)parents / num_sms);
 }
 
 size_t backward_tree_smem_bytes(int n, int nb) {

@@ -51,6 +51,6 @@ cudaError_t launch_backward_reduce(const BackwardArgs& b, int nparts, cudaStream
 size_t backward_tree_smem_bytes(int n, int nb);
 size_t backward_leaf_smem_bytes(int mF);
 // Whether the leaves' inverses go through the Hessenberg form of each parent's C.
-bool backward_hess_suits(int mF, long long parents, long long half, int num_sms);
+bool backward_hess_suits(int mF, long long parents, long long half, int num_sms, bool df);
 
 }  // namespace gbsbin

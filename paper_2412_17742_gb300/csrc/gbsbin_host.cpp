@@ -1072,7 +1072,7 @@ int backward_tree_setup(gbsbin_plan* P) {
   t.D = n + 1;
   t.A0 = P->btree.mat[0];
   t.half = half;
-  t.hess = backward_hess_suits(mF, parents, half, P->num_sms);
+  t.hess = backward_hess_suits(mF, parents, half, P->num_sms, P->kernel == GBSBIN_KERNEL_BTREE_DF32);
   t.pstride = (long long)n * n + 2LL * n + (long long)mF * mF + 4LL * mF;
   t.lstride = (t.hess ? 1LL : 2LL) * mF * mF + 2LL * mF + 1;
   int off = 0;
