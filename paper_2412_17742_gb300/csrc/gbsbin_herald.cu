@@ -16,7 +16,8 @@
 // complement is A'_F = X_F M, its row u' = l and its corner 2 e, and the pivots' product the determinant.  So the
 // points share eliminations like those of the binned tables: the traced rows go on the host once per
 // state (w = 1), the first group by its spectral form for all roots of its axis in one launch (k_tree_root), and a
-// CTA per point sweeps the other groups, from the first group's result of its root.  Then the Taylor
+// CTA per point sweeps the other groups, from the first group's result of its root (or, where the first axis is so long
+// that its results would not fit the plan's memory, all groups).  Then the Taylor
 // coefficients of exp(xi^T M xi / 2 + l^T xi) by (p_i + 1) c_{p + e_i} = l_i c_p + sum_j M_ij c_{p - e_j}
 // (shells of equal total degree in parallel, in shared memory, seven warps), while the eighth warp continues
 // the elimination into the kept block - its Schur complement is I - A'_F - for the heralding probability's
@@ -61,6 +62,8 @@ __device__ double2 record_value(double2 p, float e2, float args, double2 x) {
 
 __device__ __forceinline__ void taylor_sync() { asm volatile("bar.sync 1, %0;" ::"n"(TAYLOR_THREADS) : "memory"); }
 
+// DEEP: the sweep starts at the first group (no depth 1 in memory).
+template <bool DEEP>
 __global__ void __launch_bounds__(HT) k_herald_points(HeraldArgs a, TreeArgs t) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   __shared__ double2 blk[(GBSBIN_HERALD_MAX_F + 1) * (GBSBIN_HERALD_MAX_F + 1)];   // [[A'_F, c'], [u', .]]
@@ -70,7 +73,7 @@ __global__ void __launch_bounds__(HT) k_herald_points(HeraldArgs a, TreeArgs t) 
   __shared__ PathRec<double2> s_rec;
   const long long k = blockIdx.x;
   const int nf = a.nf, f1 = nf + 1, tid = threadIdx.x;
-  if (a.L == 1) {                                     // the only group: its spectral form gives the kept block
+  if (!DEEP && a.L == 1) {                            // the only group: its spectral form gives the kept block
     double2* d = reinterpret_cast<double2*>(sm_raw);
     double2* dB = d + t.nb[0];
     const double2 w = root_at<ArF64>(t, 0, (int)k);
@@ -86,13 +89,14 @@ __global__ void __launch_bounds__(HT) k_herald_points(HeraldArgs a, TreeArgs t) 
     __syncthreads();
     if (tid == 0) s_rec.ex = ArF64::add(s_rec.ex, blk[f1 * f1 - 1]);
   } else {
-    const Sweep<double2> w = level_sweep<ArF64, false, GBSBIN_MAX_L - 1>(t, 1, a.L - 1, k, sm_raw);
+    constexpr int l0 = DEEP ? 0 : 1;
+    const Sweep<double2> w = level_sweep<ArF64, false, GBSBIN_MAX_L - l0>(t, l0, a.L - l0, k, sm_raw);
     for (int q = tid; q < f1 * f1; q += HT) {
       const int i = q / f1, j = q - q / f1 * f1;
       blk[q] = (i < nf && j < nf) || t.has_gamma ? w.G[(w.nb + i) * w.cols + w.nb + j] : ArF64::zero();
     }
     if (tid < 32) {
-      const PathRec<double2> pr = sweep_path<ArF64, false>(t, 1, w);
+      const PathRec<double2> pr = sweep_path<ArF64, false>(t, l0, w);
       if (tid == 0) s_rec = pr;
     }
   }
@@ -298,7 +302,8 @@ __global__ void k_herald_dft_axis(HeraldArgs a, int l, int slots, const double2*
 
 }  // namespace
 
-size_t herald_sweep_smem(int L, int nb0, int m1) {
+size_t herald_sweep_smem(int L, int nb0, int m1, bool deep) {
+  if (deep) return tree_level_smem_bytes(nb0 + m1, nb0 + m1);
   if (L == 1) return sizeof(double2) * (size_t)nb0 * (m1 + 2);
   return tree_level_smem_bytes(m1, m1);
 }
@@ -307,16 +312,18 @@ cudaError_t launch_herald(const HeraldArgs& a, const TreeArgs& t, int num_sms, d
                           cudaStream_t s, int* launches) {
   cudaError_t err = cudaSuccess;
   *launches = 0;
-  if (a.L > 1) {
+  const bool deep = a.L > 1 && !t.A[1];
+  if (a.L > 1 && !deep) {
     if ((err = launch_tree_root_fp64(t, num_sms, s)) != cudaSuccess) return err;
     ++*launches;
   }
-  const size_t sweep = herald_sweep_smem(a.L, t.nb[0], t.m[1]);
+  const size_t sweep = herald_sweep_smem(a.L, t.nb[0], t.m[1], deep);
   const size_t coef = a.ncoef <= SMEM_COEF ? sizeof(double2) * (size_t)a.ncoef : 0, smem = sweep > coef ? sweep : coef;
+  auto points = deep ? k_herald_points<true> : k_herald_points<false>;
   if (smem > 32 * 1024 &&
-      (err = cudaFuncSetAttribute(k_herald_points, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+      (err = cudaFuncSetAttribute(points, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
     return err;
-  k_herald_points<<<(unsigned)a.npts, HT, smem, s>>>(a, t);
+  points<<<(unsigned)a.npts, HT, smem, s>>>(a, t);
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
   ++*launches;
   int l = 0;

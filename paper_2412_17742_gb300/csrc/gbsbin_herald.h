@@ -7,7 +7,7 @@ namespace gbsbin {
 
 // The traced modes are eliminated on the host (w = 1 at every point); the rest are ordered by heralding group,
 // the kept modes (nf rows, both halves) last, and the groups run as the levels of a tree of block eliminations
-// (TreeArgs, gbsbin_tree.cuh).  The Taylor coefficients are visited in order of total degree from a table
+// (TreeArgs, gbsbin_tree.cuh; A[1] = nullptr: without depth 1 in memory, each point from the first group).  The Taylor coefficients are visited in order of total degree from a table
 // built with the plan: entry t of shell s (s = 1 .. nf cut, entries shell[s] .. shell[s + 1] - 1) is
 // coefficient q = tq[t], computed from p - e_i0 (index tqm[t], i0 = ti0[t] the first non-zero digit,
 // p_i0 = tp[t]) and its neighbours p - e_i0 - e_j (tnb[t nf + j], -1 where that digit is zero).  A channel is
@@ -39,7 +39,7 @@ struct HeraldArgs {
   double* minpiv;                    // npts: smallest pivot real part of both eliminations
   double* prob_own;                  // table: the plan's copy of Pr(b) (diagnostics)
 };
-size_t herald_sweep_smem(int L, int nb0, int m1);   // shared memory of a point's elimination
+size_t herald_sweep_smem(int L, int nb0, int m1, bool deep);   // shared memory of a point's elimination
 cudaError_t launch_herald(const HeraldArgs& a, const TreeArgs& t, int num_sms, double2* out, double* prob,
                           cudaStream_t s, int* launches);
 

@@ -315,12 +315,15 @@ int gbsbin_herald_plan_create(const gbsbin_herald_problem* p, const gbsbin_optio
   P->upload_bytes = b.bytes.size();
   if ((st = dalloc(&P->d_const, b.bytes.size())) || (st = dalloc(&P->d_gcoef, (size_t)(a.npts * (ncoef + 1)))) ||
       (st = dalloc(&P->d_scratch, (size_t)(a.npts * (ncoef + 1)))) || (st = dalloc(&P->d_minpiv, (size_t)a.npts)) ||
-      (st = dalloc(&P->d_prob, (size_t)a.table)) ||
-      (st = dalloc(&P->d_depth1, L > 1 ? (size_t)a.radix[0] * ((size_t)t.m[1] * (t.m[1] + 2) + 3) : 0))) {
+      (st = dalloc(&P->d_prob, (size_t)a.table))) {
     free_all(P);
     delete P;
     return st;
   }
+  // depth 1 of the tree, within the same 8 GiB and where there is room for it; without it every point sweeps all groups
+  const double depth1 = L > 1 ? (double)a.radix[0] * ((double)t.m[1] * (t.m[1] + 2) + 3) : 0.0;
+  const bool kept_roots = L > 1 && 2.0 * (double)a.npts * (double)(ncoef + 1) + depth1 <= (double)(1LL << 29) &&
+                          dalloc(&P->d_depth1, (size_t)depth1) == GBSBIN_OK;
   int device = 0;
   if (cudaGetDevice(&device) != cudaSuccess ||
       cudaDeviceGetAttribute(&P->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
@@ -345,7 +348,7 @@ int gbsbin_herald_plan_create(const gbsbin_herald_problem* p, const gbsbin_optio
   t.tw = a.tw;
   t.grid.L = L;
   for (int l = 0; l < L; ++l) t.grid.radix[l] = a.radix[l];
-  if (L > 1) {
+  if (kept_roots) {
     float4* q = reinterpret_cast<float4*>(P->d_depth1);
     const size_t R0 = (size_t)a.radix[0], m1 = (size_t)t.m[1];
     t.A[1] = q;
