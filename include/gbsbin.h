@@ -131,8 +131,9 @@ typedef struct gbsbin_plan gbsbin_plan;
 typedef struct {
   double sum_P;              /* sum of the returned table (1 up to rounding on the folded grid) */
   double max_imag;           /* max |Im P~| before the real part is taken (round-off probe)    */
-  double min_pivot_re;       /* min over evaluated points of min_i Re u_ii (one group: of the factors
-                                1 - w lambda_i); > 0 in theory                                 */
+  double min_pivot_re;       /* min over evaluated points of min_i Re u_ii; > 0 in theory.  For one group, and for the
+                                first group of kernels 11 and 12 (where they start from its spectral form, and
+                                rounded to FP32 there) and of heralded states, of the factors 1 - w lambda_i  */
   long long n_bad_points;    /* evaluated points with a pivot Re <= 0 or a non-finite value    */
   long long n_points;        /* grid points prod(oversample (N_l + 1))                         */
   long long n_evaluated;     /* points evaluated: conjugate symmetry halves the last axis      */

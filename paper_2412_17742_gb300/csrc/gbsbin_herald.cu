@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(HT) k_herald_points(HeraldArgs a, TreeArgs t) 
   __shared__ double2 Mq[GBSBIN_HERALD_MAX_F * GBSBIN_HERALD_MAX_F], lq[GBSBIN_HERALD_MAX_F];
   __shared__ double2 s_pref;
   __shared__ PathRec<double2> s_rec;
+  __shared__ double s_min;                            // the smallest pivot real part so far
   const long long k = blockIdx.x;
   const int nf = a.nf, f1 = nf + 1, tid = threadIdx.x;
   if (!DEEP && a.L == 1) {                            // the only group: its spectral form gives the kept block
@@ -86,6 +87,7 @@ __global__ void __launch_bounds__(HT) k_herald_points(HeraldArgs a, TreeArgs t) 
       const PathRec<double2> pr = root_path<ArF64>(t, w);
       if (tid == 0) s_rec = pr;                       // with the traced rows' exponent
     }
+    if (tid == 32) s_min = fmin(a.tmin, 1.0 - fmax(w.x * a.lam_min, w.x * a.lam_max));
     __syncthreads();
     if (tid == 0) s_rec.ex = ArF64::add(s_rec.ex, blk[f1 * f1 - 1]);
   } else {
@@ -98,6 +100,18 @@ __global__ void __launch_bounds__(HT) k_herald_points(HeraldArgs a, TreeArgs t) 
     if (tid < 32) {
       const PathRec<double2> pr = sweep_path<ArF64, false>(t, l0, w);
       if (tid == 0) s_rec = pr;
+    } else if (tid < 64) {                            // (the record's smallest pivot is FP32)
+      double mn = a.tmin;
+      if (!DEEP) {
+        const double2 r = root_at<ArF64>(t, 0, (int)w.parent);
+        mn = fmin(mn, 1.0 - fmax(r.x * a.lam_min, r.x * a.lam_max));
+      }
+      for (int q = tid - 32; q < w.nb; q += 32) {
+        const double2 z = w.pivots[q];
+        mn = z.x == z.x && z.y == z.y ? fmin(mn, z.x) : -1.0e300;
+      }
+      for (int o = 16; o > 0; o >>= 1) mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+      if (tid == 32) s_min = mn;
     }
   }
   __syncthreads();
@@ -128,14 +142,14 @@ __global__ void __launch_bounds__(HT) k_herald_points(HeraldArgs a, TreeArgs t) 
     }
     __syncwarp();
     double2 prod = rec.prod;
-    float e2 = rec.meta.y, args = rec.meta.x, mn = rec.meta.z;
+    float e2 = rec.meta.y, args = rec.meta.x;
+    double mn = s_min;
     for (int c = 0; c < nf; ++c) {
       const double2 piv = fin[c * f1 + c], r = ArF64::recip(piv);
       prod = ArF64::mul(prod, piv);
       e2 += (float)ArF64::normalise(prod);
       args += atan2f((float)piv.y, (float)piv.x);
-      mn = fminf(mn, (float)piv.x);
-      if (!(piv.x == piv.x) || !(piv.y == piv.y)) mn = -3.0e38f;
+      mn = piv.x == piv.x && piv.y == piv.y ? fmin(mn, piv.x) : -1.0e300;
       const int n1 = nf - c;
       for (int q = lane; q < n1 * n1; q += 32) {
         const int i = c + 1 + q / n1, j = c + 1 + q - q / n1 * n1;
@@ -150,7 +164,7 @@ __global__ void __launch_bounds__(HT) k_herald_points(HeraldArgs a, TreeArgs t) 
                                      make_double2(0.5 * x.x, 0.5 * x.y));
       if (lane) {
         slot[a.ncoef] = v;
-        a.minpiv[k] = isfinite(v.x) && isfinite(v.y) ? (double)mn : -1.0e300;
+        a.minpiv[k] = isfinite(v.x) && isfinite(v.y) ? mn : -1.0e300;
       } else {
         s_pref = v;
       }

@@ -24,6 +24,8 @@ struct HeraldArgs {
   int nchan;                         // channels with u <= v, then one for the heralding probability
   long long table;                   // prod nout
   double pr0;                        // Pr(0) of the whole state
+  double tmin;                       // the traced rows' smallest pivot (1e300: none)
+  double lam_min, lam_max;           // the ends of the first group's spectrum
   const double2* tw;                 // exp(-2 pi i d / radix[l]), d < radix[l], group after group
   const double* chscale;             // [ncoef] prod_i sqrt(p_i!)
   const int* chan;                   // [nchan - 1] the channels with u <= v

@@ -168,7 +168,7 @@ int gbsbin_herald_plan_create(const gbsbin_herald_problem* p, const gbsbin_optio
     Z[(size_t)n2 * W + i] = i < nt ? -gamma[order[i]] : gamma[order[i]];
   }
   cd tprod = 1.0;
-  double targ = 0.0, tmin = 3.0e38;
+  double targ = 0.0, tmin = 1.0e300;
   int te2 = 0;
   for (int k = 0; k < nt; ++k) {
     const cd piv = Z[(size_t)k * W + k];
@@ -209,6 +209,9 @@ int gbsbin_herald_plan_create(const gbsbin_herald_problem* p, const gbsbin_optio
       }
     }
     if (!hermitian_spectrum(A00, nb0, ev, xr.data(), xi.data(), X)) return GBSBIN_ERR_NUMERIC;
+    a.tmin = tmin;
+    a.lam_min = *std::min_element(ev.begin(), ev.end());
+    a.lam_max = *std::max_element(ev.begin(), ev.end());
     for (int k = 0; k < nb0; ++k) {
       const double *yr = &xr[(size_t)k * X], *yi = &xi[(size_t)k * X];
       rlam[k] = ev[k];
@@ -220,7 +223,7 @@ int gbsbin_herald_plan_create(const gbsbin_herald_problem* p, const gbsbin_optio
     double2 prod;
     float4 meta;
     double2 ex;
-  } path0 = {make_double2(tprod.real(), tprod.imag()), make_float4((float)targ, (float)te2, (float)tmin, 0.f),
+  } path0 = {make_double2(tprod.real(), tprod.imag()), make_float4((float)targ, (float)te2, (float)std::min(tmin, 3.0e38), 0.f),
              make_double2(Z[(size_t)n2 * W + n2].real(), Z[(size_t)n2 * W + n2].imag())};
   // the Taylor coefficients in order of total degree, each with its predecessor p - e_i0 (i0
   // its first non-zero digit) and that predecessor's neighbours p - e_i0 - e_j
