@@ -544,7 +544,8 @@ int gbsbin_prob_distinguishable_device(const gbsbin_problem* p, const int* patte
  * points, each factor O(L).  Where it costs less (no shard, automatic kernel choice), the plan takes
  * the table's coefficients directly instead: the product of half the factors (B(z) x)_j as a polynomial in z
  * per sub-multiset of the photons, for both halves, then the sum over complementary sub-multisets, in
- * integer arithmetic of 50 bits or more for either precision (kernel 9 or 10 is reported as asked for).
+ * integer arithmetic for either precision (kernel 9 or 10 is reported as asked for): a state's monomials in 56 bits under
+ * one exponent, where the nodes' values have one each, and the sum's factors in 60 bits (FP64, or many photons) or 56.
  * Options: precision GBSBIN_FP64 (kernel 9) or
  * GBSBIN_FP32_REFINE, which here selects pairs of FP32 (kernel 10); oversample,
  * want_diagnostics, want_timing and tile_override (9 or 10) as for gbsbin_plan_create;

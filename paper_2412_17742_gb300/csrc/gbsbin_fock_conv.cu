@@ -12,16 +12,19 @@
 // states of 165 monomials each) and 3.5e8 for the sum over states, against 1.4e9 complex products and
 // 4e9 additions of the walk over 2^15 nodes x 2601 grid points (gbsbin_fock.cu), which shards keep.
 //
-// Arithmetic: 64-bit integer sums of products of digits (mad.wide.s32).  A state's monomials are 52-bit
-// integers with one exponent per state, in two 26-bit digits; a complex product is three real ones (Karatsuba),
+// Arithmetic: 64-bit integer sums of products of digits (mad.wide.s32).  A state's monomials are 56-bit
+// integers with one exponent per state, in two 28-bit digits; a complex product is three real ones (Karatsuba),
 // each three digit products (the lo x lo term lies below the rounding), summed exactly over (k, t) and
 // rounded once per layer.  On the unit circle sum_m |F_r[m](z)|^2 <= 1 for a contraction T (the amplitudes of
 // r photons), so nothing cancels against larger intermediate terms.  The sum over states takes each
-// monomial at its column's exponent, in 2 x 25 bits for plans of FP32 pairs and 3 x 20 bits for FP64 plans
-// (12,870 states lie up to a few bits below their column's largest, and 50 bits then leave FP64's accuracy).
-// Errors of the total count under uniform loss (binomial), relative 2-norm, 8 / 12 / 16 photons in two groups:
-// pairs 1.1e-15 / 3.4e-15 / 4.8e-14 against 1.6e-13 / 2.2e-13 / 1.8e-13 by the walk.  Measured in a
-// register-tiled loop, a complex multiply-add takes a scheduler 47 clocks with two digits, 68 in pairs of FP32
+// monomial at its column's exponent, in 2 x 28 bits for plans of FP32 pairs of up to 2^14 states (the sums' upper parts
+// moved out every 16 states) and 3 x 20 bits for the others, where products of two small entries must not be lost.
+// (With states of 52 bits and the pairs' sum in 2 x 25 bits, pairs plans of 14 photons through a circuit of 2 to 5%
+// transmission, whose small entries' products are all lo x lo, had 50 times the walk's error.)
+// Relative error of whole tables against 80-bit arithmetic, 6 / 8 / 10 / 11 photons in two groups: transmissions of 40 to 90%
+// 4.0 / 4.3 / 4.6 / 4.6e-16 (the walk: FP64 6.3 / 8.7 / 12 / 13e-16, pairs 4.0e-14 / 2.9e-14 / 1.5e-14 / 1.1e-14), of 2 to 5% 1.3 / 1.7 / 2.1 / 2.5e-16
+// (pairs 1.1 / 1.7 / 3.4 / 3.3e-16; the walk 5.1 / 7.4 / 9.9 / 11e-16 and 4.7e-14 to 1.1e-14).
+// Measured in a register-tiled loop, a complex multiply-add takes a scheduler 47 clocks with two digits, 68 in pairs of FP32
 // and 424 in FP64.
 //
 // k_conv_layer: a warp per state (of either half); lane k finds the predecessor m - e_k; the factor's digits,
@@ -96,8 +99,8 @@ __global__ void __launch_bounds__(kLayerWarps * 32, 8) k_conv_layer(FockConvArgs
       const int s = min(63, emax - ek);
       const long long br = shift_round(b.x, s), bi = shift_round(b.y, s);
       int* o = s_b + 6 * q;
-      digits<26>(br, o[0], o[1]);
-      digits<26>(bi, o[2], o[3]);
+      digits<kConvDigit>(br, o[0], o[1]);
+      digits<kConvDigit>(bi, o[2], o[3]);
       o[4] = o[0] + o[2];
       o[5] = o[1] + o[3];
     }
@@ -157,16 +160,16 @@ __global__ void __launch_bounds__(kLayerWarps * 32, 8) k_conv_layer(FockConvArgs
         if (e < y.nc) {
           const long long rh = m1h[c] - m2h[c], rl = m1l[c] - m2l[c];
           const long long ih = m3h[c] - m1h[c] - m2h[c], il = m3l[c] - m1l[c] - m2l[c];
-          const longlong2 v = make_longlong2(rh + shift_round(rl, 26), ih + shift_round(il, 26));
+          const longlong2 v = make_longlong2(rh + shift_round(rl, kConvDigit), ih + shift_round(il, kConvDigit));
           raw[e] = v;
           big |= (v.x < 0 ? -v.x : v.x) | (v.y < 0 ? -v.y : v.y);
         }
       }
     }
-    // the state's exponent: its largest component in [2^51, 2^52)
+    // the state's exponent: its largest component in [2^55, 2^56)
     const unsigned bh = __reduce_or_sync(kAll, (unsigned)(big >> 32)), bl = __reduce_or_sync(kAll, (unsigned)big);
-    const int len = bit_length((long long)bh << 32 | bl), s = len - 52;
-    const int eo = len == 0 || emax == GBSBIN_FC_NONE ? GBSBIN_FC_NONE : emax + s - (kConvRowBits - 52);
+    const int len = bit_length((long long)bh << 32 | bl), s = len - kConvBits;
+    const int eo = len == 0 || emax == GBSBIN_FC_NONE ? GBSBIN_FC_NONE : emax + s - (kConvRowBits - kConvBits);
     if (lane == 0) {
       a.E[half][out][i] = eo;
       Fout[y.nc] = make_int4(0, 0, 0, 0);
@@ -175,12 +178,12 @@ __global__ void __launch_bounds__(kLayerWarps * 32, 8) k_conv_layer(FockConvArgs
       const longlong2 v = raw[e];
       long long x = eo == GBSBIN_FC_NONE ? 0 : shift_round(v.x, s), z = eo == GBSBIN_FC_NONE ? 0 : shift_round(v.y, s);
       int4 f;
-      digits<26>(x, f.x, f.y);
-      digits<26>(z, f.z, f.w);
+      digits<kConvDigit>(x, f.x, f.y);
+      digits<kConvDigit>(z, f.z, f.w);
       Fout[e] = f;
       if (y.last[half]) {
         const int lx = max(bit_length(x), bit_length(z));
-        if (lx > 0) atomicMax(s_max + half * y.nc + e, eo + lx - 52);
+        if (lx > 0) atomicMax(s_max + half * y.nc + e, eo + lx - kConvBits);
       }
     }
   }
@@ -208,9 +211,9 @@ __global__ void __launch_bounds__(256) k_conv_scale(FockConvArgs a) {
     int4 d = make_int4(0, 0, 0, 0);
     int2 d2 = make_int2(0, 0);
     if (col > GBSBIN_FC_NONE && ex != GBSBIN_FC_NONE) {
-      constexpr int B = ND == 3 ? 20 : 25;
-      const int s = min(63, 52 - ND * B + col - ex);
-      long long x = shift_round(((long long)f.x << 26) + f.y, s), z = shift_round(((long long)f.z << 26) + f.w, s);
+      constexpr int B = ND == 3 ? 20 : 28;
+      const int s = min(63, kConvBits - ND * B + col - ex);
+      long long x = shift_round(((long long)f.x << kConvDigit) + f.y, s), z = shift_round(((long long)f.z << kConvDigit) + f.w, s);
       if (ND == 3) {
         int lo;
         lo = ((int)((unsigned)x << (32 - B))) >> (32 - B);
@@ -245,7 +248,10 @@ __device__ __forceinline__ void mad_digits(long long (&m)[ND], const int (&x)[ND
 }
 
 // Sums over a chunk of states of F1[m][a] F2[p - m][b] for a 24 x 16 tile of (a, b); two stages of
-// kStage states in flight.
+// kStage states in flight.  With two digits of 28 bits a stage's sums reach 16 x 2^29 x 2^29 = 2^62, so after each their
+// parts from bit kUpper on move to 32-bit sums (at most 2^22 a stage, 2^28 in all); three digits of 20 bits stay below
+// 2^54 over all states.
+constexpr int kUpper = 40;
 template <int ND>
 __global__ void __launch_bounds__(kSumThreads, ND == 3 ? 4 : 5) k_conv_sum(FockConvArgs a) {
   __shared__ int4 sx[2][kStage][kConvRows], sy[2][kStage][kConvCols];
@@ -257,6 +263,12 @@ __global__ void __launch_bounds__(kSumThreads, ND == 3 ? 4 : 5) k_conv_sum(FockC
   // warp w and lane / 8 give two rows, lane % 8 two columns
   const int r = (threadIdx.x >> 5) * 8 + ((threadIdx.x & 31) >> 3) * 2, q = (threadIdx.x & 7) * 2;
   long long m1s[2][2][ND] = {}, m2s[2][2][ND] = {}, m3s[2][2][ND] = {};
+  constexpr int NU = ND == 2 ? 2 : 1;
+  int u1s[2][2][NU] = {}, u2s[2][2][NU] = {}, u3s[2][2][NU] = {};
+  auto move_up = [](long long& m, int& u) {
+    u += (int)(m >> kUpper);
+    m &= (1ll << kUpper) - 1;
+  };
   // 24 threads per row of the first half (in order), 16 per row of the second (the complement's)
   const int xc = threadIdx.x % kConvRows, xs = threadIdx.x / kConvRows;
   const int yc = threadIdx.x % kConvCols, ys = threadIdx.x / kConvCols;
@@ -317,11 +329,23 @@ __global__ void __launch_bounds__(kSumThreads, ND == 3 ? 4 : 5) k_conv_sum(FockC
         }
       }
     }
+    if constexpr (ND == 2) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+          for (int w = 0; w < 2; ++w) {
+            move_up(m1s[i][j][w], u1s[i][j][w]);
+            move_up(m2s[i][j][w], u2s[i][j][w]);
+            move_up(m3s[i][j][w], u3s[i][j][w]);
+          }
+    }
     __syncthreads();                             // the buffer is refilled by the next iteration's stage
   }
   double2* out = a.parts + (size_t)blockIdx.z * a.n1 * a.n2;
   const int exponent = *a.exponent;
-  constexpr int B = ND == 3 ? 20 : 25;
+  constexpr int B = ND == 3 ? 20 : 28;
   const double k = 1.0 / (double)(1 << B);
 #pragma unroll
   for (int i = 0; i < 2; ++i)
@@ -335,8 +359,14 @@ __global__ void __launch_bounds__(kSumThreads, ND == 3 ? 4 : 5) k_conv_sum(FockC
         double re = 0.0, im = 0.0;               // from the lowest weight up
 #pragma unroll
         for (int w = ND - 1; w >= 0; --w) {
-          re = fma(re, k, (double)(m1s[i][j][w] - m2s[i][j][w]));
-          im = fma(im, k, (double)(m3s[i][j][w] - m1s[i][j][w] - m2s[i][j][w]));
+          double r = (double)(m1s[i][j][w] - m2s[i][j][w]), q = (double)(m3s[i][j][w] - m1s[i][j][w] - m2s[i][j][w]);
+          if constexpr (ND == 2) {
+            constexpr double up = (double)(1ll << kUpper);
+            r = fma((double)(u1s[i][j][w] - u2s[i][j][w]), up, r);
+            q = fma((double)(u3s[i][j][w] - u1s[i][j][w] - u2s[i][j][w]), up, q);
+          }
+          re = fma(re, k, r);
+          im = fma(im, k, q);
         }
         const int s = ca + cb + exponent - 2 * B;
         v = make_double2(ldexp(re, s), ldexp(im, s));

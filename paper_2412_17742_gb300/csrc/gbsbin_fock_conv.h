@@ -13,10 +13,13 @@ namespace gbsbin {
 
 #define GBSBIN_FC_NONE (-(1 << 28))       // exponent of an all-zero state or column
 
-// Coefficients in fixed point, round(b 2^kConvRowBits / 2^e) with e the row's exponent: components up to 2^55, so that
-// a high digit of 26 bits is at most 2^29 and the sum of two (the third factor of a complex product by three
-// real ones) at most 2^30, and a row's sum of component magnitudes below 2^59, which keeps a layer's 64-bit sums below
-// 2^62 and its results three bits finer than a state's 52.
+// A state's monomials are integers of kConvBits bits, value x 2^(exponent - kConvBits), in two digits of kConvDigit.
+// Coefficients in fixed point, round(b 2^kConvRowBits / 2^e) with e the row's exponent: components up to 2^55, high
+// digits up to 2^27 and the sum of two (the third factor of a complex product by three real ones) up to 2^28, and a
+// row's sum of component magnitudes below 2^59. A layer's 64-bit sums then stay below 2^63 for up to kConvMaxTerms
+// terms (the largest: sums of 2^29 x 2^28 per term and 2^28 x 2^31), and its results are three bits finer than a state's.
+constexpr int kConvDigit = 28, kConvBits = 2 * kConvDigit;
+constexpr int kConvMaxTerms = 56;         // photons of a layer, or occupied inputs, times L + 1
 constexpr int kConvRowBits = 55;
 // e of a row whose largest component is `big` and whose component magnitudes add to `all`: big < 2^e, all < 16 x 2^e
 inline int conv_row_exponent(double big, double all) {
@@ -41,11 +44,11 @@ struct FockConvArgs {
   const int* down;                        // [t][e]: monomial e without z_{t-1} (t = 0: e itself), -1: none
   int ndown;                              // monomials of degree <= h[1] (the stride of `down`)
   const longlong2* B;                     // [row][k][t], fixed point
-  const int4* F0;                         // the empty product: digits of 2^51, and its exponent 1
+  const int4* F0;                         // the empty product: digits of 2^(kConvBits - 1), and its exponent 1
   const int* E0;
   int4* F[2][2];                          // [half][parity]: state x monomial, digits (re hi, lo, im hi, lo)
   int* E[2][2];                           // [half][parity]: the state's exponent
-  int nd;                                 // digits of the sum over states: 2 (25 bits) or 3 (20 bits)
+  int nd;                                 // digits of the sum over states: 2 (28 bits; pairs, up to 2^14 states) or 3 (20 bits)
   int2* F3[2];                            // with three: the last layers' third digits (re, im)
   int* colexp[2];                         // per monomial of the last layer: exponent of its largest entry
   int states, first, n1, n2;              // last layer of the first half: states, its codes in order; monomials
@@ -68,7 +71,7 @@ struct FockConvLayer {
   int last[2];
 };
 constexpr int kConvRows = 24, kConvCols = 16;   // monomials of either half per contraction CTA
-constexpr int kConvMaxChunk = 1024;       // states per CTA: the 64-bit sums stay below 2^62
+constexpr int kConvMaxChunk = 1024;       // states per CTA: the sums' range (k_conv_sum)
 int fock_conv_slots_per_sm(int nd);           // resident contraction CTAs of an SM
 size_t fock_conv_layer_smem(int nin, int L, int nc);
 cudaError_t launch_fock_conv(const FockConvArgs& a, const FockConvLayer* layers, int nlayers, int num_sms,

@@ -180,7 +180,6 @@ bool conv_layout(gbsbin_fock_plan* P) {
   c.nin = a.nin;
   c.L = a.L;
   c.N = N;
-  c.nd = P->df ? 2 : 3;
   c.h[0] = N / 2;
   c.h[1] = N - N / 2;
   std::vector<double> mono(c.h[1] + 1, 1.0);            // monomials of degree <= r in L variables
@@ -188,6 +187,7 @@ bool conv_layout(gbsbin_fock_plan* P) {
     mono[r] = mono[r - 1] * (r + a.L) / r;
     if (mono[r] > 4096.0) return false;
   }
+  if (std::min(c.h[1], a.nin) * (a.L + 1) > kConvMaxTerms) return false;
   c.n1 = (int)std::lround(mono[c.h[0]]);
   c.n2 = (int)std::lround(mono[c.h[1]]);
   if ((double)c.n1 * c.n2 > (double)(1 << 20) || fock_conv_layer_smem(a.nin, a.L, c.n2) > 48 * 1024) return false;
@@ -199,6 +199,9 @@ bool conv_layout(gbsbin_fock_plan* P) {
       for (int v = 0; v <= a.pw[j]; ++v) nx[u + v] += cnt[u];
     cnt.swap(nx);
   }
+  // two digits leave out lo x lo, up to 2^-57 a product: of many states' small entries that adds up (pairs, 2 to 5%
+  // transmission, 16 photons in two groups 9e-15 of the table, the walk 3e-15)
+  c.nd = P->df && cnt[c.h[0]] < (double)(1 << 14) ? 2 : 3;
   std::vector<int> row;
   for (int j = 0; j < a.nin; ++j)
     for (int v = 0; v < a.pw[j]; ++v) row.push_back(j);
@@ -366,7 +369,7 @@ int conv_setup(gbsbin_fock_plan* P) {
   const int st = dalloc(&P->d_conv, at);
   if (st) return st;
   unsigned char* d = P->d_conv;
-  const int f0[8] = {1 << 25, 0, 0, 0, 0, 0, 0, 0}, e0 = 1;   // 1 = 2^51 2^-52 2^1, then the row's zero entry
+  const int f0[8] = {1 << (kConvDigit - 1), 0, 0, 0, 0, 0, 0, 0}, e0 = 1;   // 1 = 2^55 2^-56 2^1, then the row's zero entry
   std::vector<unsigned char> tables(o_c0);               // the tables come first: one copy
   auto put = [&tables](size_t o, const void* src, size_t bytes) { std::memcpy(tables.data() + o, src, bytes); };
   put(o_rank, rank.data(), rank.size() * 4);

@@ -72,8 +72,8 @@ int main() {                       // rows "n big all", then n pairs (re, im): t
       double re, im;
       if (std::scanf("%la %la", &re, &im) != 2) return 1;
       int h[2], l[2];
-      digits<26>(conv_fixed(re, e), h[0], l[0]);
-      digits<26>(conv_fixed(im, e), h[1], l[1]);
+      digits<kConvDigit>(conv_fixed(re, e), h[0], l[0]);
+      digits<kConvDigit>(conv_fixed(im, e), h[1], l[1]);
       worst = std::max(worst, std::llabs((long long)h[0] + h[1]));
     }
   }
