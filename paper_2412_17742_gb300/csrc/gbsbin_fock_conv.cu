@@ -44,7 +44,6 @@ namespace gbsbin {
 namespace {
 
 constexpr int kLayerWarps = 4;
-constexpr int kSlots = 1;                  // monomials per lane and pass
 constexpr int kSumThreads = 96;
 constexpr int kStage = 16;                 // states staged at a time by k_conv_sum
 constexpr unsigned kAll = 0xffffffffu;
@@ -109,37 +108,29 @@ __global__ void __launch_bounds__(kLayerWarps * 32, 8) k_conv_layer(FockConvArgs
     int4* Fout = a.F[half][out] + (size_t)i * (y.nc + 1);
     longlong2* raw = reinterpret_cast<longlong2*>(Fout);     // a lane's own entries, until the state's exponent is known
     long long big = 0;
-    for (int c0 = 0; c0 < y.nc; c0 += 32 * kSlots) {
-      long long m1h[kSlots] = {}, m1l[kSlots] = {}, m2h[kSlots] = {}, m2l[kSlots] = {}, m3h[kSlots] = {}, m3l[kSlots] = {};
-      int dn[CT1 ? CT1 : 1][kSlots];
-      auto offsets = [&](int t, int (&d)[kSlots]) {
-#pragma unroll
-        for (int c = 0; c < kSlots; ++c) {
-          const int e = c0 + lane + 32 * c;
-          d[c] = e < y.nc ? s_down[t * y.nc + e] : y.nc0;
-        }
-      };
+    for (int c0 = 0; c0 < y.nc; c0 += 32) {                  // a monomial a lane
+      const int e = c0 + lane;
+      long long m1h = 0, m1l = 0, m2h = 0, m2l = 0, m3h = 0, m3l = 0;
+      auto offset = [&](int t) { return e < y.nc ? s_down[t * y.nc + e] : y.nc0; };
+      int dn[CT1 ? CT1 : 1];
       if (CT1) {
 #pragma unroll
-        for (int t = 0; t < CT1; ++t) offsets(t, dn[t]);
+        for (int t = 0; t < CT1; ++t) dn[t] = offset(t);
       }
-      auto term = [&](const int4* src, int k, int t, const int (&d)[kSlots]) {
+      auto term = [&](const int4* src, int k, int t, int d) {
         const int2* bp = reinterpret_cast<const int2*>(s_b + 6 * (k * T1 + t));
         const int2 br = bp[0], bi = bp[1], bs = bp[2];
-#pragma unroll
-        for (int c = 0; c < kSlots; ++c) {
-          const int4 f = src[d[c]];
-          mad(m1h[c], f.x, br.x);
-          mad(m1l[c], f.x, br.y);
-          mad(m1l[c], f.y, br.x);
-          mad(m2h[c], f.z, bi.x);
-          mad(m2l[c], f.z, bi.y);
-          mad(m2l[c], f.w, bi.x);
-          const int sh = f.x + f.z, sl = f.y + f.w;
-          mad(m3h[c], sh, bs.x);
-          mad(m3l[c], sh, bs.y);
-          mad(m3l[c], sl, bs.x);
-        }
+        const int4 f = src[d];
+        mad(m1h, f.x, br.x);
+        mad(m1l, f.x, br.y);
+        mad(m1l, f.y, br.x);
+        mad(m2h, f.z, bi.x);
+        mad(m2l, f.z, bi.y);
+        mad(m2l, f.w, bi.x);
+        const int sh = f.x + f.z, sl = f.y + f.w;
+        mad(m3h, sh, bs.x);
+        mad(m3l, sh, bs.y);
+        mad(m3l, sl, bs.x);
       };
       for (unsigned left = mask; left; left &= left - 1) {
         const int k = __ffs(left) - 1;
@@ -148,22 +139,15 @@ __global__ void __launch_bounds__(kLayerWarps * 32, 8) k_conv_layer(FockConvArgs
 #pragma unroll
           for (int t = 0; t < CT1; ++t) term(src, k, t, dn[t]);
         } else {
-          for (int t = 0; t < T1; ++t) {
-            offsets(t, dn[0]);
-            term(src, k, t, dn[0]);
-          }
+          for (int t = 0; t < T1; ++t) term(src, k, t, offset(t));
         }
       }
-#pragma unroll
-      for (int c = 0; c < kSlots; ++c) {
-        const int e = c0 + lane + 32 * c;
-        if (e < y.nc) {
-          const long long rh = m1h[c] - m2h[c], rl = m1l[c] - m2l[c];
-          const long long ih = m3h[c] - m1h[c] - m2h[c], il = m3l[c] - m1l[c] - m2l[c];
-          const longlong2 v = make_longlong2(rh + shift_round(rl, kConvDigit), ih + shift_round(il, kConvDigit));
-          raw[e] = v;
-          big |= (v.x < 0 ? -v.x : v.x) | (v.y < 0 ? -v.y : v.y);
-        }
+      if (e < y.nc) {
+        const long long rh = m1h - m2h, rl = m1l - m2l;
+        const long long ih = m3h - m1h - m2h, il = m3l - m1l - m2l;
+        const longlong2 v = make_longlong2(rh + shift_round(rl, kConvDigit), ih + shift_round(il, kConvDigit));
+        raw[e] = v;
+        big |= (v.x < 0 ? -v.x : v.x) | (v.y < 0 ? -v.y : v.y);
       }
     }
     // the state's exponent: its largest component in [2^55, 2^56)
