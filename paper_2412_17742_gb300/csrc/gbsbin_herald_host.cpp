@@ -1,6 +1,6 @@
-// Host side of heralded states (arXiv:2412.17742, Sec. VII): validation, the adjacency blocks
-// A = X XA split by mode role, the heralding grid's twiddles, Pr(0), device buffers and the
-// two launches (points, then the inverse DFT over the heralding grid).
+// Host side of heralded states (arXiv:2412.17742, Sec. VII): validation, XA ordered by mode role with its traced
+// rows eliminated, the first heralding group's spectral form, the grid's twiddles, Pr(0), device buffers and the
+// launches (the first group's roots, the points, the inverse DFT over the heralding grid).
 #include <algorithm>
 #include <cmath>
 #include <complex>

@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(kSpectralThreads) k_points_spectral(PointArgs 
   spectral_point<TP, DISP>(a, e, threadIdx.x % TP, e < a.grid.n_eval);
 }
 
-// A batch: block j takes the points e0 .. e0 + kSpectralBatchPoints - 1 of its job's problem.
+// A batch: block j takes the points e0 .. e0 + GBSBIN_SPECTRAL_BATCH_POINTS - 1 of its job's problem.
 constexpr int kBatchTP = kSpectralThreads / GBSBIN_SPECTRAL_BATCH_POINTS;
 __global__ void __launch_bounds__(kSpectralThreads) k_points_spectral_batch(PointBatch b) {
   const PointJob job = b.jobs[blockIdx.x];

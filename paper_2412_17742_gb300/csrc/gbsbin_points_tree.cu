@@ -24,7 +24,8 @@
 // whose pivots are those of B's unpivoted LU.  log q = 1/2 sum(u_0^T y) - 1/2 sum Log(pivots).
 // Each node carries a path record - the pivot product (scaled by a power of two), the FP32
 // sum of the pivots' arguments, the exponent sum and the smallest pivot real part - and
-// leaves write the unfinished form that the inverse DFT's first stage finishes in FP64.
+// leaves write the unfinished form from which the inverse DFT takes G (undisplaced plans' leaves write G themselves)
+// and log q is finished in FP64 when asked for.
 //
 // Arithmetic: every kernel is written once over an arithmetic (gbsbin_df.cuh): pairs of
 // FP32 (about 46 bits) on the FMA pipe, or FP64.  The chains here are short and dependent;
