@@ -279,7 +279,7 @@ __device__ __forceinline__ Sweep<typename Ar::E> level_sweep(const TreeArgs& a, 
     } else {
       // entries (i, s), i in (kk, rows), s in (kk + 1, cols), over threads 32..; two
       // independent entries per pass.  floor(idx / w_) from a float reciprocal: idx < 2^14
-      // and w_ <= 65, so (idx + 1/2) / w_ stays more than 1/(2 w_) from an integer
+      // and w_ <= 96 (heralded states), so (idx + 1/2) / w_ stays 1/(2 w_) from an integer, the product's error below 2^-16
       const int t = tid - 32, LO = LT - 32;
       const int w_ = cols - kk - 2, total = (rows - kk - 1) * w_;
       const float rw = 1.0f / (float)(w_ > 0 ? w_ : 1);

@@ -20,6 +20,8 @@ def _problem(seed, bins, cut, disp):
 @pytest.mark.parametrize("bins,cut,precision,spectral", [
     ([0] * 24 + [1] * 8, [5, 2], 0, False),              # 48 of 64 rows: 0.19 ms of host for 0.11 of the table
     ([0] * 24 + [1] * 8, [5, 2], 1, False),
+    ([0] * 24 + [1] * 8, [199, 1], 0, True),             # two turns of the SMs, eigenvalues in two rounds of the path record
+    ([0] * 24 + [1] * 8, [799, 1], 1, True),
     ([0] * 12 + [1] * 4, [4, 4], 0, False),              # 24 of 32 rows: 28 us for 20
     ([0] * 8 + [1] * 8, [4, 4], 1, False),               # 16 of 32 rows in pairs: 14 us for 6
     ([0] * 8 + [1] * 8, [4, 4], 0, True),                # in FP64 15
