@@ -37,7 +37,7 @@
 // thread, the states copied asynchronously two stages ahead; the chunk is set so that the CTAs fill the SMs
 // once.  (24 x 24 with 2 x 3 outputs: 646 us for the launch against 600, with fewer warps to hide the chains.)
 // k_conv_table: a warp per table entry adds its monomial pairs over all chunks in a fixed order.
-// N = 16, three groups, whole table: 6807 us by the walk in pairs of FP32 (31000 in FP64), 1340 us here.
+// N = 16, three groups, whole table: 6807 us by the walk in pairs of FP32 (31000 in FP64), 1350 us here.
 #include "gbsbin_fock_conv.h"
 
 namespace gbsbin {
